@@ -2,12 +2,15 @@
 
 Every function here has the name of the C entry point it calls
 (include/fpq.h) and passes torch tensors' device pointers and the current CUDA
-stream.  All arithmetic runs in the library's kernels.  There is no fallback:
-if the shared library is missing the import of a symbol fails.
+stream: the calls a running model makes per layer through a small CPython
+extension (csrc/fpq_torch.cpp), the others through ctypes.  All arithmetic runs
+in the library's kernels.  There is no fallback: if the shared library is
+missing the import of a symbol fails.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -15,6 +18,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _SO = os.path.join(_HERE, "libfpq.so")
+_BINDING = os.path.join(_HERE, "_fpq_torch.so")
 
 OK = 0
 ERR_NULL, ERR_FORMAT, ERR_SHAPE, ERR_ALIGN, ERR_UNSUPPORTED = -1, -2, -3, -4, -5
@@ -165,6 +169,23 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_layers = None
+
+
+def _load_layers():
+    """The CPython extension with the per-layer calls; raises if it has not been built."""
+    global _layers
+    if not os.path.exists(_BINDING):
+        raise FileNotFoundError(
+            f"{_BINDING} is missing: build it with `python -m paper_2408_06995_b200.build` "
+            "(there is no CPU or PyTorch fallback)")
+    spec = importlib.util.spec_from_file_location("_fpq_torch", _BINDING)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    _layers = module
+    return module
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -240,14 +261,14 @@ def fpq_linear_workspace_size(M, N, K, fx: Format, fw: Format) -> int:
 
 
 def fpq_linear(x, w_prepared, w_scale, x_scale, fx: Format, fw: Format, bias, N: int, y=None, workspace=None):
-    assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.dim() == 2
-    M, K = x.shape
     if y is None:
-        y = torch.empty((M, N), dtype=torch.float32, device=x.device)
+        y = torch.empty((x.shape[0], N), dtype=torch.float32, device=x.device)
     if workspace is None:
+        M, K = x.shape
         workspace = torch.empty(max(1, fpq_linear_workspace_size(M, N, K, fx, fw)), dtype=torch.uint8, device=x.device)
-    _check(lib().fpq_linear(_ptr(x), _ptr(w_prepared), _ptr(w_scale), float(x_scale), fx.c(), fw.c(), _ptr(bias),
-                            _ptr(y), M, N, K, _ptr(workspace), workspace.numel(), _stream()), "fpq_linear")
+    code = (_layers or _load_layers()).linear(x, w_prepared, w_scale, x_scale, fx, fw, bias, N, y, workspace)
+    if code:
+        raise FpqError(code, "fpq_linear")
     return y
 
 
@@ -257,18 +278,18 @@ def fpq_conv2d_workspace_size(B, C, H, W, C_out, R, S, pad, stride, fx: Format, 
 
 def fpq_conv2d(x, w_prepared, w_scale, x_scale, fx: Format, fw: Format, bias, C_out, R, S, pad, stride, y=None,
                workspace=None):
-    assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.dim() == 4
-    B, C, H, W = x.shape
-    Ho = (H + 2 * pad - R) // stride + 1
-    Wo = (W + 2 * pad - S) // stride + 1
-    if y is None:
-        y = torch.empty((B, C_out, Ho, Wo), dtype=torch.float32, device=x.device)
-    if workspace is None:
-        workspace = torch.empty(max(1, fpq_conv2d_workspace_size(B, C, H, W, C_out, R, S, pad, stride, fx, fw)),
-                                dtype=torch.uint8, device=x.device)
-    _check(lib().fpq_conv2d(_ptr(x), _ptr(w_prepared), _ptr(w_scale), float(x_scale), fx.c(), fw.c(), _ptr(bias),
-                            _ptr(y), B, C, H, W, C_out, R, S, pad, stride, _ptr(workspace), workspace.numel(),
-                            _stream()), "fpq_conv2d")
+    if y is None or workspace is None:
+        B, C, H, W = x.shape
+        if y is None:
+            y = torch.empty((B, C_out, (H + 2 * pad - R) // stride + 1, (W + 2 * pad - S) // stride + 1),
+                            dtype=torch.float32, device=x.device)
+        if workspace is None:
+            workspace = torch.empty(max(1, fpq_conv2d_workspace_size(B, C, H, W, C_out, R, S, pad, stride, fx, fw)),
+                                    dtype=torch.uint8, device=x.device)
+    code = (_layers or _load_layers()).conv2d(x, w_prepared, w_scale, x_scale, fx, fw, bias, C_out, R, S, pad, stride, y,
+                                              workspace)
+    if code:
+        raise FpqError(code, "fpq_conv2d")
     return y
 
 
@@ -353,12 +374,10 @@ def fpq_conv2d_split_workspace_size(B, C1, C2, H, W, C_out, R, S, pad, stride, f
 def fpq_conv2d_split(x1, x1_scale, x2, x2_scale, w_prepared, w_scale, fx: Format, fw: Format, bias, y, R, S, pad,
                      stride, workspace):
     """Convolution over the channel concatenation of x1 and x2, quantized with their own scales."""
-    B, C1, H, W = x1.shape
-    C2 = x2.shape[1]
-    C_out = y.shape[1]
-    _check(lib().fpq_conv2d_split(_ptr(x1), C1, float(x1_scale), _ptr(x2), C2, float(x2_scale), _ptr(w_prepared),
-                                  _ptr(w_scale), fx.c(), fw.c(), _ptr(bias), _ptr(y), B, H, W, C_out, R, S, pad, stride,
-                                  _ptr(workspace), workspace.numel(), _stream()), "fpq_conv2d_split")
+    code = (_layers or _load_layers()).conv2d_split(x1, x1_scale, x2, x2_scale, w_prepared, w_scale, fx, fw, bias, y, R, S,
+                                                    pad, stride, workspace)
+    if code:
+        raise FpqError(code, "fpq_conv2d_split")
     return y
 
 
