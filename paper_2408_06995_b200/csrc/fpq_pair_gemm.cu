@@ -69,7 +69,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
     float* s_scale = reinterpret_cast<float*>(smem + (bars - smem_base) + 512);   // [n_pad] x_scale * w_scale, then [n_pad] bias
     float* s_bias = s_scale + g.n_pad;
 
-    asm volatile("griddepcontrol.launch_dependents;");
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();

@@ -344,6 +344,7 @@ __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const float* __
                                                                  int64_t Kp, float rinv, uint8_t* __restrict__ codes,
                                                                  int* status)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     bool nan = false;
     int64_t vec_per_row = Kp / 16;
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_e4m3_kernel(const f
     __shared__ __align__(16) uint8_t tile[32][128 + 16];
     // the contraction queued behind this kernel may start its set-up (it waits for this grid
     // to finish before it reads the codes)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     bool nan = false;
     const int HW = H * W, Wp = W + 2 * pad, Hp = H + 2 * pad;
@@ -599,39 +601,24 @@ cudaError_t launch_quantize_rows_e4m3(const float* x, int64_t M, int64_t K, int6
                                       cudaStream_t st, int e5m2)
 {
     int64_t total = M * (Kp / 16);
-    if (e5m2)
-        quantize_rows_e4m3_kernel<false, true><<<grid_for(total, 256), 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, codes,
-                                                                                    status_word());
-    else
-        quantize_rows_e4m3_kernel<false, false><<<grid_for(total, 256), 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, codes,
-                                                                                     status_word());
-    return cudaGetLastError();
+    return launch_overlapped(e5m2 ? quantize_rows_e4m3_kernel<false, true> : quantize_rows_e4m3_kernel<false, false>,
+                             dim3(grid_for(total, 256)), 256, 0, st, x, M, K, Kp, 1.0f / scale, codes, status_word());
 }
 
 cudaError_t launch_quantize_rows_e4m3_twice(const float* x, int64_t M, int64_t K, int64_t Kp, float scale, uint8_t* codes,
                                             cudaStream_t st, int e5m2)
 {
     int64_t total = M * (Kp / 16);
-    if (e5m2)
-        quantize_rows_e4m3_kernel<true, true><<<grid_for(total, 256), 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, codes,
-                                                                                   status_word());
-    else
-        quantize_rows_e4m3_kernel<true, false><<<grid_for(total, 256), 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, codes,
-                                                                                    status_word());
-    return cudaGetLastError();
+    return launch_overlapped(e5m2 ? quantize_rows_e4m3_kernel<true, true> : quantize_rows_e4m3_kernel<true, false>,
+                             dim3(grid_for(total, 256)), 256, 0, st, x, M, K, Kp, 1.0f / scale, codes, status_word());
 }
 
 cudaError_t launch_quantize_nchw_to_nhwc_e4m3(const float* x, int B, int C, int H, int W, int pad, int Cp, int row,
                                               int c_off, float scale, uint8_t* codes, cudaStream_t st, int e5m2)
 {
     dim3 grid((H * W + 31) / 32, (Cp + 127) / 128, B);
-    if (e5m2)
-        quantize_nchw_to_nhwc_e4m3_kernel<true><<<grid, 256, 0, st>>>(x, C, H, W, pad, Cp, row, c_off, 1.0f / scale, codes,
-                                                                      status_word());
-    else
-        quantize_nchw_to_nhwc_e4m3_kernel<false><<<grid, 256, 0, st>>>(x, C, H, W, pad, Cp, row, c_off, 1.0f / scale, codes,
-                                                                       status_word());
-    return cudaGetLastError();
+    return launch_overlapped(e5m2 ? quantize_nchw_to_nhwc_e4m3_kernel<true> : quantize_nchw_to_nhwc_e4m3_kernel<false>, grid, 256,
+                             0, st, x, C, H, W, pad, Cp, row, c_off, 1.0f / scale, codes, status_word());
 }
 
 // ---------------------------------------------------------------------------------
@@ -673,6 +660,7 @@ __global__ void __launch_bounds__(256) quantize_rows_terms_kernel(const float* _
     s1[threadIdx.x] = tab1.t[threadIdx.x];
     s2[threadIdx.x] = tab2.t[threadIdx.x];
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     bool nan = false;
     const int64_t vec_per_row = Kp / 16;
@@ -730,6 +718,7 @@ __global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_terms_kernel(const 
     s1[threadIdx.x] = tab1.t[threadIdx.x];
     s2[threadIdx.x] = tab2.t[threadIdx.x];
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     bool nan = false;
     const int HW = H * W, Wp = W + 2 * pad, Hp = H + 2 * pad;

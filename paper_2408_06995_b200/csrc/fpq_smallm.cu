@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(SMALLM_THREADS) small_m_linear_kernel(const fl
     constexpr int PER = W4 ? 8 : 4;                   // reduction elements per lane and step
     constexpr int STEP = 32 * PER;
     constexpr int U = (MR * PER >= 32) ? 2 : (MR * PER >= 16 ? 4 : 8);     // steps in flight
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     bool nan = false;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row_bytes = W4 ? Kp / 2 : Kp;
@@ -124,8 +125,8 @@ template <bool W4, int MR>
 static void launch_small(int blocks, const float* x, int M, int K, int Kp, const uint8_t* w, int N, const float* w_scale,
                          float x_scale, const float* bias, float* y, cudaStream_t st)
 {
-    small_m_linear_kernel<W4, MR><<<blocks, SMALLM_THREADS, 0, st>>>(x, M, K, Kp, w, N, w_scale, x_scale, 1.0f / x_scale,
-                                                                     bias, y, status_word());
+    (void)launch_overlapped(small_m_linear_kernel<W4, MR>, dim3(blocks), SMALLM_THREADS, 0, st, x, M, K, Kp, w, N, w_scale,
+                            x_scale, 1.0f / x_scale, bias, y, status_word());
 }
 
 fpq_status launch_small_m_linear(const float* x, int M, int K, const void* w_prepared, int w4, int N, const float* w_scale,
