@@ -290,7 +290,7 @@ fpq_status fpq_linear_static(const float* x, const void* w_prepared, const float
  * fpq_prepared_size_split bytes, 128-byte aligned): that copy starts x2's channels at a multiple
  * of 128 so that no 128-wide chunk of the reduction mixes the two scales.
  * workspace: fpq_conv2d_split_workspace_size bytes, 128-byte aligned, scratch.
- * Formats, alignment, errors and stream behaviour as fpq_conv2d (three kernels).
+ * Formats, alignment, errors and stream behaviour as fpq_conv2d (two kernels).
  */
 size_t fpq_prepared_size_split(fpq_format fmt, int32_t N, int32_t C1, int32_t C2, int32_t R, int32_t S);
 fpq_status fpq_prepare_weight_split(const uint8_t* codes, fpq_format fmt, int32_t N, int32_t C1, int32_t C2,

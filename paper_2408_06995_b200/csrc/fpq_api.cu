@@ -1065,10 +1065,8 @@ fpq_status fpq_conv2d_split(const float* x1, int C1, float x1_scale, const float
     // each tensor is quantized with its own scale into its own channel range of the framed
     // channels-last codes; the concatenated FP32 tensor is never formed
     const int e5 = is_e5m2_native(fx) ? 1 : 0;
-    if (launch_quantize_nchw_to_nhwc_e4m3(x1, B, C1, H, W, pad, C1p, (int)row, 0, x1_scale, (uint8_t*)workspace, st, e5) !=
-            cudaSuccess ||
-        launch_quantize_nchw_to_nhwc_e4m3(x2, B, C2, H, W, pad, (int)round_up(C2, 16), (int)row, C1p, x2_scale,
-                                          (uint8_t*)workspace, st, e5) != cudaSuccess)
+    if (launch_quantize_nchw_split(x1, C1, C1p, x1_scale, x2, C2, (int)round_up(C2, 16), x2_scale, B, H, W, pad,
+                                   (uint8_t*)workspace, st, e5) != cudaSuccess)
         return FPQ_ERR_CUDA;
     GemmProblem p{};
     p.conv = 1;
@@ -1097,6 +1095,11 @@ fpq_status fpq_conv2d_split(const float* x1, int C1, float x1_scale, const float
     p.c_seg = C1p / 128;
     p.bias = bias;
     p.y = y;
+    if (g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && pair_gemm_preferred(p)) {
+        const fpq_status sp = launch_pair_gemm(p, st);
+        if (sp != FPQ_ERR_UNSUPPORTED)
+            return sp;
+    }
     return launch_gemm(p, st);
 }
 

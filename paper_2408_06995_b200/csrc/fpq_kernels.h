@@ -17,6 +17,9 @@ cudaError_t launch_quantize_rows_e4m3(const float* x, int64_t M, int64_t K, int6
                                       cudaStream_t st, int e5m2 = 0);
 cudaError_t launch_quantize_nchw_to_nhwc_e4m3(const float* x, int B, int C, int H, int W, int pad, int Cp, int row,
                                               int c_off, float scale, uint8_t* codes, cudaStream_t st, int e5m2 = 0);
+// two tensors with their own scales into one list of pixels, [Cp1 positions of x1 | Cp2 of x2] each
+cudaError_t launch_quantize_nchw_split(const float* x1, int C1, int Cp1, float scale1, const float* x2, int C2, int Cp2,
+                                       float scale2, int B, int H, int W, int pad, uint8_t* codes, cudaStream_t st, int e5m2);
 cudaError_t launch_zero_census(const uint8_t* codes, int64_t n, int four_bit, unsigned long long* count, cudaStream_t st);
 // Code-to-code table of an exact re-encode (weight format -> E4M3), passed to the kernel by value.
 struct CodeTable {

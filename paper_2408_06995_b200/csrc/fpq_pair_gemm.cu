@@ -11,6 +11,9 @@
 // one memory latency whatever its size), warp 1 tensor-memory owner (and, in the pair's first CTA, the
 // MMA issuer for both), warps 2-9 epilogue (tcgen05.ld -> acc * (x_scale * w_scale[n]) + bias[n] -> NCHW).
 // Two accumulators: a unit's epilogue overlaps the next unit's MMAs.  Every wait is bounded; no TMA multicast.
+//
+// A layer whose input is two concatenated tensors with their own scales keeps one accumulator per tensor, joined in the
+// epilogue.
 #include <cuda.h>
 
 #include <mutex>
@@ -31,7 +34,11 @@ constexpr int SMEM_BUDGET = 227 * 1024;
 
 struct PGArgs {
     int64_t M;                 // framed pixels B * Hp * Wp
-    int N, BN;                 // outputs; column tile (128 or 256), BN / 2 weight rows per CTA
+    int N, BN;                 // outputs; column tile (a multiple of 32), BN / 2 weight rows per CTA
+    int seg_chunk;             // two input tensors: chunks from here on belong to the second one (0: one tensor)
+    float x_scale2;
+    double estimate;           // host side only: cycles of the launch
+    int acc_cols, acc_bufs;    // TMEM columns of a unit's accumulator(s); units whose accumulators fit at once (1 or 2)
     int cchunks, taps, S;
     int tgroup, ngroups;       // taps per weight stage, weight stages per chunk
     int Wp, HpWp;
@@ -68,6 +75,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + (bars - smem_base) + 288);
     float* s_scale = reinterpret_cast<float*>(smem + (bars - smem_base) + 512);   // [n_pad] x_scale * w_scale, then [n_pad] bias
     float* s_bias = s_scale + g.n_pad;
+    float* s_scale2 = s_bias + g.n_pad;            // two input tensors: x_scale2 * w_scale[n]
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -144,18 +152,22 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
     } else if (warp == 1) {
         // ---------------- MMA issuer: one thread of the pair's first CTA ----------------
         if (rank == 0 && elect_one()) {
-            uint32_t sa = 0, pa = 0, sb = 0, pb = 0, it = 0;
+            uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
             bool dead = false;
             const uint32_t HI = SMEM_DESC_HI_K_SW128;
             const uint32_t TSTEP = (uint32_t)g.b_tap_bytes >> 4;
             const uint32_t row_wrap8 = (uint32_t)(g.Wp - g.S) * 8u;
-            for (int u = u_lo; u < u_hi && !dead; ++u, ++it) {
-                const uint32_t buf = it & 1, aph = (it >> 1) & 1;
+            uint32_t buf = 0, aph = 0;
+            for (int u = u_lo; u < u_hi && !dead; ++u) {
                 if (!mbar_wait_cluster(acc_empty + 8 * buf, aph ^ 1)) { dead = true; break; }
                 tc_fence_after();
-                const uint32_t d = tmem_base + buf * (uint32_t)g.BN;
+                uint32_t d = tmem_base + buf * (uint32_t)g.acc_cols;
                 bool first = true;
                 for (int cc = 0; cc < g.cchunks && !dead; ++cc) {
+                    if (cc == g.seg_chunk && cc != 0) {
+                        d += (uint32_t)g.BN;                       // the second tensor's accumulator
+                        first = true;
+                    }
                     if (!mbar_wait_cluster(a_full + 8 * sa, pa)) { dead = true; break; }
                     tc_fence_after();
                     const uint32_t abase = smem_desc_lo(a_ring + sa * g.a_stage_bytes);
@@ -189,6 +201,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
                 if (dead)
                     break;
                 mma_commit_pair(acc_full + 8 * buf, 3);
+                if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
             }
             if (dead)
                 flag_status(g.status, FPQ_ERR_TIMEOUT);
@@ -202,15 +215,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
         for (int i = threadIdx.x - 32 * EPI_W0; i < g.n_pad; i += 32 * NUM_EPI) {
             s_scale[i] = (i < g.N) ? g.x_scale * __ldg(g.w_scale + i) : 0.f;
             s_bias[i] = (g.bias && i < g.N) ? __ldg(g.bias + i) : 0.f;
+            if (g.seg_chunk)
+                s_scale2[i] = (i < g.N) ? g.x_scale2 * __ldg(g.w_scale + i) : 0.f;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * NUM_EPI) : "memory");
-        uint32_t it = 0;
+        uint32_t buf = 0, aph = 0;
         bool dead = false;
-        for (int u = u_lo; u < u_hi && !dead; ++u, ++it) {
+        for (int u = u_lo; u < u_hi && !dead; ++u) {
             int mu, nt;
             decode(u, mu, nt);
             const int mt = 2 * mu + (int)rank;
-            const uint32_t buf = it & 1, aph = (it >> 1) & 1;
             const uint32_t q = (uint32_t)mt * BM + row;
             const uint32_t b = fdiv(q, g.div_HpWp);
             const uint32_t rem = q - b * (uint32_t)g.HpWp;
@@ -220,10 +234,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
             float* yrow = g.y + ((int64_t)b * g.N * g.Ho + oy) * g.Wo + ox;
             if (!mbar_wait(acc_full + 8 * buf, aph)) { dead = true; break; }
             tc_fence_after();
-            const int ncol0 = half * BNh;                          // first column of this warp within the tile
-            const uint32_t t_addr = tmem_base + buf * (uint32_t)g.BN + (uint32_t)ncol0 + ((uint32_t)(quarter * 32) << 16);
-            for (int c = 0; c < BNh; c += 32) {
-                const int nb = nt * g.BN + ncol0 + c;              // output channel of the chunk's first column
+            const uint32_t t_addr = tmem_base + buf * (uint32_t)g.acc_cols + ((uint32_t)(quarter * 32) << 16);
+            for (int c = 32 * half; c < g.BN; c += 64) {           // (every second 32 columns of the tile)
+                const int nb = nt * g.BN + c;                      // output channel of the chunk's first column
                 if (nb >= g.N)
                     break;
                 uint32_t r[32];
@@ -238,6 +251,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
                     r[4 * k + 1] = __float_as_uint(fmaf(__uint_as_float(r[4 * k + 1]), sv.y, bv.y));
                     r[4 * k + 2] = __float_as_uint(fmaf(__uint_as_float(r[4 * k + 2]), sv.z, bv.z));
                     r[4 * k + 3] = __float_as_uint(fmaf(__uint_as_float(r[4 * k + 3]), sv.w, bv.w));
+                }
+                if (g.seg_chunk) {
+                    uint32_t r2[32];
+                    tmem_ld32(t_addr + g.BN + c, r2);
+                    tmem_ld_wait();
+                    const float4* t4 = reinterpret_cast<const float4*>(s_scale2 + nb);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 tv = t4[k];
+                        r[4 * k + 0] = __float_as_uint(fmaf(__uint_as_float(r2[4 * k + 0]), tv.x, __uint_as_float(r[4 * k + 0])));
+                        r[4 * k + 1] = __float_as_uint(fmaf(__uint_as_float(r2[4 * k + 1]), tv.y, __uint_as_float(r[4 * k + 1])));
+                        r[4 * k + 2] = __float_as_uint(fmaf(__uint_as_float(r2[4 * k + 2]), tv.z, __uint_as_float(r[4 * k + 2])));
+                        r[4 * k + 3] = __float_as_uint(fmaf(__uint_as_float(r2[4 * k + 3]), tv.w, __uint_as_float(r[4 * k + 3])));
+                    }
                 }
                 if (row_valid) {
                     float* dst = yrow + (int64_t)nb * nstride;
@@ -257,6 +284,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
             __syncwarp();
             if (lane == 0)
                 mbar_arrive_cluster(racc_empty + 8 * buf);
+            if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
         }
         if (dead)
             flag_status(g.status, FPQ_ERR_TIMEOUT);
@@ -271,17 +299,45 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
     }
 }
 
+// Column tile of a layer: the one with the shortest estimate, in SM cycles.  A chunk of the reduction takes its MMAs
+// (0.53 cycles per column and 32 reduction elements, 52 at least) or the arrival of its operands (some 43 bytes per clock
+// and SM); an epilogue stores some 15 bytes per clock and SM and is hidden behind the next unit's MMAs, except the last
+// one's.  A width that just fits the columns and the SM pairs beats the widest one: 640 -> 320 channels at 64 x 64, batch
+// 2, whole layer: 35 units x 3 tiles of 128 in two rounds 24.1 us, x 2 of 160 in one 19.3 us; 256 -> 256 at 32 x 32,
+// batch 16: 15.5 us with 128, 18.6 us with 64 or 192.
+int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_bytes, int accs, double* cycles)
+{
+    int pick = 128;
+    double best = 0.0;
+    for (int bn = 64; bn <= 256; bn += 32) {
+        if (bn - 32 >= N)
+            break;
+        const int64_t units = (int64_t)m_units * ((N + bn - 1) / bn);
+        const double waves = (double)((units + nclusters - 1) / nclusters);
+        const double mmas = taps * 4 * (bn * 0.53 > 52.0 ? bn * 0.53 : 52.0);
+        const double fill = (taps * bn * 64.0 + a_bytes) / 43.0;
+        const double unit = 800.0 + cchunks * (mmas > fill ? mmas : fill), epi = 128.0 * bn * 4 / 15;
+        const bool hidden = 2 * bn * accs <= 512;
+        const double cost = hidden ? waves * (waves > 1 && epi > unit ? epi : unit) + epi : waves * (unit + epi);
+        if (best == 0.0 || cost < best) {
+            best = cost;
+            pick = bn;
+        }
+    }
+    *cycles = best;
+    return pick;
+}
+
 // geometry and shared-memory plan; FPQ_ERR_UNSUPPORTED outside the kernel's range
 fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
 {
-    if (!p.conv || p.x != nullptr || p.stride != 1 || p.c_seg != 0 || p.N < 1 || p.R * p.S > 64)
+    if (!p.conv || p.x != nullptr || p.stride != 1 || p.N < 1 || p.R * p.S > 64)
         return FPQ_ERR_UNSUPPORTED;
     const int Hp = p.H + 2 * p.pad, Wp = p.W + 2 * p.pad;
     const int64_t framed = (int64_t)p.B * Hp * Wp;
     const int halo_rows = BM + (p.R - 1) * Wp + (p.S - 1);
     const int64_t flat_tiles = (framed + BM - 1) / BM;
-    const int64_t exact_tiles = ((int64_t)p.B * p.Ho * p.Wo + BM - 1) / BM;
-    if (halo_rows > 2 * 256 - 16 || flat_tiles * 4 > exact_tiles * 5 + 4 || framed >= 0x7fffff00ll)
+    if (halo_rows > 2 * 256 - 16 || framed >= 0x7fffff00ll)
         return FPQ_ERR_UNSUPPORTED;
     g = PGArgs{};
     g.M = framed;
@@ -299,9 +355,13 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
     g.m_tiles = (int)flat_tiles;
     const int m_units = (g.m_tiles + 1) / 2;
     const int nclusters = nsm / 2;
-    // 256-wide column tiles halve the weight traffic per MMA, but a cluster needs at least two units for its
-    // epilogue to overlap the next unit's MMAs
-    g.BN = (p.N > 128 && (int64_t)m_units * ((p.N + 255) / 256) >= 2ll * nclusters) ? 256 : 128;
+    g.seg_chunk = p.c_seg;
+    g.x_scale2 = p.x_scale2;
+    const int accs = p.c_seg ? 2 : 1;
+    const int a_bytes = (int)round_up(halo_rows, 8) * 128;
+    g.BN = choose_tile(p.N, m_units, nclusters, g.cchunks, g.taps, a_bytes, accs, &g.estimate);
+    g.acc_cols = g.BN * accs;
+    g.acc_bufs = 2 * g.acc_cols <= 512 ? 2 : 1;
     g.n_tiles = (p.N + g.BN - 1) / g.BN;
     g.div_nt = make_fastdiv((uint32_t)g.n_tiles);
     g.units = m_units * g.n_tiles;
@@ -315,7 +375,7 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
     g.n_pad = g.n_tiles * g.BN;
     if (g.n_pad * 8 > 32 * 1024)
         return FPQ_ERR_UNSUPPORTED;
-    const int ctl = 512 + 1024 + g.n_pad * 8;
+    const int ctl = 512 + 1024 + g.n_pad * 4 * (1 + accs);
     g.a_stages = 2;
     g.b_stages = (SMEM_BUDGET - ctl - g.a_stages * g.a_stage_bytes) / g.b_stage_bytes;
     if (g.b_stages > 8)
@@ -330,7 +390,9 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
             g.b_stages = 8;
     }
     g.idesc = idesc_f8f6f4_pair(p.a_e5m2 ? 1u : 0u, p.w4 ? 5u : (p.w_e5m2 ? 1u : 0u), (uint32_t)g.BN);
-    g.tmem_cols = 2u * (uint32_t)g.BN;
+    g.tmem_cols = 32;
+    while ((int)g.tmem_cols < g.acc_bufs * g.acc_cols)
+        g.tmem_cols *= 2;
     g.wait_prior_grid = p.after_stage1;
     *dyn_bytes = ctl + g.a_stages * g.a_stage_bytes + g.b_stages * g.b_stage_bytes;
     return FPQ_OK;
@@ -338,15 +400,49 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
 
 }  // namespace
 
-// The layers this kernel is meant for: enough units to fill the GPU's SM pairs and a reduction long enough for the
-// tensor cores to be the bound (measured on B200 against the general contraction).
+// Whether this kernel is expected to be faster than the general contraction.
 bool pair_gemm_preferred(const GemmProblem& p)
 {
     PGArgs g;
     int dyn = 0;
-    if (plan_pg(p, 148, g, &dyn) != FPQ_OK)
+    constexpr int SMS = 148;
+    if (plan_pg(p, SMS, g, &dyn) != FPQ_OK)
         return false;
-    return g.units >= 60 && g.cchunks * g.taps >= 12;
+    const int blocks = g.cchunks * g.taps;
+    // one tap: both kernels are bound by their epilogues and the fetch of the activations; the pairs win where they get
+    // through in one round (320 channels at 64 x 64, batch 2: 10.0 against 11.0 us; 960 -> 320: 15.1 against 17.1) and
+    // lose in several (1024 -> 1024 at 32 x 32, batch 16: 48.6 against 43.9) or to a split reduction (2560 -> 1280 at
+    // 16 x 16: 14.5 against 12.4)
+    if (g.taps < 4)
+        return p.N > 64 && g.units >= 40 && g.units <= SMS / 2 && blocks >= 3 && blocks <= 12;
+    // otherwise against an estimate of the general one: 128 x 128 tiles whose blocks of 128 reduction elements take some
+    // 520 cycles each, the reduction split over clusters when the tiles leave SMs idle.  (1280 channels at 16 x 16, batch
+    // 2: 17.1 against 20.3 us; batch 1: 16.6 against 15.0; 256 channels at 16 x 16: 8.0 against 11.1; 1280 -> 128 at
+    // 32 x 32: 17.7 against 14.2.)
+    // (where the frame is much of the image it tiles the image itself, in powers of two, and loads every tap apart:
+    // 416 -> 608 channels at 11 x 11, batch 50: 49.8 us so, 24.3 us on pairs with the framed pixels)
+    int64_t m_tiles = g.m_tiles;
+    double block = 520.0;
+    if (m_tiles * 4 > ((int64_t)p.B * p.Ho * p.Wo + BM - 1) / BM * 5 + 4) {
+        int wt = 1, ht = 1;
+        while (wt < p.Wo && wt < BM) wt *= 2;
+        while (ht < p.Ho && ht < BM / wt) ht *= 2;
+        const int bt = BM / (wt * ht);
+        m_tiles = (int64_t)((p.Wo + wt - 1) / wt) * ((p.Ho + ht - 1) / ht) * ((p.B + bt - 1) / bt);
+        block = 700.0;
+    }
+    if (p.N <= 64)
+        block *= 0.65;         // (its column tile is 64 wide there)
+    const int64_t tiles = m_tiles * ((p.N + 127) / 128);
+    double general;
+    if (2 * tiles <= SMS && g.cchunks >= 2) {
+        int64_t sp = SMS / tiles < 8 ? SMS / tiles : 8;
+        if (sp > g.cchunks) sp = g.cchunks;
+        general = block * (double)((g.cchunks + sp - 1) / sp) * g.taps + 2000.0;
+    } else {
+        general = block * (double)((tiles + SMS - 1) / SMS) * blocks;
+    }
+    return g.estimate <= general + 4300.0;
 }
 
 fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)

@@ -391,11 +391,17 @@ __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const float* __
 // shared memory: loads are coalesced along pixels (16 in flight per thread), stores
 // are whole 128-byte channel rows.  The blocks also share out the frame pixels.
 // ---------------------------------------------------------------------------------
+// Two input tensors of a layer go in one launch, blockIdx.y counting the first one's 128-channel groups, then the second's
+// (640 + 320 channels at 64 x 64, batch 2: 9.2 us, two launches 11.8).
+struct NchwSource {
+    const float* x;
+    float rinv;
+    int C, Cp, c_off;          // channels; channels to fill; first position in a pixel's row
+};
 template <bool E5>
-__global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_e4m3_kernel(const float* __restrict__ x, int C, int H,
-                                                                         int W, int pad, int Cp, int row, int c_off,
-                                                                         float rinv, uint8_t* __restrict__ codes,
-                                                                         int* status)
+__global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_e4m3_kernel(const NchwSource first, const NchwSource second,
+                                                                         int groups1, int H, int W, int pad, int row,
+                                                                         uint8_t* __restrict__ codes, int* status)
 {
     __shared__ __align__(16) uint8_t tile[32][128 + 16];
     // the contraction queued behind this kernel may start its set-up (it waits for this grid
@@ -405,7 +411,11 @@ __global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_e4m3_kernel(const f
     bool nan = false;
     const int HW = H * W, Wp = W + 2 * pad, Hp = H + 2 * pad;
     const int b = blockIdx.z;
-    const int c0 = blockIdx.y * 128;
+    const bool one = (int)blockIdx.y < groups1;
+    const float* x = one ? first.x : second.x;
+    const float rinv = one ? first.rinv : second.rinv;
+    const int C = one ? first.C : second.C, Cp = one ? first.Cp : second.Cp, c_off = one ? first.c_off : second.c_off;
+    const int c0 = ((int)blockIdx.y - (one ? 0 : groups1)) * 128;
     const int p0 = blockIdx.x * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 pixels x 8 channel groups of 16
     const float* xb = x + (int64_t)b * C * HW;
@@ -613,12 +623,26 @@ cudaError_t launch_quantize_rows_e4m3_twice(const float* x, int64_t M, int64_t K
                              dim3(grid_for(total, 256)), 256, 0, st, x, M, K, Kp, 1.0f / scale, codes, status_word());
 }
 
+static cudaError_t launch_nchw(const NchwSource& first, const NchwSource& second, int B, int H, int W, int pad, int row,
+                               uint8_t* codes, cudaStream_t st, int e5m2)
+{
+    const int groups1 = (first.Cp + 127) / 128, groups2 = (second.Cp + 127) / 128;
+    return launch_overlapped(e5m2 ? quantize_nchw_to_nhwc_e4m3_kernel<true> : quantize_nchw_to_nhwc_e4m3_kernel<false>,
+                             dim3((H * W + 31) / 32, groups1 + groups2, B), 256, 0, st, first, second, groups1, H, W, pad, row,
+                             codes, status_word());
+}
+
 cudaError_t launch_quantize_nchw_to_nhwc_e4m3(const float* x, int B, int C, int H, int W, int pad, int Cp, int row,
                                               int c_off, float scale, uint8_t* codes, cudaStream_t st, int e5m2)
 {
-    dim3 grid((H * W + 31) / 32, (Cp + 127) / 128, B);
-    return launch_overlapped(e5m2 ? quantize_nchw_to_nhwc_e4m3_kernel<true> : quantize_nchw_to_nhwc_e4m3_kernel<false>, grid, 256,
-                             0, st, x, C, H, W, pad, Cp, row, c_off, 1.0f / scale, codes, status_word());
+    return launch_nchw({x, 1.0f / scale, C, Cp, c_off}, {x, 0.f, 0, 0, 0}, B, H, W, pad, row, codes, st, e5m2);
+}
+
+cudaError_t launch_quantize_nchw_split(const float* x1, int C1, int Cp1, float scale1, const float* x2, int C2, int Cp2,
+                                       float scale2, int B, int H, int W, int pad, uint8_t* codes, cudaStream_t st, int e5m2)
+{
+    return launch_nchw({x1, 1.0f / scale1, C1, Cp1, 0}, {x2, 1.0f / scale2, C2, Cp2, Cp1}, B, H, W, pad, Cp1 + Cp2, codes, st,
+                       e5m2);
 }
 
 // ---------------------------------------------------------------------------------

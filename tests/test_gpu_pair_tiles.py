@@ -1,0 +1,71 @@
+"""Convolutions on CTA pairs with column tiles of every width the library picks (64 .. 256 in steps of 32, a last tile of
+less), one and two input tensors, one and two accumulators in tensor memory, and frames that are much of the image:
+against the general contraction, whose products and order of additions are the same, bit for bit where it does not split
+the reduction over a cluster, else within the rounding of the FP32 sums; and against the CPU oracle at one size."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2408_06995_b200 as fpq
+from paper_2408_06995_b200 import inputs as I
+from _helpers import assert_close, gpu_layer, layer_scales, oracle_layer, sample_indices
+
+pytestmark = pytest.mark.gpu
+
+
+def _both(call):
+    try:
+        fpq.fpq_set_path_policy(fpq.PATH_TWO_KERNELS_NARROW)
+        want = call().clone()
+        fpq.fpq_set_path_policy(fpq.PATH_TWO_KERNELS)
+        got = call().clone()
+    finally:
+        fpq.fpq_set_path_policy(fpq.PATH_AUTO)
+    assert fpq.fpq_read_status() == fpq.OK
+    # FP32 sums of at most 2^15 exact products in another order: 2^15 * 2^-24 of the sum of magnitudes at worst, a
+    # hundredth of that in practice; outputs here are sums of K terms of random sign, so relative to the largest one
+    assert float((got - want).abs().max()) <= 2e-5 * float(want.abs().max())
+
+
+def _weights(gen, Co, K, fw):
+    w = torch.randn(Co, K, generator=gen, device="cuda") * 0.05
+    scale = (w.abs().amax(dim=1) / fpq.fpq_format_max(fw)).contiguous()
+    return fpq.fpq_quantize_weight(w, scale, fw), scale
+
+
+@pytest.mark.parametrize("B,C,H,W,Co", [(2, 320, 64, 64, 320), (2, 640, 32, 32, 640), (64, 192, 32, 32, 192), (8, 512, 32, 32, 512),
+                                        (3, 320, 45, 45, 324), (5, 136, 30, 17, 100), (50, 416, 11, 11, 608), (2, 192, 7, 5, 288),
+                                        (1, 256, 13, 96, 70), (16, 256, 32, 32, 256)])
+@pytest.mark.parametrize("fw", [fpq.E4M3, fpq.E2M1])
+def test_one_tensor(B, C, H, W, Co, fw):
+    gen = torch.Generator(device="cuda").manual_seed(C + Co)
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda")
+    codes, scale = _weights(gen, Co, C * 9, fw)
+    prep = fpq.fpq_prepare_weight(codes, fw, fpq.CONV2D, Co, C, 3, 3)
+    bias = torch.randn(Co, generator=gen, device="cuda")
+    _both(lambda: fpq.fpq_conv2d(x, prep, scale, 0.01, fpq.E4M3, fw, bias, Co, 3, 3, 1, 1))
+
+
+@pytest.mark.parametrize("B,C1,C2,res,Co,R", [(2, 640, 320, 64, 320, 3), (2, 640, 320, 32, 640, 3), (2, 1280, 640, 16, 1280, 3),
+                                              (4, 100, 7, 33, 250, 3), (3, 128, 300, 9, 96, 3), (2, 320, 640, 64, 320, 1)])
+def test_two_tensors(B, C1, C2, res, Co, R):
+    fw = fpq.E2M1
+    gen = torch.Generator(device="cuda").manual_seed(C1 + C2)
+    x1 = torch.randn(B, C1, res, res, generator=gen, device="cuda")
+    x2 = torch.randn(B, C2, res, res, generator=gen, device="cuda") * 3
+    codes, scale = _weights(gen, Co, (C1 + C2) * R * R, fw)
+    prep = fpq.fpq_prepare_weight_split(codes, fw, Co, C1, C2, R, R)
+    bias = torch.randn(Co, generator=gen, device="cuda")
+    y = torch.empty(B, Co, res, res, device="cuda")
+    ws = torch.empty(fpq.fpq_conv2d_split_workspace_size(B, C1, C2, res, res, Co, R, R, R // 2, 1, fpq.E4M3, fw),
+                     dtype=torch.uint8, device="cuda")
+    _both(lambda: fpq.fpq_conv2d_split(x1, 0.01, x2, 0.03, prep, scale, fpq.E4M3, fw, bias, y, R, R, R // 2, 1, ws))
+
+
+def test_small_frame_against_the_oracle():
+    L = I.draw(I.conv_layer("frame", 9, 150, 7, 9, 104, 3, wfmt="e2m1", rounding=True), 21, 0, "silu", 0.03, True)
+    ws, xs = layer_scales(L)
+    y = gpu_layer(L, ws, xs).reshape(-1)
+    idx = sample_indices(y.size, 20000, 5)
+    yr, ab = oracle_layer(L, ws, xs, idx)
+    assert_close(y[idx], np.asarray(yr), np.asarray(ab))
