@@ -5,11 +5,12 @@
 // FMA contractions on the CUDA cores (register-tiled, 128 x 128 x 16 tiles), not reduced-precision
 // tensor-core products.
 //
-//   soft_weight_kernel      E = Wq(alpha) - W and dWq/dalpha per weight; sum of lambda
+//   prepare_kernel          E = Wq(alpha) - W and dWq/dalpha per weight; A^T for the tensor-core routes
 //   sgemm128<true>          D = A E^T            (= Yq - Y by linearity), sum of D^2; with few output tiles the
 //                           reduction is cut into slices that reduce_d_kernel adds
 //   sgemm128<false>         partial sums of D^T A over slices of the M rows
-//   grad_finalize_kernel    slices added in a fixed order, chain rule, optional descent update
+//   grad_finalize_kernel    slices added in a fixed order, chain rule, sum of lambda, optional descent update
+// With many calibration rows D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are fewer products: see gram_preferred.
 //   harden_kernel           the inference rule: decision bit = (sigma(alpha) >= 0.5)
 //   unfold_kernel           a convolution's input rows, so that the same step serves convolution weights
 #include <math.h>
@@ -84,45 +85,77 @@ __device__ __forceinline__ void block_atomic_add(double v, double* dst)
     }
 }
 
-// Learned-rounding equation of Sec. V-B with the sigmoid kept soft.  One thread per weight.
-__global__ void __launch_bounds__(256) soft_weight_kernel(const float* __restrict__ w, const float* __restrict__ scale,
-                                                          QFormat f, const float* __restrict__ alpha,
-                                                          float* __restrict__ E, float* __restrict__ DQ,
-                                                          double* __restrict__ reg_sum, int64_t N, int64_t K,
-                                                          int* __restrict__ status)
+// Learned-rounding equation of Sec. V-B with the sigmoid kept soft, for one weight.
+struct SoftWeight {
+    float e, dq;               // Wq(alpha) - w, dWq/dalpha
+};
+__device__ __forceinline__ SoftWeight soft_weight(float wv, float al, float g, float r, float c, const QFormat& f, bool& nan)
 {
-    int64_t total = N * K;
-    float lam_acc = 0.f;
-    const float c = __uint_as_float(f.cmax_bits);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t n = i / K;
-        float g = __ldg(scale + n);
-        float r = __fdiv_rn(1.0f, g);
-        float wv = __ldg(w + i);
-        float t = __fmul_rn(wv, r);
-        float al = __ldg(alpha + i);
-        SoftTerms st = soft_terms(al);
-        float sig = st.sig, u = st.u;
-        float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
-        lam_acc += 1.0f - u16 * u4;
-        if (t != t) {
-            E[i] = 0.f;
-            DQ[i] = 0.f;
-            flag_status(status, FPQ_ERR_NAN_INPUT);
-            continue;
-        }
-        float a = fminf(fmaxf(t, -c), c);
-        int Eb = (int)((__float_as_uint(a) >> 23) & 0xffu);
-        int e_eff = max(Eb - 127, 1 - f.B);                               // binade whose step applies
-        float s = __uint_as_float((uint32_t)(e_eff - f.m + 127) << 23);     // step, a power of two
-        float s_inv = __uint_as_float((uint32_t)(f.m - e_eff + 127) << 23);
-        float fl = floorf(a * s_inv);                                       // exact: power-of-two scaling
-        float pre = s * (fl + sig);
-        float q = fminf(fmaxf(pre, -c), c);
-        E[i] = fmaf(g, q, -wv);
-        DQ[i] = (pre >= -c && pre <= c) ? g * s * st.sp : 0.f;
+    const float t = __fmul_rn(wv, r);
+    if (t != t) {
+        nan = true;
+        return {0.f, 0.f};
     }
-    block_atomic_add((double)lam_acc, reg_sum);
+    const SoftTerms st = soft_terms(al);
+    const float a = fminf(fmaxf(t, -c), c);
+    const int Eb = (int)((__float_as_uint(a) >> 23) & 0xffu);
+    const int e_eff = max(Eb - 127, 1 - f.B);                                 // binade whose step applies
+    const float s = __uint_as_float((uint32_t)(e_eff - f.m + 127) << 23);     // step, a power of two
+    const float s_inv = __uint_as_float((uint32_t)(f.m - e_eff + 127) << 23);
+    const float fl = floorf(a * s_inv);                                       // exact: power-of-two scaling
+    const float pre = s * (fl + st.sig);
+    const float q = fminf(fmaxf(pre, -c), c);
+    return {fmaf(g, q, -wv), (pre >= -c && pre <= c) ? g * s * st.sp : 0.f};
+}
+
+// The first blocks: E and dWq/dalpha, four weights per thread (VEC, rows of a multiple of four) or one; block 0 empties
+// the losses.  The others, where A is transposed: one 32 x 32 tile of A^T each.  One launch: both are short.
+template <bool VEC>
+__global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ w, const float* __restrict__ scale, QFormat f,
+                                                      const float* __restrict__ alpha, float* __restrict__ E,
+                                                      float* __restrict__ DQ, double* __restrict__ loss, int64_t N, int64_t K,
+                                                      int weight_blocks, const float* __restrict__ A, int64_t M,
+                                                      float* __restrict__ AT, int64_t Mp, int* __restrict__ status)
+{
+    __shared__ float tile[32][33];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if ((int)blockIdx.x >= weight_blocks) {
+        const int64_t tiles_k = (K + 31) / 32, id = (int64_t)blockIdx.x - weight_blocks;
+        const int64_t m0 = id / tiles_k * 32, k0 = (id - id / tiles_k * tiles_k) * 32;
+        const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+        for (int r = ty; r < 32; r += 8)
+            tile[r][tx] = (m0 + r < M && k0 + tx < K) ? A[(m0 + r) * K + k0 + tx] : 0.f;
+        __syncthreads();
+#pragma unroll
+        for (int r = ty; r < 32; r += 8)
+            if (k0 + r < K && m0 + tx < M)
+                AT[(k0 + r) * Mp + m0 + tx] = tile[tx][r];
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 2)
+        loss[threadIdx.x] = 0.0;
+    constexpr int V = VEC ? 4 : 1;
+    const float c = __uint_as_float(f.cmax_bits);
+    const int64_t per_row = K / V, total = N * per_row;
+    bool nan = false;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (int64_t)weight_blocks * 256) {
+        const int64_t n = total < 0x80000000ll ? (int64_t)((uint32_t)i / (uint32_t)per_row) : i / per_row;
+        const float g = __ldg(scale + n), r = __fdiv_rn(1.0f, g);
+        if (VEC) {
+            const float4 wv = __ldg(reinterpret_cast<const float4*>(w) + i), al = __ldg(reinterpret_cast<const float4*>(alpha) + i);
+            const SoftWeight o0 = soft_weight(wv.x, al.x, g, r, c, f, nan), o1 = soft_weight(wv.y, al.y, g, r, c, f, nan),
+                             o2 = soft_weight(wv.z, al.z, g, r, c, f, nan), o3 = soft_weight(wv.w, al.w, g, r, c, f, nan);
+            reinterpret_cast<float4*>(E)[i] = make_float4(o0.e, o1.e, o2.e, o3.e);
+            reinterpret_cast<float4*>(DQ)[i] = make_float4(o0.dq, o1.dq, o2.dq, o3.dq);
+        } else {
+            const SoftWeight o = soft_weight(__ldg(w + i), __ldg(alpha + i), g, r, c, f, nan);
+            E[i] = o.e;
+            DQ[i] = o.dq;
+        }
+    }
+    if (nan)
+        flag_status(status, FPQ_ERR_NAN_INPUT);
 }
 
 // C[i][j] = sum_r P(i, r) Q(j, r) over r in [z * r_per_split, min(R, (z + 1) * r_per_split)), z = blockIdx.z,
@@ -137,6 +170,7 @@ __global__ void __launch_bounds__(256, 2) sgemm128(const float* __restrict__ P, 
 {
     __shared__ __align__(16) float Ps[2][BK][LDS];
     __shared__ __align__(16) float Qs[2][BK][LDS];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const int t = threadIdx.x;
     const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
@@ -287,28 +321,101 @@ __global__ void __launch_bounds__(256, 2) sgemm128(const float* __restrict__ P, 
 }
 
 // grad = (2 / (M N)) (sum of the slices of D^T A) * dWq/dalpha + reg * dlambda/dalpha; alpha -= lr * grad when
-// lr != 0.  Thread 0 of block 0 turns the sum of squares into the mean.
+// lr != 0; sum of lambda.  E == NULL: thread 0 of block 0 turns the sum of squares into the mean; otherwise the mean is
+// <D^T A, E> / (M N), as sum D^2 = sum D (A E^T).
+// VEC: four weights per thread.  Few blocks, each ending in two atomics: those of a thousand blocks took longer than the
+// rest (7.7 us for 960 x 320 weights).
+template <bool VEC>
 __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restrict__ GP, int splits,
-                                                            const float* __restrict__ DQ, float* __restrict__ alpha,
-                                                            float* __restrict__ grad, double* __restrict__ loss,
-                                                            int64_t total, float coef, double inv_mn, float reg, float lr)
+                                                            const float* __restrict__ DQ, const float* __restrict__ E,
+                                                            float* __restrict__ alpha, float* __restrict__ grad,
+                                                            double* __restrict__ loss, int64_t total, float coef,
+                                                            double inv_mn, float reg, float lr)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    constexpr int V = VEC ? 4 : 1;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!E && blockIdx.x == 0 && threadIdx.x == 0)
         loss[0] *= inv_mn;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        float g = 0.f;
-        for (int z = 0; z < splits; ++z)
-            g += GP[(int64_t)z * total + i];
-        float al = alpha[i];
-        SoftTerms st = soft_terms(al);
-        float u = st.u;
-        float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
-        float u19 = u16 * u2 * u;
-        float dlam = -40.0f * u19 * (al > 0.f ? 1.f : (al < 0.f ? -1.f : 0.f)) * st.sp;
-        float gr = fmaf(coef * g, DQ[i], reg * dlam);
-        grad[i] = gr;
+    float lam = 0.f;
+    double sq = 0.0;
+    auto load = [](const float* p, float (&v)[V]) {
+        if (VEC) {
+            const float4 t = *reinterpret_cast<const float4*>(p);
+            v[0] = t.x, v[V > 1 ? 1 : 0] = t.y, v[V > 2 ? 2 : 0] = t.z, v[V > 3 ? 3 : 0] = t.w;
+        } else {
+            v[0] = *p;
+        }
+    };
+    auto store = [](float* p, const float (&v)[V]) {
+        if (VEC)
+            *reinterpret_cast<float4*>(p) = make_float4(v[0], v[V > 1 ? 1 : 0], v[V > 2 ? 2 : 0], v[V > 3 ? 3 : 0]);
+        else
+            *p = v[0];
+    };
+    for (int64_t i = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < total; i += V * ((int64_t)gridDim.x * blockDim.x)) {
+        float g[V] = {}, dq[V], al[V], gr[V], e[V];
+        load(DQ + i, dq);
+        load(alpha + i, al);
+        if (E)
+            load(E + i, e);
+#pragma unroll 4
+        for (int z = 0; z < splits; ++z) {
+            float t[V];
+            load(GP + (int64_t)z * total + i, t);
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                g[v] += t[v];
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            if (E)
+                sq = fma((double)g[v], (double)e[v], sq);
+            const SoftTerms st = soft_terms(al[v]);
+            const float u = st.u;
+            const float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
+            lam += 1.0f - u16 * u4;
+            const float u19 = u16 * u2 * u;
+            const float dlam = -40.0f * u19 * (al[v] > 0.f ? 1.f : (al[v] < 0.f ? -1.f : 0.f)) * st.sp;
+            gr[v] = fmaf(coef * g[v], dq[v], reg * dlam);
+            al[v] = al[v] - lr * gr[v];
+        }
+        store(grad + i, gr);
         if (lr != 0.f)
-            alpha[i] = al - lr * gr;
+            store(alpha + i, al);
+    }
+    block_atomic_add((double)lam, loss + 1);
+    if (E) {
+        __syncthreads();                               // (the helper's shared memory is used again)
+        block_atomic_add(sq * inv_mn, loss);
+    }
+}
+
+// S = sum of the slices of A^T A [K][K] (fixed order; the sums in double).  Eight threads share four floats, each adding
+// every eighth slice: a whole wave of loads is in flight at once.
+__global__ void __launch_bounds__(256) reduce_gram_kernel(const float4* __restrict__ SP, int splits, float4* __restrict__ S,
+                                                          int64_t total4)
+{
+    __shared__ double4 part[8][32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    double4 t = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (i < total4) {
+#pragma unroll 8
+        for (int k = group; k < splits; k += 8) {
+            const float4 v = SP[(int64_t)k * total4 + i];
+            t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+        }
+    }
+    part[group][lane] = t;
+    __syncthreads();
+    if (group == 0 && i < total4) {
+#pragma unroll
+        for (int k = 1; k < 8; ++k) {
+            const double4 v = part[k][lane];
+            t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+        }
+        S[i] = make_float4((float)t.x, (float)t.y, (float)t.z, (float)t.w);
     }
 }
 
@@ -316,6 +423,7 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
 __global__ void __launch_bounds__(256) reduce_d_kernel(const float* __restrict__ DP, int splits, float* __restrict__ D,
                                                        int64_t total, int64_t N, int64_t N4, double* __restrict__ sq_sum)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     float sq = 0.f;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         if (i % N4 >= N)
@@ -386,7 +494,19 @@ struct Plan {
     int kb_per_split_tc, splits_tc;
     int kb_per_split1_tc, splits1_tc;       // first contraction: sliced too when it has few output tiles
     size_t off_AT, off_DT;
+    // with A^T A: slices of M in it, slices of its K rows in the product with E
+    int gram, tc_s, tc_g, splits_s, splits_g;      // tc_*: on the tensor cores (slices in 32-wide blocks), else FP32 multiply-adds
+    int64_t per_s, per_g;                          // 32-wide blocks or elements per slice
+    size_t off_SP, off_S;
 };
+
+// E (A^T A) in place of (A E^T)^T A: M K^2 + N K^2 products instead of 2 M N K (calibration rows: QKV 320 -> 960 with
+// 4096 rows 0.5 G instead of 2.5 G).  Only with clearly more rows than columns: A^T A is then well away from singular, and
+// the mean square, <E (A^T A), E>, keeps its relative accuracy.
+bool gram_preferred(int64_t M, int64_t N, int64_t K)
+{
+    return K % 4 == 0 && M >= 2 * K && (double)K * (double)(M + N) * 1.25 <= 2.0 * (double)M * (double)N;
+}
 
 // As many slices of a reduction of length R as still fit into one wave of two resident blocks per SM (one more
 // would add a second, nearly empty wave), each at least 128 long.
@@ -453,6 +573,47 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     o += (size_t)round_up(K * p.Mp * 4, 256);
     p.off_DT = o;
     o += (size_t)round_up(N * p.Mp * 4, 256);
+    p.gram = gram_preferred(M, N, K);
+    if (p.gram) {
+        auto cut = [](int64_t tiles, int64_t kblocks, int64_t least, int64_t* per, int* splits) {
+            int64_t want = 148 / tiles;
+            want = want < 1 ? 1 : (want > 64 ? 64 : want);
+            int64_t each = (kblocks + want - 1) / want;
+            *per = each < least ? least : each;
+            *splits = (int)((kblocks + *per - 1) / *per);
+        };
+        // multiply-adds: a 16-wide stage takes some 1200 cycles however few there are, so slices are short
+        auto cut_short = [](int64_t tiles, int64_t R, int64_t* per, int* splits) {
+            const int64_t least = tiles > 8 ? 64 : 32;
+            int64_t want = 2 * 148 / tiles;
+            want = want < 1 ? 1 : (want > 32 ? 32 : want);
+            const int64_t each = (R + want - 1) / want;
+            *per = round_up(each < least ? least : each, BK);
+            *splits = (int)((R + *per - 1) / *per);
+        };
+        // (the tensor-core kernel has some 10 us of its own: 128 x 256 tiles filled, split, drained and stored; the
+        // multiply-adds take about 6 us per 10^8 products.  960 x 320 x 320: 12.6 us against 9.9)
+        const int64_t tk = (K + 127) / 128;
+        p.tc_s = M * K * K >= 100000000;
+        if (p.tc_s)
+            cut(tk * ((K + 255) / 256), (M + 31) / 32, 4, &p.per_s, &p.splits_s);
+        else
+            cut_short(tk * tk, M, &p.per_s, &p.splits_s);
+        p.tc_g = N * K * K >= 130000000;
+        if (p.tc_g)
+            cut(tk * ((N + 255) / 256), (K + 31) / 32, 1, &p.per_g, &p.splits_g);
+        else
+            cut_short(tk * ((N + 127) / 128), K, &p.per_g, &p.splits_g);
+        p.off_SP = o;
+        o += (size_t)round_up((int64_t)p.splits_s * K * K * 4, 256);
+        p.off_S = o;
+        o += (size_t)round_up(K * K * 4, 256);
+        const int64_t gp = (int64_t)round_up((int64_t)p.splits_g * N * K * 4, 256);
+        if (gp > (int64_t)(p.off_AT - p.off_GP)) {
+            p.off_GP = o;
+            o += (size_t)gp;
+        }
+    }
     p.bytes = o;
     return p;
 }
@@ -475,38 +636,75 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
     int* status = status_word();
     if (!status)
         return FPQ_ERR_CUDA;
-    if (cudaMemsetAsync(loss, 0, 2 * sizeof(double), st) != cudaSuccess)
-        return FPQ_ERR_CUDA;
-    soft_weight_kernel<<<grid_for(N * K), 256, 0, st>>>(w, scale, f, alpha, E, DQ, loss + 1, N, K, status);
-    double inv_mn = 1.0 / ((double)M * (double)N);
-    if (tf32x3_applies(a, K, E, K, M, N, K) && M <= (1 << 21) && N <= (1 << 21) && K <= (1 << 21)) {
-        // Both contractions on the tensor cores (three TF32 products per FP32 product): D^T = (A E^T)^T is written
-        // transposed by the first one's epilogue and A^T by a transpose kernel, so that the second one, D^T A,
-        // again reduces over the contiguous index of both operands.
-        float* AT = (float*)(ws + p.off_AT);
-        float* DT = (float*)(ws + p.off_DT);
-        if (launch_transpose(a, K, M, K, AT, p.Mp, st) != cudaSuccess)
+    const double inv_mn = 1.0 / ((double)M * (double)N);
+    const float coef = (float)(2.0 * inv_mn);
+    const bool tc = tf32x3_applies(a, K, E, K, M, N, K) && M <= (1 << 21) && N <= (1 << 21) && K <= (1 << 21);
+    float* AT = (float*)(ws + p.off_AT);
+    {
+        const bool vec = K % 4 == 0 && (uintptr_t)w % 16 == 0 && (uintptr_t)alpha % 16 == 0;
+        const int weight_blocks = grid_for(vec ? N * K / 4 : N * K);
+        const int64_t blocks = weight_blocks + (tc && !(p.gram && !p.tc_s) ? ((M + 31) / 32) * ((K + 31) / 32) : 0);
+        if (blocks > 0x7fffffff)
+            return FPQ_ERR_SHAPE;
+        if (launch_overlapped(vec ? prepare_kernel<true> : prepare_kernel<false>, dim3((unsigned)blocks), 256, 0, st, w, scale, f,
+                              alpha, E, DQ, loss, N, K, weight_blocks, a, M, AT, p.Mp, status) != cudaSuccess)
             return FPQ_ERR_CUDA;
+    }
+    auto finalize = [&](int splits, const float* e) {
+        const bool vec = N * K % 4 == 0 && (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
+        int blocks = grid_for(vec ? N * K / 4 : N * K);
+        blocks = blocks > 2 * 148 ? 2 * 148 : blocks;
+        return launch_overlapped(vec ? grad_finalize_kernel<true> : grad_finalize_kernel<false>, dim3(blocks), 256, 0, st, GP,
+                                 splits, DQ, e, alpha, grad, loss, N * K, coef, inv_mn, reg, lr) == cudaSuccess
+                   ? FPQ_OK
+                   : FPQ_ERR_CUDA;
+    };
+    if (tc && p.gram) {
+        const int64_t tk = (K + TILE - 1) / TILE;
+        float* SP = (float*)(ws + p.off_SP);
+        float* S = (float*)(ws + p.off_S);
+        // (chunks of 4 blocks: half the bias of the truncating additions, which enters twice here)
+        fpq_status sg = FPQ_OK;
+        if (p.tc_s)
+            sg = launch_tf32x3(AT, p.Mp, AT, p.Mp, K, K, M, (int)p.per_s, 1, SP, K, K * K, nullptr, st, 3, nullptr, 1.0f, nullptr,
+                               0, 4);
+        else if (launch_overlapped(sgemm128<false>, dim3((unsigned)tk, (unsigned)tk, (unsigned)p.splits_s), 256, 0, st, a, K, a, K, SP,
+                                   K, (int)K, (int)K, M, p.per_s, nullptr) != cudaSuccess)
+            sg = FPQ_ERR_CUDA;
+        if (sg != FPQ_OK)
+            return sg;
+        if (launch_overlapped(reduce_gram_kernel, dim3((unsigned)((K * K / 4 + 31) / 32)), 256, 0, st, (const float4*)SP, p.splits_s,
+                              (float4*)S, K * K / 4) != cudaSuccess)
+            return FPQ_ERR_CUDA;
+        if (p.tc_g)
+            sg = launch_tf32x3(S, K, E, K, K, N, K, (int)p.per_g, 1, GP, K, N * K, nullptr, st, 3, nullptr, 1.0f, nullptr, 0, 4);
+        else if (launch_overlapped(sgemm128<true>, dim3((unsigned)((N + TILE - 1) / TILE), (unsigned)tk, (unsigned)p.splits_g), 256, 0,
+                                   st, E, K, S, K, GP, K, (int)N, (int)K, K, p.per_g, nullptr) != cudaSuccess)
+            sg = FPQ_ERR_CUDA;
+        return sg != FPQ_OK ? sg : finalize(p.splits_g, E);
+    }
+    if (tc) {
+        // Both contractions on the tensor cores (three TF32 products per FP32 product): D^T = (A E^T)^T is written
+        // transposed by the first one's epilogue, so that the second one, D^T A, again reduces over the contiguous
+        // index of both operands (it reads A^T).
+        float* DT = (float*)(ws + p.off_DT);
         fpq_status s1;
         if (p.splits1_tc == 1) {
             s1 = launch_tf32x3(a, K, E, K, M, N, K, p.kb_per_split1_tc, 1, DT, p.Mp, 0, loss, st);
         } else {
             // few output tiles and a long reduction: slices of it, added up in a fixed order, then transposed
             s1 = launch_tf32x3(a, K, E, K, M, N, K, p.kb_per_split1_tc, 0, DP, p.N4, M * p.N4, nullptr, st);
-            if (s1 == FPQ_OK) {
-                reduce_d_kernel<<<grid_for(M * p.N4), 256, 0, st>>>(DP, p.splits1_tc, D, M * p.N4, N, p.N4, loss);
-                if (launch_transpose(D, p.N4, M, N, DT, p.Mp, st) != cudaSuccess)
-                    return FPQ_ERR_CUDA;
-            }
+            if (s1 == FPQ_OK && (launch_overlapped(reduce_d_kernel, dim3(grid_for(M * p.N4)), 256, 0, st, DP, p.splits1_tc, D,
+                                                   M * p.N4, N, p.N4, loss) != cudaSuccess ||
+                                 launch_transpose(D, p.N4, M, N, DT, p.Mp, st) != cudaSuccess))
+                return FPQ_ERR_CUDA;
         }
         if (s1 != FPQ_OK)
             return s1;
         s1 = launch_tf32x3(DT, p.Mp, AT, p.Mp, N, K, M, p.kb_per_split_tc, 0, GP, K, N * K, nullptr, st);
         if (s1 != FPQ_OK)
             return s1;
-        grad_finalize_kernel<<<grid_for(N * K), 256, 0, st>>>(GP, p.splits_tc, DQ, alpha, grad, loss, N * K,
-                                                              (float)(2.0 * inv_mn), inv_mn, reg, lr);
-        return cudaGetLastError() == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
+        return finalize(p.splits_tc, nullptr);
     }
     dim3 g1((unsigned)((M + TILE - 1) / TILE), (unsigned)((N + TILE - 1) / TILE), (unsigned)p.splits1);
     if (p.splits1 == 1) {
@@ -517,9 +715,7 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
     }
     dim3 g2((unsigned)((N + TILE - 1) / TILE), (unsigned)((K + TILE - 1) / TILE), (unsigned)p.splits);
     sgemm128<false><<<g2, 256, 0, st>>>(D, p.N4, a, K, GP, K, (int)N, (int)K, M, p.r_per_split, nullptr);
-    grad_finalize_kernel<<<grid_for(N * K), 256, 0, st>>>(GP, p.splits, DQ, alpha, grad, loss, N * K,
-                                                          (float)(2.0 * inv_mn), inv_mn, reg, lr);
-    return cudaGetLastError() == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? finalize(p.splits, nullptr) : FPQ_ERR_CUDA;
 }
 
 fpq_status launch_round_harden(const float* alpha, int64_t N, int64_t K, uint8_t* bits, cudaStream_t st)
