@@ -2,8 +2,9 @@
 
 Every function here has the name of the C entry point it calls
 (include/fpq.h) and passes torch tensors' device pointers and the current CUDA
-stream: the calls a running model makes per layer through a small CPython
-extension (csrc/fpq_torch.cpp), the others through ctypes.  All arithmetic runs
+stream: the calls a running model makes per layer, the encoding search and the
+rounding-learning step through a small CPython extension (csrc/fpq_torch.cpp),
+the others through ctypes.  All arithmetic runs
 in the library's kernels.  There is no fallback: if the shared library is
 missing the import of a symbol fails.
 """
@@ -406,19 +407,16 @@ def fpq_search_format(x: torch.Tensor, encodings, clip: torch.Tensor, mse: torch
                       best: torch.Tensor = None, workspace: torch.Tensor = None):
     """Mean squared error of every (encoding, clipping value) candidate on x and Algorithm 1's
     choice.  Returns (mse [n_enc][n_clip] float64, best [2] int32), both on the device."""
-    assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous()
-    assert clip.is_cuda and clip.dtype == torch.float32 and clip.is_contiguous()
     n_enc, n_clip = len(encodings), clip.numel()
-    enc = (_CFormat * n_enc)(*[f.c() for f in encodings])
     if mse is None:
         mse = torch.empty((n_enc, n_clip), dtype=torch.float64, device=x.device)
     if best is None:
         best = torch.empty(2, dtype=torch.int32, device=x.device)
     if workspace is None:
         workspace = torch.empty(max(8, fpq_search_workspace_size(n_enc, n_clip)), dtype=torch.uint8, device=x.device)
-    _check(lib().fpq_search_format(_ptr(x), x.numel(), ctypes.cast(enc, ctypes.c_void_p), n_enc, _ptr(clip), n_clip,
-                                   _ptr(mse), _ptr(best), _ptr(workspace), workspace.numel(), _stream()),
-           "fpq_search_format")
+    code = (_layers or _load_layers()).search(x, encodings, clip, mse, best, workspace)
+    if code:
+        raise FpqError(code, "fpq_search_format")
     return mse, best
 
 
@@ -431,20 +429,16 @@ def fpq_round_learn_step(w: torch.Tensor, scale: torch.Tensor, fmt: Format, alph
                          workspace: torch.Tensor = None):
     """One evaluation of the rounding-learning objective and its gradient (Sec. V-B); alpha is updated in
     place when lr != 0.  Returns (grad [N][K] float32, loss [2] float64 = {mse, sum of lambda}), on the device."""
-    for t_ in (w, scale, alpha, a):
-        assert t_.is_cuda and t_.dtype == torch.float32 and t_.is_contiguous()
-    N, K = w.shape
-    M = a.shape[0]
-    assert a.shape == (M, K) and alpha.shape == (N, K) and scale.shape == (N,)
     if grad is None:
-        grad = torch.empty((N, K), dtype=torch.float32, device=w.device)
+        grad = torch.empty(w.shape, dtype=torch.float32, device=w.device)
     if loss is None:
         loss = torch.empty(2, dtype=torch.float64, device=w.device)
     if workspace is None:
-        workspace = torch.empty(max(256, fpq_round_learn_workspace_size(M, N, K)), dtype=torch.uint8, device=w.device)
-    _check(lib().fpq_round_learn_step(_ptr(w), _ptr(scale), fmt.c(), _ptr(alpha), _ptr(a), M, N, K, float(reg),
-                                      float(lr), _ptr(grad), _ptr(loss), _ptr(workspace), workspace.numel(),
-                                      _stream()), "fpq_round_learn_step")
+        size = fpq_round_learn_workspace_size(a.shape[0], *w.shape)
+        workspace = torch.empty(max(256, size), dtype=torch.uint8, device=w.device)
+    code = (_layers or _load_layers()).learn_step(w, scale, fmt, alpha, a, reg, lr, grad, loss, workspace)
+    if code:
+        raise FpqError(code, "fpq_round_learn_step")
     return grad, loss
 
 

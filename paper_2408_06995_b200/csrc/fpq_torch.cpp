@@ -207,10 +207,70 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
     return PyLong_FromLong(status);
 }
 
+// search(x, encodings, clip, mse, best, workspace) -> status
+PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    const at::Tensor *x, *clip;
+    void *xp, *clipp, *mse, *best, *work, *st;
+    fpq_format enc[16];
+    if (!arguments(n, 6) || !fp32_cuda(a[0], 0, &x) || !fp32_cuda(a[2], 0, &clip) || !pointer(a[0], &xp) || !pointer(a[2], &clipp) ||
+        !pointer(a[3], &mse) || !pointer(a[4], &best) || !pointer(a[5], &work) || !stream(&st))
+        return nullptr;
+    PyObject* seq = PySequence_Fast(a[1], "encodings must be a sequence");
+    if (!seq)
+        return nullptr;
+    // (more encodings than the library takes: the count is passed on and rejected there, before any is read)
+    const Py_ssize_t count_enc = PySequence_Fast_GET_SIZE(seq);
+    for (Py_ssize_t i = 0; i < count_enc && i < 16; ++i)
+        if (!format(PySequence_Fast_GET_ITEM(seq, i), &enc[i])) {
+            Py_DECREF(seq);
+            return nullptr;
+        }
+    Py_DECREF(seq);
+    const int64_t elements = x->numel();
+    const int32_t n_enc = count_enc > 1000000 ? 1000000 : (int32_t)count_enc;
+    const int32_t n_clip = clip->numel() > 1000000 ? 1000000 : (int32_t)clip->numel();
+    const size_t work_bytes = (size_t)count(a[5]);
+    fpq_status status;
+    Py_BEGIN_ALLOW_THREADS
+    status = fpq_search_format((const float*)xp, elements, enc, n_enc, (const float*)clipp, n_clip, (double*)mse, (int32_t*)best,
+                               work, work_bytes, st);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(status);
+}
+
+// learn_step(w, scale, fmt, alpha, a, reg, lr, grad, loss, workspace) -> status
+PyObject* learn_step(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    const at::Tensor *w, *scale, *alpha, *rows;
+    void *wp, *scalep, *alphap, *rowsp, *grad, *loss, *work, *st;
+    fpq_format fmt;
+    float reg, lr;
+    if (!arguments(n, 10) || !fp32_cuda(a[0], 2, &w) || !fp32_cuda(a[1], 1, &scale) || !format(a[2], &fmt) ||
+        !fp32_cuda(a[3], 2, &alpha) || !fp32_cuda(a[4], 2, &rows) || !real(a[5], &reg) || !real(a[6], &lr) || !pointer(a[0], &wp) ||
+        !pointer(a[1], &scalep) || !pointer(a[3], &alphap) || !pointer(a[4], &rowsp) || !pointer(a[7], &grad) ||
+        !pointer(a[8], &loss) || !pointer(a[9], &work) || !stream(&st))
+        return nullptr;
+    const int64_t M = rows->size(0), N = w->size(0), K = w->size(1);
+    if (rows->size(1) != K || alpha->size(0) != N || alpha->size(1) != K || scale->size(0) != N) {
+        PyErr_SetString(PyExc_AssertionError, "expected w and alpha [N][K], a [M][K], scale [N]");
+        return nullptr;
+    }
+    const size_t work_bytes = (size_t)count(a[9]);
+    fpq_status status;
+    Py_BEGIN_ALLOW_THREADS
+    status = fpq_round_learn_step((const float*)wp, (const float*)scalep, fmt, (float*)alphap, (const float*)rowsp, M, N, K, reg, lr,
+                                  (float*)grad, (double*)loss, work, work_bytes, st);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(status);
+}
+
 PyMethodDef methods[] = {
     {"linear", (PyCFunction)(void (*)(void))linear, METH_FASTCALL, nullptr},
     {"conv2d", (PyCFunction)(void (*)(void))conv2d, METH_FASTCALL, nullptr},
     {"conv2d_split", (PyCFunction)(void (*)(void))conv2d_split, METH_FASTCALL, nullptr},
+    {"search", (PyCFunction)(void (*)(void))search, METH_FASTCALL, nullptr},
+    {"learn_step", (PyCFunction)(void (*)(void))learn_step, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
 
