@@ -383,6 +383,32 @@ __global__ void __launch_bounds__(256) quantize_rows_e4m3_kernel(const float* __
         flag_status(status, FPQ_ERR_NAN_INPUT);
 }
 
+// The same where rows are whole 16-byte pieces of codes (K a multiple of 16): the codes are x's values in order, so a block
+// takes 4096 of them, a thread four groups of four 256 groups apart, and loads and stores are whole lines.
+// (320 columns: 8192 rows 2.5 us, 65536 rows 15.4 us; sixteen values per thread behind a 64-bit division 3.8 and 17.4 us)
+template <bool E5>
+__global__ void __launch_bounds__(256) quantize_flat_kernel(const float4* __restrict__ x, int64_t groups, float rinv,
+                                                            uint32_t* __restrict__ codes, int* status)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    bool nan = false;
+    for (int64_t base = (int64_t)blockIdx.x * 1024 + threadIdx.x; base < groups; base += (int64_t)gridDim.x * 1024) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (base + u * 256 < groups)
+                v[u] = __ldg(x + base + u * 256);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (base + u * 256 < groups)
+                codes[base + u * 256] = fp8x4_from_scaled<E5>(__fmul_rn(v[u].x, rinv), __fmul_rn(v[u].y, rinv),
+                                                              __fmul_rn(v[u].z, rinv), __fmul_rn(v[u].w, rinv), nan);
+    }
+    if (nan)
+        flag_status(status, FPQ_ERR_NAN_INPUT);
+}
+
 // ---------------------------------------------------------------------------------
 // NCHW FP32 -> channels-last codes with a zero frame: [B][H+2p][W+2p][row] (channel padding
 // and frame = code 0), the A operand of the implicit-GEMM convolution.  The kernel fills the
@@ -610,6 +636,11 @@ cudaError_t launch_quantize_weight(const float* w, int64_t N, int64_t K, const f
 cudaError_t launch_quantize_rows_e4m3(const float* x, int64_t M, int64_t K, int64_t Kp, float scale, uint8_t* codes,
                                       cudaStream_t st, int e5m2)
 {
+    if (K == Kp && (uintptr_t)x % 16 == 0) {
+        const int64_t groups = M * (K / 4);
+        return launch_overlapped(e5m2 ? quantize_flat_kernel<true> : quantize_flat_kernel<false>, dim3(grid_for(groups, 1024)), 256,
+                                 0, st, (const float4*)x, groups, 1.0f / scale, (uint32_t*)codes, status_word());
+    }
     int64_t total = M * (Kp / 16);
     return launch_overlapped(e5m2 ? quantize_rows_e4m3_kernel<false, true> : quantize_rows_e4m3_kernel<false, false>,
                              dim3(grid_for(total, 256)), 256, 0, st, x, M, K, Kp, 1.0f / scale, codes, status_word());
