@@ -1232,7 +1232,16 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     // several column tiles per row tile: try to keep the row tile's whole activation panel in the
     // ring (read / quantized once) and stream the weights
     bool done = false;
-    if (g.ksplit == 1 && !g.pair && g.n_tiles > 1 && g.mode != MODE_TAPS) {
+    // row-major output with several column tiles whose weights fit: CTA b keeps the weights of column tile b % n_tiles and
+    // goes through every (grid / n_tiles)-th row tile, so that at any time the whole GPU writes one compact piece of the
+    // output (a plain store kernel with these tiles: 112 us for 671 MB so, 126 us with a contiguous range of tiles per CTA;
+    // 320 -> 2560, M = 65536, whole layer: 164.7 -> 144.3 us; 320 -> 960, M = 8192: 15.4 -> 14.8).  Not with many SMs left
+    // over (40 column tiles, 120 of 148: 640 -> 5120, M = 16384, 122.6 -> 131.8 us), nor where the weights leave no room
+    // for two chunks per activation stage (768 -> 3200, M = 8192: 45.5 -> 55.5 us).
+    const int col_grid = di->sms / g.n_tiles * g.n_tiles;
+    const bool by_column = MODE == MODE_ROWS && !FUSED && g.ksplit == 1 && g.n_tiles > 1 && col_grid * 10 >= di->sms * 9 &&
+                           (int64_t)g.m_tiles * g.n_tiles > col_grid && b_all + 2 * (g.cchunks < 2 ? 1 : 2) * (int64_t)g.a_chunk_bytes <= budget;
+    if (!by_column && g.ksplit == 1 && !g.pair && g.n_tiles > 1 && g.mode != MODE_TAPS) {
         const bool conv9 = g.mode == MODE_FLAT && g.taps == 9 && g.S == 3;
         if (conv9 || g.taps == 1) {
             const int cps = conv9 ? 1 : (g.cchunks >= 3 ? 3 : g.cchunks);      // chunks per A stage
@@ -1261,7 +1270,7 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
         g.b_resident = 1;
         g.b_span = g.nblk;
         g.b_stages = 1;
-        g.m_fastest = 1;
+        g.m_fastest = by_column ? 0 : 1;
         const int room = budget - (int)b_all;
         int chunks = room / (2 * g.a_chunk_bytes);            // chunks (TAPS: boxes) per stage
         const int want = (g.mode == MODE_FLAT && g.taps >= 4) ? 1 : 4;
@@ -1300,7 +1309,7 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     g.b_stage_bytes = g.b_span * b_block;
     if (g.a_stages < 1 || g.b_stages < 1 || (!g.b_resident && g.b_stages < 2))
         return FPQ_ERR_UNSUPPORTED;
-    g.contiguous = (g.a_resident || (g.b_resident && g.n_tiles > 1)) ? 1 : 0;
+    g.contiguous = (g.a_resident || (g.b_resident && g.n_tiles > 1 && !by_column)) ? 1 : 0;
     g.div_tiles = make_fastdiv((uint32_t)(g.m_fastest ? g.m_tiles : g.n_tiles));
     // the partial sums of a split tile are staged over the rings
     if (g.ksplit > 1 && g.a_stages * g.a_stage_bytes + g.b_stages * g.b_stage_bytes < BN * BM * 4)
@@ -1354,7 +1363,7 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     const int64_t tiles = (int64_t)g.m_tiles * g.n_tiles;
     if (g.ksplit > 1 && tiles * g.ksplit > 0x7fffff00ll)
         return FPQ_ERR_SHAPE;
-    const int grid = g.ksplit > 1 ? (int)tiles * g.ksplit : (int)(tiles < di->sms ? tiles : di->sms);
+    const int grid = g.ksplit > 1 ? (int)tiles * g.ksplit : by_column ? col_grid : (int)(tiles < di->sms ? tiles : di->sms);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(num_threads(FUSED));
