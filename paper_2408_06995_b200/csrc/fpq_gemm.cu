@@ -37,15 +37,15 @@ namespace fpq {
 
 constexpr int BM = 128;        // output rows per tile (TMEM lanes)
 constexpr int BK = 128;        // reduction elements per block (one 128-byte swizzled row)
-// Warp roles.  Plain form: producer, MMA issuer, 8 epilogue warps (two per TMEM lane quarter,
-// each half of the columns).  Fused form: producer, MMA issuer, 4 epilogue warps and 16
+// Warp roles.  Plain form: activation producer, MMA issuer, 8 epilogue warps (two per TMEM lane quarter,
+// each half of the columns), weight producer.  Fused form: weight producer, MMA issuer, 4 epilogue warps and 16
 // transform warps that quantize FP32 activations into the A ring - the conversion is bound by
 // instruction issue, so it gets most of the SM's warps.
 constexpr int NUM_XFORM_WARPS = 16;
 __host__ __device__ constexpr int epi_warps(bool fused) { return fused ? 4 : 8; }
 __host__ __device__ constexpr int num_threads(bool fused)
 {
-    return 64 + 32 * epi_warps(fused) + (fused ? 32 * NUM_XFORM_WARPS + 32 : 0);   // + one L2-prefetch warp
+    return 64 + 32 * epi_warps(fused) + 32 + (fused ? 32 * NUM_XFORM_WARPS : 0);   // (+ 32: weight producer / L2 prefetch)
 }
 constexpr int SMEM_BUDGET = 227 * 1024;   // the most dynamic shared memory a CTA can have on sm_100
 
@@ -76,6 +76,8 @@ struct GemmArgs {
     // one weight load covers b_box_t taps x b_box_c chunks of the column tile (a TMA load costs its SM about 400
     // cycles whatever its size): b_box_t > 1 inside a chunk's taps, b_box_c > 1 over chunks of a tap-less layer
     int b_box_t, b_box_c;
+    int b_loads;               // loads of a full weight stage
+    int a_chunks;              // chunks of a full activation stage (not TAPS)
     int a_box_c;               // row-major activations: one load covers the a_box_c chunks of a stage (1 = one per chunk)
     int y_tma;                 // row-major output leaves through TMA stores
     int vec_scale;             // w_scale / bias are 16-byte aligned
@@ -362,97 +364,62 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
 
     // Every wait below is bounded; a role whose wait expires records FPQ_ERR_TIMEOUT and
     // leaves its loop, the other roles then run into their own limits and follow.
-    if (warp == 0) {
-        // ---------------- TMA producer (one thread; its loops never divide) ----------------
+    if (!FUSED && warp == 0) {
+        // ---------------- activation producer (one thread; its loops never divide) ----------------
         if (elect_one()) {
-            uint32_t sa = 0, pa = 0, sb = 0, pb = 0;   // stage and phase of the next load per ring
-            uint32_t na = 0, nb = 0;                   // stages issued (for the abort path)
-            int resident_nt = -1, resident_mt = -1;
+            // the activation codes are written by the preceding grid
+            if (g.wait_prior_grid)
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+            uint32_t sa = 0, pa = 1, na = 0;           // stage and (inverted) phase of the next load; stages issued
+            int resident_mt = -1;
             bool dead = false;
-            bool prior_done = !g.wait_prior_grid;
-            // `count` consecutive weight blocks (chunk c2, tap t2 onward; taps fastest) of column tile n0, one load per box
-            const int b_box = g.b_box_t * g.b_box_c;
-            auto load_weights = [&](uint32_t dst, uint32_t bar, int n0, int c2, int t2, int count) {
-                for (int l = 0; l < count; l += b_box, dst += b_box * B_BLOCK_BYTES) {
-                    tma_load_4d(dst, &tmB, bar, 0, n0, t2, c2);
-                    t2 += g.b_box_t;
-                    if (t2 >= g.taps) { t2 = 0; c2 += g.b_box_c; }
-                }
-            };
+            const int chunks = MODE == MODE_TAPS ? 0 : g.a_chunks;       // chunks of a full stage
+            const bool a_wide = MODE == MODE_ROWS && g.a_box_c > 1;
             for (int t = t_lo; t < t_hi && !dead; t += t_step) {
                 int mt, nt;
                 decode_tile(t, mt, nt);
-                const int n0 = nt * BN;
-                int x0 = 0, y0 = 0, b0 = 0;
+                if (g.a_resident && resident_mt == mt)
+                    continue;                          // the panel is still in the ring
+                resident_mt = mt;
                 if (MODE == MODE_TAPS) {
                     const uint32_t r1 = fdiv((uint32_t)mt, g.div_tx);
-                    x0 = (mt - (int)r1 * g.tiles_x) * g.Wt * g.stride;
+                    const int x0 = (mt - (int)r1 * g.tiles_x) * g.Wt * g.stride;
                     const uint32_t r2 = fdiv(r1, g.div_ty);
-                    y0 = ((int)r1 - (int)r2 * g.tiles_y) * g.Ht * g.stride;
-                    b0 = (int)r2 * g.Bt;
-                }
-                const bool load_b = !(g.b_resident && resident_nt == nt);
-                resident_nt = nt;
-                const bool load_a = !(g.a_resident && resident_mt == mt);
-                resident_mt = mt;
-                int cc = c_lo, tap = 0, r = 0, sx = 0; // block j = (cc, tap), tap = (r, sx)
-                int ja = 0, jb = 0;                    // position inside the current A / B stage
-                bool early_b = false;
-                for (int j = 0; j < nblk; ++j) {
-                    if (jb == 0 && load_b && !prior_done && g.b_resident) {
-                        // the weights do not depend on the kernel in front: fetch them before waiting for it
-                        if (!mbar_wait(b_empty + 8 * sb, pb ^ 1)) { dead = true; break; }
-                        mbar_expect_tx(b_full + 8 * sb, (uint32_t)g.nblk * g.b_block_tx);
-                        load_weights(b_ring + sb * g.b_stage_bytes, b_full + 8 * sb, n0, 0, 0, g.nblk);
-                        ++nb;
-                        if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
-                        early_b = true;
-                    }
-                    if (!prior_done) {
-                        // the activation codes are written by the preceding grid
-                        asm volatile("griddepcontrol.wait;" ::: "memory");
-                        prior_done = true;
-                    }
-                    if (ja == 0 && !FUSED && load_a) {
-                        // activation stage: the data of the next a_span blocks
-                        if (!mbar_wait(a_empty + 8 * sa, pa ^ 1)) { dead = true; break; }
-                        const int nblocks = min(g.a_span, nblk - j);
-                        const int nloads = (MODE == MODE_TAPS) ? nblocks : nblocks / g.taps;
-                        const bool a_wide = MODE == MODE_ROWS && g.a_box_c > 1;
-                        mbar_expect_tx(a_full + 8 * sa, (uint32_t)(a_wide ? g.a_box_c : nloads) * g.a_chunk_tx);
+                    const int y0 = ((int)r1 - (int)r2 * g.tiles_y) * g.Ht * g.stride;
+                    const int b0 = (int)r2 * g.Bt;
+                    int c2 = c_lo, t2 = 0, ry = 0, sx = 0;               // next block = (chunk, tap), tap = (ry, sx)
+                    for (int left = nblk; left > 0; left -= g.a_span) {
+                        if (!mbar_wait(a_empty + 8 * sa, pa)) { dead = true; break; }
+                        const int nloads = min(g.a_span, left);
+                        mbar_expect_tx(a_full + 8 * sa, (uint32_t)nloads * g.a_chunk_tx);
                         uint32_t dst = a_ring + sa * g.a_stage_bytes;
-                        if (a_wide) {
-                            // all chunks of the stage in one box (chunks past the last one read as zeros)
-                            tma_load_4d(dst, &tmA, a_full + 8 * sa, 0, mt * tile_rows, cc, 0);
-                        } else if (MODE == MODE_TAPS) {
-                            int c2 = cc, t2 = tap, r2 = r, s2 = sx;
-                            for (int l = 0; l < nloads; ++l, dst += g.a_chunk_bytes) {
-                                tma_load_4d(dst, &tmA, a_full + 8 * sa, c2 * BK, x0 + s2, y0 + r2, b0);
-                                if (++s2 == g.S) { s2 = 0; ++r2; }
-                                if (++t2 == g.taps) { t2 = 0; r2 = 0; s2 = 0; ++c2; }
-                            }
-                        } else {
-                            for (int l = 0; l < nloads; ++l, dst += g.a_chunk_bytes)
-                                for (int bx = 0; bx < g.a_boxes; ++bx)
-                                    tma_load_4d(dst + bx * g.a_box_rows * 128, &tmA, a_full + 8 * sa, (cc + l) * BK,
-                                                mt * tile_rows + bx * g.a_box_rows, 0, 0);
+                        for (int l = 0; l < nloads; ++l, dst += g.a_chunk_bytes) {
+                            tma_load_4d(dst, &tmA, a_full + 8 * sa, c2 * BK, x0 + sx, y0 + ry, b0);
+                            if (++sx == g.S) { sx = 0; ++ry; }
+                            if (++t2 == g.taps) { t2 = 0; ry = 0; sx = 0; ++c2; }
                         }
                         ++na;
                         if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
                     }
-                    if (jb == 0 && load_b && !early_b) {
-                        if (!mbar_wait(b_empty + 8 * sb, pb ^ 1)) { dead = true; break; }
-                        // (a box that reaches past the last chunk is filled with zeros there and reports its full size)
-                        const int nblocks = (min(g.b_span, nblk - j) + b_box - 1) / b_box * b_box;
-                        mbar_expect_tx(b_full + 8 * sb, (uint32_t)nblocks * g.b_block_tx);
-                        load_weights(b_ring + sb * g.b_stage_bytes, b_full + 8 * sb, n0, cc, tap, nblocks);
-                        ++nb;
-                        if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
+                } else {
+                    const int row = mt * tile_rows;
+                    for (int cc = c_lo; cc < c_hi; cc += chunks) {
+                        if (!mbar_wait(a_empty + 8 * sa, pa)) { dead = true; break; }
+                        const int nloads = min(chunks, c_hi - cc);
+                        const uint32_t bar = a_full + 8 * sa;
+                        mbar_expect_tx(bar, (uint32_t)(a_wide ? g.a_box_c : nloads) * g.a_chunk_tx);
+                        uint32_t dst = a_ring + sa * g.a_stage_bytes;
+                        if (a_wide) {
+                            // all chunks of the stage in one box (chunks past the last one read as zeros)
+                            tma_load_4d(dst, &tmA, bar, 0, row, cc, 0);
+                        } else {
+                            for (int l = 0; l < nloads; ++l, dst += g.a_chunk_bytes)
+                                for (int bx = 0; bx < g.a_boxes; ++bx)
+                                    tma_load_4d(dst + bx * g.a_box_rows * 128, &tmA, bar, (cc + l) * BK, row + bx * g.a_box_rows, 0, 0);
+                        }
+                        ++na;
+                        if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
                     }
-                    if (++ja == g.a_span) ja = 0;
-                    if (++jb == g.b_span) jb = 0;
-                    if (++sx == g.S) { sx = 0; ++r; }
-                    if (++tap == g.taps) { tap = 0; r = 0; sx = 0; ++cc; }
                 }
             }
             if (dead) {
@@ -460,6 +427,49 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                 // let the copies still in flight land before the CTA's shared memory is released
                 for (uint32_t i = (na > (uint32_t)g.a_stages ? na - g.a_stages : 0); i < na; ++i)
                     (void)mbar_wait(a_full + 8 * (i % g.a_stages), (i / g.a_stages) & 1);
+            }
+        }
+    } else if (warp == (FUSED ? 0 : 2 + NUM_EPI_WARPS)) {
+        // ---------------- weight producer: a thread of its own ----------------
+        // The weights do not depend on the quantize kernel in front (what wrote them was complete when that one let this
+        // kernel start): the ring is filled while it still runs.  With both operands loaded by one thread every stage
+        // cost it some 0.5 us of dependent instructions, which is what small layers were bound by.
+        if (elect_one()) {
+            uint32_t sb = 0, pb = 1, nb = 0;
+            int resident_nt = -1;
+            bool dead = false;
+            const int b_box = g.b_box_t * g.b_box_c;
+            for (int t = t_lo; t < t_hi && !dead; t += t_step) {
+                int mt, nt;
+                decode_tile(t, mt, nt);
+                if (g.b_resident && resident_nt == nt)
+                    continue;
+                resident_nt = nt;
+                const int n0 = nt * BN;
+                int c2 = c_lo, t2 = 0;                 // next block = (chunk, tap), taps fastest
+                for (int left = nblk; left > 0; left -= g.b_span) {
+                    // (the limits of its waits start counting once the kernel in front has finished)
+                    if (nb == (uint32_t)g.b_stages && g.wait_prior_grid)
+                        asm volatile("griddepcontrol.wait;" ::: "memory");
+                    if (!mbar_wait(b_empty + 8 * sb, pb)) { dead = true; break; }
+                    // one load per box; one that reaches past the last chunk is filled with zeros there and reports its
+                    // full size
+                    const int count = min(g.b_span, left);
+                    const int loads = count == g.b_span ? g.b_loads : (count + b_box - 1) / b_box;
+                    const uint32_t bar = b_full + 8 * sb;
+                    mbar_expect_tx(bar, (uint32_t)(loads * b_box) * g.b_block_tx);
+                    uint32_t dst = b_ring + sb * g.b_stage_bytes;
+                    for (int l = 0; l < loads; ++l, dst += b_box * B_BLOCK_BYTES) {
+                        tma_load_4d(dst, &tmB, bar, 0, n0, t2, c2);
+                        t2 += g.b_box_t;
+                        if (t2 >= g.taps) { t2 = 0; c2 += g.b_box_c; }
+                    }
+                    ++nb;
+                    if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
+                }
+            }
+            if (dead) {
+                flag_status(g.status, FPQ_ERR_TIMEOUT);
                 for (uint32_t i = (nb > (uint32_t)g.b_stages ? nb - g.b_stages : 0); i < nb; ++i)
                     (void)mbar_wait(b_full + 8 * (i % g.b_stages), (i / g.b_stages) & 1);
             }
@@ -1331,6 +1341,8 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     } else if (g.b_span > 1) {
         g.b_box_c = g.b_span;
     }
+    g.b_loads = (g.b_span + g.b_box_t * g.b_box_c - 1) / (g.b_box_t * g.b_box_c);
+    g.a_chunks = g.mode == MODE_TAPS ? 0 : g.a_span / g.taps;
     // prepared weights [N][taps][Cp] as (position in chunk, output, tap, chunk): a box lands as [chunk][tap][output][128 B]
     CUtensorMap tmB, tmA2 = tmA;
     g.a_box_c = 1;
