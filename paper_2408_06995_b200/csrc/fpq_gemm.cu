@@ -80,6 +80,7 @@ struct GemmArgs {
     int a_chunks;              // chunks of a full activation stage (not TAPS)
     int a_box_c;               // row-major activations: one load covers the a_box_c chunks of a stage (1 = one per chunk)
     int y_tma;                 // row-major output leaves through TMA stores
+    int y_stage;               // bytes of each epilogue warp's staging: two 4 KiB buffers, or one where a warp stores once
     int vec_scale;             // w_scale / bias are 16-byte aligned
     int stage_scales;          // x_scale * w_scale[n] and bias[n] of all N columns sit in shared memory
     int contiguous;            // tile order: 1 = every CTA walks a contiguous range, 0 = CTAs interleave
@@ -246,12 +247,12 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
 
-    // layout: [A ring][B ring][epilogue staging for TMA stores, 2 x 4 KiB per warp][barriers + flags]
+    // layout: [A ring][B ring][epilogue staging for TMA stores, 1 or 2 x 4 KiB per warp][barriers + flags]
     //         [x_scale * w_scale | bias, all N columns, when they fit]
     const uint32_t a_ring = smem_base;
     const uint32_t b_ring = a_ring + g.a_stages * g.a_stage_bytes;
     const uint32_t ctl_off = g.a_stages * g.a_stage_bytes + g.b_stages * g.b_stage_bytes;
-    const uint32_t bars = smem_base + ctl_off + (g.y_tma ? NUM_EPI_WARPS * 8192 : 0);
+    const uint32_t bars = smem_base + ctl_off + (g.y_tma ? NUM_EPI_WARPS * g.y_stage : 0);
     // barrier slots (8 bytes each): a_full[8] a_empty[8] b_full[8] b_empty[8] acc_full[2] acc_empty[2]
     const uint32_t a_full = bars, a_empty = bars + 64, b_full = bars + 128, b_empty = bars + 192;
     const uint32_t acc_full = bars + 256, acc_empty = bars + 272;
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
         // row-major output: the warp's 32 x 32 block goes through a 128-byte-swizzled staging
         // buffer and leaves as one TMA store (whole 128-byte lines; rows past M and columns
         // past N are clipped by the tensor map)
-        uint8_t* stage0 = smem + ctl_off + (warp - 2) * 8192;     // two 4 KiB buffers, used in turn
+        uint8_t* stage0 = smem + ctl_off + (warp - 2) * g.y_stage;     // two 4 KiB buffers, used in turn (or one)
         // (as in the MMA role: bounded waits start counting after the kernel in front)
         if (g.wait_prior_grid)
             asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1181,7 +1182,10 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     g.stage_scales = (n_pad * 8 <= 16384) ? 1 : 0;
     // (without the table of all columns: every epilogue warp's copy of its own columns' scales and biases, 2 * BN floats
     // per group of four warps)
-    const int ctl = 512 + 1024 + (g.y_tma ? epi_warps(FUSED) * 8192 : 0) + (g.stage_scales ? n_pad * 8 : 4 * 2 * BN * 4);
+    // a row-major layer with at most one tile per CTA: nothing stays resident, both operands stream
+    const bool one_tile = MODE == MODE_ROWS && !FUSED && (int64_t)g.m_tiles * g.n_tiles <= di->sms;
+    g.y_stage = one_tile && BN == 64 ? 4096 : 8192;
+    const int ctl = 512 + 1024 + (g.y_tma ? epi_warps(FUSED) * g.y_stage : 0) + (g.stage_scales ? n_pad * 8 : 4 * 2 * BN * 4);
     const int budget = SMEM_BUDGET - ctl;
     const int b_block = BN * BK;
     const int a_min_span = (g.mode == MODE_FLAT) ? g.taps : 1;
@@ -1251,7 +1255,23 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
     const int col_grid = di->sms / g.n_tiles * g.n_tiles;
     const bool by_column = MODE == MODE_ROWS && !FUSED && g.ksplit == 1 && g.n_tiles > 1 && col_grid * 10 >= di->sms * 9 &&
                            (int64_t)g.m_tiles * g.n_tiles > col_grid && b_all + 2 * (g.cchunks < 2 ? 1 : 2) * (int64_t)g.a_chunk_bytes <= budget;
-    if (!by_column && g.ksplit == 1 && !g.pair && g.n_tiles > 1 && g.mode != MODE_TAPS) {
+    if (one_tile && g.ksplit == 1) {
+        // the whole reduction in flight if it fits, two chunks per stage, so that the MMAs start with the first of them
+        const int span = g.cchunks >= 4 ? 2 : 1, want = (g.cchunks + span - 1) / span;
+        const int stage = span * (g.a_chunk_bytes + b_block);
+        int n = budget / stage;
+        if (n > 8) n = 8;
+        if (n > want) n = want;
+        if (n >= 2 || n == want) {
+            g.b_resident = 0;
+            g.m_fastest = 0;
+            g.a_span = g.b_span = span;
+            g.a_stage_bytes = span * g.a_chunk_bytes;
+            g.a_stages = g.b_stages = n < 2 ? 2 : n;
+            done = true;
+        }
+    }
+    if (!done && !by_column && g.ksplit == 1 && !g.pair && g.n_tiles > 1 && g.mode != MODE_TAPS) {
         const bool conv9 = g.mode == MODE_FLAT && g.taps == 9 && g.S == 3;
         if (conv9 || g.taps == 1) {
             const int cps = conv9 ? 1 : (g.cchunks >= 3 ? 3 : g.cchunks);      // chunks per A stage
@@ -1450,7 +1470,8 @@ fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st)
     g.status = status_word();
     g.wait_prior_grid = p.after_stage1;
 
-    const int BN = (p.N <= 64) ? 64 : 128;
+    // (64-wide column tiles as well where a linear layer's 128-wide ones would leave half of the SMs idle)
+    const int BN = (p.N <= 64 || (!p.conv && p.x == nullptr && (p.M + BM - 1) / BM * ((p.N + 63) / 64) <= 148)) ? 64 : 128;
     g.n_tiles = (p.N + BN - 1) / BN;
     g.idesc = idesc_f8f6f4(p.a_e5m2 ? 1u : 0u, p.w4 ? 5u : (p.w_e5m2 ? 1u : 0u), (uint32_t)BN);
     g.b_block_tx = (uint32_t)(BN * BK) / (p.w4 ? 2 : 1);
