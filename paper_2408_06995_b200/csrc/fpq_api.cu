@@ -541,6 +541,11 @@ static fpq_status linear_contract_impl(const void* workspace, size_t ws_bytes, c
     p.x_scale = x_scale;
     p.bias = bias;
     p.y = y;
+    if (p.x == nullptr && g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && pair_rows_preferred(p, 1)) {
+        const fpq_status sp = launch_pair_rows(p, 1, (cudaStream_t)stream);
+        if (sp != FPQ_ERR_UNSUPPORTED)
+            return sp;
+    }
     return launch_gemm(p, (cudaStream_t)stream);
 }
 
@@ -635,6 +640,25 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
             return FPQ_ERR_ALIGN;
         if (!status_word())
             return FPQ_ERR_CUDA;
+        {
+            // long reductions: CTA pairs, both terms on one copy of the codes
+            GemmProblem p{};
+            p.after_stage1 = 1;
+            p.w_e5m2 = is_e5m2_native(term) ? 1 : 0;
+            p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
+            p.M = M, p.N = (int)N, p.C = (int)K;
+            p.Cp = (int)K2;
+            p.Ca = (int)round_up(K, 16);
+            p.R = p.S = 1, p.stride = 1;
+            p.a_codes = (const uint8_t*)workspace;
+            p.w_prepared = w_prepared, p.w_scale = w_scale, p.x_scale = x_scale * two_term_unshift(fw), p.bias = bias, p.y = y;
+            if (g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && pair_rows_preferred(p, 2)) {
+                if (launch_quantize_rows_e4m3(x, M, K, p.Ca, x_scale, (uint8_t*)workspace, (cudaStream_t)stream, p.a_e5m2) !=
+                    cudaSuccess)
+                    return FPQ_ERR_CUDA;
+                return launch_pair_rows(p, 2, (cudaStream_t)stream);
+            }
+        }
         if (launch_quantize_rows_e4m3_twice(x, M, K, K2 / 2, x_scale, (uint8_t*)workspace, (cudaStream_t)stream,
                                             is_e5m2_native(fx) ? 1 : 0) != cudaSuccess)
             return FPQ_ERR_CUDA;

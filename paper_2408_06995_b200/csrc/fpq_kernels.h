@@ -86,6 +86,11 @@ bool pair_conv_preferred(const GemmProblem& p);   // ... and it measured faster 
 fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st);
 bool pair_gemm_preferred(const GemmProblem& p);   // in range, and faster than the general contraction on shapes like this
 
+// The contraction of a linear layer (activation codes already in the workspace, written once whatever the terms) on CTA
+// pairs; weights of two terms share the activations.  FPQ_ERR_UNSUPPORTED when out of range (nothing was enqueued).
+fpq_status launch_pair_rows(const GemmProblem& p, int terms, cudaStream_t st);
+bool pair_rows_preferred(const GemmProblem& p, int terms);   // in range, and faster than the general contraction
+
 // Linear layer with at most 8 rows on the CUDA cores (one pass over the weights).
 bool small_m_linear_applies(int64_t M, int64_t K);
 fpq_status launch_small_m_linear(const float* x, int M, int K, const void* w_prepared, int w4, int N, const float* w_scale,
