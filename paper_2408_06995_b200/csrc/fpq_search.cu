@@ -29,16 +29,17 @@ constexpr int SEARCH_CHUNK = SEARCH_THREADS * SEARCH_PER_THREAD;
 constexpr int SEARCH_DIRECT_BLOCKS = 1184;     // most blocks of the direct form
 // Sorted form: bins of |x| by exponent and the leading 10 mantissa bits, over the 16 binades below (and with) the
 // one of the largest clipping value.  Steps are at least 2^-6 of the value, so a threshold cuts one bin in 16 or fewer.
-// (11 bits: twice the table for half the elements in cut bins; 47 against 41 us for 3.7 M elements and 222 candidates,
-// 53 against 50 us for 1 M elements and 444 candidates.)
 constexpr int LOW_BITS = 13;                   // mantissa bits inside a bin
 constexpr int BINS = 16 << (23 - LOW_BITS);
 constexpr int SORT_THREADS = 1024;
-constexpr int SORT_PIECE = 32768;              // most elements sorted at a time (offsets are 16 bits)
+constexpr int SORT_ROUND = 4 * SORT_THREADS;   // elements: four a thread
+constexpr int SORT_FLIGHT = 4;                 // rounds whose loads are in flight together
+constexpr int SORT_PIECE = 15 * SORT_ROUND;    // most elements sorted at a time
 constexpr int SORT_LIST = 4096;                // elements outside the bins, handled one by one
 constexpr int SORT_BLOCKS = 148;
 constexpr int MAX_THRESHOLDS = 128;            // per candidate, padded
-constexpr size_t SORT_SMEM = (size_t)BINS * 2 + SORT_PIECE * 2 + SORT_LIST * sizeof(float) + SEARCH_MAX_CAND * sizeof(double);
+constexpr int SORT_SLOTS = SORT_PIECE + BINS;       // every bin padded to an even number
+constexpr size_t SORT_SMEM = (size_t)BINS * 4 + SORT_SLOTS * 2 + SEARCH_MAX_CAND * sizeof(double);
 constexpr int PACK_SHIFT = 37;                 // a bin's count above its sum of low bits
 constexpr int64_t PACK_MAX = 1 << 24;          // ... which holds up to this many elements
 
@@ -65,6 +66,7 @@ struct SearchArgs {
     double* spread_sq;               // [blocks]: sum of squared distances from the bins' centres
     unsigned long long* bin_sum;     // [BINS]: sum of low bits, with the count above it
     uint32_t* threshold;             // [candidates][MAX_THRESHOLDS]: smallest |x| (bit pattern) above each threshold
+    char4* nudge;                    // [candidates][32]: threshold k = 32 q + lane less midpoint * scale, component q
     ulonglong2* below;               // [BINS + MAX_THRESHOLDS]: what Prefix holds (search_prefix_kernel)
     ulonglong2* below_sq;            // [BINS + MAX_THRESHOLDS]
     unsigned* ticket;
@@ -334,6 +336,8 @@ __global__ void __launch_bounds__(256) search_tables_kernel(const SearchArgs a)
             ++at;
     }
     a.threshold[id] = at;
+    reinterpret_cast<signed char*>(a.nudge + c * 32 + k % 32)[k / 32] =
+        k < a.enc[i].thresholds ? (signed char)(at - __float_as_uint(__fmul_rn(code_midpoint(a.enc[i], k), scale))) : 0;
 }
 
 // Sums over a range of bins, in units of the last place of the lowest binade (so that all elements are whole numbers
@@ -406,24 +410,31 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t mine, uint32_t* s_warp, 
 // grid value instead of the one of the bin's lower edge (which is what search_eval_kernel gives to the whole bin).
 // The change is -2 D * sum(x - mu) over those elements, D the step and mu the midpoint, both times the scale.
 // blockIdx.y: the share of the candidates (every share sorts for itself).
-static_assert(BINS % (8 * SORT_THREADS) == 0, "offsets of a thread are whole 16-byte words");
-static_assert(SORT_PIECE / SORT_THREADS <= 32, "one bit per element of a thread");
+// What bounds it: instructions (0.7 issued per cycle and scheduler), more than half of them in the candidates' walk below.
+// So a bin's slots start at an even place and are padded with zeros, and a threshold walks its bin two elements to a
+// register and two registers a step; the thresholds themselves are worked out again (a multiplication and a stored offset
+// in ulps) rather than read, 57 instead of 227 KB per block; a warp's candidates are neighbours, so that it seldom changes
+// the encoding; and a piece may have 61440 elements, because half of the walk does not depend on them.  3.7 M elements,
+// 444 candidates, whole search: 69.8 -> 60.4 us (walk 73 K -> 56 K of the block's 105 K cycles); 1 M: 47.5 -> 41.2 us;
+// 262144: 35.3 -> 33.6 us.  (Four elements a step from slots in fours: 59.2 us there, but more pieces above 4.2 M.)
+static_assert(BINS == 16 * SORT_THREADS, "four 16-byte words of a thread");
+static_assert(4 * SORT_PIECE / SORT_ROUND <= 64, "one bit per element of a thread");
+static_assert(SORT_PIECE < 65536 && SORT_SLOTS / 2 < 65536, "a bin's word");
+static_assert(SORT_SLOTS * 2 >= SORT_LIST * 4 + SORT_THREADS * 8, "the list lies where the elements will");
+static_assert(SEARCH_MAX_CAND <= 32 * (SORT_THREADS / 32), "a lane per candidate of its warp");
 __global__ void __launch_bounds__(SORT_THREADS, 1) search_sort_kernel(const SearchArgs a)
 {
     extern __shared__ __align__(16) uint8_t s_raw[];
-    uint32_t* words = reinterpret_cast<uint32_t*>(s_raw);                            // two 16-bit offsets each
-    const uint16_t* ends = reinterpret_cast<const uint16_t*>(s_raw);
-    uint16_t* sorted = reinterpret_cast<uint16_t*>(s_raw + BINS * 2);                // low bits, bin after bin
-    float* list = reinterpret_cast<float*>(s_raw + BINS * 2 + SORT_PIECE * 2);
-    double* acc = reinterpret_cast<double*>(list + SORT_LIST);                       // [candidates]
+    uint32_t* words = reinterpret_cast<uint32_t*>(s_raw);                            // start / 2 << 16 | count
+    uint16_t* sorted = reinterpret_cast<uint16_t*>(s_raw + BINS * 4);                // low bits, bin after bin
+    double* acc = reinterpret_cast<double*>(s_raw + BINS * 4 + SORT_SLOTS * 2);      // [candidates]
+    float* list = reinterpret_cast<float*>(sorted);                                  // (before there are sorted elements)
+    double* s_part = reinterpret_cast<double*>(list + SORT_LIST);
     __shared__ uint32_t s_warp[32];
-    __shared__ double s_red[32], s_part[SORT_THREADS];
+    __shared__ double s_red[32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ncand = a.n_enc * a.n_clip;
     const int c_lo = (int)((int64_t)blockIdx.y * ncand / gridDim.y), c_hi = (int)((int64_t)(blockIdx.y + 1) * ncand / gridDim.y);
-    const int base = first_key(a, lane);
-    for (int c = tid; c < c_hi - c_lo; c += SORT_THREADS)
-        acc[c] = 0.0;
 
     // four consecutive elements' magnitudes; 0 (which no candidate changes) past the end
     const bool vec = ((uintptr_t)a.x % 16) == 0;
@@ -444,45 +455,57 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) search_sort_kernel(const Sear
     const int64_t share = round_up((a.n + gridDim.x - 1) / gridDim.x, 4);
     const int64_t lo = min((int64_t)blockIdx.x * share, a.n), hi = min(lo + share, a.n);
     const int pieces = (int)((hi - lo + SORT_PIECE - 1) / SORT_PIECE);
+    const int base = first_key(a, lane);
+    for (int c = tid; c < c_hi - c_lo; c += SORT_THREADS)
+        acc[c] = 0.0;
     double spread_sq = 0.0;
     bool nan = false;
     for (int piece = 0; piece < pieces; ++piece) {
         const int64_t p_lo = lo + round_up((hi - lo) * piece / pieces, 4);
         const int64_t p_hi = piece + 1 == pieces ? hi : lo + round_up((hi - lo) * (piece + 1) / pieces, 4);
-        for (int w = tid; w < BINS / 8; w += SORT_THREADS)
-            reinterpret_cast<uint4*>(words)[w] = make_uint4(0, 0, 0, 0);
+        uint32_t v[SORT_FLIGHT][4];
+        auto load = [&](int64_t k) {
+#pragma unroll
+            for (int f = 0; f < SORT_FLIGHT; ++f)
+                load4(k + f * SORT_ROUND + 4 * tid, p_hi, v[f]);
+        };
+        load(p_lo);
+#pragma unroll
+        for (int w = 0; w < BINS / 4; w += SORT_THREADS)
+            reinterpret_cast<uint4*>(words)[w + tid] = make_uint4(0, 0, 0, 0);
         __syncthreads();
 
         // counts per bin; one bit of `outside` per element of this thread that has none
-        uint32_t outside = 0;
-        uint32_t v[4], next[4];
-        load4(p_lo + 4 * tid, p_hi, v);
-        int round = 0;
-        for (int64_t k = p_lo + 4 * tid; k < p_hi; k += 4 * SORT_THREADS, ++round) {
-            load4(k + 4 * SORT_THREADS, p_hi, next);
+        uint64_t outside = 0;
+        for (int64_t k = p_lo; k < p_hi; k += SORT_FLIGHT * SORT_ROUND) {
+            if (k > p_lo)
+                load(k);
+            const int first = (int)(k - p_lo) / SORT_ROUND * 4;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int key = (int)(v[q] >> LOW_BITS) - base;
-                if ((unsigned)key < (unsigned)BINS && v[q] != 0) {
-                    atomicAdd(words + (key >> 1), 1u << ((key & 1) * 16));
-                    const float centre = __uint_as_float((v[q] & ~((1u << LOW_BITS) - 1)) | (1u << (LOW_BITS - 1)));
-                    const double d = (double)(__uint_as_float(v[q]) - centre);
-                    spread_sq = fma(d, d, spread_sq);
-                } else if (v[q] != 0) {
-                    outside |= 1u << (4 * round + q);
+            for (int f = 0; f < SORT_FLIGHT; ++f)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t bits = v[f][q];
+                    const int key = (int)(bits >> LOW_BITS) - base;
+                    if ((unsigned)key < (unsigned)BINS && bits != 0) {
+                        atomicAdd(words + key, 1u);
+                        const float centre = __uint_as_float((bits & ~((1u << LOW_BITS) - 1)) | (1u << (LOW_BITS - 1)));
+                        const double d = (double)(__uint_as_float(bits) - centre);
+                        spread_sq = fma(d, d, spread_sq);
+                    } else if (bits != 0) {
+                        outside |= 1ull << (first + 4 * f + q);
+                    }
                 }
-                v[q] = next[q];
-            }
         }
         if (__syncthreads_or(outside != 0)) {
             // elements below or above the bins (and infinities and NaNs): every thread puts its own into the list, in
             // thread order, then applies its candidates to the whole list; more than the list holds: in several turns
-            uint32_t total, at = block_scan((uint32_t)__popc(outside), s_warp, total);
+            uint32_t total, at = block_scan((uint32_t)__popcll(outside), s_warp, total);
             for (uint32_t first = 0; first < total; first += SORT_LIST) {
                 while (outside && at < first + SORT_LIST) {
-                    const int e = __ffs(outside) - 1;
+                    const int e = __ffsll((long long)outside) - 1;
                     outside &= outside - 1;
-                    const uint32_t bits = __float_as_uint(__ldg(a.x + p_lo + (int64_t)(e >> 2) * (4 * SORT_THREADS) + 4 * tid + (e & 3)));
+                    const uint32_t bits = __float_as_uint(__ldg(a.x + p_lo + (int64_t)(e >> 2) * SORT_ROUND + 4 * tid + (e & 3)));
                     nan |= (bits & 0x7fffffffu) > 0x7f800000u;
                     list[at++ - first] = __uint_as_float(bits & 0x7fffffffu);
                 }
@@ -553,115 +576,153 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) search_sort_kernel(const Sear
             }
         }
 
-        // exclusive offsets, in place
+        // starts, in place of the counts, which the elements' placing counts up again; zeros in all slots
         {
-            uint4* mine = reinterpret_cast<uint4*>(words) + tid * (BINS / 8 / SORT_THREADS);
-            uint32_t sum = 0;
+            uint4* mine = reinterpret_cast<uint4*>(words) + warp * 128 + lane;
+            auto padded = [](uint32_t count) { return (count + 1) & ~1u; };
+            uint32_t below[4], run = 0;
+            uint4 t[4];
 #pragma unroll
-            for (int q = 0; q < BINS / 8 / SORT_THREADS; ++q) {
-                const uint4 t = mine[q];
-                const uint32_t s2 = (t.x & 0xffff) + (t.x >> 16) + (t.y & 0xffff) + (t.y >> 16) + (t.z & 0xffff) +
-                                    (t.z >> 16) + (t.w & 0xffff) + (t.w >> 16);
-                sum += s2;
+            for (int q = 0; q < 4; ++q) {
+                t[q] = mine[32 * q];
+                const uint32_t sum = padded(t[q].x) + padded(t[q].y) + padded(t[q].z) + padded(t[q].w);
+                uint32_t incl = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+                    incl += lane >= o ? u : 0u;
+                }
+                below[q] = run + incl - sum;
+                run += __shfl_sync(0xffffffffu, incl, 31);
             }
-            uint32_t total, run = block_scan(sum, s_warp, total);
-            auto step = [&](uint32_t& t) {
-                const uint32_t first = run, second = run + (t & 0xffff);
-                run = second + (t >> 16);
-                t = first | (second << 16);
+            if (lane == 0)
+                s_warp[warp] = run;
+            __syncthreads();
+            const uint32_t of_warp = s_warp[lane], total = __reduce_add_sync(0xffffffffu, of_warp);
+            const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0u);
+            uint32_t at = 0;
+            auto place = [&](uint32_t& word) {
+                const uint32_t count = word;
+                word = at << 15;
+                at += padded(count);
             };
 #pragma unroll
-            for (int q = 0; q < BINS / 8 / SORT_THREADS; ++q) {
-                uint4 t = mine[q];
-                step(t.x), step(t.y), step(t.z), step(t.w);
-                mine[q] = t;
+            for (int q = 0; q < 4; ++q) {
+                at = before + below[q];
+                place(t[q].x), place(t[q].y), place(t[q].z), place(t[q].w);
+                mine[32 * q] = t[q];
             }
+            for (uint32_t w = tid; w * 8 < total; w += SORT_THREADS)
+                reinterpret_cast<uint4*>(sorted)[w] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
 
-        // low bits to their places; afterwards a bin's 16-bit offset is where it ends
-        load4(p_lo + 4 * tid, p_hi, v);
-        for (int64_t k = p_lo + 4 * tid; k < p_hi; k += 4 * SORT_THREADS) {
-            load4(k + 4 * SORT_THREADS, p_hi, next);
+        // low bits to their places
+        for (int64_t k = p_lo; k < p_hi; k += SORT_FLIGHT * SORT_ROUND) {
+            load(k);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int key = (int)(v[q] >> LOW_BITS) - base;
-                if ((unsigned)key < (unsigned)BINS && v[q] != 0) {
-                    const int sh = (key & 1) * 16;
-                    const uint32_t at = (atomicAdd(words + (key >> 1), 1u << sh) >> sh) & 0xffffu;
-                    sorted[at] = (uint16_t)(v[q] & ((1u << LOW_BITS) - 1));
+            for (int f = 0; f < SORT_FLIGHT; ++f)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t bits = v[f][q];
+                    const int key = (int)(bits >> LOW_BITS) - base;
+                    if ((unsigned)key < (unsigned)BINS && bits != 0) {
+                        const uint32_t word = atomicAdd(words + key, 1u);
+                        sorted[(word >> 16) * 2 + (word & 0xffffu)] = (uint16_t)(bits & ((1u << LOW_BITS) - 1));
+                    }
                 }
-                v[q] = next[q];
-            }
         }
         __syncthreads();
 
         // the block's share of the global table (which the kernel in front empties)
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        for (int b = blockIdx.y == 0 ? tid : BINS; b < BINS; b += SORT_THREADS) {
-            const int s0 = b ? ends[b - 1] : 0, s1 = ends[b];
-            if (s1 > s0) {
-                unsigned long long sum = 0;
-                for (int e = s0; e < s1; ++e)
-                    sum += sorted[e];
-                atomicAdd(a.bin_sum + b, sum | ((unsigned long long)(s1 - s0) << PACK_SHIFT));
+        // (every block starts elsewhere: atomics of many blocks on one bin wait for each other)
+        for (int turn = blockIdx.y == 0 ? 0 : BINS / SORT_THREADS; turn < BINS / SORT_THREADS; ++turn) {
+            const int b = (turn + (int)blockIdx.x) % (BINS / SORT_THREADS) * SORT_THREADS + tid;
+            const uint32_t word = words[b], count = word & 0xffffu;
+            if (count) {
+                const uint32_t* at = reinterpret_cast<const uint32_t*>(sorted) + (word >> 16);
+                uint32_t sum = 0;                               // (below 2^29)
+#pragma unroll 1
+                for (uint32_t e = 0; e < count; e += 2) {
+                    const uint32_t l = *at++;
+                    sum += (l & 0xffffu) + (l >> 16);
+                }
+                atomicAdd(a.bin_sum + b, sum | ((unsigned long long)count << PACK_SHIFT));
             }
         }
 
         // What the thresholds change: a warp per candidate, four thresholds per lane (their look-ups in flight
         // together).  x - mu = (low bits of x - low bits of the threshold) * ulp - (mu - threshold), the last difference
         // with a single rounding, so FP32 is enough.
-        int known = -1;
-        float mid[4], step[4];
-        for (int c = c_lo + warp; c < c_hi; c += SORT_THREADS / 32) {
-            uint32_t at[4], span[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                at[q] = __ldcg(a.threshold + c * MAX_THRESHOLDS + 32 * q + lane);
-            int i;
-            float scale;
-            candidate_scale(a, c, i, scale);
+        // Lane j has the encoding, the scale and the result of the warp's j-th candidate.  (Neighbouring candidates: most
+        // warps stay with one encoding.)
+        const int per_warp = (c_hi - c_lo + SORT_THREADS / 32 - 1) / (SORT_THREADS / 32);
+        const int c_first = c_lo + warp * per_warp, count_c = min(per_warp, c_hi - c_first);
+        int known = -1, its_enc = 0;
+        float its_scale = 0.f, its_sum = 0.f, mid[4], step[4];
+        if (lane < count_c)
+            candidate_scale(a, c_first + lane, its_enc, its_scale);
+        const char4* nudges = a.nudge + c_first * 32 + lane;
+        char4 next = count_c > 0 ? __ldcg(nudges) : char4{};
+        for (int turn = 0; turn < count_c; ++turn) {
+            const char4 nudge = next;
+            nudges += 32;
+            if (turn + 1 < count_c)
+                next = __ldcg(nudges);
+            const int i = __shfl_sync(0xffffffffu, its_enc, turn);
+            const float scale = __shfl_sync(0xffffffffu, its_scale, turn);
             if (i != known) {
                 known = i;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int k = 32 * q + lane;
-                    mid[q] = code_midpoint(a.enc[i], k);
+                    mid[q] = k >= a.enc[i].thresholds ? INFINITY : code_midpoint(a.enc[i], k);
                     step[q] = k >= a.enc[i].thresholds ? 0.f
                               : __uint_as_float((uint32_t)((max(k >> a.enc[i].m, 1) - a.enc[i].m) << 23) + a.enc[i].bias_bits);
                 }
             }
+            uint32_t at[4], span[4];
+            const int off[4] = {nudge.x, nudge.y, nudge.z, nudge.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
+                at[q] = __float_as_uint(__fmul_rn(mid[q], scale)) + (uint32_t)off[q];
                 const int key = (int)(at[q] >> LOW_BITS) - base;
-                // (a threshold on a bin's edge has the whole bin above it; 0xffffffff, no threshold, has no bin)
+                // (a threshold on a bin's edge has the whole bin above it; one that is not there, at infinity, has no bin)
                 const bool cuts = (unsigned)key < (unsigned)BINS && (at[q] & ((1u << LOW_BITS) - 1)) != 0;
-                span[q] = cuts ? (uint32_t)(key ? ends[key - 1] : 0) | ((uint32_t)ends[key] << 16) : 0u;
+                span[q] = cuts ? words[key] : 0u;
             }
             float s = 0.f;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint32_t low = at[q] & ((1u << LOW_BITS) - 1), s1 = span[q] >> 16;
-                uint32_t cnt = 0, over = 0;
-                for (uint32_t e = span[q] & 0xffffu; e < s1; ++e) {
-                    const uint32_t l = sorted[e];
-                    if (l >= low) {
-                        ++cnt;
-                        over += l - low;
-                    }
-                }
-                if (cnt) {
+                const uint32_t count = span[q] & 0xffffu;
+                if (count) {
+                    const uint32_t less = ((1u - (at[q] & ((1u << LOW_BITS) - 1))) & 0xffffu) * 0x10001u;
+                    const uint32_t* p = reinterpret_cast<const uint32_t*>(sorted) + (span[q] >> 16);
+                    const uint32_t* const end = p + (count + 1) / 2;
+                    uint32_t hits = 0, over = 0;                // (hits: two halves)
+#pragma unroll 1
+                    do {
+                        // per half: 0 below the threshold, else 1 + by how much above
+                        const uint32_t l = p + 1 < end ? p[1] : 0u;
+                        const uint32_t d0 = __viaddmax_s16x2_relu(p[0], less, 0u), d1 = __viaddmax_s16x2_relu(l, less, 0u);
+                        hits += __vminu2(d0, 0x00010001u) + __vminu2(d1, 0x00010001u);
+                        over = __dp2a_lo(d0 + d1, 0x0101u, over);
+                        p += 2;
+                    } while (p < end);
+                    const uint32_t cnt = (hits & 0xffffu) + (hits >> 16);
                     const float ulp_up = __uint_as_float(max(at[q] & 0x7f800000u, 1u << 23));       // 2^23 ulps
                     const float past = __fmaf_rn(scale, mid[q], -__uint_as_float(at[q]));           // mu - threshold
-                    s = __fmaf_rn(step[q] * scale, __fmaf_rn((float)over * 0x1p-23f, ulp_up, -(float)cnt * past), s);
+                    s = __fmaf_rn(step[q] * scale, __fmaf_rn((float)(over - cnt) * 0x1p-23f, ulp_up, -(float)cnt * past), s);
                 }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
                 s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0)
-                acc[c - c_lo] -= 2.0 * (double)s;
+            its_sum = lane == turn ? s : its_sum;
         }
+        if (lane < count_c)
+            acc[c_first - c_lo + lane] -= 2.0 * (double)its_sum;
         __syncthreads();
     }
 
@@ -838,7 +899,7 @@ size_t search_workspace_bytes(int n_enc, int n_clip)
 
 // Scratch of the sorted form inside the workspace (which is 8-byte aligned): offsets from its first 16-byte boundary.
 struct SortScratch {
-    size_t below, below_sq, bin_sum, threshold, spread_sq, partial, ticket, bytes;
+    size_t below, below_sq, bin_sum, threshold, nudge, spread_sq, partial, ticket, bytes;
 };
 static SortScratch sort_scratch(int ncand)
 {
@@ -847,7 +908,8 @@ static SortScratch sort_scratch(int ncand)
     s.below_sq = s.below + sizeof(ulonglong2) * (BINS + MAX_THRESHOLDS);
     s.bin_sum = s.below_sq + sizeof(ulonglong2) * (BINS + MAX_THRESHOLDS);
     s.threshold = s.bin_sum + sizeof(unsigned long long) * BINS;
-    s.spread_sq = s.threshold + sizeof(uint32_t) * MAX_THRESHOLDS * (size_t)ncand;
+    s.nudge = s.threshold + sizeof(uint32_t) * MAX_THRESHOLDS * (size_t)ncand;
+    s.spread_sq = s.nudge + sizeof(char4) * 32 * (size_t)ncand;
     s.partial = s.spread_sq + sizeof(double) * SORT_BLOCKS;
     s.ticket = s.partial + sizeof(double) * SORT_BLOCKS * (size_t)ncand;
     s.bytes = s.ticket + sizeof(unsigned) + 8;
@@ -855,21 +917,24 @@ static SortScratch sort_scratch(int ncand)
 }
 
 // In how many shares the candidates are walked: every share sorts all elements again, and walks fewer candidates.  Pays
-// while a block's elements are few (444 candidates, 262144 elements: 54 us alone, 46 in two, 41 in four shares; 3.7 M
-// elements: 75, 104, 154 us).
-static int sort_shares(int64_t n)
+// while a block's elements are few beside the candidates (444 candidates in 1, 2, 4, 8 shares: 262144 elements 45.5, 37.9,
+// 33.6, 32.3 us, 1 M elements 48.6, 42.0, 41.2, 48.5, 1.6 M elements 50.5, 47.1, 47.7, 72.1; 222 candidates: 400000 elements
+// 31.2, 28.5, 27.9, 31.7, 1 M elements 32.2, 30.2, 33.2, 42.3).
+static int sort_shares(int64_t n, int ncand)
 {
     int shares = 4;
-    while (shares > 1 && n * shares > (int64_t)SORT_BLOCKS * (SORT_PIECE / 2))
+    while (shares > 1 && n * shares > (int64_t)7000 * ncand)
         shares /= 2;
     return shares;
 }
 
-// The sorted form has a fixed cost (444 candidates: 30 us direct and 34 us sorted at 131072 elements, 45 and 34 us at
-// 196608; 222 candidates: 32 and 31 us at 262144), and its tables have to fit the workspace (170 candidates or more).
+// The sorted form has a fixed cost that grows less with the candidates than the direct form's time (444 candidates: 29.7 us
+// direct and 31.9 us sorted at 131072 elements, 41.7 and 33.5 at 200000; 222 candidates: 26.6 and 26.9 us at 200000, 32.5
+// and 26.9 at 262144), and its tables have to fit the workspace (90 candidates or more).
 static bool sorted_form(int64_t n, int n_enc, int n_clip)
 {
-    return n * n_enc * n_clip >= 75000000 && sort_scratch(n_enc * n_clip).bytes <= search_workspace_bytes(n_enc, n_clip);
+    const int64_t ncand = n_enc * n_clip;
+    return n * ncand >= 26000000 + 86000 * ncand && sort_scratch((int)ncand).bytes <= search_workspace_bytes(n_enc, n_clip);
 }
 
 static fpq_status launch_sorted(SearchArgs a, void* workspace, cudaStream_t st)
@@ -881,6 +946,7 @@ static fpq_status launch_sorted(SearchArgs a, void* workspace, cudaStream_t st)
     a.below_sq = (ulonglong2*)(ws + s.below_sq);
     a.bin_sum = (unsigned long long*)(ws + s.bin_sum);
     a.threshold = (uint32_t*)(ws + s.threshold);
+    a.nudge = (char4*)(ws + s.nudge);
     a.spread_sq = (double*)(ws + s.spread_sq);
     a.partial = (double*)(ws + s.partial);
     a.ticket = (unsigned*)(ws + s.ticket);
@@ -895,7 +961,7 @@ static fpq_status launch_sorted(SearchArgs a, void* workspace, cudaStream_t st)
         done += a.n;
         a.add_to = part > 0;
         a.divide_by = part + 1 == parts ? (double)total : 0.0;
-        const int shares = sort_shares(a.n);
+        const int shares = sort_shares(a.n, ncand);
         a.blocks = SORT_BLOCKS / shares;
         search_tables_kernel<<<(ncand * MAX_THRESHOLDS + 255) / 256, 256, 0, st>>>(a);
         cudaLaunchConfig_t cfg = {};

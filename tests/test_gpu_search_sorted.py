@@ -93,3 +93,26 @@ def test_nan_in_a_large_tensor():
     got, best = _search(x, FP8, O.clip_candidates(4.0, 111))
     assert fpq.fpq_read_status() == fpq.ERR_NAN_INPUT
     assert np.isnan(got).all() and best == (-1, -1)
+
+
+def _crowd(n, rng):
+    # most elements in one bin, some of its neighbours with odd counts, thresholds of many candidates through it
+    x = (1.0 + rng.integers(0, 4096, n) * 2.0 ** -23).astype(np.float32)
+    x[:: 1000] = rng.uniform(0.25, 2.0, x[:: 1000].size)
+    return x * rng.choice([-1.0, 1.0], n).astype(np.float32)
+
+
+# 180 candidates: from 230445 elements on sorted, four shares up to 315000 and two up to 630000; a block sorts up to 61440
+# elements at a time
+@pytest.mark.parametrize("kind", ["normal", "crowd"])
+@pytest.mark.parametrize("n", [230444, 230445, 315000, 315001, 630001, 148 * 61440, 148 * 61440 + 1])
+def test_shares_and_pieces(kind, n):
+    rng = np.random.default_rng(n)
+    x = _data("normal", n, rng) if kind == "normal" else _crowd(n, rng)
+    clips = O.clip_candidates(float(np.abs(x).max()), 30)
+    pick = [3, 20] if n > 1000000 else [0, 7, 14, 21, 29]
+    got, best = _search(torch.from_numpy(x).cuda(), FP8 + FP4, clips)
+    assert fpq.fpq_read_status() == fpq.OK
+    want = O.search_mse(x, O.FP8_ENCODINGS + O.FP4_ENCODINGS, clips[pick])
+    np.testing.assert_allclose(got[:, pick], want, rtol=RTOL, atol=0)
+    assert best == O.select_encoding_and_bias(got)
