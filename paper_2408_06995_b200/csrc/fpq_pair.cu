@@ -576,11 +576,32 @@ bool pair_conv_applies(const GemmProblem& p)
     return plan_pair(p, g, &dyn) == FPQ_OK;
 }
 
-// Shapes on which this kernel measured faster than quantize kernel + contraction kernel on B200: one 128-channel
-// chunk (with two chunks the two-kernel route's split reduction still wins).
+// Shapes on which this kernel is faster than quantize kernel + contraction kernel (both measured, us, one / two kernels;
+// two chunks of channels or more go to the two kernels, whose contraction may split the reduction).
+//  - A few tiles per SM or less cannot fill the chain of load, conversion, MMA and store: 128 -> 128 channels at 32 x 32,
+//    batch 2 (19 tiles) 8.6 / 7.0, 9 (82 tiles) 9.1 / 9.2, 35 (317 tiles) 15.5 / 16.3, 64 (578 tiles) 22.0 / 23.1.
+//  - Several taps: the accumulators and weights of more than 128 outputs leave the activations too little shared memory
+//    (128 -> 256 at 32 x 32, batch 35: 27.6 / 20.8; at 64 x 64, batch 18: 54.7 / 35.1).
+//  - Half a warp converts 16 pixel pairs of a channel: narrow rows leave lanes idle (128 -> 128 at 20 x 20, batch 45:
+//    13.1 / 11.6; 28 x 28, batch 23: 12.0 / 11.5, with 64 channels to convert 11.8 / 12.0).  With a full chunk of channels
+//    rows above 32 leave a box a single row (64 x 64, batch 18: 25.1 / 24.3; 64 channels there 24.0 / 25.3), and up to 64
+//    outputs the two kernels' narrow column tile is as fast (128 -> 64 at 32 x 32, batch 35: 13.6 / 13.1; from 64: 13.3 / 13.6).
+//  - One tap: 128 -> 128 at 64 x 64, batch 1 (32 tiles) 6.1 / 6.2, 18 (576) 14.9 / 18.5; at 32 x 32, batch 2 (16) 6.6 / 6.2,
+//    9 (72) 6.9 / 7.0; at 28 x 28, batch 46: 12.2 / 11.5.  -> 256 at 64 x 64, batch 2 (64) 7.7 / 7.3, 4 (128) 8.3 / 9.9; at
+//    28 x 28, batch 46 14.4 / 15.4; at 20 x 20, batch 45 10.9 / 10.2.  More outputs: slower at any size.
 bool pair_conv_preferred(const GemmProblem& p)
 {
-    return pair_conv_applies(p) && p.Cp / BK == 1;
+    PairArgs g;
+    int dyn = 0;
+    if (plan_pair(p, g, &dyn) != FPQ_OK || g.cchunks != 1)
+        return false;
+    if (g.taps < 4 && p.N > 128)
+        return p.W >= 28 && g.m_tiles >= 128;
+    if (g.taps < 4)
+        return p.W >= 32 && g.m_tiles >= (p.W >= 64 ? 32 : 64);
+    if (p.N > 128 || g.m_tiles < 80)
+        return false;
+    return p.C <= 64 ? p.W >= 28 : p.N > 64 && p.W == 32;
 }
 
 fpq_status launch_pair_conv(const GemmProblem& p, cudaStream_t st)
