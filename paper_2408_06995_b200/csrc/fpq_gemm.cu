@@ -62,7 +62,7 @@ struct GemmArgs {
     int nblk;                  // blocks per tile = cchunks * taps
     int Wp, HpWp;              // framed geometry
     FastDiv div_HpWp, div_Wp, div_tiles, div_Wt, div_Ht, div_tx, div_ty;
-    int Wt, Ht, Bt;            // TAPS: tile of Wt * Ht * Bt = 128 output pixels
+    int Wt, Ht, Bt;            // TAPS: tile of Wt * Ht * Bt <= 128 output pixels (choose_taps_tile)
     int tiles_x, tiles_y;
     int Ho, Wo, B;
     int m_tiles, n_tiles;
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                 ox = x0 + (row - (int)q1 * g.Wt);
                 const uint32_t q2 = fdiv(q1, g.div_Ht);
                 oy = y0 + ((int)q1 - (int)q2 * g.Ht);
-                b = b0 + (int)q2;
+                b = (int)q2 < g.Bt ? b0 + (int)q2 : g.B;
             }
             row_valid = ox < g.Wo && oy < g.Ho && b < g.B;
             nstride = (int64_t)g.Ho * g.Wo;
@@ -1087,12 +1087,30 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
 // ---- host side --------------------------------------------------------------------------
 static EncodeTiledFn encode_fn() { return tensor_map_encoder(); }
 
-static int pow2_at_least(int v)
+// Tile of output pixels of a convolution whose taps are loaded apart: rows of the image cut into equal parts of at most
+// 128 pixels, then as many image rows and images as 128 pixels hold, the cut with the fewest tiles.
+// (Powers of two would use 25 of 32 pixels of a row; 64 -> 64 channels at 33 x 33, stride 2, batch 30: 12.2 us so, 10.7 now.)
+TapsTile choose_taps_tile(int B, int Ho, int Wo, int stride)
 {
-    int p = 1;
-    while (p < v)
-        p <<= 1;
-    return p;
+    int wcap = 256 / stride;                           // (a box spans at most 256 framed pixels)
+    if (wcap > BM)
+        wcap = BM;
+    TapsTile best = {};
+    for (int cut = (Wo + wcap - 1) / wcap; cut <= Wo; ++cut) {
+        TapsTile t;
+        t.w = (Wo + cut - 1) / cut;
+        t.tiles_x = (Wo + t.w - 1) / t.w;
+        const int hmax = BM / t.w < wcap ? BM / t.w : wcap;
+        t.tiles_y = (Ho + hmax - 1) / hmax;
+        t.h = (Ho + t.tiles_y - 1) / t.tiles_y;
+        t.b = BM / (t.w * t.h) < B ? BM / (t.w * t.h) : B;
+        t.tiles = (int64_t)t.tiles_x * t.tiles_y * ((B + t.b - 1) / t.b);
+        if (best.w == 0 || t.tiles < best.tiles)
+            best = t;
+        if (t.w <= 8)
+            break;                                     // (narrower: short runs of memory)
+    }
+    return best;
 }
 
 struct DeviceInfo {
@@ -1538,20 +1556,13 @@ fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st)
             if (p.stride < 1 || p.stride > 8)
                 return FPQ_ERR_UNSUPPORTED;
             g.mode = MODE_TAPS;
-            int wcap = 256 / p.stride;
-            if (wcap > BM)
-                wcap = BM;
-            g.Wt = pow2_at_least(p.Wo);
-            if (g.Wt > wcap)
-                g.Wt = wcap;
-            g.Ht = pow2_at_least(p.Ho);
-            if (g.Ht > BM / g.Wt)
-                g.Ht = BM / g.Wt;
-            g.Bt = BM / (g.Wt * g.Ht);
-            g.tiles_x = (p.Wo + g.Wt - 1) / g.Wt;
-            g.tiles_y = (p.Ho + g.Ht - 1) / g.Ht;
-            const int tiles_b = (p.B + g.Bt - 1) / g.Bt;
-            mtiles = (int64_t)g.tiles_x * g.tiles_y * tiles_b;
+            const TapsTile t = choose_taps_tile(p.B, p.Ho, p.Wo, p.stride);
+            g.Wt = t.w;
+            g.Ht = t.h;
+            g.Bt = t.b;
+            g.tiles_x = t.tiles_x;
+            g.tiles_y = t.tiles_y;
+            mtiles = t.tiles;
             g.a_boxes = 1;
             g.a_box_rows = BM;
             dimsA[0] = (cuuint64_t)p.Ca; dimsA[1] = (cuuint64_t)Wp; dimsA[2] = (cuuint64_t)Hp; dimsA[3] = (cuuint64_t)p.B;
@@ -1573,7 +1584,7 @@ fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st)
     g.div_tx = make_fastdiv((uint32_t)g.tiles_x);
     g.div_ty = make_fastdiv((uint32_t)g.tiles_y);
     g.a_chunk_bytes = g.a_boxes * g.a_box_rows * 128;
-    g.a_chunk_tx = (uint32_t)g.a_chunk_bytes;
+    g.a_chunk_tx = g.mode == MODE_TAPS ? (uint32_t)(g.Wt * g.Ht * g.Bt * 128) : (uint32_t)g.a_chunk_bytes;
     if (enc(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, (void*)p.a_codes, dimsA, stridesA, boxA, estrA,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)

@@ -72,6 +72,12 @@ struct GemmProblem {
     float x_scale2;
 };
 
+struct TapsTile {
+    int w, h, b, tiles_x, tiles_y;   // w * h * b <= 128 output pixels
+    int64_t tiles;
+};
+TapsTile choose_taps_tile(int B, int Ho, int Wo, int stride);   // B, Ho, Wo >= 1
+
 // Returns FPQ_OK or an error; enqueues one kernel.
 fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st);
 

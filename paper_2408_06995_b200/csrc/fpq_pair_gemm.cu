@@ -1,4 +1,4 @@
-// The low-bit contraction of a stride-1 convolution on CTA pairs (tcgen05 cta_group::2, M = 256): the
+// The low-bit contraction of a convolution on CTA pairs (tcgen05 cta_group::2, M = 256): the
 // wide-MMA form for layers whose time is the tensor cores' (long reductions, many output channels).
 // Activation codes come from the quantize kernel (zero-framed channels-last E4M3, as for the general
 // contraction), weights from the prepared copy; both are streamed by TMA.
@@ -14,6 +14,14 @@
 //
 // A layer whose input is two concatenated tensors with their own scales keeps one accumulator per tensor, joined in the
 // epilogue.
+//
+// 3 x 3 windows at stride 2 (PHASED): the framed image falls into four sub-images by the parities of row and column, and
+// within one of them the taps are rows of one loaded operand again.  Per chunk four boxes of every second pixel are
+// fetched instead of nine, into operands that all taps of a phase share: the general contraction, which loads every tap
+// apart, is bound by that fetch (some 43 bytes per clock and SM: 32 KB per block of 4 MMAs).  A tile is a box of
+// output pixels whose rows and columns in the operand are one longer than its own.  The many small loads need a thread
+// per operand.  320 -> 320 channels, batch 3 at 45 x 77, whole layer: 16.2 -> 12.5 us; batch 2 at 64 x 64: 17.0 -> 11.6;
+// 512 -> 1280, batch 7 at 48 x 48: 41.7 -> 28.0.
 #include <cuda.h>
 
 #include <mutex>
@@ -29,7 +37,8 @@ namespace {
 constexpr int BM = 128;
 constexpr int BK = 128;
 constexpr int EPI_W0 = 2, NUM_EPI = 8;
-constexpr int NTHREADS = 32 * (EPI_W0 + NUM_EPI);
+constexpr int B_WARP = EPI_W0 + NUM_EPI;       // stride 2 only
+constexpr int num_threads(bool phased) { return 32 * (B_WARP + (phased ? 1 : 0)); }
 constexpr int SMEM_BUDGET = 227 * 1024;
 
 struct PGArgs {
@@ -49,7 +58,9 @@ struct PGArgs {
     int b_tap_bytes, b_stage_bytes, b_stages;
     uint32_t a_tx, b_tx;       // bytes one CTA's loads of a stage report
     uint32_t idesc, tmem_cols;
-    int wait_prior_grid;
+    // stride 2: a tile of w x h x nb output pixels, row (ib * h2 + iy) * w2 + ix of its operand (w2 = w + 1, h2 = h + 1)
+    int w, h, nb, w2, h2, tiles_x, tiles_y;
+    FastDiv div_tx, div_ty, div_w2, div_h2;
     int n_pad;                 // N rounded up to the column tile: x_scale * w_scale[n] and bias[n] of all columns sit in shared memory
     const float* w_scale;
     float x_scale;
@@ -58,7 +69,15 @@ struct PGArgs {
     int* status;
 };
 
-__global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
+// The nine taps of a 3 x 3 window at stride 2, those of one phase (parity of the framed row and column) together: the
+// phases' sub-images are loaded one after the other, and a tap reads its phase's operand whole rows further down.
+__device__ constexpr int TAP_ORDER[9] = {0, 2, 6, 8, 1, 7, 3, 5, 4};
+__device__ constexpr int TAP_DOWN[9] = {0, 0, 1, 1, 0, 1, 0, 0, 0}, TAP_RIGHT[9] = {0, 1, 0, 1, 0, 0, 0, 1, 0};
+__device__ constexpr bool phase_first(int i) { return i == 0 || i == 4 || i == 6 || i == 8; }
+__device__ constexpr bool phase_last(int i) { return i == 3 || i == 5 || i == 7 || i == 8; }
+
+template <bool PHASED>
+__global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                     const __grid_constant__ CUtensorMap tmB,
                                                                     const PGArgs g)
 {
@@ -117,8 +136,64 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
         mu = (int)fdiv((uint32_t)u, g.div_nt);
         nt = u - mu * g.n_tiles;
     };
+    auto tile_origin = [&](int mt, int& x0, int& y0, int& b0) {
+        const uint32_t r1 = fdiv((uint32_t)mt, g.div_tx), r2 = fdiv(r1, g.div_ty);
+        x0 = (mt - (int)r1 * g.tiles_x) * g.w;
+        y0 = ((int)r1 - (int)r2 * g.tiles_y) * g.h;
+        b0 = (int)r2 * g.nb;
+    };
 
-    if (warp == 0) {
+    if (PHASED && warp == 0) {
+        // ---------------- stride 2: activation producer, four phases per chunk ----------------
+        if (elect_one()) {
+            uint32_t sa = 0, pa = 1;
+            bool dead = false;
+            const uint32_t full = leader(a_full);
+            for (int u = u_lo; u < u_hi && !dead; ++u) {
+                int mu, nt, x0, y0, b0;
+                decode(u, mu, nt);
+                tile_origin(2 * mu + (int)rank, x0, y0, b0);
+                for (int cc = 0; cc < g.cchunks && !dead; ++cc)
+                    for (int ph = 0; ph < 4; ++ph) {
+                        if (!mbar_wait(a_empty + 8 * sa, pa)) { dead = true; break; }
+                        if (rank == 0)
+                            mbar_expect_tx(a_full + 8 * sa, 2u * g.a_tx);
+                        tma_load_4d_pair(a_ring + sa * g.a_stage_bytes, &tmA, full + 8 * sa, cc * BK, 2 * x0 + (ph & 1),
+                                         2 * y0 + (ph >> 1), b0);
+                        if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
+                    }
+            }
+            if (dead)
+                flag_status(g.status, FPQ_ERR_TIMEOUT);
+        }
+    } else if (PHASED && warp == B_WARP) {
+        // ---------------- stride 2: weight producer ----------------
+        if (elect_one()) {
+            uint32_t sb = 0, pb = 1;
+            bool dead = false;
+            const uint32_t full = leader(b_full);
+            for (int u = u_lo; u < u_hi && !dead; ++u) {
+                int mu, nt;
+                decode(u, mu, nt);
+                const int n0 = nt * g.BN + (int)rank * BNh;
+                for (int cc = 0; cc < g.cchunks && !dead; ++cc) {
+#pragma unroll
+                    for (int i = 0; i < 9; i += 3) {
+                        if (!mbar_wait(b_empty + 8 * sb, pb)) { dead = true; break; }
+                        if (rank == 0)
+                            mbar_expect_tx(b_full + 8 * sb, 2u * g.b_tx);
+                        const uint32_t dst = b_ring + sb * g.b_stage_bytes;
+#pragma unroll
+                        for (int t = 0; t < 3; ++t)
+                            tma_load_3d_pair(dst + t * g.b_tap_bytes, &tmB, full + 8 * sb, cc * BK, n0, TAP_ORDER[i + t]);
+                        if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
+                    }
+                }
+            }
+            if (dead)
+                flag_status(g.status, FPQ_ERR_TIMEOUT);
+        }
+    } else if (!PHASED && warp == 0) {
         // ---------------- TMA producer: loads in the order the MMAs consume them ----------------
         if (elect_one()) {
             uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
@@ -163,7 +238,42 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
                 tc_fence_after();
                 uint32_t d = tmem_base + buf * (uint32_t)g.acc_cols;
                 bool first = true;
-                for (int cc = 0; cc < g.cchunks && !dead; ++cc) {
+                if (PHASED) {
+                    const uint32_t down8 = (uint32_t)g.w2 * 8u;
+                    for (int cc = 0; cc < g.cchunks && !dead; ++cc) {
+                        uint32_t abase = 0, bbase = 0;
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) {
+                            if (phase_first(i)) {
+                                if (!mbar_wait_cluster(a_full + 8 * sa, pa)) { dead = true; break; }
+                                abase = smem_desc_lo(a_ring + sa * g.a_stage_bytes);
+                            }
+                            if (i % 3 == 0) {
+                                if (!mbar_wait_cluster(b_full + 8 * sb, pb)) { dead = true; break; }
+                                bbase = smem_desc_lo(b_ring + sb * g.b_stage_bytes);
+                            }
+                            if (phase_first(i) || i % 3 == 0)
+                                tc_fence_after();
+                            const uint32_t al = abase + TAP_DOWN[i] * down8 + TAP_RIGHT[i] * 8u, bl = bbase + (i % 3) * TSTEP;
+                            if (i == 0 && cc == 0)
+                                mma_f8f6f4_pair<false>(d, al, bl, HI, g.idesc);
+                            else
+                                mma_f8f6f4_pair<true>(d, al, bl, HI, g.idesc);
+                            mma_f8f6f4_pair<true>(d, al + 2, bl + 2, HI, g.idesc);
+                            mma_f8f6f4_pair<true>(d, al + 4, bl + 4, HI, g.idesc);
+                            mma_f8f6f4_pair<true>(d, al + 6, bl + 6, HI, g.idesc);
+                            if (i % 3 == 2) {
+                                mma_commit_pair(b_empty + 8 * sb, 3);
+                                if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
+                            }
+                            if (phase_last(i)) {
+                                mma_commit_pair(a_empty + 8 * sa, 3);
+                                if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
+                            }
+                        }
+                    }
+                }
+                for (int cc = 0; !PHASED && cc < g.cchunks && !dead; ++cc) {
                     if (cc == g.seg_chunk && cc != 0) {
                         d += (uint32_t)g.BN;                       // the second tensor's accumulator
                         first = true;
@@ -225,12 +335,25 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_gemm_kernel(const __grid
             int mu, nt;
             decode(u, mu, nt);
             const int mt = 2 * mu + (int)rank;
-            const uint32_t q = (uint32_t)mt * BM + row;
-            const uint32_t b = fdiv(q, g.div_HpWp);
-            const uint32_t rem = q - b * (uint32_t)g.HpWp;
-            const int oy = (int)fdiv(rem, g.div_Wp);
-            const int ox = (int)rem - oy * g.Wp;
-            const bool row_valid = (int64_t)q < g.M && ox < g.Wo && oy < g.Ho && (int)b < g.B;
+            uint32_t b;
+            int oy, ox;
+            bool row_valid = true;
+            if (PHASED) {
+                const uint32_t q1 = fdiv((uint32_t)row, g.div_w2), q2 = fdiv(q1, g.div_h2);
+                const int ix = row - (int)q1 * g.w2, iy = (int)q1 - (int)q2 * g.h2;
+                int b0;
+                tile_origin(mt, ox, oy, b0);
+                ox += ix, oy += iy, b = (uint32_t)b0 + q2;
+                row_valid = ix < g.w && iy < g.h && (int)q2 < g.nb;
+            } else {
+                const uint32_t q = (uint32_t)mt * BM + row;
+                b = fdiv(q, g.div_HpWp);
+                const uint32_t rem = q - b * (uint32_t)g.HpWp;
+                oy = (int)fdiv(rem, g.div_Wp);
+                ox = (int)rem - oy * g.Wp;
+                row_valid = (int64_t)q < g.M;
+            }
+            row_valid = row_valid && ox < g.Wo && oy < g.Ho && (int)b < g.B;
             float* yrow = g.y + ((int64_t)b * g.N * g.Ho + oy) * g.Wo + ox;
             if (!mbar_wait(acc_full + 8 * buf, aph)) { dead = true; break; }
             tc_fence_after();
@@ -328,16 +451,43 @@ int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_
     return pick;
 }
 
+// Stride 2: image rows cut into equal parts, then as many image rows and images as the 128 operand rows hold, one column
+// and row of each sub-image more than the tile's (the second and third taps' reach); the cut with the fewest tiles.
+void choose_phase_tile(PGArgs& g)
+{
+    int64_t best = 0;
+    for (int cut = (g.Wo + 126) / 127; cut <= g.Wo; ++cut) {
+        const int w = (g.Wo + cut - 1) / cut, w2 = w + 1;
+        const int hmax = (BM - w) / w2 + 1, tiles_x = (g.Wo + w - 1) / w, tiles_y = (g.Ho + hmax - 1) / hmax;
+        const int h = (g.Ho + tiles_y - 1) / tiles_y, h2 = h + 1;
+        int nb = (BM - w - (h - 1) * w2) / (h2 * w2) + 1;
+        if (nb > g.B)
+            nb = g.B;
+        const int64_t tiles = (int64_t)tiles_x * tiles_y * ((g.B + nb - 1) / nb);
+        if (h2 <= 128 && (best == 0 || tiles < best)) {
+            best = tiles;
+            g.w = w, g.h = h, g.nb = nb, g.w2 = w2, g.h2 = h2, g.tiles_x = tiles_x, g.tiles_y = tiles_y;
+        }
+        if (w <= 8)
+            break;
+    }
+    g.m_tiles = (int)best;
+    g.div_tx = make_fastdiv((uint32_t)g.tiles_x);
+    g.div_ty = make_fastdiv((uint32_t)g.tiles_y);
+    g.div_w2 = make_fastdiv((uint32_t)g.w2);
+    g.div_h2 = make_fastdiv((uint32_t)g.h2);
+}
+
 // geometry and shared-memory plan; FPQ_ERR_UNSUPPORTED outside the kernel's range
 fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
 {
-    if (!p.conv || p.x != nullptr || p.stride != 1 || p.N < 1 || p.R * p.S > 64)
+    const bool phased = p.stride == 2;
+    if (!p.conv || p.x != nullptr || p.N < 1 || p.R * p.S > 64 ||
+        !(p.stride == 1 || (phased && p.R == 3 && p.S == 3 && p.c_seg == 0)))
         return FPQ_ERR_UNSUPPORTED;
     const int Hp = p.H + 2 * p.pad, Wp = p.W + 2 * p.pad;
     const int64_t framed = (int64_t)p.B * Hp * Wp;
-    const int halo_rows = BM + (p.R - 1) * Wp + (p.S - 1);
-    const int64_t flat_tiles = (framed + BM - 1) / BM;
-    if (halo_rows > 2 * 256 - 16 || framed >= 0x7fffff00ll)
+    if (framed >= 0x7fffff00ll)
         return FPQ_ERR_UNSUPPORTED;
     g = PGArgs{};
     g.M = framed;
@@ -352,23 +502,36 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
     g.div_Wp = make_fastdiv((uint32_t)Wp);
     g.div_HpWp = make_fastdiv((uint32_t)g.HpWp);
     g.B = p.B; g.Ho = p.Ho; g.Wo = p.Wo;
-    g.m_tiles = (int)flat_tiles;
+    int halo_rows;
+    if (phased) {
+        choose_phase_tile(g);
+        halo_rows = BM + g.w2 + 1;                     // (the last tap's reach; the box itself may be shorter)
+        if (g.nb * g.h2 * g.w2 > halo_rows)
+            halo_rows = g.nb * g.h2 * g.w2;
+        g.a_tx = (uint32_t)(g.nb * g.h2 * g.w2 * 128);
+    } else {
+        halo_rows = BM + (p.R - 1) * Wp + (p.S - 1);
+        g.m_tiles = (int)((framed + BM - 1) / BM);
+    }
+    if (halo_rows > 2 * 256 - 16)
+        return FPQ_ERR_UNSUPPORTED;
     const int m_units = (g.m_tiles + 1) / 2;
     const int nclusters = nsm / 2;
     g.seg_chunk = p.c_seg;
     g.x_scale2 = p.x_scale2;
     const int accs = p.c_seg ? 2 : 1;
-    const int a_bytes = (int)round_up(halo_rows, 8) * 128;
+    const int a_bytes = phased ? 4 * (int)g.a_tx : (int)round_up(halo_rows, 8) * 128;
     g.BN = choose_tile(p.N, m_units, nclusters, g.cchunks, g.taps, a_bytes, accs, &g.estimate);
     g.acc_cols = g.BN * accs;
     g.acc_bufs = 2 * g.acc_cols <= 512 ? 2 : 1;
     g.n_tiles = (p.N + g.BN - 1) / g.BN;
     g.div_nt = make_fastdiv((uint32_t)g.n_tiles);
     g.units = m_units * g.n_tiles;
-    g.a_boxes = halo_rows > 256 ? 2 : 1;
+    g.a_boxes = halo_rows > 256 && !phased ? 2 : 1;
     g.a_box_rows = (int)round_up((halo_rows + g.a_boxes - 1) / g.a_boxes, 8);
     g.a_stage_bytes = g.a_boxes * g.a_box_rows * 128;
-    g.a_tx = (uint32_t)g.a_stage_bytes;
+    if (!phased)
+        g.a_tx = (uint32_t)g.a_stage_bytes;
     g.b_tap_bytes = (g.BN / 2) * BK;
     g.b_stage_bytes = g.tgroup * g.b_tap_bytes;
     g.b_tx = (uint32_t)g.b_stage_bytes / (p.w4 ? 2 : 1);
@@ -382,8 +545,13 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
         g.b_stages = 8;
     if (g.b_stages < 2)
         return FPQ_ERR_UNSUPPORTED;
-    // a third activation stage if the weights still keep three
-    if (g.b_stages >= 4 && SMEM_BUDGET - ctl - 3 * g.a_stage_bytes - 3 * g.b_stage_bytes >= 0) {
+    // a third activation stage if the weights still keep three (stride 2: one per phase)
+    if (phased && SMEM_BUDGET - ctl - 4 * g.a_stage_bytes - 3 * g.b_stage_bytes >= 0) {
+        g.a_stages = 4;
+        g.b_stages = (SMEM_BUDGET - ctl - g.a_stages * g.a_stage_bytes) / g.b_stage_bytes;
+        if (g.b_stages > 8)
+            g.b_stages = 8;
+    } else if (g.b_stages >= 4 && SMEM_BUDGET - ctl - 3 * g.a_stage_bytes - 3 * g.b_stage_bytes >= 0) {
         g.a_stages = 3;
         g.b_stages = (SMEM_BUDGET - ctl - g.a_stages * g.a_stage_bytes) / g.b_stage_bytes;
         if (g.b_stages > 8)
@@ -393,7 +561,6 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
     g.tmem_cols = 32;
     while ((int)g.tmem_cols < g.acc_bufs * g.acc_cols)
         g.tmem_cols *= 2;
-    g.wait_prior_grid = p.after_stage1;
     *dyn_bytes = ctl + g.a_stages * g.a_stage_bytes + g.b_stages * g.b_stage_bytes;
     return FPQ_OK;
 }
@@ -419,16 +586,12 @@ bool pair_gemm_preferred(const GemmProblem& p)
     // 520 cycles each, the reduction split over clusters when the tiles leave SMs idle.  (1280 channels at 16 x 16, batch
     // 2: 17.1 against 20.3 us; batch 1: 16.6 against 15.0; 256 channels at 16 x 16: 8.0 against 11.1; 1280 -> 128 at
     // 32 x 32: 17.7 against 14.2.)
-    // (where the frame is much of the image it tiles the image itself, in powers of two, and loads every tap apart:
-    // 416 -> 608 channels at 11 x 11, batch 50: 49.8 us so, 24.3 us on pairs with the framed pixels)
+    // (at stride 2, and where the frame is much of the image, it tiles the image itself and loads every tap apart: 416 -> 608 channels at
+    // 11 x 11, batch 50: 49.8 us so, 24.3 us on pairs with the framed pixels)
     int64_t m_tiles = g.m_tiles;
     double block = 520.0;
-    if (m_tiles * 4 > ((int64_t)p.B * p.Ho * p.Wo + BM - 1) / BM * 5 + 4) {
-        int wt = 1, ht = 1;
-        while (wt < p.Wo && wt < BM) wt *= 2;
-        while (ht < p.Ho && ht < BM / wt) ht *= 2;
-        const int bt = BM / (wt * ht);
-        m_tiles = (int64_t)((p.Wo + wt - 1) / wt) * ((p.Ho + ht - 1) / ht) * ((p.B + bt - 1) / bt);
+    if (p.stride > 1 || m_tiles * 4 > ((int64_t)p.B * p.Ho * p.Wo + BM - 1) / BM * 5 + 4) {
+        m_tiles = choose_taps_tile(p.B, p.Ho, p.Wo, p.stride).tiles;
         block = 700.0;
     }
     if (p.N <= 64)
@@ -442,7 +605,8 @@ bool pair_gemm_preferred(const GemmProblem& p)
     } else {
         general = block * (double)((tiles + SMS - 1) / SMS) * blocks;
     }
-    return g.estimate <= general + 4300.0;
+    // (stride 2 in several rounds: 256 -> 1280 channels at 16 x 16, batch 57: 20.4 us there, 22.8 here)
+    return g.estimate <= general + (p.stride > 1 && g.units > SMS / 2 ? 2000.0 : 4300.0);
 }
 
 fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
@@ -462,8 +626,10 @@ fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
             return FPQ_ERR_CUDA;
         if (!attr_set[dev]) {
-            if (cudaFuncSetAttribute(fpq_pair_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET) !=
-                cudaSuccess)
+            if (cudaFuncSetAttribute(fpq_pair_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET) !=
+                    cudaSuccess ||
+                cudaFuncSetAttribute(fpq_pair_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET) !=
+                    cudaSuccess)
                 return FPQ_ERR_CUDA;
             int v = 0;
             if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 2)
@@ -486,8 +652,20 @@ fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
     if (!g.status)
         return FPQ_ERR_CUDA;
 
+    const bool phased = p.stride == 2;
     CUtensorMap tmA, tmB;
-    {
+    if (phased) {
+        // every second pixel of every second row of the zero-framed images
+        const int Hp = p.H + 2 * p.pad;
+        cuuint64_t dims[4] = {(cuuint64_t)p.Ca, (cuuint64_t)g.Wp, (cuuint64_t)Hp, (cuuint64_t)p.B};
+        cuuint64_t strides[3] = {(cuuint64_t)p.Ca, (cuuint64_t)p.Ca * g.Wp, (cuuint64_t)p.Ca * g.Wp * Hp};
+        cuuint32_t box[4] = {BK, (cuuint32_t)(2 * g.w2), (cuuint32_t)(2 * g.h2), (cuuint32_t)g.nb};
+        cuuint32_t estr[4] = {1, 2, 2, 1};
+        if (enc(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, (void*)p.a_codes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return FPQ_ERR_CUDA;
+    } else {
         // activation codes: the zero-framed channels-last pixel list [B Hp Wp][Ca]
         cuuint64_t dims[4] = {(cuuint64_t)p.Ca, (cuuint64_t)g.M, 1, 1};
         cuuint64_t strides[3] = {(cuuint64_t)p.Ca, (cuuint64_t)p.Ca * (cuuint64_t)g.M, (cuuint64_t)p.Ca * (cuuint64_t)g.M};
@@ -503,7 +681,7 @@ fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
         cuuint64_t dims[3] = {(cuuint64_t)p.Cp, (cuuint64_t)p.N, (cuuint64_t)g.taps};
         const cuuint64_t rowB = p.w4 ? (cuuint64_t)p.Cp / 2 : (cuuint64_t)p.Cp;
         cuuint64_t strides[2] = {rowB * g.taps, rowB};
-        cuuint32_t box[3] = {BK, (cuuint32_t)(g.BN / 2), (cuuint32_t)g.tgroup};
+        cuuint32_t box[3] = {BK, (cuuint32_t)(g.BN / 2), phased ? 1u : (cuuint32_t)g.tgroup};
         cuuint32_t estr[3] = {1, 1, 1};
         if (enc(&tmB, p.w4 ? CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B : CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void*)p.w_prepared,
                 dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -515,7 +693,7 @@ fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
         nclusters = g.units;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * nclusters));
-    cfg.blockDim = dim3(NTHREADS);
+    cfg.blockDim = dim3((unsigned)num_threads(phased));
     cfg.dynamicSmemBytes = (size_t)dyn;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -527,7 +705,8 @@ fpq_status launch_pair_gemm(const GemmProblem& p, cudaStream_t st)
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, fpq_pair_gemm_kernel, tmA, tmB, (const PGArgs)g) == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, phased ? fpq_pair_gemm_kernel<true> : fpq_pair_gemm_kernel<false>, tmA, tmB,
+                              (const PGArgs)g) == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
 }
 
 }  // namespace fpq

@@ -69,3 +69,26 @@ def test_small_frame_against_the_oracle():
     idx = sample_indices(y.size, 20000, 5)
     yr, ab = oracle_layer(L, ws, xs, idx)
     assert_close(y[idx], np.asarray(yr), np.asarray(ab))
+
+
+# stride 2: tiles of whole rows, parts of rows, several images; odd and even frames; one and several rounds
+@pytest.mark.parametrize("B,C,H,W,Co", [(3, 320, 45, 77, 320), (2, 320, 64, 64, 320), (13, 128, 9, 8, 100), (1, 200, 7, 120, 256),
+                                        (1, 64, 3, 253, 64), (40, 96, 4, 3, 72), (9, 320, 31, 30, 640), (24, 192, 48, 48, 320)])
+@pytest.mark.parametrize("fw,pad", [(fpq.E4M3, 1), (fpq.E2M1, 1), (fpq.E2M1, 0)])
+def test_stride_two(B, C, H, W, Co, fw, pad):
+    gen = torch.Generator(device="cuda").manual_seed(C + Co)
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda")
+    codes, scale = _weights(gen, Co, C * 9, fw)
+    prep = fpq.fpq_prepare_weight(codes, fw, fpq.CONV2D, Co, C, 3, 3)
+    bias = torch.randn(Co, generator=gen, device="cuda")
+    _both(lambda: fpq.fpq_conv2d(x, prep, scale, 0.01, fpq.E4M3, fw, bias, Co, 3, 3, pad, 2))
+
+
+@pytest.mark.parametrize("B,C,H,W,Co", [(3, 130, 25, 41, 96), (7, 64, 11, 9, 40)])
+def test_stride_two_against_the_oracle(B, C, H, W, Co):
+    L = I.draw(I.conv_layer("down", B, C, H, W, Co, 3, stride=2, wfmt="e2m1", rounding=True), 22, 0, "silu", 0.03, True)
+    ws, xs = layer_scales(L)
+    y = gpu_layer(L, ws, xs).reshape(-1)
+    idx = sample_indices(y.size, 20000, 5)
+    yr, ab = oracle_layer(L, ws, xs, idx)
+    assert_close(y[idx], np.asarray(yr), np.asarray(ab))
