@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                 mbar_arrive(acc_empty + 8 * buf);
         }
         if (g.y_tma && lane == 0)
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the staging buffer must outlive its stores
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the staging buffer must outlive its stores
         if (dead)
             flag_status(g.status, FPQ_ERR_TIMEOUT);
     } else if (FUSED && warp == 2 + NUM_EPI_WARPS + NUM_XFORM_WARPS) {

@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
     // global memory before that kernel has completed and its writes are visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
+    bool failed = false;                               // a wait of this thread's role ran out
     // the pair's first CTA's copy of a barrier, as a cluster-space address
     auto leader = [&](uint32_t bar) { return peer_smem_addr(bar, 0u); };
 
@@ -219,8 +220,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
             }
             if (!b_issued)
                 issue_weights();
+            failed = dead;
             if (dead) {
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
                 for (uint32_t i = (nx > (uint32_t)g.x_stages ? nx - g.x_stages : 0); i < nx; ++i)
                     (void)mbar_wait(x_full + 8 * (i % g.x_stages), (i / g.x_stages) & 1);
             }
@@ -272,8 +273,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
                     break;
                 mma_commit_pair(acc_full + 8 * buf, 3);
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (warp == 3) {
         // ---------------- second CTA: tell the MMA issuer when this CTA's weights have landed ----------------
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
             const uint32_t rb = leader(b_peer);
             for (int cc = 0; cc < g.cchunks; ++cc) {
                 if (!mbar_wait(b_full + 8 * cc, 0)) {
-                    flag_status(g.status, FPQ_ERR_TIMEOUT);
+                    failed = true;
                     break;
                 }
                 mbar_arrive_cluster(rb + 8 * cc);
@@ -370,11 +370,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
             // hand the accumulator back to the MMA issuer (in the pair's first CTA)
             tc_fence_before();
             __syncwarp();
-            if (lane == 0)
+            if (lane == 0 && step + 2 < g.tiles_per_cta)           // (somebody waits for it)
                 mbar_arrive_cluster(racc_empty + 8 * buf);
         }
-        if (dead)
-            flag_status(g.status, FPQ_ERR_TIMEOUT);
+        failed = dead;
     } else if (warp >= XF_W0) {
         // ---------------- transform: staged FP32 image rows -> E4M3 codes of the operand ----------------
         // Thread item = (pair of neighbouring pixels, 16-channel group): 16 eight-byte loads (half a warp reads
@@ -482,15 +481,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
         }
         if (nan)
             flag_status(g.status, FPQ_ERR_NAN_INPUT);
-        if (dead)
-            flag_status(g.status, FPQ_ERR_TIMEOUT);
+        failed = dead;
     }
 
-    // nobody leaves while the other CTA may still arrive on this CTA's barriers or read its shared memory,
-    // and both CTAs give their tensor memory back together
+    // Nobody leaves while the other CTA may still arrive on this CTA's barriers or read its shared memory, and both CTAs
+    // give their tensor memory back together.  Every arrival but a failed role's has been waited for, so the barrier
+    // need not wait for the stores of the output (128 -> 128 channels at 32 x 32, batch 64: 19.1 -> 18.7 us; one tap,
+    // 128 -> 256 at 64 x 64, batch 8: 10.9 -> 10.1).
     tc_fence_before();
-    __syncwarp();
-    cluster_sync_all();
+    if (failed)
+        flag_status(g.status, FPQ_ERR_TIMEOUT);
+    if (__any_sync(0xffffffffu, failed))
+        cluster_arrive();
+    else
+        cluster_arrive_relaxed();
+    cluster_wait();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, g.tmem_cols);

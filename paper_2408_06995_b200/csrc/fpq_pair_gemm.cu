@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
     // the activation codes are written by the kernel in front (and the output may alias something it reads)
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
+    bool failed = false;                               // a wait of this thread's role ran out
     auto leader = [&](uint32_t bar) { return peer_smem_addr(bar, 0u); };
     auto decode = [&](int u, int& mu, int& nt) {
         mu = (int)fdiv((uint32_t)u, g.div_nt);
@@ -163,8 +164,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                         if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
                     }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (PHASED && warp == B_WARP) {
         // ---------------- stride 2: weight producer ----------------
@@ -190,8 +190,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                     }
                 }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (!PHASED && warp == 0) {
         // ---------------- TMA producer: loads in the order the MMAs consume them ----------------
@@ -221,8 +220,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                     }
                 }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: one thread of the pair's first CTA ----------------
@@ -313,8 +311,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                 mma_commit_pair(acc_full + 8 * buf, 3);
                 if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else {
         // ---------------- epilogue: y = acc * (x_scale * w_scale[n]) + bias[n], NCHW ----------------
@@ -405,17 +402,24 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0)
+            if (lane == 0 && u + g.acc_bufs < u_hi)                // (somebody waits for it)
                 mbar_arrive_cluster(racc_empty + 8 * buf);
             if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
         }
-        if (dead)
-            flag_status(g.status, FPQ_ERR_TIMEOUT);
+        failed = dead;
     }
 
+    // Nobody leaves while the other CTA may still arrive on its barriers.  Every arrival but a failed role's has been waited
+    // for, so the barrier need not wait for the stores of the output: the next kernel's blocks move in that much earlier
+    // (320 -> 320 channels at 64 x 64, batch 1, whole layer: 11.2 -> 10.5 us).
     tc_fence_before();
-    __syncwarp();
-    cluster_sync_all();
+    if (failed)
+        flag_status(g.status, FPQ_ERR_TIMEOUT);
+    if (__any_sync(0xffffffffu, failed))
+        cluster_arrive();
+    else
+        cluster_arrive_relaxed();
+    cluster_wait();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, g.tmem_cols);

@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
     if (!(g.early_weights && warp == B_WARP))
         asm volatile("griddepcontrol.wait;" ::: "memory");
 
+    bool failed = false;                               // a wait of this thread's role ran out
     auto leader = [&](uint32_t bar) { return peer_smem_addr(bar, 0u); };
 
     if (warp == 0) {
@@ -122,8 +123,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
                     if (++s == (uint32_t)g.a_stages) { s = 0; ph ^= 1; }
                 }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (warp == B_WARP) {
         // ---------------- weight producer ----------------
@@ -146,8 +146,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
                         if (++s == (uint32_t)g.b_stages) { s = 0; ph ^= 1; }
                     }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: one thread of the pair's first CTA ----------------
@@ -192,8 +191,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
                 mma_commit_pair(acc_full + 8 * buf, 3);
                 if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
             }
-            if (dead)
-                flag_status(g.status, FPQ_ERR_TIMEOUT);
+            failed = dead;
         }
     } else {
         // ---------------- epilogue ----------------
@@ -256,19 +254,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0)
+            if (lane == 0 && u + g.acc_bufs < u_hi)                // (somebody waits for it)
                 mbar_arrive_cluster(racc_empty + 8 * buf);
             if (++buf == (uint32_t)g.acc_bufs) { buf = 0; aph ^= 1; }
         }
         if (lane == 0)
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // the staging must outlive its stores
-        if (dead)
-            flag_status(g.status, FPQ_ERR_TIMEOUT);
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); // the staging must outlive its stores
+        failed = dead;
     }
 
+    // Nobody leaves while the other CTA may still arrive on its barriers.  Every arrival but a failed role's has been waited
+    // for, so the barrier need not wait for the stores of the output: the next kernel's blocks move in that much earlier
+    // (2048 x 2560 -> 640, whole layer: 13.5 -> 12.6 us).
     tc_fence_before();
-    __syncwarp();
-    cluster_sync_all();
+    if (failed)
+        flag_status(g.status, FPQ_ERR_TIMEOUT);
+    if (__any_sync(0xffffffffu, failed))
+        cluster_arrive();
+    else
+        cluster_arrive_relaxed();
+    cluster_wait();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, g.tmem_cols);
