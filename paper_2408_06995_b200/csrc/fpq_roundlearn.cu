@@ -10,10 +10,13 @@
 //                           reduction is cut into slices that reduce_d_kernel adds
 //   sgemm128<false>         partial sums of D^T A over slices of the M rows
 //   grad_finalize_kernel    slices added in a fixed order, chain rule, sum of lambda, optional descent update
-// With many calibration rows D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are fewer products: see gram_preferred.
+// With many calibration rows D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are fewer products: see gram_preferred;
+// gram_grad_kernel then takes the place of the last two.
 //   harden_kernel           the inference rule: decision bit = (sigma(alpha) >= 0.5)
 //   unfold_kernel           a convolution's input rows, so that the same step serves convolution weights
 #include <math.h>
+
+#include <mutex>
 
 #include "fpq_kernels.h"
 
@@ -320,6 +323,18 @@ __global__ void __launch_bounds__(256, 2) sgemm128(const float* __restrict__ P, 
         block_atomic_add((double)sq, sq_sum);
 }
 
+// gradient of one weight's alpha: g * dWq/dalpha + reg * dlambda/dalpha; lam += lambda(alpha)
+__device__ __forceinline__ float weight_gradient(float g, float dq, float al, float reg, float& lam)
+{
+    const SoftTerms st = soft_terms(al);
+    const float u = st.u;
+    const float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
+    lam += 1.0f - u16 * u4;
+    const float u19 = u16 * u2 * u;
+    const float dlam = -40.0f * u19 * (al > 0.f ? 1.f : (al < 0.f ? -1.f : 0.f)) * st.sp;
+    return fmaf(g, dq, reg * dlam);
+}
+
 // grad = (2 / (M N)) (sum of the slices of D^T A) * dWq/dalpha + reg * dlambda/dalpha; alpha -= lr * grad when
 // lr != 0; sum of lambda.  E == NULL: thread 0 of block 0 turns the sum of squares into the mean; otherwise the mean is
 // <D^T A, E> / (M N), as sum D^2 = sum D (A E^T).
@@ -370,13 +385,7 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
         for (int v = 0; v < V; ++v) {
             if (E)
                 sq = fma((double)g[v], (double)e[v], sq);
-            const SoftTerms st = soft_terms(al[v]);
-            const float u = st.u;
-            const float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
-            lam += 1.0f - u16 * u4;
-            const float u19 = u16 * u2 * u;
-            const float dlam = -40.0f * u19 * (al[v] > 0.f ? 1.f : (al[v] < 0.f ? -1.f : 0.f)) * st.sp;
-            gr[v] = fmaf(coef * g[v], dq[v], reg * dlam);
+            gr[v] = weight_gradient(coef * g[v], dq[v], al[v], reg, lam);
             al[v] = al[v] - lr * gr[v];
         }
         store(grad + i, gr);
@@ -388,6 +397,149 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
         __syncthreads();                               // (the helper's shared memory is used again)
         block_atomic_add(sq * inv_mn, loss);
     }
+}
+
+// The gradient from S = A^T A in one kernel: a 4 RA x 64 tile of E S per block, reduced over all of K, then what
+// grad_finalize_kernel does.  S is symmetric, so both operands are read as they lie.  64 reduction elements per stage, three
+// stages of asynchronous copies; each of the eight warps takes eight elements of a stage and has a sum of its own for the
+// whole tile, RA x 8 outputs per thread (shared memory gives 128 bytes per clock whatever part of them is broadcast: with 4 x
+// 4 outputs the loads took twice the time of the multiply-adds).  With 128 x 128 tiles the reduction had to be sliced to
+// fill the SMs, and writing, reading and adding the slices took as long again (9.9 + 5.2 us for 960 x 320 weights, 11.3 here;
+// the whole step with 4096 rows 37.1 -> 33.2 us, 512 x 256 weights and 1024 rows 20.3 -> 18.4, 555 x 128 and 431 17.9 -> 15.2).
+constexpr int GK = 64, GR = 64, G_STAGES = 3;
+constexpr int GE_LD = GR + 4;                          // rows of E in shared memory (floats)
+__host__ __device__ constexpr int gram_stage(int ra) { return 4 * ra * GE_LD + GR * GK; }      // floats
+constexpr int gram_smem(int ra)                        // the stages, and afterwards the warps' sums
+{
+    return 4 * (G_STAGES * gram_stage(ra) > 8 * 4 * ra * GK ? G_STAGES * gram_stage(ra) : 8 * 4 * ra * GK);
+}
+template <int RA>
+__global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restrict__ E, const float* __restrict__ S,
+                                                           const float* __restrict__ DQ, float* __restrict__ alpha,
+                                                           float* __restrict__ grad, double* __restrict__ loss, int64_t N,
+                                                           int64_t K, float coef, double inv_mn, float reg, float lr, int vec)
+{
+    constexpr int GN = 4 * RA, G_STAGE = gram_stage(RA);
+    extern __shared__ __align__(16) float gsm[];
+    const int t = threadIdx.x, warp = t >> 5, ty = (t >> 3) & 3, tx = t & 7;
+    const int64_t n0 = (int64_t)blockIdx.x * GN, k0 = (int64_t)blockIdx.y * GK;
+    auto fetch = [&](int stage, int64_t r0) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(gsm + stage * G_STAGE);
+        auto copy = [](uint32_t to, const float* from, bool there) {       // (zeros where there is nothing)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
+        };
+        const int row = t / (GR / 4), c = t % (GR / 4) * 4;
+#pragma unroll
+        for (int q = 0; q < GN; q += 16) {
+            if (GN % 16 && row + q >= GN)
+                break;
+            const bool there = n0 + row + q < N && r0 + c < K;
+            copy(dst + ((row + q) * GE_LD + c) * 4, there ? E + (n0 + row + q) * K + r0 + c : E, there);
+        }
+#pragma unroll
+        for (int q = 0; q < GR; q += 16) {
+            const bool there = r0 + row + q < K && k0 + c < K;
+            copy(dst + (GN * GE_LD + (row + q) * GK + c) * 4, there ? S + (r0 + row + q) * K + k0 + c : S, there);
+        }
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int stages = (int)((K + GR - 1) / GR);
+#pragma unroll
+    for (int i = 0; i < G_STAGES - 1; ++i) {
+        if (i < stages)
+            fetch(i, (int64_t)i * GR);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    unsigned long long acc[RA][4];                     // rows ty + 4 a; columns 4 tx + 0 .. 3, 32 + 4 tx + 0 .. 3
+#pragma unroll
+    for (int a = 0; a < RA; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            acc[a][b] = 0ull;
+    for (int i = 0; i < stages; ++i) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(G_STAGES - 2) : "memory");
+        __syncthreads();                               // (and everybody is done with the stage that is filled next)
+        if (i + G_STAGES - 1 < stages)
+            fetch((i + G_STAGES - 1) % G_STAGES, (int64_t)(i + G_STAGES - 1) * GR);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* es = gsm + i % G_STAGES * G_STAGE + ty * GE_LD + warp * 8;
+        const float* ss = gsm + i % G_STAGES * G_STAGE + GN * GE_LD + warp * 8 * GK + tx * 4;
+#pragma unroll
+        for (int r4 = 0; r4 < 8; r4 += 4) {
+            float e[RA][4];
+#pragma unroll
+            for (int a = 0; a < RA; ++a) {
+                const float4 v = *reinterpret_cast<const float4*>(es + a * 4 * GE_LD + r4);
+                e[a][0] = v.x, e[a][1] = v.y, e[a][2] = v.z, e[a][3] = v.w;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const ulonglong2 v0 = *reinterpret_cast<const ulonglong2*>(ss + (r4 + q) * GK);
+                const ulonglong2 v1 = *reinterpret_cast<const ulonglong2*>(ss + (r4 + q) * GK + 32);
+#pragma unroll
+                for (int a = 0; a < RA; ++a) {
+                    const unsigned long long ee = pack2(e[a][q], e[a][q]);
+                    fma2(acc[a][0], ee, v0.x);
+                    fma2(acc[a][1], ee, v0.y);
+                    fma2(acc[a][2], ee, v1.x);
+                    fma2(acc[a][3], ee, v1.y);
+                }
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < RA; ++a) {
+        float* to = gsm + warp * GN * GK + (ty + 4 * a) * GK + tx * 4;
+        *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(acc[a][0], acc[a][1]);
+        *reinterpret_cast<ulonglong2*>(to + 32) = make_ulonglong2(acc[a][2], acc[a][3]);
+    }
+    __syncthreads();
+    float lam = 0.f;
+    double sq = 0.0;
+    for (int id = t; id < GN * GK / 4; id += 256) {
+        const int row = id / (GK / 4), c = id % (GK / 4) * 4;
+        if (n0 + row >= N || k0 + c >= K)
+            continue;
+        const int64_t at = (n0 + row) * K + k0 + c;
+        const float4 dq = *reinterpret_cast<const float4*>(DQ + at), e = *reinterpret_cast<const float4*>(E + at);
+        float al[4], gr[4], g[4] = {0.f, 0.f, 0.f, 0.f};
+        if (vec) {
+            const float4 v = *reinterpret_cast<const float4*>(alpha + at);
+            al[0] = v.x, al[1] = v.y, al[2] = v.z, al[3] = v.w;
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                al[v] = alpha[at + v];
+        }
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float4 v = *reinterpret_cast<const float4*>(gsm + w * GN * GK + row * GK + c);
+            g[0] += v.x, g[1] += v.y, g[2] += v.z, g[3] += v.w;
+        }
+        const float d[4] = {dq.x, dq.y, dq.z, dq.w}, ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            sq = fma((double)g[v], (double)ev[v], sq);
+            gr[v] = weight_gradient(coef * g[v], d[v], al[v], reg, lam);
+            al[v] = al[v] - lr * gr[v];
+        }
+        if (vec) {
+            *reinterpret_cast<float4*>(grad + at) = make_float4(gr[0], gr[1], gr[2], gr[3]);
+            if (lr != 0.f)
+                *reinterpret_cast<float4*>(alpha + at) = make_float4(al[0], al[1], al[2], al[3]);
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                grad[at + v] = gr[v];
+                if (lr != 0.f)
+                    alpha[at + v] = al[v];
+            }
+        }
+    }
+    block_atomic_add((double)lam, loss + 1);
+    __syncthreads();                                   // (the helper's shared memory is used again)
+    block_atomic_add(sq * inv_mn, loss);
 }
 
 // S = sum of the slices of A^T A [K][K] (fixed order; the sums in double).  Eight threads share four floats, each adding
@@ -508,6 +660,16 @@ bool gram_preferred(int64_t M, int64_t N, int64_t K)
     return K % 4 == 0 && M >= 2 * K && (double)K * (double)(M + N) * 1.25 <= 2.0 * (double)M * (double)N;
 }
 
+// Rows of gram_grad_kernel's tiles: the fewest whose blocks all run at once, one per SM (150 blocks of 32 rows take 15.5 us
+// where 120 of 40 take 11.3: two SMs have two of them); 0: not even with 64.
+int gram_tile_rows(int64_t N, int64_t K)
+{
+    for (int rows : {32, 40, 48, 64})
+        if ((N + rows - 1) / rows * ((K + 63) / 64) <= 148)
+            return rows;
+    return 0;
+}
+
 // As many slices of a reduction of length R as still fit into one wave of two resident blocks per SM (one more
 // would add a second, nearly empty wave), each at least 128 long.
 void slice(int64_t tiles, int64_t R, int* splits, int64_t* per)
@@ -591,19 +753,20 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
             *per = round_up(each < least ? least : each, BK);
             *splits = (int)((R + *per - 1) / *per);
         };
-        // (the tensor-core kernel has some 10 us of its own: 128 x 256 tiles filled, split, drained and stored; the
-        // multiply-adds take about 6 us per 10^8 products.  960 x 320 x 320: 12.6 us against 9.9)
+        // (the tensor-core kernel has some 10 us of its own: 128 x 256 tiles filled, split, drained and stored)
         const int64_t tk = (K + 127) / 128;
         p.tc_s = M * K * K >= 100000000;
         if (p.tc_s)
             cut(tk * ((K + 255) / 256), (M + 31) / 32, 4, &p.per_s, &p.splits_s);
         else
             cut_short(tk * tk, M, &p.per_s, &p.splits_s);
-        p.tc_g = N * K * K >= 130000000;
+        // the product with E: gram_grad_kernel, some 4 us and 35 ns per row of its tiles and 64 of K, unless it has several
+        // rounds of blocks, or the tensor cores and grad_finalize_kernel (some 17.5 us) are faster
+        const int rows = gram_tile_rows(N, K);
+        p.tc_g = rows ? (K + 63) / 64 * rows > 385 : N * K * K >= 130000000;
+        p.splits_g = 1;
         if (p.tc_g)
             cut(tk * ((N + 255) / 256), (K + 31) / 32, 1, &p.per_g, &p.splits_g);
-        else
-            cut_short(tk * ((N + 127) / 128), K, &p.per_g, &p.splits_g);
         p.off_SP = o;
         o += (size_t)round_up((int64_t)p.splits_s * K * K * 4, 256);
         p.off_S = o;
@@ -616,6 +779,39 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     }
     p.bytes = o;
     return p;
+}
+
+template <int RA>
+fpq_status launch_gram_grad_rows(const float* E, const float* S, const float* DQ, float* alpha, float* grad, double* loss,
+                                 int64_t N, int64_t K, float coef, double inv_mn, float reg, float lr, cudaStream_t st)
+{
+    {
+        static std::mutex mu;
+        static bool attr_set[64] = {};
+        std::lock_guard<std::mutex> lock(mu);
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+            return FPQ_ERR_CUDA;
+        if (!attr_set[dev]) {
+            if (cudaFuncSetAttribute(gram_grad_kernel<RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, gram_smem(RA)) != cudaSuccess)
+                return FPQ_ERR_CUDA;
+            attr_set[dev] = true;
+        }
+    }
+    const int vec = (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
+    return launch_overlapped(gram_grad_kernel<RA>, dim3((unsigned)((N + 4 * RA - 1) / (4 * RA)), (unsigned)((K + GK - 1) / GK)), 256,
+                             gram_smem(RA), st, E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, vec) == cudaSuccess
+               ? FPQ_OK
+               : FPQ_ERR_CUDA;
+}
+
+fpq_status launch_gram_grad(const float* E, const float* S, const float* DQ, float* alpha, float* grad, double* loss, int64_t N,
+                            int64_t K, float coef, double inv_mn, float reg, float lr, cudaStream_t st)
+{
+    const int rows = gram_tile_rows(N, K);
+    const auto launch = rows == 32 ? launch_gram_grad_rows<8> : rows == 40 ? launch_gram_grad_rows<10>
+                        : rows == 48 ? launch_gram_grad_rows<12> : launch_gram_grad_rows<16>;
+    return launch(E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, st);
 }
 
 }  // namespace
@@ -676,11 +872,9 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
         if (launch_overlapped(reduce_gram_kernel, dim3((unsigned)((K * K / 4 + 31) / 32)), 256, 0, st, (const float4*)SP, p.splits_s,
                               (float4*)S, K * K / 4) != cudaSuccess)
             return FPQ_ERR_CUDA;
-        if (p.tc_g)
-            sg = launch_tf32x3(S, K, E, K, K, N, K, (int)p.per_g, 1, GP, K, N * K, nullptr, st, 3, nullptr, 1.0f, nullptr, 0, 4);
-        else if (launch_overlapped(sgemm128<true>, dim3((unsigned)((N + TILE - 1) / TILE), (unsigned)tk, (unsigned)p.splits_g), 256, 0,
-                                   st, E, K, S, K, GP, K, (int)N, (int)K, K, p.per_g, nullptr) != cudaSuccess)
-            sg = FPQ_ERR_CUDA;
+        if (!p.tc_g)
+            return launch_gram_grad(E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, st);
+        sg = launch_tf32x3(S, K, E, K, K, N, K, (int)p.per_g, 1, GP, K, N * K, nullptr, st, 3, nullptr, 1.0f, nullptr, 0, 4);
         return sg != FPQ_OK ? sg : finalize(p.splits_g, E);
     }
     if (tc) {

@@ -48,3 +48,33 @@ def test_repeated_calls_agree_and_descend():
     for _ in range(20):
         _, loss = fpq.fpq_round_learn_step(w, scale, fpq.E2M1, alpha, a, 0.0, lr=1e5)
     assert 0.0 < float(loss[0]) < first
+
+
+# the product with E in one kernel: tiles of 32, 40, 48 and 64 rows, several rounds of them, the last one ragged in rows and
+# columns; the tensor cores instead; step sizes and decisions that are not 16-byte aligned
+@pytest.mark.parametrize("M,N,K,lr", [(700, 33, 68, 0.0), (700, 961, 316, 1e4), (700, 1700, 256, 0.0), (600, 2350, 252, 1e4),
+                                      (200, 9500, 60, 0.0), (1100, 1500, 400, 0.0)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_gradient_tiles(M, N, K, lr, offset):
+    gen = torch.Generator(device="cuda").manual_seed(N + K)
+    w = torch.randn(N, K, generator=gen, device="cuda") * 0.02
+    a = torch.randn(M, K, generator=gen, device="cuda") + 0.2
+    scale = (w.abs().amax(dim=1) / 6).contiguous()
+    alpha = torch.empty(N * K + offset, device="cuda")[offset:].view(N, K)
+    alpha.copy_(torch.randn(N, K, generator=gen, device="cuda") * 1.5)
+    start = alpha.clone()
+    grad, loss = fpq.fpq_round_learn_step(w, scale, fpq.E2M1, alpha, a, 1e-6, lr=lr)
+    assert fpq.fpq_read_status() == fpq.OK
+    wq, dwq = O.soft_weight(w.cpu().numpy(), scale.cpu().numpy(), O.E2M1, start.cpu().numpy())
+    e = (torch.from_numpy(np.asarray(wq, dtype=np.float64)) - w.cpu().double()).cuda()
+    d = torch.from_numpy(np.asarray(dwq, dtype=np.float64)).cuda()
+    y = a.double() @ e.T
+    assert float(loss[0]) == pytest.approx(float((y * y).mean()), rel=1e-5)
+    data = 2.0 / (M * N) * (y.T @ a.double()) * d
+    # what the regulariser adds, from a step on activations of zero
+    reg, _ = fpq.fpq_round_learn_step(w, scale, fpq.E2M1, start.clone(), torch.zeros_like(a), 1e-6)
+    assert float((grad.double() - reg.double() - data).norm()) <= 1e-5 * float(data.norm())
+    if lr:
+        assert torch.equal(alpha, start - lr * grad) or float((alpha - (start - lr * grad)).abs().max()) <= 1e-6 * float(alpha.abs().max())
+    else:
+        assert torch.equal(alpha, start)
