@@ -757,7 +757,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
         const int64_t tk = (K + 127) / 128;
         p.tc_s = M * K * K >= 100000000;
         if (p.tc_s)
-            cut(tk * ((K + 255) / 256), (M + 31) / 32, 4, &p.per_s, &p.splits_s);
+            cut(tk * ((K + tf32x3_columns(K) - 1) / tf32x3_columns(K)), (M + 31) / 32, 4, &p.per_s, &p.splits_s);
         else
             cut_short(tk * tk, M, &p.per_s, &p.splits_s);
         // the product with E: gram_grad_kernel, some 4 us and 35 ns per row of its tiles and 64 of K, unless it has several
@@ -863,7 +863,7 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
         fpq_status sg = FPQ_OK;
         if (p.tc_s)
             sg = launch_tf32x3(AT, p.Mp, AT, p.Mp, K, K, M, (int)p.per_s, 1, SP, K, K * K, nullptr, st, 3, nullptr, 1.0f, nullptr,
-                               0, 4);
+                               0, 4, tf32x3_columns(K));
         else if (launch_overlapped(sgemm128<false>, dim3((unsigned)tk, (unsigned)tk, (unsigned)p.splits_s), 256, 0, st, a, K, a, K, SP,
                                    K, (int)K, (int)K, M, p.per_s, nullptr) != cudaSuccess)
             sg = FPQ_ERR_CUDA;

@@ -8,8 +8,8 @@
 // accumulated, lo * hi + hi * lo + hi * hi: what is left out (lo * lo and the bits of lo below its 11th) is
 // below 2^-19 of |p| |q| per term.
 //
-// Per CTA one 128 x 256 output tile and one slice of the reduction.  Warp 0: TMA producer (FP32 tiles of P
-// and Q, 128 / 256 rows x 32 floats, 128-byte swizzled; these are the hi operands as they are).  Warps 2-9:
+// Per CTA one 128 x 256 (or 128 x 160) output tile and one slice of the reduction.  Warp 0: TMA producer (FP32 tiles of P
+// and Q, 128 / 256 (160) rows x 32 floats, 128-byte swizzled; these are the hi operands as they are).  Warps 2-9:
 // write lo of each landed tile beside it (the same element-wise map whatever the swizzle); they are also
 // the epilogue.  Warp 1: tensor-memory owner and MMA issuer (kind::tf32, N = 256, 12 MMAs of K = 8 per
 // 32-wide block: at N = 128 the operand reads of the MMAs alone would take all of the shared-memory bandwidth).
@@ -29,15 +29,21 @@ namespace fpq {
 
 namespace {
 
-constexpr int TM = 128, TN = 256, TK = 32;           // TK floats = one 128-byte row
-constexpr int T_P_BYTES = TM * 128, T_Q_BYTES = TN * 128;
-constexpr int T_RAW_BYTES = T_P_BYTES + T_Q_BYTES;
-constexpr int T_STAGE_BYTES = 2 * T_RAW_BYTES;       // P | Q as loaded (read by the tensor core as their TF32 heads) | P lo | Q lo
-constexpr int T_STAGES = 2;
+constexpr int TM = 128, TK = 32;                     // TK floats = one 128-byte row
 constexpr int T_XF_W0 = 2, T_NUM_XF = 8;
 constexpr int T_THREADS = 32 * (T_XF_W0 + T_NUM_XF);
-constexpr int T_SCALE_BYTES = T_NUM_XF * 2 * (TN / 2) * 4;      // per epilogue warp: scales and biases of its columns (epi 2)
-constexpr int T_SMEM = T_STAGES * T_STAGE_BYTES + 1024 + 256 + T_SCALE_BYTES;
+// Output tiles are 128 x 256, or 128 x 160 where those cover the columns with less padding: 320 columns are two of them,
+// and three stages fit (two of 256): A^T A of 4096 x 320, 16.6 us with 256, 12.3 with 160; of 8192 x 320 23.2 and 17.4.
+template <int TN>
+struct Tile {
+    static constexpr int P_BYTES = TM * 128, Q_BYTES = TN * 128, RAW = P_BYTES + Q_BYTES;
+    static constexpr int STAGE = 2 * RAW;            // P | Q as loaded (read by the tensor core as their TF32 heads) | P lo | Q lo
+    static constexpr int STAGES = TN > 160 ? 2 : 3;
+    static constexpr int CHUNKS = (TN / 32 + 1) / 2; // a warp's 32-column chunks: every second one
+    static constexpr int SCALES = T_NUM_XF * 2 * CHUNKS * 32 * 4;   // per epilogue warp: scales and biases of its columns (epi 2)
+    static constexpr int SMEM = STAGES * STAGE + 1024 + 256 + SCALES;
+    static_assert(RAW % (16 * 32 * T_NUM_XF) == 0 && 2 * TN <= 512 && SMEM <= 227 * 1024, "tile");
+};
 
 struct Tf32Args {
     int I, J;                  // rows of P (output rows), rows of Q (output columns)
@@ -94,10 +100,13 @@ __device__ __forceinline__ float4 tail4(const float4 v)
     return make_float4(tail_tf32(v.x), tail_tf32(v.y), tail_tf32(v.z), tail_tf32(v.w));
 }
 
+template <int TN>
 __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_constant__ CUtensorMap tmP,
                                                                    const __grid_constant__ CUtensorMap tmQ,
                                                                    const Tf32Args g)
 {
+    using T = Tile<TN>;
+    constexpr int T_STAGES = T::STAGES, T_STAGE_BYTES = T::STAGE, T_P_BYTES = T::P_BYTES, T_RAW_BYTES = T::RAW;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -127,7 +136,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
         tma_prefetch_desc(&tmQ);
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32((const void*)tmem_slot), 2 * TN);
+        tmem_alloc(smem_u32((const void*)tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -196,9 +205,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
     } else {
         // ---------------- split warps, then epilogue ----------------
         const int tid = threadIdx.x - 32 * T_XF_W0;
-        // as epilogue, warp w owns tensor-memory lane quarter w % 4 and half of the columns
-        constexpr int HALF = TN / 2;
-        const int quarter = warp & 3, half = (warp - T_XF_W0) >> 2;
+        // as epilogue, warp w owns tensor-memory lane quarter w % 4 and every second 32-column chunk
+        constexpr int HALF = T::CHUNKS * 32;
+        auto first_column = [&](int h) { return (2 * h + ((warp - T_XF_W0) >> 2)) * 32; };
+        const int quarter = warp & 3;
         const int i = ti * TM + quarter * 32 + lane;
         float sum[HALF];
 #pragma unroll
@@ -214,8 +224,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
             tc_fence_after();
 #pragma unroll
             for (int h = 0; h < HALF / 32; ++h) {
+                if (TN / 32 % 2 && first_column(h) >= TN)
+                    break;
                 uint32_t r[32];
-                tmem_ld32(tmem_base + buf * TN + (uint32_t)(half * HALF + h * 32) + ((uint32_t)(quarter * 32) << 16), r);
+                tmem_ld32(tmem_base + buf * TN + (uint32_t)first_column(h) + ((uint32_t)(quarter * 32) << 16), r);
                 tmem_ld_wait();
 #pragma unroll
                 for (int v = 0; v < 32; ++v)
@@ -232,9 +244,9 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
 #pragma unroll
             for (int q = 0; q < 2 * HALF / 32; ++q) {
                 const int e = q * 32 + lane;                       // [0, HALF): scale, [HALF, 2 HALF): bias
-                const int col = tj * TN + half * HALF + (e < HALF ? e : e - HALF);
+                const int own = e < HALF ? e : e - HALF, col = tj * TN + first_column(own / 32) + own % 32;
                 float v = 0.f;
-                if (col < g.J)
+                if (col < g.J && (TN / 32 % 2 == 0 || first_column(own / 32) < TN))
                     v = e < HALF ? g.x_scale * __ldg(g.w_scale + col) : (g.bias ? __ldg(g.bias + col) : 0.f);
                 w_sc[e] = v;
             }
@@ -268,8 +280,8 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
         if (!dead && kb_hi > kb_lo) {
 #pragma unroll
             for (int c = 0; c < HALF / 32; ++c) {
-                const int j0 = tj * TN + half * HALF + c * 32;
-                if (j0 >= g.J)
+                const int j0 = tj * TN + first_column(c);
+                if (j0 >= g.J || (TN / 32 % 2 && first_column(c) >= TN))
                     break;
                 const float* r = sum + c * 32;
                 if (g.epi == 0) {
@@ -341,7 +353,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 2 * TN);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
@@ -388,13 +400,13 @@ bool tf32x3_applies(const float* P, int64_t ldp, const float* Q, int64_t ldq, in
 fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ldq, int64_t I, int64_t J, int64_t R,
                          int kb_per_split, int epi, float* C, int64_t ldc, int64_t split_stride, double* sq_sum,
                          cudaStream_t st, int passes, const float* w_scale, float x_scale, const float* bias, int howo,
-                         int chunk)
+                         int chunk, int columns)
 {
     static std::mutex mu;
     static EncodeTiledFn enc = nullptr;
     static bool attr_set[64] = {};
     if (!tf32x3_applies(P, ldp, Q, ldq, I, J, R) || kb_per_split < 1 || (passes != 1 && passes != 3) ||
-        epi < 0 || epi > 2 || chunk < 2)
+        epi < 0 || epi > 2 || chunk < 2 || (columns != 160 && columns != 256))
         return FPQ_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lock(mu);
@@ -407,20 +419,23 @@ fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ld
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
             return FPQ_ERR_CUDA;
         if (!attr_set[dev]) {
-            if (cudaFuncSetAttribute(tf32x3_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM) != cudaSuccess)
+            if (cudaFuncSetAttribute(tf32x3_gemm_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<256>::SMEM) !=
+                    cudaSuccess ||
+                cudaFuncSetAttribute(tf32x3_gemm_kernel<160>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<160>::SMEM) !=
+                    cudaSuccess)
                 return FPQ_ERR_CUDA;
             attr_set[dev] = true;
         }
     }
     CUtensorMap tmP, tmQ;
-    if (!encode_rows(enc, &tmP, P, I, R, ldp, TM) || !encode_rows(enc, &tmQ, Q, J, R, ldq, TN))
+    if (!encode_rows(enc, &tmP, P, I, R, ldp, TM) || !encode_rows(enc, &tmQ, Q, J, R, ldq, columns))
         return FPQ_ERR_CUDA;
     Tf32Args g{};
     g.I = (int)I;
     g.J = (int)J;
     g.kblocks = (int)((R + TK - 1) / TK);
     g.kb_per_split = kb_per_split;
-    g.tiles_j = (int)((J + TN - 1) / TN);
+    g.tiles_j = (int)((J + columns - 1) / columns);
     g.epi = epi;
     g.passes = passes;
     g.chunk = chunk;
@@ -435,8 +450,8 @@ fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ld
     g.status = status_word();
     if (!g.status)
         return FPQ_ERR_CUDA;
-    // kind::tf32: FP32 accumulator, TF32 (format 2) on both sides, K-major, N = 256, M = 128
-    g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+    // kind::tf32: FP32 accumulator, TF32 (format 2) on both sides, K-major, N = columns, M = 128
+    g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(columns >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
     const int splits = (g.kblocks + kb_per_split - 1) / kb_per_split;
     if ((sq_sum || epi == 2) && splits != 1)
         return FPQ_ERR_UNSUPPORTED;
@@ -444,7 +459,9 @@ fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ld
     if (tiles > 0x7fffffff || splits > 65535)
         return FPQ_ERR_SHAPE;
     dim3 grid((unsigned)tiles, (unsigned)splits);
-    return launch_overlapped(tf32x3_gemm_kernel, grid, T_THREADS, T_SMEM, st, tmP, tmQ, g) == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
+    const cudaError_t err = columns == 256 ? launch_overlapped(tf32x3_gemm_kernel<256>, grid, T_THREADS, Tile<256>::SMEM, st, tmP, tmQ, g)
+                                           : launch_overlapped(tf32x3_gemm_kernel<160>, grid, T_THREADS, Tile<160>::SMEM, st, tmP, tmQ, g);
+    return err == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
 }
 
 cudaError_t launch_transpose(const float* X, int64_t ldx, int64_t M, int64_t K, float* XT, int64_t ldt, cudaStream_t st)

@@ -50,10 +50,10 @@ def test_repeated_calls_agree_and_descend():
     assert 0.0 < float(loss[0]) < first
 
 
-# the product with E in one kernel: tiles of 32, 40, 48 and 64 rows, several rounds of them, the last one ragged in rows and
+# A^T A with 256- and 160-wide tiles; the product with E in one kernel: tiles of 32, 40, 48 and 64 rows, several rounds of them, the last one ragged in rows and
 # columns; the tensor cores instead; step sizes and decisions that are not 16-byte aligned
 @pytest.mark.parametrize("M,N,K,lr", [(700, 33, 68, 0.0), (700, 961, 316, 1e4), (700, 1700, 256, 0.0), (600, 2350, 252, 1e4),
-                                      (200, 9500, 60, 0.0), (1100, 1500, 400, 0.0)])
+                                      (200, 9500, 60, 0.0), (1100, 1500, 400, 0.0), (1100, 600, 316, 0.0), (1200, 700, 580, 1e4)])
 @pytest.mark.parametrize("offset", [0, 1])
 def test_gradient_tiles(M, N, K, lr, offset):
     gen = torch.Generator(device="cuda").manual_seed(N + K)
