@@ -700,7 +700,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     p.off_D = o;
     o += (size_t)round_up(M * p.N4 * 4, 256);
     {
-        const int64_t tiles1 = ((M + 127) / 128) * ((N + 255) / 256);       // 128 x 256 output tiles
+        const int64_t tiles1 = ((M + 127) / 128) * ((N + tf32x3_columns(N) - 1) / tf32x3_columns(N));
         const int64_t kblocks = (K + 31) / 32;
         p.kb_per_split1_tc = (int)kblocks;
         p.splits1_tc = 1;
@@ -720,7 +720,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     // second contraction on the tensor cores: one CTA per SM, so about 148 / tiles slices of at least 4 blocks
     p.Mp = round_up(M, 4);
     {
-        const int64_t tiles2 = ((N + 127) / 128) * ((K + 255) / 256);       // 128 x 256 output tiles
+        const int64_t tiles2 = ((N + 127) / 128) * ((K + tf32x3_columns(K) - 1) / tf32x3_columns(K));
         const int64_t kblocks = (M + 31) / 32;
         int64_t want = 148 / tiles2;
         want = want < 1 ? 1 : (want > 64 ? 64 : want);
@@ -766,7 +766,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
         p.tc_g = rows ? (K + 63) / 64 * rows > 385 : N * K * K >= 130000000;
         p.splits_g = 1;
         if (p.tc_g)
-            cut(tk * ((N + 255) / 256), (K + 31) / 32, 1, &p.per_g, &p.splits_g);
+            cut(tk * ((N + tf32x3_columns(N) - 1) / tf32x3_columns(N)), (K + 31) / 32, 1, &p.per_g, &p.splits_g);
         p.off_SP = o;
         o += (size_t)round_up((int64_t)p.splits_s * K * K * 4, 256);
         p.off_S = o;
@@ -863,7 +863,7 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
         fpq_status sg = FPQ_OK;
         if (p.tc_s)
             sg = launch_tf32x3(AT, p.Mp, AT, p.Mp, K, K, M, (int)p.per_s, 1, SP, K, K * K, nullptr, st, 3, nullptr, 1.0f, nullptr,
-                               0, 4, tf32x3_columns(K));
+                               0, 4);
         else if (launch_overlapped(sgemm128<false>, dim3((unsigned)tk, (unsigned)tk, (unsigned)p.splits_s), 256, 0, st, a, K, a, K, SP,
                                    K, (int)K, (int)K, M, p.per_s, nullptr) != cudaSuccess)
             sg = FPQ_ERR_CUDA;

@@ -400,13 +400,14 @@ bool tf32x3_applies(const float* P, int64_t ldp, const float* Q, int64_t ldq, in
 fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ldq, int64_t I, int64_t J, int64_t R,
                          int kb_per_split, int epi, float* C, int64_t ldc, int64_t split_stride, double* sq_sum,
                          cudaStream_t st, int passes, const float* w_scale, float x_scale, const float* bias, int howo,
-                         int chunk, int columns)
+                         int chunk)
 {
+    const int columns = tf32x3_columns(J);
     static std::mutex mu;
     static EncodeTiledFn enc = nullptr;
     static bool attr_set[64] = {};
     if (!tf32x3_applies(P, ldp, Q, ldq, I, J, R) || kb_per_split < 1 || (passes != 1 && passes != 3) ||
-        epi < 0 || epi > 2 || chunk < 2 || (columns != 160 && columns != 256))
+        epi < 0 || epi > 2 || chunk < 2)
         return FPQ_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lock(mu);
