@@ -97,20 +97,22 @@ __device__ __forceinline__ float2 mul2(float2 a, float r)
     return d;
 }
 
-// Sixteen codes for the MMA operand (a minus zero may stay: as an operand it only ever contributes a
-// signed zero to the sum; NaN becomes code 0).
-__device__ __forceinline__ uint32_t e4m3x4_op(float t0, float t1, float t2, float t3, bool& nan)
+// Four codes for the MMA operand (a minus zero may stay: as an operand it only ever contributes a signed zero to the sum);
+// `nan` collects the top bits of bytes that are NaN.
+__device__ __forceinline__ uint32_t e4m3x4_op(float t0, float t1, float t2, float t3, uint32_t& nan)
 {
     uint16_t lo, hi;
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(lo) : "f"(t1), "f"(t0));
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(hi) : "f"(t3), "f"(t2));
     const uint32_t v = (uint32_t)lo | ((uint32_t)hi << 16);
-    const uint32_t nan_bytes = ((v & 0x7f7f7f7fu) + 0x01010101u) & 0x80808080u;
-    if (nan_bytes) {
-        nan = true;
-        return v & ~((nan_bytes >> 7) * 0xffu);
-    }
+    nan |= (v & 0x7f7f7f7fu) + 0x01010101u;
     return v;
+}
+// NaN becomes code 0
+__device__ __forceinline__ void clear_nan(uint4& v)
+{
+    auto clear = [](uint32_t& w) { w &= ~(((((w & 0x7f7f7f7fu) + 0x01010101u) & 0x80808080u) >> 7) * 0xffu); };
+    clear(v.x), clear(v.y), clear(v.z), clear(v.w);
 }
 
 __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid_constant__ CUtensorMap tmX,
@@ -446,14 +448,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
                             for (int q = 0; q < 16; ++q)
                                 a[q] = mul2(*reinterpret_cast<const float2*>(p + q * g.W), g.rinv);
                             uint4 v0, v1;
-                            v0.x = e4m3x4_op(a[0].x, a[1].x, a[2].x, a[3].x, nan);
-                            v0.y = e4m3x4_op(a[4].x, a[5].x, a[6].x, a[7].x, nan);
-                            v0.z = e4m3x4_op(a[8].x, a[9].x, a[10].x, a[11].x, nan);
-                            v0.w = e4m3x4_op(a[12].x, a[13].x, a[14].x, a[15].x, nan);
-                            v1.x = e4m3x4_op(a[0].y, a[1].y, a[2].y, a[3].y, nan);
-                            v1.y = e4m3x4_op(a[4].y, a[5].y, a[6].y, a[7].y, nan);
-                            v1.z = e4m3x4_op(a[8].y, a[9].y, a[10].y, a[11].y, nan);
-                            v1.w = e4m3x4_op(a[12].y, a[13].y, a[14].y, a[15].y, nan);
+                            uint32_t bad = 0;
+                            v0.x = e4m3x4_op(a[0].x, a[1].x, a[2].x, a[3].x, bad);
+                            v0.y = e4m3x4_op(a[4].x, a[5].x, a[6].x, a[7].x, bad);
+                            v0.z = e4m3x4_op(a[8].x, a[9].x, a[10].x, a[11].x, bad);
+                            v0.w = e4m3x4_op(a[12].x, a[13].x, a[14].x, a[15].x, bad);
+                            v1.x = e4m3x4_op(a[0].y, a[1].y, a[2].y, a[3].y, bad);
+                            v1.y = e4m3x4_op(a[4].y, a[5].y, a[6].y, a[7].y, bad);
+                            v1.z = e4m3x4_op(a[8].y, a[9].y, a[10].y, a[11].y, bad);
+                            v1.w = e4m3x4_op(a[12].y, a[13].y, a[14].y, a[15].y, bad);
+                            if (bad & 0x80808080u) {           // (one test per item, not per word)
+                                nan = true;
+                                clear_nan(v0), clear_nan(v1);
+                            }
                             if (i0 >= tr.i_lo)
                                 *reinterpret_cast<uint4*>(dst + i0 * 128 + ((cg ^ (i0 & 7)) << 4)) = v0;
                             const int i1 = i0 + 1;
