@@ -678,7 +678,7 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
         return FPQ_ERR_ALIGN;
     // a handful of rows (time-embedding projections): one pass over the weights on the CUDA cores,
     // whatever the route policy says; the workspace is not touched
-    if (small_m_linear_applies(M, K) && N <= 0x7fffffff && !is_e5m2_native(fw) && is_e4m3_native(fx)) {
+    if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(M, K, N, is_e2m1(fw) ? 1 : 0)) {
         if (!status_word())
             return FPQ_ERR_CUDA;
         return launch_small_m_linear(x, (int)M, (int)K, w_prepared, is_e2m1(fw) ? 1 : 0, (int)N, w_scale, x_scale, bias, y,

@@ -98,7 +98,7 @@ fpq_status launch_pair_rows(const GemmProblem& p, int terms, cudaStream_t st);
 bool pair_rows_preferred(const GemmProblem& p, int terms);   // in range, and faster than the general contraction
 
 // Linear layer with at most 8 rows on the CUDA cores (one pass over the weights).
-bool small_m_linear_applies(int64_t M, int64_t K);
+bool small_m_linear_preferred(int64_t M, int64_t K, int64_t N, int w4);
 fpq_status launch_small_m_linear(const float* x, int M, int K, const void* w_prepared, int w4, int N, const float* w_scale,
                                  float x_scale, const float* bias, float* y, cudaStream_t st);
 
