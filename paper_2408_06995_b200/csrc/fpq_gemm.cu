@@ -1196,6 +1196,24 @@ struct WeightSpec {
     int64_t M;
 };
 
+// Few rows in front of many weights: M x K up to 128 KB of activation codes.  (All CTAs read the same few lines; whatever the
+// cause, a CTA's stream of chunks is then up to 1.5 times slower, the more CTAs the slower: 64-wide tiles, 5120 -> 5120, 13.6
+// us at 32 rows and 18.1 at 24; 2560 -> 8576 9.7 us at 64 rows and 13.4 at 32.)
+static bool few_codes(int64_t M, int64_t cchunks) { return M * cchunks <= 1024; }
+
+// Whether a linear layer's tile is shared by a cluster of sp CTAs with `longest` chunks each: a chunk takes some 0.22 us
+// (64-wide tiles; 0.275: 128-wide ones), the exchange 1.3 us and, as row-major outputs leave it column by column, 0.19 us per
+// column of a CTA and 128 rows (us without / with, 64-wide: 2560 -> 320 at 64 rows 9.0 / 6.6, at 128 9.2 / 7.8, 2560 -> 2560 at
+// 64 9.2 / 9.5; 5120 -> 320 at 512 14.1 / 9.9; 1280 -> 320 at 128 7.1 / 7.3).  With few codes only clusters of five and more pay (8
+// rows: 1280 -> 320 6.4 / 5.5, 2560 -> 2560 9.0 / 10.5; 128-wide, 5120 -> 2560 15.7 / 11.6, 5120 -> 5120 16.2 / 16.6).
+static bool rows_split_pays(const GemmArgs& g, int BN, int sp, int longest)
+{
+    if (few_codes(g.M, g.cchunks) && sp < 5)
+        return false;
+    const double rows = g.M < BM ? (double)g.M : (double)BM;
+    return (g.cchunks - longest) * (BN == 64 ? 0.22 : 0.275) > 1.3 + BN / sp * rows / BM * 0.19;
+}
+
 template <int BN, bool FUSED, int MODE>
 static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, const CUtensorMap& tmY, GemmArgs& g,
                                  cudaStream_t st)
@@ -1254,10 +1272,7 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
             g.seg_ranks = r1;
             g.ksplit = r1 + r2;
         }
-    } else if (g.cchunks >= 2 && base_tiles * 2 <= di->sms &&
-               (MODE != MODE_ROWS || (g.m_tiles == 1 && (g.cchunks >= 32 || (g.M <= 8 && g.cchunks >= 8))))) {
-        // (row-major outputs leave the cluster's reduction column by column, which only pays for a single
-        // row tile with a very long reduction or a handful of rows: measured on the SD-v1 linears)
+    } else if (g.cchunks >= 2 && base_tiles * 2 <= di->sms) {
         int s_max = (int)(di->sms / base_tiles);
         if (s_max > 8) s_max = 8;
         if (s_max > g.cchunks) s_max = g.cchunks;
@@ -1268,7 +1283,8 @@ static fpq_status launch_mode(const CUtensorMap& tmA, const WeightSpec& wspec, c
             int sp = s_max;
             while (sp > 2 && (g.cchunks + sp - 2) / (sp - 1) == longest)
                 --sp;
-            g.ksplit = sp;
+            if (MODE != MODE_ROWS || rows_split_pays(g, BN, sp, longest))
+                g.ksplit = sp;
         }
     }
     // several column tiles per row tile: try to keep the row tile's whole activation panel in the
@@ -1498,8 +1514,12 @@ fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st)
     g.status = status_word();
     g.wait_prior_grid = p.after_stage1;
 
-    // (64-wide column tiles as well where a linear layer's 128-wide ones would leave half of the SMs idle)
-    const int BN = (p.N <= 64 || (!p.conv && p.x == nullptr && (p.M + BM - 1) / BM * ((p.N + 63) / 64) <= 148)) ? 64 : 128;
+    // (64-wide column tiles as well where a linear layer's 128-wide ones would leave half of the SMs idle; but not for few
+    // codes and many weights: 8 rows, 5120 -> 5120 20.3 us with 64, 16.2 with 128, 5120 -> 640 8.1 and 7.7, 2560 -> 5120 12.0 and 10.7, 2560 -> 2560 9.0 and 9.4)
+    int BN = p.N <= 64 ? 64 : 128;
+    if (!p.conv && p.x == nullptr && (p.M + BM - 1) / BM * ((p.N + 63) / 64) <= 148 &&
+        !(few_codes(p.M, g.cchunks) && p.N > (g.cchunks >= 32 ? 512 : g.cchunks >= 20 ? 2560 : 5120)))
+        BN = 64;
     g.n_tiles = (p.N + BN - 1) / BN;
     g.idesc = idesc_f8f6f4(p.a_e5m2 ? 1u : 0u, p.w4 ? 5u : (p.w_e5m2 ? 1u : 0u), (uint32_t)BN);
     g.b_block_tx = (uint32_t)(BN * BK) / (p.w4 ? 2 : 1);

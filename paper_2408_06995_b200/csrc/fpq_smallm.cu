@@ -162,7 +162,7 @@ SmallPlan plan_small(int64_t M, int64_t K, int64_t N, int w4)
     static const double step[2][4] = {{0.061, 0.10, 0.17, 0.32}, {0.185, 0.266, 0.41, 0.754}};
     static const double column[2][4] = {{0.085, 0.17, 0.19, 0.29}, {0.115, 0.124, 0.16, 0.36}};
     static const double chain[2][4] = {{107, 127, 190, 330}, {150, 255, 430, 690}};
-    p.ns = 1400.0 + (double)N * (p.steps * step[w4][i] + column[w4][i]) + 0.5 * ((p.steps + p.ks - 1) / p.ks) * chain[w4][i];
+    p.ns = 1400.0 + (double)N * (p.steps * step[w4][i] + column[w4][i]) + ((p.steps + p.ks - 1) / p.ks) * chain[w4][i];
     return p;
 }
 

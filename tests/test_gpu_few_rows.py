@@ -33,3 +33,15 @@ def test_nan_in_a_row_is_reported():
     assert fpq.fpq_read_status() == fpq.ERR_NAN_INPUT
     assert fpq.fpq_read_status() == fpq.OK
     assert bool(torch.isfinite(y).all())
+
+
+# tiles shared by clusters with several row tiles, ragged in rows, columns and chunks; few codes with 128-wide and 64-wide tiles
+@pytest.mark.parametrize("M,K,N", [(200, 5120, 321), (513, 4990, 100), (129, 2560, 70), (16, 5100, 2600), (9, 2700, 3000), (25, 5120, 513),
+                                   (64, 2304, 200)])
+@pytest.mark.parametrize("wfmt", ["e2m1", "e4m3"])
+def test_shared_tiles(M, K, N, wfmt):
+    L = I.draw(I.linear_layer("shared", M, K, N, wfmt), 32, M, "silu", 0.02, True)
+    ws, xs = layer_scales(L)
+    y = gpu_layer(L, ws, xs)
+    yo, ab = oracle_layer(L, ws, xs)
+    assert_close(y, yo, ab)
