@@ -81,7 +81,7 @@ struct GemmArgs {
     int b_loads;               // loads of a full weight stage
     int a_chunks;              // chunks of a full activation stage (not TAPS)
     int a_box_c;               // row-major activations: one load covers the a_box_c chunks of a stage (1 = one per chunk)
-    int y_tma;                 // row-major output leaves through TMA stores
+    int y_tma;                 // row-major output: 1 through TMA stores, 2 (N no multiple of 4) row by row, both from staging
     int y_stage;               // bytes of each epilogue warp's staging: two 4 KiB buffers, or one where a warp stores once
     int vec_scale;             // w_scale / bias are 16-byte aligned
     int stage_scales;          // x_scale * w_scale[n] and bias[n] of all N columns sit in shared memory
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
-        if (g.y_tma)
+        if (g.y_tma == 1)
             tma_prefetch_desc(&tmY);
     }
     if (warp == 1) {
@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                                     r[cl][j] = __float_as_uint(fmaf(__uint_as_float(r2[j]), sv, __uint_as_float(r[cl][j])));
                                 }
                             }
-                            if (g.y_tma) {
+                            if (g.y_tma == 1) {
                                 // the buffer is free once the store before the previous one has read it
                                 uint8_t* stage = stage0 + (nstore & 1u) * 4096;
                                 ++nstore;
@@ -856,36 +856,42 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                                         : "memory");
                                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                                 }
+                            } else if (MODE == MODE_ROWS) {
+                                // rows start anywhere, so a TMA store cannot take them: through the staging all the same,
+                                // then 32 neighbouring floats of a row per instruction (a lane storing along its own
+                                // row: 12263 x 1536 -> 2570, whole layer, 227.6 us, 84.9 so; 8192 x 320 -> 637 39.3 and
+                                // 12.8; 300 x 768 -> 333 9.8 and 6.2)
+                                const uint8_t* stage = stage0;
+                                __syncwarp();
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    *reinterpret_cast<uint4*>(stage0 + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                                        make_uint4(r[cl][4 * j], r[cl][4 * j + 1], r[cl][4 * j + 2], r[cl][4 * j + 3]);
+                                __syncwarp();
+                                const int64_t m0 = (int64_t)mt * BM + quarter * 32;
+                                const int rows = (int)min((int64_t)32, g.M - m0);
+                                float* dst = g.y + m0 * g.N + nb + lane;
+                                if (nb + lane < g.N) {
+#pragma unroll 8
+                                    for (int k = 0; k < rows; ++k, dst += g.N)
+                                        *dst = *reinterpret_cast<const float*>(stage + k * 128 + (((lane >> 2) ^ (k & 7)) << 4) + (lane & 3) * 4);
+                                }
                             } else if (row_valid) {
-                                if (MODE == MODE_ROWS) {
-                                    if (full && g.N % 4 == 0) {
-                                        uint4* dst = reinterpret_cast<uint4*>(yrow + nb);
+                                float* dst = yrow + (int64_t)nb * nstride;
+                                if (full) {
 #pragma unroll
-                                        for (int j = 0; j < 8; ++j)
-                                            dst[j] = make_uint4(r[cl][4 * j], r[cl][4 * j + 1], r[cl][4 * j + 2], r[cl][4 * j + 3]);
-                                    } else {
-#pragma unroll
-                                        for (int j = 0; j < 32; ++j)
-                                            if (nb + j < g.N)
-                                                yrow[nb + j] = __uint_as_float(r[cl][j]);
+                                    for (int j = 0; j < 32; j += 4) {
+                                        dst[0] = __uint_as_float(r[cl][j]);
+                                        dst[nstride] = __uint_as_float(r[cl][j + 1]);
+                                        dst[2 * nstride] = __uint_as_float(r[cl][j + 2]);
+                                        dst[3 * nstride] = __uint_as_float(r[cl][j + 3]);
+                                        dst += 4 * nstride;
                                     }
                                 } else {
-                                    float* dst = yrow + (int64_t)nb * nstride;
-                                    if (full) {
 #pragma unroll
-                                        for (int j = 0; j < 32; j += 4) {
-                                            dst[0] = __uint_as_float(r[cl][j]);
-                                            dst[nstride] = __uint_as_float(r[cl][j + 1]);
-                                            dst[2 * nstride] = __uint_as_float(r[cl][j + 2]);
-                                            dst[3 * nstride] = __uint_as_float(r[cl][j + 3]);
-                                            dst += 4 * nstride;
-                                        }
-                                    } else {
-#pragma unroll
-                                        for (int j = 0; j < 32; ++j)
-                                            if (nb + j < g.N)
-                                                dst[(int64_t)j * nstride] = __uint_as_float(r[cl][j]);
-                                    }
+                                    for (int j = 0; j < 32; ++j)
+                                        if (nb + j < g.N)
+                                            dst[(int64_t)j * nstride] = __uint_as_float(r[cl][j]);
                                 }
                             }
                         }
@@ -898,7 +904,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
             if (lane == 0)
                 mbar_arrive(acc_empty + 8 * buf);
         }
-        if (g.y_tma && lane == 0)
+        if (g.y_tma == 1 && lane == 0)
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the staging buffer must outlive its stores
         if (dead)
             flag_status(g.status, FPQ_ERR_TIMEOUT);
@@ -1099,26 +1105,38 @@ static EncodeTiledFn encode_fn() { return tensor_map_encoder(); }
 
 // Tile of output pixels of a convolution whose taps are loaded apart: rows of the image cut into equal parts of at most
 // 128 pixels, then as many image rows and images as 128 pixels hold, the cut with the fewest tiles.
-// (Powers of two would use 25 of 32 pixels of a row; 64 -> 64 channels at 33 x 33, stride 2, batch 30: 12.2 us so, 10.7 now.)
+// (64 -> 64 channels at 33 x 33, stride 2, batch 30, 17 of 32 pixels of a row in use with powers of two: 12.2 us so, 10.7 now.)
+// Powers of two where that is no fewer, and nothing narrower than 16: 416 -> 800 channels, one tap at stride 2, 51 x 51,
+// batch 31: 58 us with 32 x 4, 67 with the fewer tiles of 13 x 9.
 TapsTile choose_taps_tile(int B, int Ho, int Wo, int stride)
 {
     int wcap = 256 / stride;                           // (a box spans at most 256 framed pixels)
     if (wcap > BM)
         wcap = BM;
-    TapsTile best = {};
-    for (int cut = (Wo + wcap - 1) / wcap; cut <= Wo; ++cut) {
+    auto tile = [&](int w, int hmax) {
         TapsTile t;
-        t.w = (Wo + cut - 1) / cut;
-        t.tiles_x = (Wo + t.w - 1) / t.w;
-        const int hmax = BM / t.w < wcap ? BM / t.w : wcap;
+        t.w = w;
+        t.tiles_x = (Wo + w - 1) / w;
         t.tiles_y = (Ho + hmax - 1) / hmax;
         t.h = (Ho + t.tiles_y - 1) / t.tiles_y;
         t.b = BM / (t.w * t.h) < B ? BM / (t.w * t.h) : B;
         t.tiles = (int64_t)t.tiles_x * t.tiles_y * ((B + t.b - 1) / t.b);
-        if (best.w == 0 || t.tiles < best.tiles)
+        return t;
+    };
+    int w = 1, h = 1;
+    while (w < Wo && w < wcap) w *= 2;
+    while (h < Ho && h < BM / w && h < wcap) h *= 2;
+    TapsTile best = tile(w, h);
+    best.h = h;
+    best.b = BM / (w * h);
+    best.tiles = (int64_t)best.tiles_x * best.tiles_y * ((B + best.b - 1) / best.b);
+    for (int cut = (Wo + wcap - 1) / wcap; cut <= Wo; ++cut) {
+        const int part = (Wo + cut - 1) / cut;
+        const TapsTile t = tile(part, BM / part < wcap ? BM / part : wcap);
+        if (part < 16)
+            break;                                     // (short runs of memory)
+        if (t.tiles < best.tiles)
             best = t;
-        if (t.w <= 8)
-            break;                                     // (narrower: short runs of memory)
     }
     return best;
 }
@@ -1625,7 +1643,7 @@ fpq_status launch_gemm(const GemmProblem& p, cudaStream_t st)
 
     // row-major output through TMA stores
     CUtensorMap tmY = tmA;
-    g.y_tma = 0;
+    g.y_tma = p.conv ? 0 : 2;
     g.vec_scale = ((uintptr_t)p.w_scale % 16 == 0) && (p.bias == nullptr || (uintptr_t)p.bias % 16 == 0);
     if (!p.conv && p.N % 4 == 0 && (uintptr_t)p.y % 16 == 0) {
         cuuint64_t dimsY[2] = {(cuuint64_t)p.N, (cuuint64_t)p.M};
