@@ -961,10 +961,9 @@ fpq_status fpq_conv2d(const float* x, const void* w_prepared, const float* w_sca
             return FPQ_ERR_CUDA;
         cudaStream_t st = (cudaStream_t)stream;
         const int e5 = is_e5m2_native(fx) ? 1 : 0;
-        if (launch_quantize_nchw_to_nhwc_e4m3(x, B, C, H, W, pad, Cp, C2, 0, x_scale, (uint8_t*)workspace, st, e5) !=
-                cudaSuccess ||
-            launch_quantize_nchw_to_nhwc_e4m3(x, B, C, H, W, pad, Cp, C2, Cp, x_scale, (uint8_t*)workspace, st, e5) !=
-                cudaSuccess)
+        // (as if it were the concatenation of the tensor with itself: one launch)
+        if (launch_quantize_nchw_split(x, C, Cp, x_scale, x, C, Cp, x_scale, B, H, W, pad, (uint8_t*)workspace, st, e5) !=
+            cudaSuccess)
             return FPQ_ERR_CUDA;
         return conv2d_contract_impl(workspace, ws_bytes, w_prepared, w_scale, x_scale * two_term_unshift(fw), fx, term, bias,
                                     y, B, C2, H, W, C_out, R, S, pad, stride, stream, 1, nullptr);

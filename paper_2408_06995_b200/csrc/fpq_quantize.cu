@@ -908,6 +908,8 @@ __global__ void __launch_bounds__(256) quantize_nchw_to_nhwc_terms_kernel(const 
 __global__ void __launch_bounds__(256) repeat_rows_kernel(const uint4* __restrict__ src, int64_t rows, int64_t vec_per_row,
                                                           uint4* __restrict__ dst)
 {
+    // (the quantize kernel behind it starts when this one ends: let in early, 992 -> 192 channels at 38 x 38 took 26.0 us, not 20.9)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t total = rows * vec_per_row;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = i / vec_per_row, c = i - r * vec_per_row;
@@ -921,11 +923,8 @@ cudaError_t launch_quantize_rows_terms(const float* x, int64_t M, int64_t K, int
                                        const CodeTable& t1, const CodeTable* t2, uint8_t* codes, cudaStream_t st)
 {
     const int grid = grid_for(M * (Kp / 16), 256);
-    if (t2)
-        quantize_rows_terms_kernel<2><<<grid, 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, f, t1, *t2, codes, status_word());
-    else
-        quantize_rows_terms_kernel<1><<<grid, 256, 0, st>>>(x, M, K, Kp, 1.0f / scale, f, t1, t1, codes, status_word());
-    return cudaGetLastError();
+    return launch_overlapped(t2 ? quantize_rows_terms_kernel<2> : quantize_rows_terms_kernel<1>, dim3(grid), 256, 0, st, x, M, K, Kp,
+                             1.0f / scale, f, t1, t2 ? *t2 : t1, codes, status_word());
 }
 
 cudaError_t launch_quantize_nchw_to_nhwc_terms(const float* x, int B, int C, int H, int W, int pad, int Cp, float scale,
@@ -933,20 +932,14 @@ cudaError_t launch_quantize_nchw_to_nhwc_terms(const float* x, int B, int C, int
                                                cudaStream_t st)
 {
     dim3 grid((H * W + 31) / 32, (Cp + 127) / 128, B);
-    if (t2)
-        quantize_nchw_to_nhwc_terms_kernel<2><<<grid, 256, 0, st>>>(x, C, H, W, pad, Cp, 1.0f / scale, f, t1, *t2, codes,
-                                                                     status_word());
-    else
-        quantize_nchw_to_nhwc_terms_kernel<1><<<grid, 256, 0, st>>>(x, C, H, W, pad, Cp, 1.0f / scale, f, t1, t1, codes,
-                                                                     status_word());
-    return cudaGetLastError();
+    return launch_overlapped(t2 ? quantize_nchw_to_nhwc_terms_kernel<2> : quantize_nchw_to_nhwc_terms_kernel<1>, grid, 256, 0, st, x, C,
+                             H, W, pad, Cp, 1.0f / scale, f, t1, t2 ? *t2 : t1, codes, status_word());
 }
 
 cudaError_t launch_repeat_rows(const void* src, int64_t rows, int64_t row_bytes, void* dst, cudaStream_t st)
 {
     const int64_t vec = row_bytes / 16;
-    repeat_rows_kernel<<<grid_for(rows * vec, 256), 256, 0, st>>>((const uint4*)src, rows, vec, (uint4*)dst);
-    return cudaGetLastError();
+    return launch_overlapped(repeat_rows_kernel, dim3(grid_for(rows * vec, 256)), 256, 0, st, (const uint4*)src, rows, vec, (uint4*)dst);
 }
 
 // ---------------------------------------------------------------------------------
