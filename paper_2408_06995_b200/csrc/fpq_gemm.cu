@@ -236,6 +236,19 @@ __device__ __forceinline__ void fill_chunk_rows(const GemmArgs& g, uint8_t* dst,
 // FUSED = false: the activation operand is read as codes (TMA, written by a quantize kernel).
 // FUSED = true : 16 more warps read the FP32 activations and quantize them straight into the
 //                activation ring, so the codes never exist in global memory.
+// 32 x 32 floats from an epilogue warp's swizzled staging to rows m0 .. and columns n0 .. of y [M][N].  (Out of line: in the
+// epilogue's loop its code cost the layers that do not need it 2-3 %.)
+__device__ __noinline__ void store_rows(const uint8_t* stage, float* y, int64_t m0, int64_t M, int n0, int N, int lane)
+{
+    const int rows = (int)min((int64_t)32, M - m0);
+    float* dst = y + m0 * N + n0 + lane;
+    if (n0 + lane < N) {
+#pragma unroll 8
+        for (int k = 0; k < rows; ++k, dst += N)
+            *dst = *reinterpret_cast<const float*>(stage + k * 128 + (((lane >> 2) ^ (k & 7)) << 4) + (lane & 3) * 4);
+    }
+}
+
 template <int BN, bool FUSED, int MODE>
 __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                   const __grid_constant__ CUtensorMap tmB,
@@ -836,7 +849,7 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                                     r[cl][j] = __float_as_uint(fmaf(__uint_as_float(r2[j]), sv, __uint_as_float(r[cl][j])));
                                 }
                             }
-                            if (g.y_tma == 1) {
+                            if (MODE == MODE_ROWS) {
                                 // the buffer is free once the store before the previous one has read it
                                 uint8_t* stage = stage0 + (nstore & 1u) * 4096;
                                 ++nstore;
@@ -847,34 +860,22 @@ __global__ void __launch_bounds__(num_threads(FUSED), 1) fpq_gemm_kernel(const _
                                 for (int j = 0; j < 8; ++j)
                                     *reinterpret_cast<uint4*>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) =
                                         make_uint4(r[cl][4 * j], r[cl][4 * j + 1], r[cl][4 * j + 2], r[cl][4 * j + 3]);
-                                fence_proxy_async();
-                                __syncwarp();
-                                if (lane == 0) {
-                                    asm volatile(
-                                        "cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                        ::"l"(&tmY), "r"(smem_u32(stage)), "r"(nb), "r"(mt * BM + quarter * 32)
-                                        : "memory");
-                                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                                }
-                            } else if (MODE == MODE_ROWS) {
-                                // rows start anywhere, so a TMA store cannot take them: through the staging all the same,
-                                // then 32 neighbouring floats of a row per instruction (a lane storing along its own
-                                // row: 12263 x 1536 -> 2570, whole layer, 227.6 us, 84.9 so; 8192 x 320 -> 637 39.3 and
-                                // 12.8; 300 x 768 -> 333 9.8 and 6.2)
-                                const uint8_t* stage = stage0;
-                                __syncwarp();
-#pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    *reinterpret_cast<uint4*>(stage0 + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                                        make_uint4(r[cl][4 * j], r[cl][4 * j + 1], r[cl][4 * j + 2], r[cl][4 * j + 3]);
-                                __syncwarp();
-                                const int64_t m0 = (int64_t)mt * BM + quarter * 32;
-                                const int rows = (int)min((int64_t)32, g.M - m0);
-                                float* dst = g.y + m0 * g.N + nb + lane;
-                                if (nb + lane < g.N) {
-#pragma unroll 8
-                                    for (int k = 0; k < rows; ++k, dst += g.N)
-                                        *dst = *reinterpret_cast<const float*>(stage + k * 128 + (((lane >> 2) ^ (k & 7)) << 4) + (lane & 3) * 4);
+                                if (g.y_tma == 1) {
+                                    fence_proxy_async();
+                                    __syncwarp();
+                                    if (lane == 0) {
+                                        asm volatile(
+                                            "cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+                                            ::"l"(&tmY), "r"(smem_u32(stage)), "r"(nb), "r"(mt * BM + quarter * 32)
+                                            : "memory");
+                                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                                    }
+                                } else {
+                                    // rows start anywhere, so a TMA store cannot take them: 32 neighbouring floats of a row
+                                    // per instruction (a lane storing along its own row: 12263 x 1536 -> 2570, whole layer,
+                                    // 227.6 us, 84.9 so; 8192 x 320 -> 637 39.3 and 12.8; 300 x 768 -> 333 9.8 and 6.2)
+                                    __syncwarp();
+                                    store_rows(stage, g.y, (int64_t)mt * BM + quarter * 32, g.M, nb, g.N, lane);
                                 }
                             } else if (row_valid) {
                                 float* dst = yrow + (int64_t)nb * nstride;
