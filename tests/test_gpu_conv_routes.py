@@ -36,3 +36,23 @@ def test_routes_agree(B, C, H, W, Co, R, route):
     want = out[fpq.PATH_TWO_KERNELS]
     for got in out.values():
         assert float((got - want).abs().max()) <= 2e-5 * float(want.abs().max())
+
+
+# one tap: reductions shared by a cluster or not, on both sides of the rule
+@pytest.mark.parametrize("B,C,H,W,Co,stride", [(8, 256, 20, 20, 300, 2), (15, 1344, 11, 40, 357, 2), (4, 1280, 8, 8, 640, 2),
+                                               (2, 256, 16, 16, 256, 1), (2, 1280, 8, 8, 1280, 1)])
+def test_one_tap_reductions(B, C, H, W, Co, stride):
+    gen = torch.Generator(device="cuda").manual_seed(C + Co)
+    x = torch.randn(B, C, H, W, generator=gen, device="cuda")
+    w = torch.randn(Co, C, generator=gen, device="cuda") * 0.05
+    scale = (w.abs().amax(dim=1) / fpq.fpq_format_max(fpq.E2M1)).contiguous()
+    codes = fpq.fpq_quantize_weight(w, scale, fpq.E2M1)
+    conv = fpq.fpq_prepare_weight(codes, fpq.E2M1, fpq.CONV2D, Co, C, 1, 1)
+    got = fpq.fpq_conv2d(x, conv, scale, 0.01, fpq.E4M3, fpq.E2M1, None, Co, 1, 1, 0, stride)
+    rows = x[:, :, ::stride, ::stride].permute(0, 2, 3, 1).reshape(-1, C).contiguous()
+    lin = fpq.fpq_prepare_weight(codes, fpq.E2M1, fpq.LINEAR, Co, C)
+    want = fpq.fpq_linear(rows, lin, scale, 0.01, fpq.E4M3, fpq.E2M1, None, Co)
+    assert fpq.fpq_read_status() == fpq.OK
+    got = got.permute(0, 2, 3, 1).reshape(-1, Co)
+    # the same products, FP32 sums of at most 1344 of them in another order (as above)
+    assert float((got - want).abs().max()) <= 2e-5 * float(want.abs().max())
