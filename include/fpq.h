@@ -367,13 +367,15 @@ fpq_status fpq_search_clip_candidates(float maxabs, int32_t count, float* clip_h
  * The paper prints "+ lambda(alpha)" without saying how the per-weight terms combine or how they
  * are weighted: they are summed and the caller gives the weight `reg`.  The activations are used as
  * given (FP32, the same on both sides of the difference, as in the paper's equations).
- * Everything is computed at FP32 accuracy, the precision the method is stated in.  The two
- * contractions (A (Wq - W)^T, which is A Wq^T - A W^T by linearity, and its transpose product with A; or, with at
- * least 2 K rows and where that is fewer products, A^T A and its product with Wq - W)
- * run on the tensor cores when K is a multiple of 4 and `a` is 16-byte aligned: every FP32 product as
- * the sum of three TF32 products of exact operand splits, the reduction added up in FP32 (errors of a
- * few 1e-6 of the sum of absolute terms); otherwise they are FP32 multiply-adds on the CUDA cores.
- * The sums of squares and of lambda are accumulated in double.
+ * Everything is computed at FP32 accuracy, the precision the method is stated in: Wq - W is an FP32 number per
+ * weight, and the contractions are A (Wq - W)^T, which is A Wq^T - A W^T by linearity, and its transpose
+ * product with A.  They run on the tensor cores when K is a multiple of 4 and `a` is 16-byte aligned: every
+ * FP32 product as the sum of three TF32 products of exact operand splits, the reduction added up in FP32
+ * (errors of a few 1e-6 of the sum of absolute terms); or, where that is less work (many calibration rows),
+ * A^T A and its product with Wq - W in double, whose own errors are far below those of Wq - W.  Otherwise they
+ * are FP32 multiply-adds on the CUDA cores.  The sums of squares and of lambda are accumulated in double.
+ * mse is never negative.  Where the errors cancel along correlated calibration rows, what remains of it is
+ * as accurate as the FP32 differences Wq - W are (2^-22 of the weights in each at worst).
  *   w       [N][K] FP32 weights, scale [N] (as fpq_quantize_weight)
  *   fmt     weight format (any valid format; the paper learns rounding for FP4 only)
  *   alpha   [N][K] FP32, read; overwritten by alpha - lr * grad when lr != 0 (plain gradient descent)

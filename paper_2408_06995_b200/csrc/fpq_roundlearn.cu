@@ -1,17 +1,20 @@
 // Rounding learning (Sec. V-B): one evaluation of the objective
 //     mean((A Wq(alpha)^T - A W^T)^2) + reg * sum_i lambda(alpha_i)
 // and of its gradient with respect to alpha, for a bias-free linear layer with FP32 calibration
-// activations A [M][K].  The paper runs this step in FP32, so the two contractions here are FP32
-// FMA contractions on the CUDA cores (register-tiled, 128 x 128 x 16 tiles), not reduced-precision
-// tensor-core products.
+// activations A [M][K].  The paper runs this step in FP32, and the contractions keep at least that: the
+// direct form as three TF32 tensor-core products per FP32 product (fpq_tf32.cu), or FP32 multiply-adds on the CUDA cores
+// where rows are no multiple of 4 floats; the form with A^T A in double.
 //
-//   prepare_kernel          E = Wq(alpha) - W and dWq/dalpha per weight; A^T for the tensor-core routes
-//   sgemm128<true>          D = A E^T            (= Yq - Y by linearity), sum of D^2; with few output tiles the
-//                           reduction is cut into slices that reduce_d_kernel adds
-//   sgemm128<false>         partial sums of D^T A over slices of the M rows
+//   prepare_kernel          E = Wq(alpha) - W and dWq/dalpha per weight; A^T for the TF32 contractions
+// direct form
+//   tf32x3_gemm_kernel, or  D = A E^T            (= Yq - Y by linearity), sum of D^2; with few output tiles the
+//   sgemm128<true>          reduction is cut into slices that reduce_d_kernel adds
+//   the same, <false>       partial sums of D^T A over slices of the M rows
 //   grad_finalize_kernel    slices added in a fixed order, chain rule, sum of lambda, optional descent update
-// With many calibration rows D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are fewer products: see gram_preferred;
-// gram_grad_kernel then takes the place of the last two.
+// with many calibration rows (gram_preferred), where D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are less work
+//   gram_kernel             A^T A in double, slices of rows; gram_reduce_kernel adds them
+//   gram_grad_kernel        E (A^T A) in double, both losses, chain rule, optional descent update
+//
 //   harden_kernel           the inference rule: decision bit = (sigma(alpha) >= 0.5)
 //   unfold_kernel           a convolution's input rows, so that the same step serves convolution weights
 #include <math.h>
@@ -118,7 +121,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ 
                                                       const float* __restrict__ alpha, float* __restrict__ E,
                                                       float* __restrict__ DQ, double* __restrict__ loss, int64_t N, int64_t K,
                                                       int weight_blocks, const float* __restrict__ A, int64_t M,
-                                                      float* __restrict__ AT, int64_t Mp, int* __restrict__ status)
+                                                      float* __restrict__ AT, int64_t Mp, unsigned* __restrict__ ticket,
+                                                      int* __restrict__ status)
 {
     __shared__ float tile[32][33];
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -138,6 +142,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ 
     }
     if (blockIdx.x == 0 && threadIdx.x < 2)
         loss[threadIdx.x] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 2)
+        *ticket = 0;
     constexpr int V = VEC ? 4 : 1;
     const float c = __uint_as_float(f.cmax_bits);
     const int64_t per_row = K / V, total = N * per_row;
@@ -336,23 +342,20 @@ __device__ __forceinline__ float weight_gradient(float g, float dq, float al, fl
 }
 
 // grad = (2 / (M N)) (sum of the slices of D^T A) * dWq/dalpha + reg * dlambda/dalpha; alpha -= lr * grad when
-// lr != 0; sum of lambda.  E == NULL: thread 0 of block 0 turns the sum of squares into the mean; otherwise the mean is
-// <D^T A, E> / (M N), as sum D^2 = sum D (A E^T).
+// lr != 0; sum of lambda.  Thread 0 of block 0 turns the sum of squares into the mean.
 // VEC: four weights per thread.  Few blocks, each ending in two atomics: those of a thousand blocks took longer than the
 // rest (7.7 us for 960 x 320 weights).
 template <bool VEC>
 __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restrict__ GP, int splits,
-                                                            const float* __restrict__ DQ, const float* __restrict__ E,
-                                                            float* __restrict__ alpha, float* __restrict__ grad,
-                                                            double* __restrict__ loss, int64_t total, float coef,
-                                                            double inv_mn, float reg, float lr)
+                                                            const float* __restrict__ DQ, float* __restrict__ alpha,
+                                                            float* __restrict__ grad, double* __restrict__ loss,
+                                                            int64_t total, float coef, double inv_mn, float reg, float lr)
 {
     constexpr int V = VEC ? 4 : 1;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!E && blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0)
         loss[0] *= inv_mn;
     float lam = 0.f;
-    double sq = 0.0;
     auto load = [](const float* p, float (&v)[V]) {
         if (VEC) {
             const float4 t = *reinterpret_cast<const float4*>(p);
@@ -368,11 +371,9 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
             *p = v[0];
     };
     for (int64_t i = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < total; i += V * ((int64_t)gridDim.x * blockDim.x)) {
-        float g[V] = {}, dq[V], al[V], gr[V], e[V];
+        float g[V] = {}, dq[V], al[V], gr[V];
         load(DQ + i, dq);
         load(alpha + i, al);
-        if (E)
-            load(E + i, e);
 #pragma unroll 4
         for (int z = 0; z < splits; ++z) {
             float t[V];
@@ -383,8 +384,6 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
         }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            if (E)
-                sq = fma((double)g[v], (double)e[v], sq);
             gr[v] = weight_gradient(coef * g[v], dq[v], al[v], reg, lam);
             al[v] = al[v] - lr * gr[v];
         }
@@ -393,53 +392,172 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
             store(alpha + i, al);
     }
     block_atomic_add((double)lam, loss + 1);
-    if (E) {
-        __syncthreads();                               // (the helper's shared memory is used again)
-        block_atomic_add(sq * inv_mn, loss);
+}
+
+// ---- the gradient from S = A^T A, in double ----------------------------------------------------------------------
+// sum D^2 = <E S, E> squares what cancels in D = A E^T, and descent makes E small along the rows' leading directions, where
+// all of it cancels.  With S and E S in FP32 the loss of 4096 rows of rank 32 was up to 93 % off and negative at times; in
+// double (products of FP32 numbers are exact) it is closer than the FP32 sum of squares.  The FP64 matrix instructions give
+// 37 TFLOP/s and bound both kernels (70 % busy in gram_kernel, 42 % in gram_grad_kernel, whose blocks are short): 4096 x 320
+// rows and 960 x 320 weights 43.8 us for the whole step; with S in TF32 products 29.5, the direct form 59.6.
+
+// d += a b: 8 x 8 += (8 x 4) (4 x 8); lane l holds a[l / 4][l % 4], b[l % 4][l / 4], d[l / 4][2 (l % 4) + 0, 1]
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
+{
+    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+// 16 bytes to shared memory, zeros where there is nothing
+__device__ __forceinline__ void copy16(uint32_t to, const void* from, bool there)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
+}
+
+// S: 64 x 64 tiles on and above the diagonal, each over slices of the rows (blockIdx.y); slice z of tile t goes to SP + (z *
+// tiles + t) * 4096.  Stages of 32 rows; four warps have 32 x 32 outputs each, twice, for half of a stage's rows.
+// Rows of shared memory are 72 floats: the 4 x 8 elements of a fragment lie in 32 banks.
+constexpr int ST = 64, S_ROWS = 32, S_STAGES = 4, S_LD = ST + 8, S_STAGE = 2 * S_ROWS * S_LD;
+constexpr int S_SMEM = S_STAGES * S_STAGE * 4;
+static_assert(S_SMEM >= ST * ST * 8, "the second half's sums");
+__global__ void __launch_bounds__(256, 2) gram_kernel(const float* __restrict__ A, int64_t M, int64_t K, int tiles, int64_t per,
+                                                      double* __restrict__ SP)
+{
+    extern __shared__ __align__(16) float gsm[];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, half = warp >> 2;
+    int ti = 0, left = (int)blockIdx.x;
+    for (; left >= tiles - ti; ++ti)
+        left -= tiles - ti;
+    const int64_t i0 = (int64_t)ti * ST, j0 = (int64_t)(ti + left) * ST;
+    const int64_t m_lo = (int64_t)blockIdx.y * per, m_hi = min(m_lo + per, M);
+    const int wi = (warp & 1) * 32, wj = (warp >> 1 & 1) * 32;
+    auto fetch = [&](int stage, int64_t m) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(gsm + stage * S_STAGE);
+        const int row = t / 16, c = t % 16 * 4;
+#pragma unroll
+        for (int q = 0; q < S_ROWS; q += 16) {
+            const int64_t at = m + row + q;
+            const uint32_t to = dst + ((row + q) * S_LD + c) * 4;
+            const bool in_i = at < m_hi && i0 + c < K, in_j = at < m_hi && j0 + c < K;
+            copy16(to, in_i ? A + at * K + i0 + c : A, in_i);
+            copy16(to + S_ROWS * S_LD * 4, in_j ? A + at * K + j0 + c : A, in_j);
+        }
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int stages = (int)((m_hi - m_lo + S_ROWS - 1) / S_ROWS);
+#pragma unroll
+    for (int s = 0; s < S_STAGES - 1; ++s) {
+        if (s < stages)
+            fetch(s, m_lo + s * S_ROWS);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    double acc[4][4][2] = {};
+    for (int s = 0; s < stages; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(S_STAGES - 2) : "memory");
+        __syncthreads();                               // (and everybody is done with the stage that is filled next)
+        if (s + S_STAGES - 1 < stages)
+            fetch((s + S_STAGES - 1) % S_STAGES, m_lo + (int64_t)(s + S_STAGES - 1) * S_ROWS);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* p = gsm + s % S_STAGES * S_STAGE + (half * (S_ROWS / 2) + (lane & 3)) * S_LD + (lane >> 2);
+#pragma unroll
+        for (int k = 0; k < S_ROWS / 2; k += 4) {
+            double a[4], b[4];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                a[f] = (double)p[k * S_LD + wi + 8 * f];
+                b[f] = (double)p[(S_ROWS + k) * S_LD + wj + 8 * f];
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    mma_f64(acc[x][y], a[x], b[y]);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    double* other = reinterpret_cast<double*>(gsm);
+    double* out = SP + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (ST * ST);
+    const int at = (wi + (lane >> 2)) * ST + wj + 2 * (lane & 3);
+    if (half) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                *reinterpret_cast<double2*>(other + at + 8 * x * ST + 8 * y) = make_double2(acc[x][y][0], acc[x][y][1]);
+    }
+    __syncthreads();
+    if (!half) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const double2 o = *reinterpret_cast<const double2*>(other + at + 8 * x * ST + 8 * y);
+                *reinterpret_cast<double2*>(out + at + 8 * x * ST + 8 * y) = make_double2(acc[x][y][0] + o.x, acc[x][y][1] + o.y);
+            }
     }
 }
 
-// The gradient from S = A^T A in one kernel: a 4 RA x 64 tile of E S per block, reduced over all of K, then what
-// grad_finalize_kernel does.  S is symmetric, so both operands are read as they lie.  64 reduction elements per stage, three
-// stages of asynchronous copies; each of the eight warps takes eight elements of a stage and has a sum of its own for the
-// whole tile, RA x 8 outputs per thread (shared memory gives 128 bytes per clock whatever part of them is broadcast: with 4 x
-// 4 outputs the loads took twice the time of the multiply-adds).  With 128 x 128 tiles the reduction had to be sliced to
-// fill the SMs, and writing, reading and adding the slices took as long again (9.9 + 5.2 us for 960 x 320 weights, 11.3 here;
-// the whole step with 4096 rows 37.1 -> 33.2 us, 512 x 256 weights and 1024 rows 20.3 -> 18.4, 555 x 128 and 431 17.9 -> 15.2).
-constexpr int GK = 64, GR = 64, G_STAGES = 3;
-constexpr int GE_LD = GR + 4;                          // rows of E in shared memory (floats)
-__host__ __device__ constexpr int gram_stage(int ra) { return 4 * ra * GE_LD + GR * GK; }      // floats
-constexpr int gram_smem(int ra)                        // the stages, and afterwards the warps' sums
+// S [K][K] = the slices added in their order, both triangles.  A block has 8 rows of a tile (blockIdx.y), a thread two columns.
+__global__ void __launch_bounds__(256) gram_reduce_kernel(const double* __restrict__ SP, int slices, int tiles, double* __restrict__ S,
+                                                          int64_t K)
 {
-    return 4 * (G_STAGES * gram_stage(ra) > 8 * 4 * ra * GK ? G_STAGES * gram_stage(ra) : 8 * 4 * ra * GK);
+    __shared__ double turn[8][ST + 1];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int ti = 0, left = (int)blockIdx.x;
+    for (; left >= tiles - ti; ++ti)
+        left -= tiles - ti;
+    const int64_t i0 = (int64_t)ti * ST + blockIdx.y * 8, j0 = (int64_t)(ti + left) * ST;
+    const int row = threadIdx.x / 32, c = threadIdx.x % 32 * 2;
+    const double* p = SP + (int64_t)blockIdx.x * (ST * ST) + (blockIdx.y * 8 + row) * ST + c;
+    double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int z = 0; z < slices; ++z) {
+        const double2 v = *reinterpret_cast<const double2*>(p + (int64_t)z * gridDim.x * (ST * ST));
+        sum.x += v.x, sum.y += v.y;
+    }
+    if (i0 + row < K && j0 + c < K)                    // (K is even)
+        *reinterpret_cast<double2*>(S + (i0 + row) * K + j0 + c) = sum;
+    turn[row][c] = sum.x, turn[row][c + 1] = sum.y;
+    __syncthreads();
+    const int col = threadIdx.x / 4, r = threadIdx.x % 4 * 2;
+    if (left && j0 + col < K && i0 + r < K)
+        *reinterpret_cast<double2*>(S + (j0 + col) * K + i0 + r) = make_double2(turn[r][col], turn[r + 1][col]);
 }
-template <int RA>
-__global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restrict__ E, const float* __restrict__ S,
-                                                           const float* __restrict__ DQ, float* __restrict__ alpha,
-                                                           float* __restrict__ grad, double* __restrict__ loss, int64_t N,
-                                                           int64_t K, float coef, double inv_mn, float reg, float lr, int vec)
+
+// The rest of the step from S in one kernel: a ROWS x 64 tile of E S per block, reduced over all of K, then what
+// grad_finalize_kernel does.  S is symmetric, so both operands are read as they lie.  64 reduction elements per stage, three
+// stages of asynchronous copies; each of the eight warps has half of the columns and a quarter of a stage's elements, and
+// the quarters' sums are added through shared memory.  Rows are padded so that a fragment's elements lie in different banks.
+constexpr int GK = 64, GR = 64, G_STAGES = 3;
+constexpr int GE_LD = GR + 4, GS_LD = GK + 4, GO_LD = GK + 2;      // floats of E, doubles of S, doubles of a sum
+__host__ __device__ constexpr int gram_stage(int rows) { return rows * GE_LD * 4 + GR * GS_LD * 8; }      // bytes
+constexpr int gram_smem(int rows)
 {
-    constexpr int GN = 4 * RA, G_STAGE = gram_stage(RA);
-    extern __shared__ __align__(16) float gsm[];
-    const int t = threadIdx.x, warp = t >> 5, ty = (t >> 3) & 3, tx = t & 7;
-    const int64_t n0 = (int64_t)blockIdx.x * GN, k0 = (int64_t)blockIdx.y * GK;
+    return G_STAGES * gram_stage(rows) > 4 * rows * GO_LD * 8 ? G_STAGES * gram_stage(rows) : 4 * rows * GO_LD * 8;
+}
+template <int ROWS>
+__global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restrict__ E, const double* __restrict__ S,
+                                                           const float* __restrict__ DQ, float* __restrict__ alpha,
+                                                           float* __restrict__ grad, double* __restrict__ loss,
+                                                           unsigned* __restrict__ ticket, int64_t N, int64_t K, double coef,
+                                                           double inv_mn, float reg, float lr, int vec)
+{
+    constexpr int F = ROWS / 8;
+    extern __shared__ __align__(16) uint8_t gsm8[];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, col0 = (warp & 1) * 32, part = warp >> 1;
+    const int64_t n0 = (int64_t)blockIdx.x * ROWS, k0 = (int64_t)blockIdx.y * GK;
     auto fetch = [&](int stage, int64_t r0) {
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(gsm + stage * G_STAGE);
-        auto copy = [](uint32_t to, const float* from, bool there) {       // (zeros where there is nothing)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
-        };
-        const int row = t / (GR / 4), c = t % (GR / 4) * 4;
+        const uint32_t e = (uint32_t)__cvta_generic_to_shared(gsm8 + stage * gram_stage(ROWS)), s = e + ROWS * GE_LD * 4;
 #pragma unroll
-        for (int q = 0; q < GN; q += 16) {
-            if (GN % 16 && row + q >= GN)
-                break;
-            const bool there = n0 + row + q < N && r0 + c < K;
-            copy(dst + ((row + q) * GE_LD + c) * 4, there ? E + (n0 + row + q) * K + r0 + c : E, there);
+        for (int id = t; id < ROWS * (GR / 4); id += 256) {
+            const int row = id / (GR / 4), c = id % (GR / 4) * 4;
+            const bool there = n0 + row < N && r0 + c < K;
+            copy16(e + (row * GE_LD + c) * 4, there ? E + (n0 + row) * K + r0 + c : E, there);
         }
 #pragma unroll
-        for (int q = 0; q < GR; q += 16) {
-            const bool there = r0 + row + q < K && k0 + c < K;
-            copy(dst + (GN * GE_LD + (row + q) * GK + c) * 4, there ? S + (r0 + row + q) * K + k0 + c : S, there);
+        for (int id = t; id < GR * (GK / 2); id += 256) {
+            const int row = id / (GK / 2), c = id % (GK / 2) * 2;
+            const bool there = r0 + row < K && k0 + c < K;
+            copy16(s + (row * GS_LD + c) * 8, there ? S + (r0 + row) * K + k0 + c : S, there);
         }
     };
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -450,60 +568,51 @@ __global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restri
             fetch(i, (int64_t)i * GR);
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    unsigned long long acc[RA][4];                     // rows ty + 4 a; columns 4 tx + 0 .. 3, 32 + 4 tx + 0 .. 3
-#pragma unroll
-    for (int a = 0; a < RA; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            acc[a][b] = 0ull;
+    double acc[F][4][2] = {};
     for (int i = 0; i < stages; ++i) {
         asm volatile("cp.async.wait_group %0;" ::"n"(G_STAGES - 2) : "memory");
         __syncthreads();                               // (and everybody is done with the stage that is filled next)
         if (i + G_STAGES - 1 < stages)
             fetch((i + G_STAGES - 1) % G_STAGES, (int64_t)(i + G_STAGES - 1) * GR);
         asm volatile("cp.async.commit_group;" ::: "memory");
-        const float* es = gsm + i % G_STAGES * G_STAGE + ty * GE_LD + warp * 8;
-        const float* ss = gsm + i % G_STAGES * G_STAGE + GN * GE_LD + warp * 8 * GK + tx * 4;
+        const uint8_t* stage = gsm8 + i % G_STAGES * gram_stage(ROWS);
+        const float* es = reinterpret_cast<const float*>(stage) + (lane >> 2) * GE_LD + part * (GR / 4) + (lane & 3);
+        const double* ss = reinterpret_cast<const double*>(stage + ROWS * GE_LD * 4) + (part * (GR / 4) + (lane & 3)) * GS_LD +
+                           col0 + (lane >> 2);
 #pragma unroll
-        for (int r4 = 0; r4 < 8; r4 += 4) {
-            float e[RA][4];
+        for (int r = 0; r < GR / 4; r += 4) {
+            double b[4];
 #pragma unroll
-            for (int a = 0; a < RA; ++a) {
-                const float4 v = *reinterpret_cast<const float4*>(es + a * 4 * GE_LD + r4);
-                e[a][0] = v.x, e[a][1] = v.y, e[a][2] = v.z, e[a][3] = v.w;
-            }
+            for (int y = 0; y < 4; ++y)
+                b[y] = ss[r * GS_LD + 8 * y];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const ulonglong2 v0 = *reinterpret_cast<const ulonglong2*>(ss + (r4 + q) * GK);
-                const ulonglong2 v1 = *reinterpret_cast<const ulonglong2*>(ss + (r4 + q) * GK + 32);
+            for (int x = 0; x < F; ++x) {
+                const double a = (double)es[8 * x * GE_LD + r];
 #pragma unroll
-                for (int a = 0; a < RA; ++a) {
-                    const unsigned long long ee = pack2(e[a][q], e[a][q]);
-                    fma2(acc[a][0], ee, v0.x);
-                    fma2(acc[a][1], ee, v0.y);
-                    fma2(acc[a][2], ee, v1.x);
-                    fma2(acc[a][3], ee, v1.y);
-                }
+                for (int y = 0; y < 4; ++y)
+                    mma_f64(acc[x][y], a, b[y]);
             }
         }
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    double* sums = reinterpret_cast<double*>(gsm8);
 #pragma unroll
-    for (int a = 0; a < RA; ++a) {
-        float* to = gsm + warp * GN * GK + (ty + 4 * a) * GK + tx * 4;
-        *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(acc[a][0], acc[a][1]);
-        *reinterpret_cast<ulonglong2*>(to + 32) = make_ulonglong2(acc[a][2], acc[a][3]);
-    }
+    for (int x = 0; x < F; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+            *reinterpret_cast<double2*>(sums + (part * ROWS + 8 * x + (lane >> 2)) * GO_LD + col0 + 8 * y + 2 * (lane & 3)) =
+                make_double2(acc[x][y][0], acc[x][y][1]);
     __syncthreads();
     float lam = 0.f;
     double sq = 0.0;
-    for (int id = t; id < GN * GK / 4; id += 256) {
+    for (int id = t; id < ROWS * GK / 4; id += 256) {
         const int row = id / (GK / 4), c = id % (GK / 4) * 4;
         if (n0 + row >= N || k0 + c >= K)
             continue;
         const int64_t at = (n0 + row) * K + k0 + c;
         const float4 dq = *reinterpret_cast<const float4*>(DQ + at), e = *reinterpret_cast<const float4*>(E + at);
-        float al[4], gr[4], g[4] = {0.f, 0.f, 0.f, 0.f};
+        float al[4], gr[4];
         if (vec) {
             const float4 v = *reinterpret_cast<const float4*>(alpha + at);
             al[0] = v.x, al[1] = v.y, al[2] = v.z, al[3] = v.w;
@@ -512,16 +621,15 @@ __global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restri
             for (int v = 0; v < 4; ++v)
                 al[v] = alpha[at + v];
         }
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            const float4 v = *reinterpret_cast<const float4*>(gsm + w * GN * GK + row * GK + c);
-            g[0] += v.x, g[1] += v.y, g[2] += v.z, g[3] += v.w;
-        }
         const float d[4] = {dq.x, dq.y, dq.z, dq.w}, ev[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            sq = fma((double)g[v], (double)ev[v], sq);
-            gr[v] = weight_gradient(coef * g[v], d[v], al[v], reg, lam);
+            double g = 0.0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                g += sums[(q * ROWS + row) * GO_LD + c + v];
+            sq = fma(g, (double)ev[v], sq);
+            gr[v] = weight_gradient((float)(coef * g), d[v], al[v], reg, lam);
             al[v] = al[v] - lr * gr[v];
         }
         if (vec) {
@@ -540,34 +648,14 @@ __global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restri
     block_atomic_add((double)lam, loss + 1);
     __syncthreads();                                   // (the helper's shared memory is used again)
     block_atomic_add(sq * inv_mn, loss);
-}
-
-// S = sum of the slices of A^T A [K][K] (fixed order; the sums in double).  Eight threads share four floats, each adding
-// every eighth slice: a whole wave of loads is in flight at once.
-__global__ void __launch_bounds__(256) reduce_gram_kernel(const float4* __restrict__ SP, int splits, float4* __restrict__ S,
-                                                          int64_t total4)
-{
-    __shared__ double4 part[8][32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
-    double4 t = make_double4(0.0, 0.0, 0.0, 0.0);
-    if (i < total4) {
-#pragma unroll 8
-        for (int k = group; k < splits; k += 8) {
-            const float4 v = SP[(int64_t)k * total4 + i];
-            t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+    // a sum of squares: rounding must not leave it below zero (the block that comes last looks)
+    if (t == 0) {
+        __threadfence();
+        if (atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1) {
+            __threadfence();
+            if (__ldcg(loss) < 0.0)
+                *loss = 0.0;
         }
-    }
-    part[group][lane] = t;
-    __syncthreads();
-    if (group == 0 && i < total4) {
-#pragma unroll
-        for (int k = 1; k < 8; ++k) {
-            const double4 v = part[k][lane];
-            t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
-        }
-        S[i] = make_float4((float)t.x, (float)t.y, (float)t.z, (float)t.w);
     }
 }
 
@@ -646,28 +734,29 @@ struct Plan {
     int kb_per_split_tc, splits_tc;
     int kb_per_split1_tc, splits1_tc;       // first contraction: sliced too when it has few output tiles
     size_t off_AT, off_DT;
-    // with A^T A: slices of M in it, slices of its K rows in the product with E
-    int gram, tc_s, tc_g, splits_s, splits_g;      // tc_*: on the tensor cores (slices in 32-wide blocks), else FP32 multiply-adds
-    int64_t per_s, per_g;                          // 32-wide blocks or elements per slice
-    size_t off_SP, off_S;
+    // with A^T A: 64-wide tiles per side, slices of M
+    int gram, tiles_s, slices_s;
+    int64_t rows_s;
+    size_t off_SP, off_S, off_ticket;
 };
 
-// E (A^T A) in place of (A E^T)^T A: M K^2 + N K^2 products instead of 2 M N K (calibration rows: QKV 320 -> 960 with
-// 4096 rows 0.5 G instead of 2.5 G).  Only with clearly more rows than columns: A^T A is then well away from singular, and
-// the mean square, <E (A^T A), E>, keeps its relative accuracy.
+// E (A^T A) in place of (A E^T)^T A: half of M K^2 and N K^2 products in double instead of 2 M N K on the TF32 tensor cores,
+// by estimates in microseconds of both whole steps (us so / direct, M x N x K: 4096 x 960 x 320 43.8 / 59.6, 8192 x 2560 x 320
+// 88.4 / 195.5, 1024 x 512 x 256 22.9 / 38.0, 139 x 1394 x 192 19.2 / 32.4, 2048 x 320 x 320 30.9 / 33.0, 8192 x 1280 x 640 194.0 / 192.6, 8192 x
+// 320 x 320 59.5 / 43.8, 2048 x 640 x 640 68.5 / 50.8, 4096 x 2560 x 1280 614 / 419).
 bool gram_preferred(int64_t M, int64_t N, int64_t K)
 {
-    return K % 4 == 0 && M >= 2 * K && (double)K * (double)(M + N) * 1.25 <= 2.0 * (double)M * (double)N;
+    const double m = (double)M, n = (double)N, k = (double)K;
+    return K % 4 == 0 && 16.0 + (0.5 * m * k * (k + 64) + n * k * k) / 11.5e6 <= 25.0 + 2.0 * m * n * k / 80e6;
 }
 
-// Rows of gram_grad_kernel's tiles: the fewest whose blocks all run at once, one per SM (150 blocks of 32 rows take 15.5 us
-// where 120 of 40 take 11.3: two SMs have two of them); 0: not even with 64.
+// Rows of gram_grad_kernel's tiles: the fewest whose blocks all run at once, one per SM; with several rounds of them, 64.
 int gram_tile_rows(int64_t N, int64_t K)
 {
-    for (int rows : {32, 40, 48, 64})
+    for (int rows : {32, 40, 48})
         if ((N + rows - 1) / rows * ((K + 63) / 64) <= 148)
             return rows;
-    return 0;
+    return 64;
 }
 
 // As many slices of a reduction of length R as still fit into one wave of two resident blocks per SM (one more
@@ -737,81 +826,54 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     o += (size_t)round_up(N * p.Mp * 4, 256);
     p.gram = gram_preferred(M, N, K);
     if (p.gram) {
-        auto cut = [](int64_t tiles, int64_t kblocks, int64_t least, int64_t* per, int* splits) {
-            int64_t want = 148 / tiles;
-            want = want < 1 ? 1 : (want > 64 ? 64 : want);
-            int64_t each = (kblocks + want - 1) / want;
-            *per = each < least ? least : each;
-            *splits = (int)((kblocks + *per - 1) / *per);
-        };
-        // multiply-adds: a 16-wide stage takes some 1200 cycles however few there are, so slices are short
-        auto cut_short = [](int64_t tiles, int64_t R, int64_t* per, int* splits) {
-            const int64_t least = tiles > 8 ? 64 : 32;
-            int64_t want = 2 * 148 / tiles;
-            want = want < 1 ? 1 : (want > 32 ? 32 : want);
-            const int64_t each = (R + want - 1) / want;
-            *per = round_up(each < least ? least : each, BK);
-            *splits = (int)((R + *per - 1) / *per);
-        };
-        // (the tensor-core kernel has some 10 us of its own: 128 x 256 tiles filled, split, drained and stored)
-        const int64_t tk = (K + 127) / 128;
-        p.tc_s = M * K * K >= 100000000;
-        if (p.tc_s)
-            cut(tk * ((K + tf32x3_columns(K) - 1) / tf32x3_columns(K)), (M + 31) / 32, 4, &p.per_s, &p.splits_s);
-        else
-            cut_short(tk * tk, M, &p.per_s, &p.splits_s);
-        // the product with E: gram_grad_kernel, some 4 us and 35 ns per row of its tiles and 64 of K, unless it has several
-        // rounds of blocks, or the tensor cores and grad_finalize_kernel (some 17.5 us) are faster
-        const int rows = gram_tile_rows(N, K);
-        p.tc_g = rows ? (K + 63) / 64 * rows > 385 : N * K * K >= 130000000;
-        p.splits_g = 1;
-        if (p.tc_g)
-            cut(tk * ((N + tf32x3_columns(N) - 1) / tf32x3_columns(N)), (K + 31) / 32, 1, &p.per_g, &p.splits_g);
-        p.off_SP = o;
-        o += (size_t)round_up((int64_t)p.splits_s * K * K * 4, 256);
-        p.off_S = o;
-        o += (size_t)round_up(K * K * 4, 256);
-        const int64_t gp = (int64_t)round_up((int64_t)p.splits_g * N * K * 4, 256);
-        if (gp > (int64_t)(p.off_AT - p.off_GP)) {
-            p.off_GP = o;
-            o += (size_t)gp;
+        // the slices with the shortest rounds of blocks (a stage of 32 rows and the sums' way out as two of them)
+        p.tiles_s = (int)((K + ST - 1) / ST);
+        const int64_t tiles = (int64_t)p.tiles_s * (p.tiles_s + 1) / 2, stages = (M + S_ROWS - 1) / S_ROWS;
+        int64_t best = 0;
+        for (int64_t want = 1; want <= 64 && want <= stages; ++want) {
+            const int64_t each = (stages + want - 1) / want, slices = (stages + each - 1) / each;
+            const int64_t cost = (tiles * slices + 147) / 148 * (each + 2);
+            if (best == 0 || cost < best) {
+                best = cost;
+                p.slices_s = (int)slices;
+                p.rows_s = each * S_ROWS;
+            }
         }
+        p.off_SP = o;
+        o += (size_t)round_up((int64_t)p.slices_s * tiles * ST * ST * 8, 256);
+        p.off_S = o;
+        o += (size_t)round_up(K * K * 8, 256);
     }
+    p.off_ticket = o;
+    o += 256;
     p.bytes = o;
     return p;
 }
 
-template <int RA>
-fpq_status launch_gram_grad_rows(const float* E, const float* S, const float* DQ, float* alpha, float* grad, double* loss,
-                                 int64_t N, int64_t K, float coef, double inv_mn, float reg, float lr, cudaStream_t st)
+// most dynamic shared memory of a kernel, set once per device
+template <typename Kernel>
+bool allow_smem(Kernel kernel, int bytes, bool (&set)[64])
 {
-    {
-        static std::mutex mu;
-        static bool attr_set[64] = {};
-        std::lock_guard<std::mutex> lock(mu);
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
-            return FPQ_ERR_CUDA;
-        if (!attr_set[dev]) {
-            if (cudaFuncSetAttribute(gram_grad_kernel<RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, gram_smem(RA)) != cudaSuccess)
-                return FPQ_ERR_CUDA;
-            attr_set[dev] = true;
-        }
-    }
-    const int vec = (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
-    return launch_overlapped(gram_grad_kernel<RA>, dim3((unsigned)((N + 4 * RA - 1) / (4 * RA)), (unsigned)((K + GK - 1) / GK)), 256,
-                             gram_smem(RA), st, E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, vec) == cudaSuccess
-               ? FPQ_OK
-               : FPQ_ERR_CUDA;
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+        return false;
+    if (!set[dev])
+        set[dev] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    return set[dev];
 }
 
-fpq_status launch_gram_grad(const float* E, const float* S, const float* DQ, float* alpha, float* grad, double* loss, int64_t N,
-                            int64_t K, float coef, double inv_mn, float reg, float lr, cudaStream_t st)
+template <int ROWS>
+cudaError_t launch_gram_grad(const float* E, const double* S, const float* DQ, float* alpha, float* grad, double* loss, unsigned* ticket,
+                             int64_t N, int64_t K, double coef, double inv_mn, float reg, float lr, cudaStream_t st)
 {
-    const int rows = gram_tile_rows(N, K);
-    const auto launch = rows == 32 ? launch_gram_grad_rows<8> : rows == 40 ? launch_gram_grad_rows<10>
-                        : rows == 48 ? launch_gram_grad_rows<12> : launch_gram_grad_rows<16>;
-    return launch(E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, st);
+    static bool set[64] = {};
+    if (!allow_smem(gram_grad_kernel<ROWS>, gram_smem(ROWS), set))
+        return cudaErrorUnknown;
+    const int vec = (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
+    return launch_overlapped(gram_grad_kernel<ROWS>, dim3((unsigned)((N + ROWS - 1) / ROWS), (unsigned)((K + GK - 1) / GK)), 256,
+                             gram_smem(ROWS), st, E, S, DQ, alpha, grad, loss, ticket, N, K, coef, inv_mn, reg, lr, vec);
 }
 
 }  // namespace
@@ -836,46 +898,41 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
     const float coef = (float)(2.0 * inv_mn);
     const bool tc = tf32x3_applies(a, K, E, K, M, N, K) && M <= (1 << 21) && N <= (1 << 21) && K <= (1 << 21);
     float* AT = (float*)(ws + p.off_AT);
+    unsigned* ticket = (unsigned*)(ws + p.off_ticket);
     {
         const bool vec = K % 4 == 0 && (uintptr_t)w % 16 == 0 && (uintptr_t)alpha % 16 == 0;
         const int weight_blocks = grid_for(vec ? N * K / 4 : N * K);
-        const int64_t blocks = weight_blocks + (tc && !(p.gram && !p.tc_s) ? ((M + 31) / 32) * ((K + 31) / 32) : 0);
+        const int64_t blocks = weight_blocks + (tc && !p.gram ? ((M + 31) / 32) * ((K + 31) / 32) : 0);
         if (blocks > 0x7fffffff)
             return FPQ_ERR_SHAPE;
         if (launch_overlapped(vec ? prepare_kernel<true> : prepare_kernel<false>, dim3((unsigned)blocks), 256, 0, st, w, scale, f,
-                              alpha, E, DQ, loss, N, K, weight_blocks, a, M, AT, p.Mp, status) != cudaSuccess)
+                              alpha, E, DQ, loss, N, K, weight_blocks, a, M, AT, p.Mp, ticket, status) != cudaSuccess)
             return FPQ_ERR_CUDA;
     }
-    auto finalize = [&](int splits, const float* e) {
+    auto finalize = [&](int splits) {
         const bool vec = N * K % 4 == 0 && (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
         int blocks = grid_for(vec ? N * K / 4 : N * K);
         blocks = blocks > 2 * 148 ? 2 * 148 : blocks;
         return launch_overlapped(vec ? grad_finalize_kernel<true> : grad_finalize_kernel<false>, dim3(blocks), 256, 0, st, GP,
-                                 splits, DQ, e, alpha, grad, loss, N * K, coef, inv_mn, reg, lr) == cudaSuccess
+                                 splits, DQ, alpha, grad, loss, N * K, coef, inv_mn, reg, lr) == cudaSuccess
                    ? FPQ_OK
                    : FPQ_ERR_CUDA;
     };
     if (tc && p.gram) {
-        const int64_t tk = (K + TILE - 1) / TILE;
-        float* SP = (float*)(ws + p.off_SP);
-        float* S = (float*)(ws + p.off_S);
-        // (chunks of 4 blocks: half the bias of the truncating additions, which enters twice here)
-        fpq_status sg = FPQ_OK;
-        if (p.tc_s)
-            sg = launch_tf32x3(AT, p.Mp, AT, p.Mp, K, K, M, (int)p.per_s, 1, SP, K, K * K, nullptr, st, 3, nullptr, 1.0f, nullptr,
-                               0, 4);
-        else if (launch_overlapped(sgemm128<false>, dim3((unsigned)tk, (unsigned)tk, (unsigned)p.splits_s), 256, 0, st, a, K, a, K, SP,
-                                   K, (int)K, (int)K, M, p.per_s, nullptr) != cudaSuccess)
-            sg = FPQ_ERR_CUDA;
-        if (sg != FPQ_OK)
-            return sg;
-        if (launch_overlapped(reduce_gram_kernel, dim3((unsigned)((K * K / 4 + 31) / 32)), 256, 0, st, (const float4*)SP, p.splits_s,
-                              (float4*)S, K * K / 4) != cudaSuccess)
+        double* SP = (double*)(ws + p.off_SP);
+        double* S = (double*)(ws + p.off_S);
+        const unsigned tiles = (unsigned)(p.tiles_s * (p.tiles_s + 1) / 2);
+        static bool set[64] = {};
+        if (!allow_smem(gram_kernel, S_SMEM, set) ||
+            launch_overlapped(gram_kernel, dim3(tiles, (unsigned)p.slices_s), 256, S_SMEM, st, a, M, K, p.tiles_s, p.rows_s, SP) !=
+                cudaSuccess ||
+            launch_overlapped(gram_reduce_kernel, dim3(tiles, ST / 8), 256, 0, st, SP, p.slices_s, p.tiles_s, S, K) != cudaSuccess)
             return FPQ_ERR_CUDA;
-        if (!p.tc_g)
-            return launch_gram_grad(E, S, DQ, alpha, grad, loss, N, K, coef, inv_mn, reg, lr, st);
-        sg = launch_tf32x3(S, K, E, K, K, N, K, (int)p.per_g, 1, GP, K, N * K, nullptr, st, 3, nullptr, 1.0f, nullptr, 0, 4);
-        return sg != FPQ_OK ? sg : finalize(p.splits_g, E);
+        const int rows = gram_tile_rows(N, K);
+        const auto launch = rows == 32 ? launch_gram_grad<32> : rows == 40 ? launch_gram_grad<40>
+                            : rows == 48 ? launch_gram_grad<48> : launch_gram_grad<64>;
+        return launch(E, S, DQ, alpha, grad, loss, ticket, N, K, 2.0 * inv_mn, inv_mn, reg, lr, st) == cudaSuccess ? FPQ_OK
+                                                                                                                  : FPQ_ERR_CUDA;
     }
     if (tc) {
         // Both contractions on the tensor cores (three TF32 products per FP32 product): D^T = (A E^T)^T is written
@@ -898,7 +955,7 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
         s1 = launch_tf32x3(DT, p.Mp, AT, p.Mp, N, K, M, p.kb_per_split_tc, 0, GP, K, N * K, nullptr, st);
         if (s1 != FPQ_OK)
             return s1;
-        return finalize(p.splits_tc, nullptr);
+        return finalize(p.splits_tc);
     }
     dim3 g1((unsigned)((M + TILE - 1) / TILE), (unsigned)((N + TILE - 1) / TILE), (unsigned)p.splits1);
     if (p.splits1 == 1) {
@@ -909,7 +966,7 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
     }
     dim3 g2((unsigned)((N + TILE - 1) / TILE), (unsigned)((K + TILE - 1) / TILE), (unsigned)p.splits);
     sgemm128<false><<<g2, 256, 0, st>>>(D, p.N4, a, K, GP, K, (int)N, (int)K, M, p.r_per_split, nullptr);
-    return cudaGetLastError() == cudaSuccess ? finalize(p.splits, nullptr) : FPQ_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? finalize(p.splits) : FPQ_ERR_CUDA;
 }
 
 fpq_status launch_round_harden(const float* alpha, int64_t N, int64_t K, uint8_t* bits, cudaStream_t st)

@@ -14,7 +14,7 @@
 // the epilogue.  Warp 1: tensor-memory owner and MMA issuer (kind::tf32, N = 256, 12 MMAs of K = 8 per
 // 32-wide block: at N = 128 the operand reads of the MMAs alone would take all of the shared-memory bandwidth).
 // The tensor core adds each MMA's result into the accumulator with truncation, a bias of about 2^-26 of the
-// running sum per MMA, so a long reduction is accumulated in chunks of 8 or 4 blocks (96 or 48 MMAs) into two
+// running sum per MMA, so a long reduction is accumulated in chunks of 8 blocks (96 MMAs) into two
 // accumulators used in turn, and the split warps add the finished chunks up in registers (FP32, round to
 // nearest).  Every wait is bounded; nothing here uses TMA multicast.
 #include <cuda.h>
@@ -32,6 +32,7 @@ namespace {
 constexpr int TM = 128, TK = 32;                     // TK floats = one 128-byte row
 constexpr int T_XF_W0 = 2, T_NUM_XF = 8;
 constexpr int T_THREADS = 32 * (T_XF_W0 + T_NUM_XF);
+constexpr int T_CHUNK = 8;                           // 32-wide blocks accumulated in tensor memory before they are added up
 // Output tiles are 128 x 256, or 128 x 160 where those cover the columns with less padding: 320 columns are two of them,
 // and three stages fit (two of 256): A^T A of 4096 x 320, 16.6 us with 256, 12.3 with 160; of 8192 x 320 23.2 and 17.4.
 template <int TN>
@@ -50,9 +51,7 @@ struct Tf32Args {
     int kblocks;               // 32-wide blocks of the reduction
     int kb_per_split;          // blocks per slice (blockIdx.y)
     int tiles_j;
-    int epi;                   // 0: C[z][i][j] = the slice's sum, row-major;  1: C[z][j][i] (transposed: 32 lanes write 32
-                               // consecutive floats), and the sum of squares if sq_sum
-    int chunk;                 // 32-wide blocks accumulated in tensor memory before they are added up
+    int epi;                   // 0: C[z][i][j] = the slice's sum, row-major;  1: C[j][i] (transposed) and the sum of squares
     int passes;                // 3: full FP32 products;  1: the operands are TF32 numbers already (hi * hi is all there is)
     // epi 2: the layer's output y = sum * (x_scale * w_scale[j]) + bias[j], row-major [I][J] (howo = 0) or NCHW with
     // i = image * howo + pixel
@@ -193,7 +192,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
                 }
                 mma_commit(empty + 8 * s);          // the stage is free once these MMAs have read it
                 if (++s == T_STAGES) { s = 0; ph ^= 1; }
-                if (++in_chunk == g.chunk || kb + 1 == kb_hi) {
+                if (++in_chunk == T_CHUNK || kb + 1 == kb_hi) {
                     mma_commit(acc_full + 8 * buf);
                     in_chunk = 0;
                     ++chunk;
@@ -214,7 +213,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
 #pragma unroll
         for (int v = 0; v < HALF; ++v)
             sum[v] = 0.f;
-        const int nchunks = (kb_hi - kb_lo + g.chunk - 1) / g.chunk;
+        const int nchunks = (kb_hi - kb_lo + T_CHUNK - 1) / T_CHUNK;
         int drained = 0;
         bool dead = false;
         // adds chunk c (complete in its accumulator) to the sums and hands the accumulator back
@@ -271,7 +270,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
             if (++s == T_STAGES) { s = 0; ph ^= 1; }
             // half a chunk later the previous chunk's MMAs are long done: add it up now, off the critical path
             const int done = kb - kb_lo + 1;
-            if (done % g.chunk == g.chunk / 2 && done / g.chunk > drained)
+            if (done % T_CHUNK == T_CHUNK / 2 && done / T_CHUNK > drained)
                 drain(drained++);
         }
         while (!dead && drained < nchunks)
@@ -331,14 +330,14 @@ __global__ void __launch_bounds__(T_THREADS, 1) tf32x3_gemm_kernel(const __grid_
                     for (int v = 0; v < 32; ++v) {
                         if (j0 + v < g.J && i < g.I) {
                             const float d = r[v];
-                            g.C[(int64_t)z * g.split_stride + (int64_t)(j0 + v) * g.ldc + i] = d;
+                            g.C[(int64_t)(j0 + v) * g.ldc + i] = d;
                             sq = fmaf(d, d, sq);
                         }
                     }
                 }
             }
         }
-        if (g.epi == 1 && g.sq_sum) {
+        if (g.epi == 1) {
             double t = (double)sq;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
@@ -396,18 +395,17 @@ bool tf32x3_applies(const float* P, int64_t ldp, const float* Q, int64_t ldq, in
 }
 
 // C = P Q^T over slices of the reduction.  epi 0: slice z goes to C + z * split_stride, row-major with leading
-// dimension ldc; epi 1: the same transposed, C[j][i]; with one slice *sq_sum += sum of squares unless NULL.
+// dimension ldc; epi 1 (one slice): C[j][i] with leading dimension ldc, and *sq_sum += sum of squares.
 fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ldq, int64_t I, int64_t J, int64_t R,
                          int kb_per_split, int epi, float* C, int64_t ldc, int64_t split_stride, double* sq_sum,
-                         cudaStream_t st, int passes, const float* w_scale, float x_scale, const float* bias, int howo,
-                         int chunk)
+                         cudaStream_t st, int passes, const float* w_scale, float x_scale, const float* bias, int howo)
 {
     const int columns = tf32x3_columns(J);
     static std::mutex mu;
     static EncodeTiledFn enc = nullptr;
     static bool attr_set[64] = {};
     if (!tf32x3_applies(P, ldp, Q, ldq, I, J, R) || kb_per_split < 1 || (passes != 1 && passes != 3) ||
-        epi < 0 || epi > 2 || chunk < 2)
+        epi < 0 || epi > 2)
         return FPQ_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lock(mu);
@@ -439,7 +437,6 @@ fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ld
     g.tiles_j = (int)((J + columns - 1) / columns);
     g.epi = epi;
     g.passes = passes;
-    g.chunk = chunk;
     g.w_scale = w_scale;
     g.x_scale = x_scale;
     g.bias = bias;
@@ -454,7 +451,7 @@ fpq_status launch_tf32x3(const float* P, int64_t ldp, const float* Q, int64_t ld
     // kind::tf32: FP32 accumulator, TF32 (format 2) on both sides, K-major, N = columns, M = 128
     g.idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(columns >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
     const int splits = (g.kblocks + kb_per_split - 1) / kb_per_split;
-    if ((sq_sum || epi == 2) && splits != 1)
+    if ((epi == 1 || epi == 2) && splits != 1)
         return FPQ_ERR_UNSUPPORTED;
     const int64_t tiles = ((I + TM - 1) / TM) * (int64_t)g.tiles_j;
     if (tiles > 0x7fffffff || splits > 65535)
