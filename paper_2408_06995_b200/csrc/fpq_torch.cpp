@@ -14,7 +14,7 @@
 
 namespace {
 
-PyObject *g_exp_bits, *g_man_bits, *g_exp_bias, *g_sat_mode, *g_data_ptr;
+PyObject *g_exp_bits, *g_man_bits, *g_exp_bias, *g_sat_mode, *g_data_ptr, *g_numel;
 
 // (torch's accessors report errors as C++ exceptions: they become Python's here)
 template <typename F>
@@ -115,9 +115,25 @@ bool tensor(PyObject* o, const at::Tensor** out)
     return false;
 }
 
-int64_t count(PyObject* o)
+// size of a workspace (bytes: its elements are): of any object whose pointer is taken, and never more than it says
+bool workspace(PyObject* o, void** p, size_t* bytes)
 {
-    return THPVariable_Check(o) ? THPVariable_Unpack(o).numel() : -1;
+    *bytes = 0;
+    if (!pointer(o, p))
+        return false;
+    if (o == Py_None)
+        return true;
+    if (THPVariable_Check(o))
+        return guarded([&] { *bytes = (size_t)THPVariable_Unpack(o).numel(); });
+    PyObject* v = PyObject_CallMethodNoArgs(o, g_numel);
+    if (!v)
+        return false;
+    const long long n = PyLong_AsLongLong(v);
+    Py_DECREF(v);
+    if (n < 0 && !PyErr_Occurred())
+        PyErr_SetString(PyExc_ValueError, "a workspace of negative size");
+    *bytes = (size_t)n;
+    return n >= 0;
 }
 
 bool arguments(Py_ssize_t given, Py_ssize_t wanted)
@@ -133,14 +149,14 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     const at::Tensor* x;
     void *xp, *w, *ws, *bias, *y, *work, *st;
+    size_t work_bytes;
     float xs;
     fpq_format fx, fw;
     int64_t N;
     if (!arguments(n, 10) || !fp32_cuda(a[0], 2, &x) || !pointer(a[1], &w) || !pointer(a[2], &ws) || !real(a[3], &xs) ||
         !format(a[4], &fx) || !format(a[5], &fw) || !pointer(a[6], &bias) || !integer(a[7], &N) || !pointer(a[8], &y) ||
-        !pointer(a[9], &work) || !pointer(a[0], &xp) || !stream(&st))
+        !workspace(a[9], &work, &work_bytes) || !pointer(a[0], &xp) || !stream(&st))
         return nullptr;
-    const size_t work_bytes = (size_t)count(a[9]);
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_linear((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, x->size(0), N,
@@ -154,6 +170,7 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     const at::Tensor* x;
     void *xp, *w, *ws, *bias, *y, *work, *st;
+    size_t work_bytes;
     float xs;
     fpq_format fx, fw;
     int g[5];
@@ -163,9 +180,8 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
     for (int i = 0; i < 5; ++i)
         if (!integer(a[7 + i], &g[i]))
             return nullptr;
-    if (!pointer(a[12], &y) || !pointer(a[13], &work) || !pointer(a[0], &xp) || !stream(&st))
+    if (!pointer(a[12], &y) || !workspace(a[13], &work, &work_bytes) || !pointer(a[0], &xp) || !stream(&st))
         return nullptr;
-    const size_t work_bytes = (size_t)count(a[13]);
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_conv2d((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, (int)x->size(0),
@@ -180,6 +196,7 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     const at::Tensor *x1, *x2, *y;
     void *x1p, *x2p, *yp, *w, *ws, *bias, *work, *st;
+    size_t work_bytes;
     float s1, s2;
     fpq_format fx, fw;
     int g[4];
@@ -194,9 +211,8 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
     for (int i = 0; i < 4; ++i)
         if (!integer(a[10 + i], &g[i]))
             return nullptr;
-    if (!pointer(a[14], &work) || !pointer(a[0], &x1p) || !pointer(a[2], &x2p) || !pointer(a[9], &yp) || !stream(&st))
+    if (!workspace(a[14], &work, &work_bytes) || !pointer(a[0], &x1p) || !pointer(a[2], &x2p) || !pointer(a[9], &yp) || !stream(&st))
         return nullptr;
-    const size_t work_bytes = (size_t)count(a[14]);
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_conv2d_split((const float*)x1p, (int)x1->size(1), s1, (const float*)x2p, (int)x2->size(1), s2, w,
@@ -212,9 +228,10 @@ PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     const at::Tensor *x, *clip;
     void *xp, *clipp, *mse, *best, *work, *st;
+    size_t work_bytes;
     fpq_format enc[16];
     if (!arguments(n, 6) || !fp32_cuda(a[0], 0, &x) || !fp32_cuda(a[2], 0, &clip) || !pointer(a[0], &xp) || !pointer(a[2], &clipp) ||
-        !pointer(a[3], &mse) || !pointer(a[4], &best) || !pointer(a[5], &work) || !stream(&st))
+        !pointer(a[3], &mse) || !pointer(a[4], &best) || !workspace(a[5], &work, &work_bytes) || !stream(&st))
         return nullptr;
     PyObject* seq = PySequence_Fast(a[1], "encodings must be a sequence");
     if (!seq)
@@ -230,7 +247,6 @@ PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
     const int64_t elements = x->numel();
     const int32_t n_enc = count_enc > 1000000 ? 1000000 : (int32_t)count_enc;
     const int32_t n_clip = clip->numel() > 1000000 ? 1000000 : (int32_t)clip->numel();
-    const size_t work_bytes = (size_t)count(a[5]);
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_search_format((const float*)xp, elements, enc, n_enc, (const float*)clipp, n_clip, (double*)mse, (int32_t*)best,
@@ -244,19 +260,19 @@ PyObject* learn_step(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     const at::Tensor *w, *scale, *alpha, *rows;
     void *wp, *scalep, *alphap, *rowsp, *grad, *loss, *work, *st;
+    size_t work_bytes;
     fpq_format fmt;
     float reg, lr;
     if (!arguments(n, 10) || !fp32_cuda(a[0], 2, &w) || !fp32_cuda(a[1], 1, &scale) || !format(a[2], &fmt) ||
         !fp32_cuda(a[3], 2, &alpha) || !fp32_cuda(a[4], 2, &rows) || !real(a[5], &reg) || !real(a[6], &lr) || !pointer(a[0], &wp) ||
         !pointer(a[1], &scalep) || !pointer(a[3], &alphap) || !pointer(a[4], &rowsp) || !pointer(a[7], &grad) ||
-        !pointer(a[8], &loss) || !pointer(a[9], &work) || !stream(&st))
+        !pointer(a[8], &loss) || !workspace(a[9], &work, &work_bytes) || !stream(&st))
         return nullptr;
     const int64_t M = rows->size(0), N = w->size(0), K = w->size(1);
     if (rows->size(1) != K || alpha->size(0) != N || alpha->size(1) != K || scale->size(0) != N) {
         PyErr_SetString(PyExc_AssertionError, "expected w and alpha [N][K], a [M][K], scale [N]");
         return nullptr;
     }
-    const size_t work_bytes = (size_t)count(a[9]);
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_round_learn_step((const float*)wp, (const float*)scalep, fmt, (float*)alphap, (const float*)rowsp, M, N, K, reg, lr,
@@ -285,5 +301,6 @@ PyMODINIT_FUNC PyInit__fpq_torch(void)
     g_exp_bias = PyUnicode_InternFromString("exp_bias");
     g_sat_mode = PyUnicode_InternFromString("sat_mode");
     g_data_ptr = PyUnicode_InternFromString("data_ptr");
+    g_numel = PyUnicode_InternFromString("numel");
     return PyModule_Create(&module);
 }
