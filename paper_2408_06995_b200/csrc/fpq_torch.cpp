@@ -16,7 +16,8 @@ namespace {
 
 PyObject *g_exp_bits, *g_man_bits, *g_exp_bias, *g_sat_mode, *g_data_ptr, *g_numel;
 
-// (torch's accessors report errors as C++ exceptions: they become Python's here)
+// (torch's accessors report errors as C++ exceptions: they become Python's here; none may leave a call, or run where the
+// interpreter lock has been given up)
 template <typename F>
 bool guarded(F f)
 {
@@ -90,27 +91,40 @@ bool integer(PyObject* o, int* out)
     return true;
 }
 
-// a contiguous FP32 CUDA tensor of `dim` dimensions (0: any)
-bool fp32_cuda(PyObject* o, int64_t dim, const at::Tensor** out)
-{
-    if (THPVariable_Check(o)) {
-        const at::Tensor& t = THPVariable_Unpack(o);
-        if (t.is_cuda() && t.scalar_type() == at::kFloat && t.is_contiguous() && (dim == 0 || t.dim() == dim)) {
-            *out = &t;
-            return true;
-        }
+// sizes and elements of a tensor (sparse, nested and traced tensors may throw instead of giving them)
+struct Shape {
+    int64_t dim, size[4], numel;
+
+    void take(const at::Tensor& t)
+    {
+        dim = t.dim();
+        for (int64_t i = 0; i < 4; ++i)
+            size[i] = i < dim ? t.size(i) : 1;
+        numel = t.numel();
     }
-    PyErr_SetString(PyExc_AssertionError, "expected a contiguous float32 CUDA tensor of the documented shape");
-    return false;
+};
+
+// a contiguous FP32 CUDA tensor of `dim` dimensions (0: any)
+bool fp32_cuda(PyObject* o, int64_t dim, Shape* out)
+{
+    bool fits = false;
+    if (THPVariable_Check(o) && !guarded([&] {
+            const at::Tensor& t = THPVariable_Unpack(o);
+            fits = t.is_cuda() && t.scalar_type() == at::kFloat && t.is_contiguous() && (dim == 0 || t.dim() == dim);
+            if (fits)
+                out->take(t);
+        }))
+        return false;
+    if (!fits)
+        PyErr_SetString(PyExc_AssertionError, "expected a contiguous float32 CUDA tensor of the documented shape");
+    return fits;
 }
 
 // any tensor: the caller's sizes are taken as they are
-bool tensor(PyObject* o, const at::Tensor** out)
+bool tensor(PyObject* o, Shape* out)
 {
-    if (THPVariable_Check(o)) {
-        *out = &THPVariable_Unpack(o);
-        return true;
-    }
+    if (THPVariable_Check(o))
+        return guarded([&] { out->take(THPVariable_Unpack(o)); });
     PyErr_SetString(PyExc_TypeError, "expected a tensor");
     return false;
 }
@@ -147,7 +161,7 @@ bool arguments(Py_ssize_t given, Py_ssize_t wanted)
 // linear(x, w_prepared, w_scale, x_scale, fx, fw, bias, N, y, workspace) -> status
 PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    const at::Tensor* x;
+    Shape x;
     void *xp, *w, *ws, *bias, *y, *work, *st;
     size_t work_bytes;
     float xs;
@@ -159,8 +173,8 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n)
         return nullptr;
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
-    status = fpq_linear((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, x->size(0), N,
-                        x->size(1), work, work_bytes, st);
+    status = fpq_linear((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, x.size[0], N,
+                        x.size[1], work, work_bytes, st);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(status);
 }
@@ -168,7 +182,7 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n)
 // conv2d(x, w_prepared, w_scale, x_scale, fx, fw, bias, C_out, R, S, pad, stride, y, workspace) -> status
 PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    const at::Tensor* x;
+    Shape x;
     void *xp, *w, *ws, *bias, *y, *work, *st;
     size_t work_bytes;
     float xs;
@@ -184,8 +198,8 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
         return nullptr;
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
-    status = fpq_conv2d((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, (int)x->size(0),
-                        (int)x->size(1), (int)x->size(2), (int)x->size(3), g[0], g[1], g[2], g[3], g[4], work, work_bytes,
+    status = fpq_conv2d((const float*)xp, w, (const float*)ws, xs, fx, fw, (const float*)bias, (float*)y, (int)x.size[0],
+                        (int)x.size[1], (int)x.size[2], (int)x.size[3], g[0], g[1], g[2], g[3], g[4], work, work_bytes,
                         st);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(status);
@@ -194,7 +208,7 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
 // conv2d_split(x1, x1_scale, x2, x2_scale, w_prepared, w_scale, fx, fw, bias, y, R, S, pad, stride, workspace) -> status
 PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    const at::Tensor *x1, *x2, *y;
+    Shape x1, x2, y;
     void *x1p, *x2p, *yp, *w, *ws, *bias, *work, *st;
     size_t work_bytes;
     float s1, s2;
@@ -204,7 +218,7 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
         !pointer(a[4], &w) || !pointer(a[5], &ws) || !format(a[6], &fx) || !format(a[7], &fw) || !pointer(a[8], &bias) ||
         !tensor(a[9], &y))
         return nullptr;
-    if (x1->dim() != 4 || x2->dim() < 2 || y->dim() < 2) {
+    if (x1.dim != 4 || x2.dim < 2 || y.dim < 2) {
         PyErr_SetString(PyExc_ValueError, "expected NCHW tensors");
         return nullptr;
     }
@@ -215,9 +229,9 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
         return nullptr;
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
-    status = fpq_conv2d_split((const float*)x1p, (int)x1->size(1), s1, (const float*)x2p, (int)x2->size(1), s2, w,
-                              (const float*)ws, fx, fw, (const float*)bias, (float*)yp, (int)x1->size(0),
-                              (int)x1->size(2), (int)x1->size(3), (int)y->size(1), g[0], g[1], g[2], g[3], work,
+    status = fpq_conv2d_split((const float*)x1p, (int)x1.size[1], s1, (const float*)x2p, (int)x2.size[1], s2, w,
+                              (const float*)ws, fx, fw, (const float*)bias, (float*)yp, (int)x1.size[0],
+                              (int)x1.size[2], (int)x1.size[3], (int)y.size[1], g[0], g[1], g[2], g[3], work,
                               work_bytes, st);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(status);
@@ -226,7 +240,7 @@ PyObject* conv2d_split(PyObject*, PyObject* const* a, Py_ssize_t n)
 // search(x, encodings, clip, mse, best, workspace) -> status
 PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    const at::Tensor *x, *clip;
+    Shape x, clip;
     void *xp, *clipp, *mse, *best, *work, *st;
     size_t work_bytes;
     fpq_format enc[16];
@@ -244,9 +258,9 @@ PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
             return nullptr;
         }
     Py_DECREF(seq);
-    const int64_t elements = x->numel();
+    const int64_t elements = x.numel;
     const int32_t n_enc = count_enc > 1000000 ? 1000000 : (int32_t)count_enc;
-    const int32_t n_clip = clip->numel() > 1000000 ? 1000000 : (int32_t)clip->numel();
+    const int32_t n_clip = clip.numel > 1000000 ? 1000000 : (int32_t)clip.numel;
     fpq_status status;
     Py_BEGIN_ALLOW_THREADS
     status = fpq_search_format((const float*)xp, elements, enc, n_enc, (const float*)clipp, n_clip, (double*)mse, (int32_t*)best,
@@ -258,7 +272,7 @@ PyObject* search(PyObject*, PyObject* const* a, Py_ssize_t n)
 // learn_step(w, scale, fmt, alpha, a, reg, lr, grad, loss, workspace) -> status
 PyObject* learn_step(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    const at::Tensor *w, *scale, *alpha, *rows;
+    Shape w, scale, alpha, rows;
     void *wp, *scalep, *alphap, *rowsp, *grad, *loss, *work, *st;
     size_t work_bytes;
     fpq_format fmt;
@@ -268,8 +282,8 @@ PyObject* learn_step(PyObject*, PyObject* const* a, Py_ssize_t n)
         !pointer(a[1], &scalep) || !pointer(a[3], &alphap) || !pointer(a[4], &rowsp) || !pointer(a[7], &grad) ||
         !pointer(a[8], &loss) || !workspace(a[9], &work, &work_bytes) || !stream(&st))
         return nullptr;
-    const int64_t M = rows->size(0), N = w->size(0), K = w->size(1);
-    if (rows->size(1) != K || alpha->size(0) != N || alpha->size(1) != K || scale->size(0) != N) {
+    const int64_t M = rows.size[0], N = w.size[0], K = w.size[1];
+    if (rows.size[1] != K || alpha.size[0] != N || alpha.size[1] != K || scale.size[0] != N) {
         PyErr_SetString(PyExc_AssertionError, "expected w and alpha [N][K], a [M][K], scale [N]");
         return nullptr;
     }

@@ -49,6 +49,21 @@ def test_sizes_that_are_none(ext, size, error):
         ext.conv2d_split(*_split_arguments(Scratch(size)))
 
 
+def test_tensors_without_sizes_raise(ext):
+    # (an exception of torch's C++ side that left the call would end the process)
+    ragged = torch.nested.nested_tensor([torch.zeros(4, 8, 8), torch.zeros(4, 8, 9)])
+    with pytest.raises(RuntimeError, match="irregular"):
+        ext.conv2d_split(*_split_arguments(torch.zeros(16, dtype=torch.uint8), ragged))
+
+
+@pytest.mark.gpu
+def test_sparse_tensors_raise():
+    x = torch.zeros(4, 320, device="cuda").to_sparse()
+    w = torch.zeros(1 << 16, dtype=torch.uint8, device="cuda")
+    with pytest.raises((RuntimeError, AssertionError)):
+        fpq.fpq_linear(x, w, torch.ones(64, device="cuda"), 1.0, fpq.E4M3, fpq.E4M3, None, 64, torch.empty(4, 64, device="cuda"), w)
+
+
 @pytest.mark.gpu
 def test_a_workspace_that_is_too_small_is_refused_whatever_holds_it():
     x = torch.randn(300, 320, device="cuda")
