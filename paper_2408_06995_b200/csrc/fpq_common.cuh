@@ -514,7 +514,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
 // Bounded wait on a barrier of this CTA that other CTAs of the cluster arrive on.  It polls with test_wait:
 // a thread suspended in try_wait was not woken by an arrival from another CTA until its time limit ran out
 // (about 2 us per wait, measured).
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, long long limit = MBAR_WAIT_LIMIT)
 {
     const long long t0 = clock64();
     for (;;) {
@@ -531,8 +531,23 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
                 return true;
             __nanosleep(20);
         }
-        if (clock64() - t0 > 4000000000ll)
+        if (clock64() - t0 > limit)
             return false;
+    }
+}
+
+// The end of a producer's role in a CTA pair, which has issued n loads over a ring of `stages`: the MMAs' arrivals on its
+// last stages are waited for, so that none is on its way to a CTA that has left.  After a wait that ran out, the pair's
+// first CTA, whose barriers count the loads of both, waits for those in flight instead (some 50 ms at most each): shared
+// memory is not given back under a copy, and the other CTA stays until the first one arrives on the cluster's barrier.
+__device__ __forceinline__ void settle_ring(uint32_t full, uint32_t empty, uint32_t n, uint32_t stages, bool first, bool& dead)
+{
+    for (uint32_t i = n > stages ? n - stages : 0; i < n; ++i) {
+        const uint32_t at = 8 * (i % stages), parity = (i / stages) & 1;
+        if (!dead && !mbar_wait_cluster(empty + at, parity))
+            dead = true;
+        if (dead && first)
+            (void)mbar_wait_cluster(full + at, parity, 100000000ll);
     }
 }
 

@@ -226,6 +226,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
             if (dead) {
                 for (uint32_t i = (nx > (uint32_t)g.x_stages ? nx - g.x_stages : 0); i < nx; ++i)
                     (void)mbar_wait(x_full + 8 * (i % g.x_stages), (i / g.x_stages) & 1);
+                for (int cc = 0; cc < g.cchunks; ++cc)
+                    (void)mbar_wait(b_full + 8 * cc, 0);
             }
         }
     } else if (warp == 1) {
@@ -486,15 +488,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
                 if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
             }
         }
+        // (one warp waits for the MMAs' arrivals on the last stages too)
+        if (warp == XF_W0) {
+            const int used = g.tiles_per_cta * g.cchunks;
+            for (int i = used > g.a_stages ? used - g.a_stages : 0; i < used && !dead; ++i)
+                dead = !mbar_wait_cluster(a_empty + 8 * (i % g.a_stages), (i / g.a_stages) & 1);
+        }
         if (nan)
             flag_status(g.status, FPQ_ERR_NAN_INPUT);
         failed = dead;
     }
 
     // Nobody leaves while the other CTA may still arrive on this CTA's barriers or read its shared memory, and both CTAs
-    // give their tensor memory back together.  Every arrival but a failed role's has been waited for, so the barrier
-    // need not wait for the stores of the output (128 -> 128 channels at 32 x 32, batch 64: 19.1 -> 18.7 us; one tap,
-    // 128 -> 256 at 64 x 64, batch 8: 10.9 -> 10.1).
+    // give their tensor memory back together.  Every arrival but a failed role's has been waited for (the MMAs' last
+    // ones by a transform warp), so the barrier need not wait for the stores of the output (128 -> 128 channels at 32 x 32,
+    // batch 64: 19.1 -> 18.7 us; one tap, 128 -> 256 at 64 x 64, batch 8: 10.9 -> 10.1).
     tc_fence_before();
     if (failed)
         flag_status(g.status, FPQ_ERR_TIMEOUT);
