@@ -454,6 +454,26 @@ int32_t fpq_conv2d_route(int B, int C, int H, int W, int C_out, int R, int S, in
                          fpq_format fx, fpq_format fw);
 
 /*
+ * Which contraction kernel runs behind the activation-quantize kernel for this shape under the current policy (for
+ * logs, benchmarks and tests; nothing is launched):
+ *   FPQ_CONTRACTION_GENERAL     128-row tiles, the reduction shared by a cluster where that pays;
+ *   FPQ_CONTRACTION_PAIRS       256-row tiles on CTA pairs;
+ *   FPQ_CONTRACTION_CUDA_CORES  a linear layer of a few rows as one kernel on the CUDA cores, no quantize kernel;
+ *   FPQ_CONTRACTION_OTHER       the FP32 grid-value route;
+ *   negative                    FPQ_ERR_FORMAT or FPQ_ERR_SHAPE.
+ * A convolution that takes FPQ_ROUTE_PAIR_FUSED or FPQ_ROUTE_FUSED runs neither kernel.
+ */
+enum {
+    FPQ_CONTRACTION_GENERAL = 0,
+    FPQ_CONTRACTION_PAIRS = 1,
+    FPQ_CONTRACTION_CUDA_CORES = 2,
+    FPQ_CONTRACTION_OTHER = 3
+};
+int32_t fpq_linear_contraction(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format fw);
+int32_t fpq_conv2d_contraction(int B, int C, int H, int W, int C_out, int R, int S, int pad, int stride,
+                               fpq_format fx, fpq_format fw);
+
+/*
  * Diagnostic (the paper has no counterpart): launches one warp that waits on a barrier nobody ever
  * arrives on, with the same bounded wait every role of the layer kernels uses, limited to
  * limit_cycles SM clock cycles (1 .. 1e9).  The wait runs out, the warp records FPQ_ERR_TIMEOUT in the

@@ -25,6 +25,7 @@ OK = 0
 ERR_NULL, ERR_FORMAT, ERR_SHAPE, ERR_ALIGN, ERR_UNSUPPORTED = -1, -2, -3, -4, -5
 ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_NAN_INPUT, ERR_TOO_LARGE, ERR_SCALE = -6, -7, -8, -9, -10, -11
 ROUTE_TWO_KERNELS, ROUTE_FUSED, ROUTE_PAIR_FUSED, ROUTE_OTHER = 0, 1, 2, 3
+CONTRACTION_GENERAL, CONTRACTION_PAIRS, CONTRACTION_CUDA_CORES, CONTRACTION_OTHER = 0, 1, 2, 3
 STATIC_SCRATCH_BYTES = 8 << 20
 SAT_PAPER, SAT_NATIVE = 0, 1
 LINEAR, CONV2D = 0, 1
@@ -78,7 +79,7 @@ EXPORTS = [
     "fpq_round_learn_workspace_size", "fpq_round_learn_step", "fpq_round_learn_harden", "fpq_round_learn_unfold",
     "fpq_zero_census", "fpq_prepared_size_split", "fpq_prepare_weight_split", "fpq_conv2d_split_workspace_size",
     "fpq_conv2d_split", "fpq_set_path_policy", "fpq_get_path_policy", "fpq_read_status", "fpq_status_string",
-    "fpq_conv2d_route", "fpq_selftest_bounded_wait",
+    "fpq_conv2d_route", "fpq_linear_contraction", "fpq_conv2d_contraction", "fpq_selftest_bounded_wait",
 ]
 
 _lib = None
@@ -162,6 +163,10 @@ def lib() -> ctypes.CDLL:
         L.fpq_selftest_bounded_wait.argtypes = [i64, vp]
         L.fpq_conv2d_route.restype = i32
         L.fpq_conv2d_route.argtypes = [i32] * 9 + [F, F]
+        L.fpq_linear_contraction.restype = i32
+        L.fpq_linear_contraction.argtypes = [i64, i64, i64, F, F]
+        L.fpq_conv2d_contraction.restype = i32
+        L.fpq_conv2d_contraction.argtypes = [i32] * 9 + [F, F]
         L.fpq_read_status.restype = i32
         L.fpq_read_status.argtypes = [vp]
         L.fpq_status_string.restype = ctypes.c_char_p
@@ -482,6 +487,22 @@ def fpq_conv2d_route(B, C, H, W, C_out, R, S, pad, stride, fx: Format, fw: Forma
     r = lib().fpq_conv2d_route(B, C, H, W, C_out, R, S, pad, stride, fx.c(), fw.c())
     if r < 0:
         _check(r, "fpq_conv2d_route")
+    return r
+
+
+def fpq_linear_contraction(M, N, K, fx: Format, fw: Format) -> int:
+    """Which contraction fpq_linear would run for this shape under the current policy (CONTRACTION_*)."""
+    r = lib().fpq_linear_contraction(M, N, K, fx.c(), fw.c())
+    if r < 0:
+        _check(r, "fpq_linear_contraction")
+    return r
+
+
+def fpq_conv2d_contraction(B, C, H, W, C_out, R, S, pad, stride, fx: Format, fw: Format) -> int:
+    """Which contraction runs behind fpq_conv2d's quantize kernel for this shape under the current policy (CONTRACTION_*)."""
+    r = lib().fpq_conv2d_contraction(B, C, H, W, C_out, R, S, pad, stride, fx.c(), fw.c())
+    if r < 0:
+        _check(r, "fpq_conv2d_contraction")
     return r
 
 

@@ -502,6 +502,32 @@ fpq_status fpq_linear_quantize_input(const float* x, float x_scale, fpq_format f
                : FPQ_ERR_CUDA;
 }
 
+// shapes and types of a contraction; the pointers, scales and flags are the caller's
+static GemmProblem linear_problem(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format fw)
+{
+    GemmProblem p{};
+    p.C = (int)K;
+    p.w4 = is_e2m1(fw) ? 1 : 0;
+    p.w_e5m2 = is_e5m2_native(fw) ? 1 : 0;
+    p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
+    p.M = M;
+    p.N = (int)N;
+    p.Cp = (int)padded_c(K);
+    p.Ca = (int)round_up(K, 16);
+    p.B = p.H = p.W = p.Ho = p.Wo = 1;
+    p.R = p.S = 1;
+    p.stride = 1;
+    return p;
+}
+
+// the same with weights of two terms of type `term` (2 * padded K prepared), whose activation codes are written once
+static GemmProblem linear_two_term_problem(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format term)
+{
+    GemmProblem p = linear_problem(M, N, K, fx, term);
+    p.Cp = (int)(2 * padded_c(K));
+    return p;
+}
+
 static fpq_status linear_contract_impl(const void* workspace, size_t ws_bytes, const void* w_prepared,
                                        const float* w_scale, float x_scale, fpq_format fx, fpq_format fw,
                                        const float* bias, float* y, int64_t M, int64_t N, int64_t K, void* stream,
@@ -519,22 +545,9 @@ static fpq_status linear_contract_impl(const void* workspace, size_t ws_bytes, c
         return FPQ_ERR_ALIGN;
     if (!status_word())
         return FPQ_ERR_CUDA;
-    GemmProblem p{};
-    p.conv = 0;
+    GemmProblem p = linear_problem(M, N, K, fx, fw);
     p.x = x_fused;
-    p.C = (int)K;
     p.after_stage1 = after_stage1;
-    p.w4 = is_e2m1(fw) ? 1 : 0;
-    p.w_e5m2 = is_e5m2_native(fw) ? 1 : 0;
-    p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
-    p.M = M;
-    p.N = (int)N;
-    p.Cp = (int)padded_c(K);
-    p.Ca = (int)round_up(K, 16);
-    p.B = p.H = p.W = p.Ho = p.Wo = 1;
-    p.R = p.S = 1;
-    p.pad = 0;
-    p.stride = 1;
     p.a_codes = (const uint8_t*)workspace;
     p.w_prepared = w_prepared;
     p.w_scale = w_scale;
@@ -642,14 +655,8 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
             return FPQ_ERR_CUDA;
         {
             // long reductions: CTA pairs, both terms on one copy of the codes
-            GemmProblem p{};
+            GemmProblem p = linear_two_term_problem(M, N, K, fx, term);
             p.after_stage1 = 1;
-            p.w_e5m2 = is_e5m2_native(term) ? 1 : 0;
-            p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
-            p.M = M, p.N = (int)N, p.C = (int)K;
-            p.Cp = (int)K2;
-            p.Ca = (int)round_up(K, 16);
-            p.R = p.S = 1, p.stride = 1;
             p.a_codes = (const uint8_t*)workspace;
             p.w_prepared = w_prepared, p.w_scale = w_scale, p.x_scale = x_scale * two_term_unshift(fw), p.bias = bias, p.y = y;
             if (g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && pair_rows_preferred(p, 2)) {
@@ -804,6 +811,23 @@ fpq_status fpq_conv2d_quantize_input(const float* x, float x_scale, fpq_format f
                : FPQ_ERR_CUDA;
 }
 
+static GemmProblem conv_problem(int B, int C, int H, int W, int C_out, int R, int S, int pad, int stride, int Ho, int Wo,
+                                fpq_format fx, fpq_format fw)
+{
+    GemmProblem p{};
+    p.conv = 1;
+    p.C = C;
+    p.w4 = is_e2m1(fw) ? 1 : 0;
+    p.w_e5m2 = is_e5m2_native(fw) ? 1 : 0;
+    p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
+    p.M = (int64_t)B * Ho * Wo;
+    p.N = C_out;
+    p.Cp = (int)padded_c(C);
+    p.Ca = (int)round_up(C, 16);
+    p.B = B, p.H = H, p.W = W, p.Ho = Ho, p.Wo = Wo, p.R = R, p.S = S, p.pad = pad, p.stride = stride;
+    return p;
+}
+
 static fpq_status conv2d_contract_impl(const void* workspace, size_t ws_bytes, const void* w_prepared,
                                        const float* w_scale, float x_scale, fpq_format fx, fpq_format fw,
                                        const float* bias, float* y, int B, int C, int H, int W, int C_out, int R,
@@ -823,27 +847,9 @@ static fpq_status conv2d_contract_impl(const void* workspace, size_t ws_bytes, c
         return FPQ_ERR_ALIGN;
     if (!status_word())
         return FPQ_ERR_CUDA;
-    GemmProblem p{};
-    p.conv = 1;
+    GemmProblem p = conv_problem(B, C, H, W, C_out, R, S, pad, stride, Ho, Wo, fx, fw);
     p.x = x_fused;
-    p.C = C;
     p.after_stage1 = after_stage1;
-    p.w4 = is_e2m1(fw) ? 1 : 0;
-    p.w_e5m2 = is_e5m2_native(fw) ? 1 : 0;
-    p.a_e5m2 = is_e5m2_native(fx) ? 1 : 0;
-    p.M = (int64_t)B * Ho * Wo;
-    p.N = C_out;
-    p.Cp = (int)padded_c(C);
-    p.Ca = (int)round_up(C, 16);
-    p.B = B;
-    p.H = H;
-    p.W = W;
-    p.Ho = Ho;
-    p.Wo = Wo;
-    p.R = R;
-    p.S = S;
-    p.pad = pad;
-    p.stride = stride;
     p.a_codes = (const uint8_t*)workspace;
     p.w_prepared = w_prepared;
     p.w_scale = w_scale;
@@ -1409,22 +1415,61 @@ int32_t fpq_conv2d_route(int B, int C, int H, int W, int C_out, int R, int S, in
     if (g_path_policy == FPQ_PATH_TWO_KERNELS || g_path_policy == FPQ_PATH_TWO_KERNELS_NARROW || B == 0 || C_out == 0 ||
         !is_e4m3_native(fx))
         return FPQ_ROUTE_TWO_KERNELS;
-    GemmProblem p{};
-    p.conv = 1;
+    GemmProblem p = conv_problem(B, C, H, W, C_out, R, S, pad, stride, Ho, Wo, fx, fw);
     p.x = reinterpret_cast<const float*>((uintptr_t)256);      // never followed: the plans only look at its alignment
-    p.C = C;
-    p.w4 = is_e2m1(fw) ? 1 : 0;
-    p.w_e5m2 = is_e5m2_native(fw) ? 1 : 0;
-    p.M = (int64_t)B * Ho * Wo;
-    p.N = C_out;
-    p.Cp = (int)padded_c(C);
-    p.Ca = (int)round_up(C, 16);
-    p.B = B, p.H = H, p.W = W, p.Ho = Ho, p.Wo = Wo, p.R = R, p.S = S, p.pad = pad, p.stride = stride;
     if (pair_conv_applies(p) && (g_path_policy == FPQ_PATH_FUSED || pair_conv_preferred(p)))
         return FPQ_ROUTE_PAIR_FUSED;
     if (g_path_policy == FPQ_PATH_FUSED && stride == 1)
         return FPQ_ROUTE_FUSED;                                  // (the general fused form; it may still fall back)
     return FPQ_ROUTE_TWO_KERNELS;
+}
+
+int32_t fpq_linear_contraction(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format fw)
+{
+    QFormat q;
+    if (!resolve_format(fx, &q) || !resolve_format(fw, &q))
+        return FPQ_ERR_FORMAT;
+    if (M < 0 || N < 0 || K < 1 || M > 0x7fffffff || N > 0x7fffffff || K > 0x3fffffff)
+        return FPQ_ERR_SHAPE;
+    if (general_pair(fx, fw))
+        return FPQ_CONTRACTION_OTHER;
+    const bool pairs = g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && M > 0 && N > 0;
+    int terms = 1;
+    if (two_term_pair(fx, fw)) {
+        const fpq_format term = classify_weight(fw).e5m2 ? kE5M2Native : kE4M3Native;
+        if (pairs && pair_rows_preferred(linear_two_term_problem(M, N, K, fx, term), 2))
+            return FPQ_CONTRACTION_PAIRS;
+        K = 2 * padded_c(K), fw = term;
+    } else if (act_terms_pair(fx, fw, &terms)) {
+        K = terms * padded_c(K), fx = classify_weight(fx).e5m2 ? kE5M2Native : kE4M3Native;
+    } else if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(M, K, N, is_e2m1(fw) ? 1 : 0)) {
+        return FPQ_CONTRACTION_CUDA_CORES;
+    }
+    return pairs && pair_rows_preferred(linear_problem(M, N, K, fx, fw), 1) ? FPQ_CONTRACTION_PAIRS : FPQ_CONTRACTION_GENERAL;
+}
+
+int32_t fpq_conv2d_contraction(int B, int C, int H, int W, int C_out, int R, int S, int pad, int stride, fpq_format fx,
+                               fpq_format fw)
+{
+    QFormat q;
+    if (!resolve_format(fx, &q) || !resolve_format(fw, &q))
+        return FPQ_ERR_FORMAT;
+    if (C < 1 || C > 0x3fffffff / 2)
+        return FPQ_ERR_SHAPE;
+    if (general_pair(fx, fw))
+        return FPQ_CONTRACTION_OTHER;
+    int terms = 1, Ho, Wo;
+    if (two_term_pair(fx, fw))
+        C = 2 * (int)padded_c(C), fw = classify_weight(fw).e5m2 ? kE5M2Native : kE4M3Native;
+    else if (act_terms_pair(fx, fw, &terms))
+        C = (int)(terms * padded_c(C)), fx = classify_weight(fx).e5m2 ? kE5M2Native : kE4M3Native;
+    const fpq_status s = conv_shape(B, C, H, W, C_out, R, S, pad, stride, &Ho, &Wo);
+    if (s != FPQ_OK)
+        return s;
+    return g_path_policy != FPQ_PATH_TWO_KERNELS_NARROW && B > 0 && C_out > 0 &&
+                   pair_gemm_preferred(conv_problem(B, C, H, W, C_out, R, S, pad, stride, Ho, Wo, fx, fw))
+               ? FPQ_CONTRACTION_PAIRS
+               : FPQ_CONTRACTION_GENERAL;
 }
 
 fpq_status fpq_selftest_bounded_wait(int64_t limit_cycles, void* stream)

@@ -1,0 +1,56 @@
+"""Which contraction the library picks, without a GPU: the shapes that the GPU tests of one kernel rely on take that kernel,
+or those tests would compare another one with itself."""
+import pytest
+
+import paper_2408_06995_b200 as fpq
+
+E4M3, E5M2, E2M1, E3M4, E2M5, E1M2 = fpq.E4M3, fpq.E5M2, fpq.E2M1, fpq.E3M4, fpq.E2M5, fpq.E1M2
+GENERAL, PAIRS, FEW_ROWS, OTHER = (fpq.CONTRACTION_GENERAL, fpq.CONTRACTION_PAIRS, fpq.CONTRACTION_CUDA_CORES,
+                                   fpq.CONTRACTION_OTHER)
+
+
+# test_gpu_pair_rows.py and test_gpu_ragged_columns.py
+@pytest.mark.parametrize("fx,fw,M,K,N", [
+    (E4M3, E3M4, 2048, 2560, 640), (E4M3, E3M4, 300, 1152, 36), (E4M3, E2M5, 700, 500, 100), (E4M3, fpq.Format(5, 2, 16), 900, 386, 200),
+    (E5M2, E3M4, 513, 700, 260), (E4M3, E2M1, 1300, 1540, 1000), (E4M3, E4M3, 2300, 900, 1030), (E5M2, E5M2, 1200, 1700, 1028),
+    (E4M3, E1M2, 9217, 1300, 324), (E4M3, E3M4, 2048, 2560, 638), (E4M3, E3M4, 700, 640, 65), (E4M3, E3M4, 1111, 1300, 1283),
+    (E4M3, E2M1, 3001, 1280, 1282), (E4M3, E4M3, 2100, 2560, 639)])
+def test_linear_layers_on_pairs(fx, fw, M, K, N):
+    assert fpq.fpq_linear_contraction(M, N, K, fx, fw) == PAIRS
+
+
+@pytest.mark.parametrize("fx,fw,M,K,N,form", [
+    (E4M3, E2M1, 8192, 320, 960, GENERAL), (E4M3, E2M1, 64, 5120, 320, GENERAL), (E4M3, E3M4, 300, 640, 65, GENERAL),
+    (E4M3, E2M1, 2, 1280, 1280, FEW_ROWS), (E4M3, E2M1, 8, 5120, 10240, GENERAL), (E4M3, fpq.Format(6, 1, 31), 64, 64, 64, OTHER)])
+def test_other_linear_layers(fx, fw, M, K, N, form):
+    assert fpq.fpq_linear_contraction(M, N, K, fx, fw) == form
+
+
+# test_gpu_pair_tiles.py
+@pytest.mark.parametrize("B,C,H,W,Co,stride", [
+    (2, 320, 64, 64, 320, 1), (2, 640, 32, 32, 640, 1), (64, 192, 32, 32, 192, 1), (8, 512, 32, 32, 512, 1), (3, 320, 45, 45, 324, 1),
+    (5, 136, 30, 17, 100, 1), (50, 416, 11, 11, 608, 1), (2, 192, 7, 5, 288, 1), (1, 256, 13, 96, 70, 1), (16, 256, 32, 32, 256, 1),
+    (9, 150, 7, 9, 104, 1), (3, 320, 45, 77, 320, 2), (2, 320, 64, 64, 320, 2), (13, 128, 9, 8, 100, 2), (1, 200, 7, 120, 256, 2),
+    (1, 64, 3, 253, 64, 2), (40, 96, 4, 3, 72, 2), (9, 320, 31, 30, 640, 2), (24, 192, 48, 48, 320, 2), (3, 130, 25, 41, 96, 2),
+    (7, 64, 11, 9, 40, 2)])
+def test_convolutions_on_pairs(B, C, H, W, Co, stride):
+    for fw in (E4M3, E2M1):
+        assert fpq.fpq_conv2d_contraction(B, C, H, W, Co, 3, 3, 1, stride, E4M3, fw) == PAIRS
+
+
+def test_policies_and_errors():
+    L = fpq.lib()
+    try:
+        fpq.fpq_set_path_policy(fpq.PATH_TWO_KERNELS_NARROW)
+        assert fpq.fpq_linear_contraction(2048, 640, 2560, E4M3, E3M4) == GENERAL
+        assert fpq.fpq_conv2d_contraction(2, 320, 64, 64, 320, 3, 3, 1, 1, E4M3, E2M1) == GENERAL
+    finally:
+        fpq.fpq_set_path_policy(fpq.PATH_AUTO)
+    assert fpq.fpq_conv2d_contraction(2, 64, 8, 8, 64, 3, 3, 1, 1, E4M3, fpq.Format(6, 1, 31)) == OTHER
+    assert fpq.fpq_linear_contraction(0, 640, 2560, E4M3, E3M4) == GENERAL
+    assert L.fpq_linear_contraction(-1, 1, 1, E4M3.c(), E4M3.c()) == fpq.ERR_SHAPE
+    assert L.fpq_linear_contraction(1, 1, 0, E4M3.c(), E4M3.c()) == fpq.ERR_SHAPE
+    assert L.fpq_linear_contraction(1, 1, 1, fpq.Format(6, 3, 7).c(), E4M3.c()) == fpq.ERR_FORMAT
+    assert L.fpq_conv2d_contraction(2, 0, 8, 8, 64, 3, 3, 1, 1, E4M3.c(), E4M3.c()) == fpq.ERR_SHAPE
+    assert L.fpq_conv2d_contraction(2, 64, 1, 1, 64, 3, 3, 0, 1, E4M3.c(), E4M3.c()) == fpq.ERR_SHAPE
+    assert L.fpq_conv2d_contraction(2, 64, 8, 8, 64, 3, 3, 1, 1, fpq.Format(6, 3, 7).c(), E4M3.c()) == fpq.ERR_FORMAT

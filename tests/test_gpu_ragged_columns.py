@@ -23,7 +23,7 @@ def test_ragged_columns(M, K, N, wfmt):
     assert_close(y[idx], yo, ab)
 
 
-@pytest.mark.parametrize("M,K,N", [(2048, 2560, 638), (300, 640, 65), (1111, 1300, 1283)])
+@pytest.mark.parametrize("M,K,N", [(2048, 2560, 638), (300, 640, 65), (1111, 1300, 1283), (700, 640, 65)])
 def test_two_terms(M, K, N):
     gen = torch.Generator(device="cuda").manual_seed(N)
     x = torch.randn(M, K, generator=gen, device="cuda")
