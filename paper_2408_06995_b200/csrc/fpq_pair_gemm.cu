@@ -437,14 +437,15 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
 // Column tile of a layer: the one with the shortest estimate, in SM cycles.  A chunk of the reduction takes its MMAs
 // (0.53 cycles per column and 32 reduction elements, 52 at least) or the arrival of its operands (some 43 bytes per clock
 // and SM); an epilogue stores some 15 bytes per clock and SM and is hidden behind the next unit's MMAs, except the last
-// one's.  A width that just fits the columns and the SM pairs beats the widest one: 640 -> 320 channels at 64 x 64, batch
+// one's.  (32 columns, whose MMAs take as long as 64's, only where there are no more.)  A width that just fits the columns and
+// the SM pairs beats the widest one: 640 -> 320 channels at 64 x 64, batch
 // 2, whole layer: 35 units x 3 tiles of 128 in two rounds 24.1 us, x 2 of 160 in one 19.3 us; 256 -> 256 at 32 x 32,
 // batch 16: 15.5 us with 128, 18.6 us with 64 or 192.
 int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_bytes, int accs, double* cycles)
 {
     int pick = 128;
     double best = 0.0;
-    for (int bn = 64; bn <= 256; bn += 32) {
+    for (int bn = N <= 32 ? 32 : 64; bn <= 256; bn += 32) {
         if (bn - 32 >= N)
             break;
         const int64_t units = (int64_t)m_units * ((N + bn - 1) / bn);
@@ -617,6 +618,12 @@ bool pair_gemm_preferred(const GemmProblem& p)
     } else {
         general = block * (double)((tiles + SMS - 1) / SMS) * blocks;
     }
+    // up to 64 outputs the general kernel has little besides its blocks (batch x channels, us here / there: 8 x 320 -> 32 at
+    // 64 x 64, stride 2 17.1 / 19.6; 16 x 256 -> 32 at 32 x 32 10.8 / 11.8; 8 x 640 -> 32 at 32 x 32 15.1 / 13.9; 15 x 992 -> 24 at 21 x 21
+    // 19.8 / 16.6; 25 x 320 -> 48 at 15 x 15 11.6 / 13.0; 2 x 320 -> 64 at 30 x 30 9.7 / 8.6; 2 x 352 -> 40 at 28 x 28 9.8 / 8.0; of 57 drawn
+    // layers five take the slower one, by 4 to 8 %; with the difference that wider layers have thirteen did, by up to 23 %)
+    if (p.N <= 64)
+        return g.estimate <= general + (p.N <= 32 ? 0.0 : 1000.0);
     // (stride 2 in several rounds: 256 -> 1280 channels at 16 x 16, batch 57: 20.4 us there, 22.8 here)
     return g.estimate <= general + (p.stride > 1 && g.units > SMS / 2 ? 2000.0 : 4300.0);
 }
