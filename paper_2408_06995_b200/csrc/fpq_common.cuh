@@ -516,8 +516,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
 // (about 2 us per wait, measured).
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, long long limit = MBAR_WAIT_LIMIT)
 {
-    const long long t0 = clock64();
-    for (;;) {
+    for (long long t0 = 0;;) {                          // (the clock only after 1024 polls: most waits are short)
         for (int i = 0; i < 1024; ++i) {
             uint32_t ok;
             asm volatile(
@@ -531,23 +530,27 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
                 return true;
             __nanosleep(20);
         }
-        if (clock64() - t0 > limit)
+        const long long now = clock64();
+        if (t0 == 0)
+            t0 = now;
+        if (now - t0 > limit)
             return false;
     }
 }
 
-// The end of a producer's role in a CTA pair, which has issued n loads over a ring of `stages`: the MMAs' arrivals on its
-// last stages are waited for, so that none is on its way to a CTA that has left.  After a wait that ran out, the pair's
+// The end of a producer's role in a CTA pair; s and ph: the ring's stage that it would fill next and the parity that it would
+// wait for.  It waits as if it went round once more: no arrival of the MMAs is then on its way to a CTA that has left.  After a wait that ran out, the pair's
 // first CTA, whose barriers count the loads of both, waits for those in flight instead (some 50 ms at most each): shared
 // memory is not given back under a copy, and the other CTA stays until the first one arrives on the cluster's barrier.
-__device__ __forceinline__ void settle_ring(uint32_t full, uint32_t empty, uint32_t n, uint32_t stages, bool first, bool& dead)
+__device__ __forceinline__ void settle_ring(uint32_t full, uint32_t empty, uint32_t s, uint32_t ph, uint32_t stages, bool first,
+                                            bool& dead)
 {
-    for (uint32_t i = n > stages ? n - stages : 0; i < n; ++i) {
-        const uint32_t at = 8 * (i % stages), parity = (i / stages) & 1;
-        if (!dead && !mbar_wait_cluster(empty + at, parity))
+    for (uint32_t i = 0; i < stages; ++i) {
+        if (!dead && !mbar_wait_cluster(empty + 8 * s, ph))
             dead = true;
-        if (dead && first)
-            (void)mbar_wait_cluster(full + at, parity, 100000000ll);
+        if (dead && first)                             // (the parity of the stage's last load is ph too)
+            (void)mbar_wait_cluster(full + 8 * s, ph, 100000000ll);
+        if (++s == stages) { s = 0; ph ^= 1; }
     }
 }
 

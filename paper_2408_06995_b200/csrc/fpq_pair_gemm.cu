@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
     if (PHASED && warp == 0) {
         // ---------------- stride 2: activation producer, four phases per chunk ----------------
         if (elect_one()) {
-            uint32_t sa = 0, pa = 1, na = 0;
+            uint32_t sa = 0, pa = 1;
             bool dead = false;
             const uint32_t full = leader(a_full);
             for (int u = u_lo; u < u_hi && !dead; ++u) {
@@ -161,17 +161,16 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                             mbar_expect_tx(a_full + 8 * sa, 2u * g.a_tx);
                         tma_load_4d_pair(a_ring + sa * g.a_stage_bytes, &tmA, full + 8 * sa, cc * BK, 2 * x0 + (ph & 1),
                                          2 * y0 + (ph >> 1), b0);
-                        ++na;
                         if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
                     }
             }
-            settle_ring(a_full, a_empty, na, g.a_stages, rank == 0, dead);
+            settle_ring(a_full, a_empty, sa, pa, g.a_stages, rank == 0, dead);
             failed = dead;
         }
     } else if (PHASED && warp == B_WARP) {
         // ---------------- stride 2: weight producer ----------------
         if (elect_one()) {
-            uint32_t sb = 0, pb = 1, nb = 0;
+            uint32_t sb = 0, pb = 1;
             bool dead = false;
             const uint32_t full = leader(b_full);
             for (int u = u_lo; u < u_hi && !dead; ++u) {
@@ -188,18 +187,17 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
 #pragma unroll
                         for (int t = 0; t < 3; ++t)
                             tma_load_3d_pair(dst + t * g.b_tap_bytes, &tmB, full + 8 * sb, cc * BK, n0, TAP_ORDER[i + t]);
-                        ++nb;
                         if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
                     }
                 }
             }
-            settle_ring(b_full, b_empty, nb, g.b_stages, rank == 0, dead);
+            settle_ring(b_full, b_empty, sb, pb, g.b_stages, rank == 0, dead);
             failed = dead;
         }
     } else if (!PHASED && warp == 0) {
         // ---------------- TMA producer: loads in the order the MMAs consume them ----------------
         if (elect_one()) {
-            uint32_t sa = 0, pa = 0, sb = 0, pb = 0, na = 0, nb = 0;
+            uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
             bool dead = false;
             const uint32_t ra_full = leader(a_full), rb_full = leader(b_full);
             for (int u = u_lo; u < u_hi && !dead; ++u) {
@@ -214,20 +212,18 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
                     for (int bx = 0; bx < g.a_boxes; ++bx)
                         tma_load_4d_pair(a_ring + sa * g.a_stage_bytes + bx * g.a_box_rows * 128, &tmA, ra_full + 8 * sa,
                                          cc * BK, mt * BM + bx * g.a_box_rows, 0, 0);
-                    ++na;
                     if (++sa == (uint32_t)g.a_stages) { sa = 0; pa ^= 1; }
                     for (int tg = 0; tg < g.ngroups; ++tg) {
                         if (!mbar_wait(b_empty + 8 * sb, pb ^ 1)) { dead = true; break; }
                         if (rank == 0)
                             mbar_expect_tx(b_full + 8 * sb, 2u * g.b_tx);
                         tma_load_3d_pair(b_ring + sb * g.b_stage_bytes, &tmB, rb_full + 8 * sb, cc * BK, n0, tg * g.tgroup);
-                        ++nb;
                         if (++sb == (uint32_t)g.b_stages) { sb = 0; pb ^= 1; }
                     }
                 }
             }
-            settle_ring(a_full, a_empty, na, g.a_stages, rank == 0, dead);
-            settle_ring(b_full, b_empty, nb, g.b_stages, rank == 0, dead);
+            settle_ring(b_full, b_empty, sb, pb ^ 1, g.b_stages, rank == 0, dead);
+            settle_ring(a_full, a_empty, sa, pa ^ 1, g.a_stages, rank == 0, dead);
             failed = dead;
         }
     } else if (warp == 1) {

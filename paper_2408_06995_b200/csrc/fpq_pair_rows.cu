@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
     if (warp == 0) {
         // ---------------- activation producer ----------------
         if (elect_one()) {
-            uint32_t s = 0, ph = 1, issued = 0;
+            uint32_t s = 0, ph = 1;
             bool dead = false;
             const uint32_t full = leader(a_full);
             for (int u = u_lo; u < u_hi && !dead; ++u) {
@@ -120,11 +120,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
                         for (int l = 0; l < loads; ++l)
                             tma_load_4d_pair(dst + l * BM * BK, &tmA, full + 8 * s, (c + l) * BK, row, 0, 0);
                     }
-                    ++issued;
                     if (++s == (uint32_t)g.a_stages) { s = 0; ph ^= 1; }
                 }
             }
-            settle_ring(a_full, a_empty, issued, g.a_stages, rank == 0, dead);
+            settle_ring(a_full, a_empty, s, ph, g.a_stages, rank == 0, dead);
             failed = dead;
         }
     } else if (warp == B_WARP) {
@@ -139,18 +138,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_rows_kernel(const __grid
                 for (int c = 0; c < g.kc && !dead; c += g.span)
                     for (int t = 0; t < g.terms; ++t) {
                         // (the limits of its waits start counting once the kernel in front has finished)
-                        if (issued == (uint32_t)g.b_stages)
+                        if (issued++ == (uint32_t)g.b_stages)
                             asm volatile("griddepcontrol.wait;" ::: "memory");
                         if (!mbar_wait(b_empty + 8 * s, ph)) { dead = true; break; }
                         if (rank == 0)
                             mbar_expect_tx(b_full + 8 * s, 2u * g.b_tx);
                         tma_load_4d_pair(b_ring + s * g.b_stage_bytes, &tmB, full + 8 * s, 0, n0, 0, t * g.kc + c);
-                        ++issued;
                         if (++s == (uint32_t)g.b_stages) { s = 0; ph ^= 1; }
                     }
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            settle_ring(b_full, b_empty, issued, g.b_stages, rank == 0, dead);
+            settle_ring(b_full, b_empty, s, ph, g.b_stages, rank == 0, dead);
             failed = dead;
         }
     } else if (warp == 1) {
