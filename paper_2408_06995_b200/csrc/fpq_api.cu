@@ -663,7 +663,9 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
                 if (launch_quantize_rows_e4m3(x, M, K, p.Ca, x_scale, (uint8_t*)workspace, (cudaStream_t)stream, p.a_e5m2) !=
                     cudaSuccess)
                     return FPQ_ERR_CUDA;
-                return launch_pair_rows(p, 2, (cudaStream_t)stream);
+                s = launch_pair_rows(p, 2, (cudaStream_t)stream);
+                if (s != FPQ_ERR_UNSUPPORTED)                  // (planned for 148 SMs above, for the device's here)
+                    return s;
             }
         }
         if (launch_quantize_rows_e4m3_twice(x, M, K, K2 / 2, x_scale, (uint8_t*)workspace, (cudaStream_t)stream,

@@ -41,6 +41,7 @@ struct PRArgs {
     uint32_t idesc, tmem_cols;
     int acc_bufs;
     int early_weights;
+    bool narrowed;             // host side only: a wider tile would be faster, but two stages of it do not fit
     const float* w_scale;
     float x_scale;
     const float* bias;
@@ -312,8 +313,10 @@ bool plan_rows(const GemmProblem& p, int terms, int nsm, PRArgs& g, double* cycl
     const int nclusters = nsm / 2;
     const int64_t m_units = (p.M + 2 * BM - 1) / (2 * BM);
     // A chunk takes its MMAs or the arrival of its operands; an epilogue stores some 21 bytes per clock and SM and is hidden
-    // behind the next unit, except the last one's.  The tile that just fits columns and SM pairs wins.
-    double best = 0.0;
+    // behind the next unit, except the last one's.  The tile that just fits columns and SM pairs wins, of those with two
+    // stages of a chunk pair and all terms' weights (two terms: up to 160 columns).
+    const int room = SMEM_BUDGET - 1024 - CTL - NUM_EPI * EPI_STAGE;
+    double best = 0.0, best_any = 0.0;
     for (int bn = 32; bn <= 256; bn += 32) {
         if (bn - 32 >= p.N)
             break;
@@ -323,11 +326,14 @@ bool plan_rows(const GemmProblem& p, int terms, int nsm, PRArgs& g, double* cycl
         const double fill = (BM * BK + g.terms * bn * 64.0) / 45.0;
         const double unit = 800.0 + g.kc * (mmas > fill ? mmas : fill), epi = 400.0 + BM * bn * 4 / 21.0;
         const double cost = waves * (waves > 1 && epi > unit ? epi : unit) + epi;
-        if (best == 0.0 || cost < best) {
+        if (best_any == 0.0 || cost < best_any)
+            best_any = cost;
+        if (2 * g.span * (BM * BK + terms * (bn / 2) * BK) <= room && (best == 0.0 || cost < best)) {
             best = cost;
             g.BN = bn;
         }
     }
+    g.narrowed = best_any < best;
     *cycles = best;
     g.n_tiles = (p.N + g.BN - 1) / g.BN;
     g.div_nt = make_fastdiv((uint32_t)g.n_tiles);
@@ -338,7 +344,6 @@ bool plan_rows(const GemmProblem& p, int terms, int nsm, PRArgs& g, double* cycl
     g.b_stage_bytes = g.span * (g.BN / 2) * BK;
     g.b_tx = (uint32_t)g.b_stage_bytes / (p.w4 ? 2 : 1);
     // as many weight stages per activation stage as there are terms
-    const int room = SMEM_BUDGET - 1024 - CTL - NUM_EPI * EPI_STAGE;
     int n = room / (g.a_stage_bytes + terms * g.b_stage_bytes);
     if (n > 8 / terms) n = 8 / terms;
     if (n < 2)
@@ -360,6 +365,9 @@ bool plan_rows(const GemmProblem& p, int terms, int nsm, PRArgs& g, double* cycl
 // M = 16384 121.6 -> 85.6 us, 1344 -> 2944 at 33076 250 -> 200, 1280 -> 320 at 65536 116 -> 108; it loses with few tiles
 // (1280 -> 1280 at 512: 7.6 -> 8.6) and to resident weights (640 -> 640 at 32768: 45.6 -> 46.6).  Two terms: from a few
 // hundred rows on (320 -> 320 at 8192 13.0 -> 9.6, 2560 -> 640 at 2048 20.7 -> 16.1, 5120 -> 1280 at 128 12.6 -> 19.4).
+// Where a wider tile than fits would be faster, only large layers of several rounds (codes written twice and one term's kernel / once and
+// both terms': 320 -> 2560 at 65536 192 / 170, 2560 -> 2560 at 8192 136 / 99, 2560 -> 640 at 16384 109 / 83, 640 -> 5120 at 2048 23.3 / 21.6, 1152 -> 512 at 6985
+// 20.7 / 17.6; in one round 2560 -> 2560 at 1024 18.6 / 19.5, 4928 -> 4192 at 425 23.6 / 24.7; small 320 -> 224 at 12215 10.5 / 11.2).
 bool pair_rows_preferred(const GemmProblem& p, int terms)
 {
     PRArgs g;
@@ -370,7 +378,7 @@ bool pair_rows_preferred(const GemmProblem& p, int terms)
     if (p.M <= 256)
         return false;
     if (terms > 1)
-        return g.kc >= 3 && p.M * g.kc >= 2500;
+        return g.kc >= 3 && p.M * g.kc >= 2500 && (!g.narrowed || (g.units > SMS / 2 && p.M * p.N * g.kc >= 20000000));
     const int64_t m_tiles = (p.M + 127) / 128, n_tiles = (p.N + 127) / 128;
     const int64_t col_grid = SMS / n_tiles * n_tiles;
     const bool resident = n_tiles > 1 && col_grid * 10 >= SMS * 9 && g.kc <= 5;

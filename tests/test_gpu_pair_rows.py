@@ -45,3 +45,26 @@ def test_against_the_oracle_and_the_general_contraction(fx, fw, M, K, N):
     idx = (rows[:, None] * N + np.arange(N)[None, :]).reshape(-1)
     yr, ab = O.linear(x, w, ws, xs, _o(fx), _o(fw), bias, None, idx)
     assert_close(y.reshape(-1)[idx], yr, ab)
+
+
+# weights of two terms whose cheapest tile leaves no room for two stages of both terms' weights: the codes are still written
+# once (the second half of the scratch stays as it was)
+@pytest.mark.parametrize("fw,M,K,N", [(fpq.E3M4, 3000, 1280, 1280), (fpq.E3M4, 2300, 2561, 2560), (fpq.E2M5, 7000, 320, 2555)])
+def test_two_terms_share_the_codes_with_wide_outputs(fw, M, K, N):
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    x = torch.randn(M, K, generator=gen, device="cuda")
+    w = torch.randn(N, K, generator=gen, device="cuda") * 0.02
+    scale = (w.abs().amax(dim=1) / fpq.fpq_format_max(fw)).contiguous()
+    prep = fpq.fpq_prepare_weight(fpq.fpq_quantize_weight(w, scale, fw), fw, fpq.LINEAR, N, K)
+    bias = torch.randn(N, generator=gen, device="cuda")
+    ws = torch.full((fpq.fpq_linear_workspace_size(M, N, K, fpq.E4M3, fw),), 0xAA, dtype=torch.uint8, device="cuda")
+    got = fpq.fpq_linear(x, prep, scale, 0.01, fpq.E4M3, fw, bias, N, workspace=ws).clone()
+    assert bool((ws[M * ((K + 15) // 16 * 16):] == 0xAA).all())
+    try:
+        fpq.fpq_set_path_policy(fpq.PATH_TWO_KERNELS_NARROW)
+        want = fpq.fpq_linear(x, prep, scale, 0.01, fpq.E4M3, fw, bias, N, workspace=ws)
+    finally:
+        fpq.fpq_set_path_policy(fpq.PATH_AUTO)
+    assert fpq.fpq_read_status() == fpq.OK
+    # exact products, FP32 sums in another order
+    assert float((got - want).abs().max()) <= 2e-5 * float(want.abs().max())
