@@ -38,13 +38,16 @@ __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return (a + 
 // ---- launches that overlap the end of the kernel in front ------------------------
 // A kernel launched this way may start while the kernel in front of it in the stream still runs, as soon as all of that
 // one's blocks have executed griddepcontrol.launch_dependents (or ended): its own griddepcontrol.wait, before the first
-// access to global memory, waits until the kernel in front is complete and its writes are visible.  Every kernel of the
-// layer calls is launched so; one launched normally starts some 2.5 us after the end of the kernel in front (QKV linear
+// access to global memory, waits until the kernel in front is complete and its writes are visible.  The kernels of the
+// layer calls are launched so, but for the general contraction when it quantizes its activations itself or is called on
+// its own; one launched normally starts some 2.5 us after the end of the kernel in front (QKV linear
 // 320 -> 960 at M = 8192, calls one after another: 18.3 -> 15.5 us).
 // The contractions leave the launch_dependents to their end: blocks of the next layer's quantize kernel that move in
-// earlier take issue slots and memory ports from their last tiles (19.5 us).  The quantize kernels execute it behind
-// their own wait, so that when their contraction starts everything in front of the layer is complete: it may fetch
-// weights before its own wait.
+// earlier take issue slots and memory ports from their last tiles (19.5 us).  The quantize kernels and the one-kernel
+// convolution on CTA pairs execute it behind their own wait.  So everything in front of a kernel is complete when the one
+// behind it starts, and that is what the early loads rest on: a contraction behind its own quantize kernel may fetch
+// weights before its own wait, because whatever wrote them came before the quantize kernel.  A kernel that executed it
+// before its wait would let its successor read what a kernel in front of both is still writing.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
                                      Args... args)

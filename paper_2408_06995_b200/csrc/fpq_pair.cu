@@ -134,9 +134,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
     float* s_scale = reinterpret_cast<float*>(smem + (bars - smem_base) + 512);
     float* s_bias = s_scale + g.BN;
 
-    // launched with programmatic stream serialization: the next kernel in the stream may be set up while this one
-    // runs (its CTAs become resident as this kernel's CTAs leave)
-    asm volatile("griddepcontrol.launch_dependents;");
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();            // 0: the pair's first CTA (issues the MMAs)
@@ -176,6 +173,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
     // everything above (barriers, tensor memory) overlapped the tail of the kernel in front; nothing below touches
     // global memory before that kernel has completed and its writes are visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The next kernel in the stream may be set up while this one runs (its CTAs become resident as this kernel's CTAs leave):
+    // 2 to 6 % of a layer (128 -> 128 channels at 32 x 32, batch 35: 15.6 us without, 14.9; one tap, 100 -> 128 at 64 x 64, batch 1:
+    // 7.2, 6.3).  Behind this kernel's own wait, and when all its CTAs have their tensor memory.
+    asm volatile("griddepcontrol.launch_dependents;");
 
     bool failed = false;                               // a wait of this thread's role ran out
     // the pair's first CTA's copy of a barrier, as a cluster-space address
@@ -604,8 +605,10 @@ bool pair_conv_applies(const GemmProblem& p)
 //    (128 -> 256 at 32 x 32, batch 35: 27.6 / 20.8; at 64 x 64, batch 18: 54.7 / 35.1).
 //  - Half a warp converts 16 pixel pairs of a channel: narrow rows leave lanes idle (128 -> 128 at 20 x 20, batch 45:
 //    13.1 / 11.6; 28 x 28, batch 23: 12.0 / 11.5, with 64 channels to convert 11.8 / 12.0).  With a full chunk of channels
-//    rows above 32 leave a box a single row (64 x 64, batch 18: 25.1 / 24.3; 64 channels there 24.0 / 25.3), and up to 64
-//    outputs the two kernels' narrow column tile is as fast (128 -> 64 at 32 x 32, batch 35: 13.6 / 13.1; from 64: 13.3 / 13.6).
+//    rows above 32 leave a box a single row (36 x 36, batch 9, 24, 64: 11.4 / 9.5, 14.2 / 13.8, 26.9 / 24.5; 40 x 40, batch 8, 20:
+//    10.7 / 9.5, 13.8 / 13.9; 48 x 48, batch 5, 14, 40: 10.6 / 9.3, 13.7 / 14.0, 28.7 / 28.3; 56 x 56, batch 12: 17.1 / 15.7; 60 x 60,
+//    batch 10, 24: 17.4 / 15.2, 25.4 / 25.5; 64 x 64, batch 18: 25.1 / 24.3; 64 channels there 24.0 / 25.3), so of the widths
+//    (multiples of 4) the one between 28 and 36 is left; and up to 64 outputs the two kernels' narrow column tile is as fast (128 -> 64 at 32 x 32, batch 35: 13.6 / 13.1; from 64: 13.3 / 13.6).
 //  - One tap: 128 -> 128 at 64 x 64, batch 1 (32 tiles) 6.1 / 6.2, 18 (576) 14.9 / 18.5; at 32 x 32, batch 2 (16) 6.6 / 6.2,
 //    9 (72) 6.9 / 7.0; at 28 x 28, batch 46: 12.2 / 11.5.  -> 256 at 64 x 64, batch 2 (64) 7.7 / 7.3, 4 (128) 8.3 / 9.9; at
 //    28 x 28, batch 46 14.4 / 15.4; at 20 x 20, batch 45 10.9 / 10.2.  More outputs: slower at any size.
@@ -621,7 +624,7 @@ bool pair_conv_preferred(const GemmProblem& p)
         return p.W >= 32 && g.m_tiles >= (p.W >= 64 ? 32 : 64);
     if (p.N > 128 || g.m_tiles < 80)
         return false;
-    return p.C <= 64 ? p.W >= 28 : p.N > 64 && p.W == 32;
+    return p.C <= 64 ? p.W >= 28 : p.N > 64 && p.W > 28 && p.W < 36;
 }
 
 fpq_status launch_pair_conv(const GemmProblem& p, cudaStream_t st)

@@ -365,9 +365,10 @@ bool plan_rows(const GemmProblem& p, int terms, int nsm, PRArgs& g, double* cycl
 // M = 16384 121.6 -> 85.6 us, 1344 -> 2944 at 33076 250 -> 200, 1280 -> 320 at 65536 116 -> 108; it loses with few tiles
 // (1280 -> 1280 at 512: 7.6 -> 8.6) and to resident weights (640 -> 640 at 32768: 45.6 -> 46.6).  Two terms: from a few
 // hundred rows on (320 -> 320 at 8192 13.0 -> 9.6, 2560 -> 640 at 2048 20.7 -> 16.1, 5120 -> 1280 at 128 12.6 -> 19.4).
-// Where a wider tile than fits would be faster, only large layers of several rounds (codes written twice and one term's kernel / once and
-// both terms': 320 -> 2560 at 65536 192 / 170, 2560 -> 2560 at 8192 136 / 99, 2560 -> 640 at 16384 109 / 83, 640 -> 5120 at 2048 23.3 / 21.6, 1152 -> 512 at 6985
-// 20.7 / 17.6; in one round 2560 -> 2560 at 1024 18.6 / 19.5, 4928 -> 4192 at 425 23.6 / 24.7; small 320 -> 224 at 12215 10.5 / 11.2).
+// Where a wider tile than fits would be faster, only large layers of several rounds (codes written twice and one term's
+// kernel / once and both terms': 320 -> 2560 at 65536 192 / 170, 2560 -> 2560 at 8192 136 / 99, 2560 -> 640 at 16384 109 / 83,
+// 640 -> 5120 at 2048 23.3 / 21.6, 1152 -> 512 at 6985 20.7 / 17.6; in one round 2560 -> 2560 at 1024 18.6 / 19.5, 4928 -> 4192 at
+// 425 23.6 / 24.7; small 320 -> 224 at 12215 10.5 / 11.2).
 bool pair_rows_preferred(const GemmProblem& p, int terms)
 {
     PRArgs g;
