@@ -437,7 +437,9 @@ __global__ void __launch_bounds__(num_threads(PHASED), 1) fpq_pair_gemm_kernel(c
 // the SM pairs beats the widest one: 640 -> 320 channels at 64 x 64, batch
 // 2, whole layer: 35 units x 3 tiles of 128 in two rounds 24.1 us, x 2 of 160 in one 19.3 us; 256 -> 256 at 32 x 32,
 // batch 16: 15.5 us with 128, 18.6 us with 64 or 192.
-int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_bytes, int accs, double* cycles)
+// loads: those of a chunk where every tap's weights are one, which takes their thread some 400 cycles each (4 x 348 -> 98
+// channels at 7 x 7, 25 taps: 22.5 us for 3 x 26 of them, the general kernel 15.7).
+int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_bytes, int accs, int loads, double* cycles)
 {
     int pick = 128;
     double best = 0.0;
@@ -446,7 +448,9 @@ int choose_tile(int N, int m_units, int nclusters, int cchunks, int taps, int a_
             break;
         const int64_t units = (int64_t)m_units * ((N + bn - 1) / bn);
         const double waves = (double)((units + nclusters - 1) / nclusters);
-        const double mmas = taps * 4 * (bn * 0.53 > 52.0 ? bn * 0.53 : 52.0);
+        double mmas = taps * 4 * (bn * 0.53 > 52.0 ? bn * 0.53 : 52.0);
+        if (mmas < 400.0 * loads)
+            mmas = 400.0 * loads;
         const double fill = (taps * bn * 64.0 + a_bytes) / 43.0;
         const double unit = 800.0 + cchunks * (mmas > fill ? mmas : fill), epi = 128.0 * bn * 4 / 15;
         const bool hidden = 2 * bn * accs <= 512;
@@ -530,13 +534,14 @@ fpq_status plan_pg(const GemmProblem& p, int nsm, PGArgs& g, int* dyn_bytes)
     g.x_scale2 = p.x_scale2;
     const int accs = p.c_seg ? 2 : 1;
     const int a_bytes = phased ? 4 * (int)g.a_tx : (int)round_up(halo_rows, 8) * 128;
-    g.BN = choose_tile(p.N, m_units, nclusters, g.cchunks, g.taps, a_bytes, accs, &g.estimate);
+    g.a_boxes = halo_rows > 256 && !phased ? 2 : 1;
+    const int loads = g.taps >= 4 && g.tgroup == 1 ? g.ngroups + g.a_boxes : 0;
+    g.BN = choose_tile(p.N, m_units, nclusters, g.cchunks, g.taps, a_bytes, accs, loads, &g.estimate);
     g.acc_cols = g.BN * accs;
     g.acc_bufs = 2 * g.acc_cols <= 512 ? 2 : 1;
     g.n_tiles = (p.N + g.BN - 1) / g.BN;
     g.div_nt = make_fastdiv((uint32_t)g.n_tiles);
     g.units = m_units * g.n_tiles;
-    g.a_boxes = halo_rows > 256 && !phased ? 2 : 1;
     g.a_box_rows = (int)round_up((halo_rows + g.a_boxes - 1) / g.a_boxes, 8);
     g.a_stage_bytes = g.a_boxes * g.a_box_rows * 128;
     if (!phased)

@@ -68,3 +68,14 @@ def test_policies_and_errors():
 def test_convolutions_of_few_outputs(B, C, H, W, Co, stride, form):
     for fw in (E4M3, E2M1):
         assert fpq.fpq_conv2d_contraction(B, C, H, W, Co, 3, 3, 1, stride, E4M3, fw) == form
+
+
+# windows whose taps do not go three to a load (16, 25, 49): a load per tap bounds the pairs (us, pairs / general: 4 x 348 -> 98 at
+# 7 x 7, 25 taps 22.5 / 15.7; 271 -> 924 at 10 x 10 22.6 / 15.1; 14 x 631 -> 85 at 18 x 18 36.9 / 25.3; 331 -> 569 at 16 x 16, 16 taps 17.0 /
+# 13.1; 22 x 107 -> 493 at 8 x 8 10.3 / 16.2; 22 x 55 -> 745 at 40 x 40 48.7 / 82.7; 4 x 249 -> 30 at 22 x 22, 49 taps 27.8 / 19.6)
+@pytest.mark.parametrize("B,C,H,W,Co,R,form", [
+    (4, 348, 7, 7, 98, 5, GENERAL), (1, 271, 10, 10, 924, 5, GENERAL), (14, 631, 18, 18, 85, 5, GENERAL), (2, 331, 16, 16, 569, 4, GENERAL),
+    (22, 107, 8, 8, 493, 4, PAIRS), (22, 55, 40, 40, 745, 4, PAIRS), (4, 249, 22, 22, 30, 7, GENERAL)])
+def test_large_windows(B, C, H, W, Co, R, form):
+    for fw in (E4M3, E2M1):
+        assert fpq.fpq_conv2d_contraction(B, C, H, W, Co, R, R, R // 2, 1, E4M3, fw) == form
