@@ -11,7 +11,7 @@
 //   sgemm128<true>          reduction is cut into slices that reduce_d_kernel adds
 //   the same, <false>       partial sums of D^T A over slices of the M rows
 //   grad_finalize_kernel    slices added in a fixed order, chain rule, sum of lambda, optional descent update
-// with many calibration rows (gram_preferred), where D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are less work
+// with many calibration rows (make_plan), where D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are less work
 //   gram_kernel             A^T A in double, slices of rows; gram_reduce_kernel adds them
 //   gram_grad_kernel        E (A^T A) in double, both losses, chain rule, optional descent update
 //
@@ -740,16 +740,6 @@ struct Plan {
     size_t off_SP, off_S, off_ticket;
 };
 
-// E (A^T A) in place of (A E^T)^T A: half of M K^2 and N K^2 products in double instead of 2 M N K on the TF32 tensor cores,
-// by estimates in microseconds of both whole steps (us so / direct, M x N x K: 4096 x 960 x 320 43.8 / 59.6, 8192 x 2560 x 320
-// 88.4 / 195.5, 1024 x 512 x 256 22.9 / 38.0, 139 x 1394 x 192 19.2 / 32.4, 2048 x 320 x 320 30.9 / 33.0, 8192 x 1280 x 640 194.0 / 192.6, 8192 x
-// 320 x 320 59.5 / 43.8, 2048 x 640 x 640 68.5 / 50.8, 4096 x 2560 x 1280 614 / 419).
-bool gram_preferred(int64_t M, int64_t N, int64_t K)
-{
-    const double m = (double)M, n = (double)N, k = (double)K;
-    return K % 4 == 0 && 16.0 + (0.5 * m * k * (k + 64) + n * k * k) / 11.5e6 <= 25.0 + 2.0 * m * n * k / 80e6;
-}
-
 // Rows of gram_grad_kernel's tiles: the fewest whose blocks all run at once, one per SM; with several rounds of them, 64.
 int gram_tile_rows(int64_t N, int64_t K)
 {
@@ -824,9 +814,13 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     o += (size_t)round_up(K * p.Mp * 4, 256);
     p.off_DT = o;
     o += (size_t)round_up(N * p.Mp * 4, 256);
-    p.gram = gram_preferred(M, N, K);
-    if (p.gram) {
-        // the slices with the shortest rounds of blocks (a stage of 32 rows and the sums' way out as two of them)
+    {
+        // E (A^T A) in place of (A E^T)^T A: half of M K^2 and N K^2 products in double instead of 2 M N K on the TF32 tensor
+        // cores.  The slices of M with the shortest rounds of blocks (a stage of 32 rows 1.25 us, the sums' way out two of
+        // them), the rounds of gram_grad_kernel's blocks over K (42 ns per row of a tile and 64 of K), against the direct
+        // form's products (us so / direct, M x N x K: 4096 x 960 x 320 43.8 / 59.6, 8192 x 2560 x 320 88.4 / 195.5, 1024 x 512 x 256 22.9 /
+        // 38.0, 139 x 1394 x 192 19.2 / 32.4, 2048 x 320 x 320 30.9 / 33.0, 8192 x 320 x 320 59.5 / 43.8, 2048 x 640 x 640 68.5 / 50.8,
+        // 1024 x 2560 x 640 132 / 72.8, 94 x 19 x 1164, whose 19 blocks reduce 19 times 64 elements each, 50.3 / 35.0).
         p.tiles_s = (int)((K + ST - 1) / ST);
         const int64_t tiles = (int64_t)p.tiles_s * (p.tiles_s + 1) / 2, stages = (M + S_ROWS - 1) / S_ROWS;
         int64_t best = 0;
@@ -839,6 +833,13 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
                 p.rows_s = each * S_ROWS;
             }
         }
+        const int rows = gram_tile_rows(N, K);
+        const int64_t rounds = ((N + rows - 1) / rows * p.tiles_s + 147) / 148;
+        const double gram = 8.0 + 1.25 * (double)best + (double)rounds * (6.0 + 0.042 * rows * p.tiles_s);
+        p.gram = K % 4 == 0 && gram <= 28.0 + 2.0 * (double)M * (double)N * (double)K / 83e6;
+    }
+    if (p.gram) {
+        const int64_t tiles = (int64_t)p.tiles_s * (p.tiles_s + 1) / 2;
         p.off_SP = o;
         o += (size_t)round_up((int64_t)p.slices_s * tiles * ST * ST * 8, 256);
         p.off_S = o;
