@@ -261,26 +261,31 @@ __global__ void __launch_bounds__(SEARCH_THREADS) search_mse_kernel(const Search
 }
 
 // Block partial sums -> mse (in a fixed order: the same whatever the timing), then the selection.  One block, whose threads
-// share a candidate's blocks as far as there are fewer candidates than threads: a thread that adds all 1184 blocks waits
-// for one load after the other (3.3 M elements, 4 candidates: 64.9 us, 14.1 so).
+// share a candidate's blocks as far as there are fewer candidates than threads, and add up their shares pairwise: a thread
+// that adds all 1184 blocks waits for one load after the other (3.3 M elements, 4 candidates: 64.9 us, 12.9 so).
 __global__ void __launch_bounds__(1024) search_finish_kernel(const SearchArgs a)
 {
     __shared__ double part[1024];
-    const int ncand = a.n_enc * a.n_clip, width = (ncand + 31) / 32 * 32, shares = 1024 / width;
-    const int share = threadIdx.x / width, c = threadIdx.x - share * width;
+    const int t = threadIdx.x, ncand = a.n_enc * a.n_clip;
+    int shares = min(1024 / ncand, a.blocks);
+    const int share = t / ncand, c = t - share * ncand;
     double s = 0.0;
-    if (share < shares && c < ncand) {
-#pragma unroll 8
+    if (share < shares) {
+#pragma unroll 4
         for (int b = share; b < a.blocks; b += shares)
             s += __ldcg(a.partial + (int64_t)b * ncand + c);
     }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x < ncand) {
-        for (int k = 1; k < shares; ++k)
-            s += part[k * width + c];
-        a.mse[c] = a.n > 0 ? s / (double)a.n : 0.0;
+    part[t] = s;
+    while (shares > 1) {
+        const int half = (shares + 1) / 2;
+        __syncthreads();
+        if (share < shares - half)
+            part[t] += part[t + half * ncand];
+        shares = half;
     }
+    __syncthreads();
+    if (t < ncand)
+        a.mse[t] = a.n > 0 ? part[t] / (double)a.n : 0.0;
     __syncthreads();
     select_best<1024>(a.mse, ncand, a.n_clip, a.best);
 }
