@@ -262,18 +262,25 @@ __global__ void __launch_bounds__(SEARCH_THREADS) search_mse_kernel(const Search
 
 // Block partial sums -> mse (in a fixed order: the same whatever the timing), then the selection.  One block, whose threads
 // share a candidate's blocks as far as there are fewer candidates than threads, and add up their shares pairwise: a thread
-// that adds all 1184 blocks waits for one load after the other (3.3 M elements, 4 candidates: 64.9 us, 12.9 so).
+// that adds all 1184 blocks waits for one load after the other (3.3 M elements, 4 candidates: 64.9 us, 12.4 so).
 __global__ void __launch_bounds__(1024) search_finish_kernel(const SearchArgs a)
 {
     __shared__ double part[1024];
     const int t = threadIdx.x, ncand = a.n_enc * a.n_clip;
-    int shares = min(1024 / ncand, a.blocks);
+    int shares = min(1024 / ncand, (a.blocks + 7) / 8);
     const int share = t / ncand, c = t - share * ncand;
     double s = 0.0;
     if (share < shares) {
-#pragma unroll 4
-        for (int b = share; b < a.blocks; b += shares)
-            s += __ldcg(a.partial + (int64_t)b * ncand + c);
+        // (eight loads in flight, whatever the count)
+        for (int b = share; b < a.blocks; b += 8 * shares) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                v[u] = b + u * shares < a.blocks ? a.partial[(int64_t)(b + u * shares) * ncand + c] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                s += v[u];
+        }
     }
     part[t] = s;
     while (shares > 1) {
