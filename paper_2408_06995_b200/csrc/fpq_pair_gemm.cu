@@ -612,7 +612,8 @@ bool pair_gemm_preferred(const GemmProblem& p)
         block *= 0.65;         // (its column tile is 64 wide there)
     const int64_t tiles = m_tiles * ((p.N + 127) / 128);
     double general;
-    if (2 * tiles <= SMS && g.cchunks >= 2) {
+    const bool split = 2 * tiles <= SMS && g.cchunks >= 2;
+    if (split) {
         int64_t sp = SMS / tiles < 8 ? SMS / tiles : 8;
         if (sp > g.cchunks) sp = g.cchunks;
         general = block * (double)((g.cchunks + sp - 1) / sp) * g.taps + 2000.0;
@@ -621,10 +622,11 @@ bool pair_gemm_preferred(const GemmProblem& p)
     }
     // up to 64 outputs the general kernel has little besides its blocks (batch x channels, us here / there: 8 x 320 -> 32 at
     // 64 x 64, stride 2 17.1 / 19.6; 16 x 256 -> 32 at 32 x 32 10.8 / 11.8; 8 x 640 -> 32 at 32 x 32 15.1 / 13.9; 15 x 992 -> 24 at 21 x 21
-    // 19.8 / 16.6; 25 x 320 -> 48 at 15 x 15 11.6 / 13.0; 2 x 320 -> 64 at 30 x 30 9.7 / 8.6; 2 x 352 -> 40 at 28 x 28 9.8 / 8.0; of 57 drawn
-    // layers five take the slower one, by 4 to 8 %; with the difference that wider layers have thirteen did, by up to 23 %)
+    // 19.8 / 16.6; 25 x 320 -> 48 at 15 x 15 11.6 / 13.0; 2 x 320 -> 64 at 30 x 30 9.7 / 8.6; 2 x 352 -> 40 at 28 x 28 9.8 / 8.0; and where it
+    // cannot split the reduction 4 x 128 -> 8 at 59 x 59 7.8 / 8.4).  Of 144 drawn 3 x 3 layers with so few outputs seven take the
+    // slower one by more than 3 %, at stride 1 by 8 % at most; with the margin of wider layers 16 do.
     if (p.N <= 64)
-        return g.estimate <= general + (p.N <= 32 ? 0.0 : 1000.0);
+        return g.estimate <= general + (split && p.N <= 32 ? 0.0 : 1000.0);
     // (stride 2 in several rounds: 256 -> 1280 channels at 16 x 16, batch 57: 20.4 us there, 22.8 here)
     return g.estimate <= general + (p.stride > 1 && g.units > SMS / 2 ? 2000.0 : 4300.0);
 }

@@ -64,7 +64,7 @@ def test_policies_and_errors():
     (2, 1280, 8, 8, 32, 1, GENERAL), (2, 1280, 8, 8, 4, 1, GENERAL), (2, 1280, 16, 16, 16, 1, GENERAL), (2, 320, 32, 32, 3, 1, GENERAL),
     (15, 992, 21, 21, 24, 1, GENERAL), (8, 640, 32, 32, 32, 1, GENERAL), (2, 1280, 16, 16, 32, 2, GENERAL), (1, 480, 27, 27, 24, 2, GENERAL),
     (2, 1280, 8, 8, 33, 1, GENERAL), (2, 320, 30, 30, 64, 1, GENERAL), (2, 352, 28, 28, 40, 1, GENERAL), (25, 320, 15, 15, 48, 1, PAIRS),
-    (4, 1312, 61, 61, 64, 1, PAIRS)])
+    (4, 1312, 61, 61, 64, 1, PAIRS), (4, 128, 59, 59, 8, 1, PAIRS)])
 def test_convolutions_of_few_outputs(B, C, H, W, Co, stride, form):
     for fw in (E4M3, E2M1):
         assert fpq.fpq_conv2d_contraction(B, C, H, W, Co, 3, 3, 1, stride, E4M3, fw) == form
