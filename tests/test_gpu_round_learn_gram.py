@@ -1,5 +1,5 @@
 """The rounding-learning step with many calibration rows, where the gradient is E (A^T A) instead of (A E^T)^T A: on both
-sides of the rule that chooses it, with each product on the multiply-add units and on the tensor cores."""
+sides of the rule that chooses it."""
 import numpy as np
 import pytest
 import torch
@@ -50,8 +50,8 @@ def test_repeated_calls_agree_and_descend():
     assert 0.0 < float(loss[0]) < first
 
 
-# A^T A with 256- and 160-wide tiles; the product with E in one kernel: tiles of 32, 40, 48 and 64 rows, several rounds of them, the last one ragged in rows and
-# columns; the tensor cores instead; step sizes and decisions that are not 16-byte aligned
+# the product with E in tiles of 32, 40, 48 and 64 rows, several rounds of them, the last one ragged in rows and columns; one
+# and many slices of A^T A; the direct form; step sizes and decisions that are not 16-byte aligned
 @pytest.mark.parametrize("M,N,K,lr", [(700, 33, 68, 0.0), (700, 961, 316, 1e4), (700, 1700, 256, 0.0), (600, 2350, 252, 1e4),
                                       (200, 9500, 60, 0.0), (1100, 1500, 400, 0.0), (1100, 600, 316, 0.0), (1200, 700, 580, 1e4)])
 @pytest.mark.parametrize("offset", [0, 1])
