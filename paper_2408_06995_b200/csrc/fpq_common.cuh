@@ -549,7 +549,7 @@ __device__ __forceinline__ void settle_ring(uint32_t full, uint32_t empty, uint3
                                             bool& dead)
 {
     for (uint32_t i = 0; i < stages; ++i) {
-        if (!dead && !mbar_wait_cluster(empty + 8 * s, ph))
+        if (!dead && !mbar_wait(empty + 8 * s, ph))      // (the loop's own wait: polling took 1 to 3 % of a layer)
             dead = true;
         if (dead && first)                             // (the parity of the stage's last load is ph too)
             (void)mbar_wait_cluster(full + 8 * s, ph, 100000000ll);

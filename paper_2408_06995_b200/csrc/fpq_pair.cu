@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fpq_pair_conv_kernel(const __grid
         if (warp == XF_W0) {
             const int used = g.tiles_per_cta * g.cchunks;
             for (int i = used > g.a_stages ? used - g.a_stages : 0; i < used && !dead; ++i)
-                dead = !mbar_wait_cluster(a_empty + 8 * (i % g.a_stages), (i / g.a_stages) & 1);
+                dead = !mbar_wait(a_empty + 8 * (i % g.a_stages), (i / g.a_stages) & 1);
         }
         if (nan)
             flag_status(g.status, FPQ_ERR_NAN_INPUT);

@@ -2,8 +2,8 @@
 // error of quantizing the tensor with every (encoding, clipping value) candidate, then
 // the selection rule of Algorithm 1.
 //
-// Two forms, 444 candidates on 3.7 M elements: 631 us (direct), 73 us (sorted).  Small tensors: every candidate is applied to every element
-// (search_mse_kernel), which is bound by instruction issue.  Large tensors: a
+// Two forms, 444 candidates on 3.7 M elements: 658 us with every candidate applied to every element, 61 us sorted.  Small
+// tensors: every candidate is applied to every element (search_mse_kernel), which is bound by instruction issue.  Large tensors: a
 // candidate's quantizer is a staircase of at most 127 steps, so between two of its
 // thresholds all elements round to the same grid value and only counts and sums of the
 // elements matter.  The elements are sorted into bins a fraction of a step wide; a bin
