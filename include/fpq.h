@@ -427,13 +427,14 @@ fpq_status fpq_round_learn_harden(const float* alpha, int64_t N, int64_t K, uint
  *                         memory (the layer of Sec. VI-A as one pass: FP32 in -> quantize -> low-bit
  *                         MAC -> FP32 out).  Stride-1 convolutions whose whole weight tensor fits in
  *                         the shared memory of a pair of SMs run on CTA pairs (tcgen05 cta_group::2);
- *                         linear layers and the other stride-1 convolutions use the general fused
- *                         form; other geometries fall back to two kernels.
+ *                         linear layers of few rows keep the codes in registers, other linear layers
+ *                         and stride-1 convolutions use the general fused form; other geometries fall
+ *                         back to two kernels.
  *   FPQ_PATH_TWO_KERNELS  always *_quantize_input followed by *_contract.
  *   FPQ_PATH_TWO_KERNELS_NARROW  the same, and the contraction never takes its CTA-pair form (M = 256
  *                         MMAs for long reductions with many tiles): for measurements and tests.
- *   FPQ_PATH_AUTO         the library's choice per shape (default): the CTA-pair kernel where it
- *                         applies and measured faster, else two kernels.
+ *   FPQ_PATH_AUTO         the library's choice per shape (default): the CTA-pair kernel, or that of
+ *                         few rows, where it applies and measured faster, else two kernels.
  */
 enum { FPQ_PATH_AUTO = 0, FPQ_PATH_FUSED = 1, FPQ_PATH_TWO_KERNELS = 2, FPQ_PATH_TWO_KERNELS_NARROW = 3 };
 fpq_status fpq_set_path_policy(int32_t policy);

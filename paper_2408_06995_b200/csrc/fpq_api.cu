@@ -570,9 +570,11 @@ fpq_status fpq_linear_contract(const void* workspace, size_t ws_bytes, const voi
                                 nullptr);
 }
 
-fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_scale, float x_scale, fpq_format fx,
-                      fpq_format fw, const float* bias, float* y, int64_t M, int64_t N, int64_t K, void* workspace,
-                      size_t ws_bytes, void* stream)
+// whole: the rows of the call that these M are part of, which decide about the kernels for few rows (so that a call cut into
+// slices gives what it would give in one piece)
+static fpq_status linear_impl(const float* x, const void* w_prepared, const float* w_scale, float x_scale, fpq_format fx,
+                              fpq_format fw, const float* bias, float* y, int64_t M, int64_t N, int64_t K, void* workspace,
+                              size_t ws_bytes, void* stream, int64_t whole)
 {
     if (bad_scale(x_scale))
         return FPQ_ERR_SCALE;
@@ -685,9 +687,22 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
     if (!aligned(x, 16) || !aligned(y, 16) || !aligned(w_prepared, 128) || !aligned(w_scale, 4) ||
         (bias && !aligned(bias, 4)))
         return FPQ_ERR_ALIGN;
+    if (g_path_policy == FPQ_PATH_FUSED || g_path_policy == FPQ_PATH_AUTO) {
+        // few rows: one kernel, the codes stay in registers
+        GemmProblem p = linear_problem(M, N, K, fx, fw);
+        p.x = x, p.w_prepared = w_prepared, p.w_scale = w_scale, p.x_scale = x_scale, p.bias = bias, p.y = y;
+        p.M = whole;
+        const bool few = few_rows_preferred(p);
+        p.M = M;
+        if (few) {
+            s = launch_few_rows(p, (cudaStream_t)stream);
+            if (s != FPQ_ERR_UNSUPPORTED)
+                return s;
+        }
+    }
     // a handful of rows (time-embedding projections): one pass over the weights on the CUDA cores,
     // whatever the route policy says; the workspace is not touched
-    if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(M, K, N, is_e2m1(fw) ? 1 : 0)) {
+    if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(whole, K, N, is_e2m1(fw) ? 1 : 0)) {
         if (!status_word())
             return FPQ_ERR_CUDA;
         return launch_small_m_linear(x, (int)M, (int)K, w_prepared, is_e2m1(fw) ? 1 : 0, (int)N, w_scale, x_scale, bias, y,
@@ -706,6 +721,13 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
         return s;
     return linear_contract_impl(workspace, ws_bytes, w_prepared, w_scale, x_scale, fx, fw, bias, y, M, N, K, stream, 1,
                                 nullptr);
+}
+
+fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_scale, float x_scale, fpq_format fx,
+                      fpq_format fw, const float* bias, float* y, int64_t M, int64_t N, int64_t K, void* workspace,
+                      size_t ws_bytes, void* stream)
+{
+    return linear_impl(x, w_prepared, w_scale, x_scale, fx, fw, bias, y, M, N, K, workspace, ws_bytes, stream, M);
 }
 
 static fpq_status conv_shape(int B, int C, int H, int W, int C_out, int R, int S, int pad, int stride, int* Ho,
@@ -1240,8 +1262,8 @@ fpq_status fpq_linear_host(const float* x_host, float* x_dev, const void* w_prep
     // (row slices stay 16-byte aligned only if whole rows are: otherwise one slice)
     const bool sliceable = (K % 4 == 0) && (N % 4 == 0);
     auto layer = [&](int64_t m0, int64_t m) {
-        return fpq_linear(x_dev + m0 * K, w_prepared, w_scale, x_scale, fx, fw, bias, y_dev + m0 * N, m, N, K, workspace,
-                          ws_bytes, stream);
+        return linear_impl(x_dev + m0 * K, w_prepared, w_scale, x_scale, fx, fw, bias, y_dev + m0 * N, m, N, K, workspace,
+                           ws_bytes, stream, M);
     };
     if (!sliceable) {
         cudaStream_t st = (cudaStream_t)stream;

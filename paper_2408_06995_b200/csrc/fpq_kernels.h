@@ -97,8 +97,15 @@ bool pair_gemm_preferred(const GemmProblem& p);   // in range, and faster than t
 fpq_status launch_pair_rows(const GemmProblem& p, int terms, cudaStream_t st);
 bool pair_rows_preferred(const GemmProblem& p, int terms);   // in range, and faster than the general contraction
 
+// Linear layer from FP32 rows (p.x) in one kernel with warp-level MMAs, for few rows.  FPQ_ERR_UNSUPPORTED when out of range
+// (nothing was enqueued).
+fpq_status launch_few_rows(const GemmProblem& p, cudaStream_t st);
+bool few_rows_preferred(const GemmProblem& p);   // in range, and faster than the other routes
+
 // Linear layer with at most 8 rows on the CUDA cores (one pass over the weights).
 bool small_m_linear_preferred(int64_t M, int64_t K, int64_t N, int w4);
+double small_m_linear_ns(int64_t M, int64_t K, int64_t N, int w4);   // its estimated time (1e30: out of range) ...
+double two_kernels_ns(int64_t K, int64_t N);                          // ... and that of a quantize kernel and a contraction of few rows
 fpq_status launch_small_m_linear(const float* x, int M, int K, const void* w_prepared, int w4, int N, const float* w_scale,
                                  float x_scale, const float* bias, float* y, cudaStream_t st);
 

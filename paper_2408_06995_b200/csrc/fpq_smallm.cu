@@ -168,18 +168,26 @@ SmallPlan plan_small(int64_t M, int64_t K, int64_t N, int w4)
 
 }  // namespace
 
+static bool in_range(int64_t M, int64_t K, int64_t N)
+{
+    // (rows are read as 16-byte pieces: K a multiple of 4)
+    return M >= 1 && M <= SMALLM_MAX_ROWS && K % 4 == 0 && K <= (1 << 20) && N >= 1 && N <= 0x7fffffff;
+}
+
+double small_m_linear_ns(int64_t M, int64_t K, int64_t N, int w4) { return in_range(M, K, N) ? plan_small(M, K, N, w4).ns : 1e30; }
+
+double two_kernels_ns(int64_t K, int64_t N)
+{
+    return 4200.0 + 2.8 * (double)(K < 320 ? K : 320) + 0.3 * (double)(K > 320 ? K - 320 : 0) + 3.3e-4 * (double)N * (double)K + 0.05 * (double)N;
+}
+
 // Whether one pass on the CUDA cores is expected to be faster than the quantize kernel and the contraction, whose
-// time in chains of its kind is fitted by the right side (us, here / there: 1280 -> 1280, 4-bit weights, 2 rows 3.9 / 6.3,
+// time in chains of its kind is fitted by two_kernels_ns (us, here / there: 1280 -> 1280, 4-bit weights, 2 rows 3.9 / 6.3,
 // 8 rows 9.4 / 6.5; 1280 -> 10240, one row 11.7 / 8.9; 5120 -> 10240, 8 rows 156 / 23; 8-bit weights: 1280 -> 10240, one row
 // 8.2 / 9.8, 8 rows 37 / 9.8; 5120 -> 320, 4 rows 5.2 / 7.2, 8 rows 8.5 / 7.3).
 bool small_m_linear_preferred(int64_t M, int64_t K, int64_t N, int w4)
 {
-    // (rows are read as 16-byte pieces: K a multiple of 4)
-    if (M < 1 || M > SMALLM_MAX_ROWS || K % 4 != 0 || K > (1 << 20) || N < 1 || N > 0x7fffffff)
-        return false;
-    const double other = 4200.0 + 2.8 * (double)(K < 320 ? K : 320) + 0.3 * (double)(K > 320 ? K - 320 : 0) +
-                         3.3e-4 * (double)N * (double)K + 0.05 * (double)N;
-    return plan_small(M, K, N, w4).ns <= other;
+    return in_range(M, K, N) && plan_small(M, K, N, w4).ns <= two_kernels_ns(K, N);
 }
 
 template <bool W4, int MR, int KS>
