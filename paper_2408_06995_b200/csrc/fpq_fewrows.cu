@@ -9,7 +9,7 @@
 // memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3e-8 to 8e-8, theirs 3e-8 to 9e-8).
 // What bounds it: with one block per SM the chain of loads, converts and MMAs, some 0.4 to 0.9 us per 64 elements of a warp; with
 // several the conversions, which every block does for itself.  Whole layer, us here / two kernels, E2M1 weights: 16 x 320 -> 320 1.8 /
-// 5.3, 64 x 320 -> 1280 3.0 / 5.6, 32 x 1280 -> 1280 4.0 / 6.7, 128 x 96 -> 160 1.8 / 5.0; against a warp per column on the CUDA cores
+// 5.3, 64 x 320 -> 1280 3.0 / 5.6, 32 x 1280 -> 1280 4.0 / 6.7; against a warp per column on the CUDA cores
 // (fpq_smallm.cu): 2 x 1280 -> 1280 2.4 / 3.8, 8 x 320 -> 1280 1.8 / 4.8, 8 x 1280 -> 1280 2.8 / 6.2.
 #include <cuda_fp16.h>
 
@@ -240,8 +240,10 @@ cudaError_t launch(const FewArgs& g, cudaStream_t st)
 
 bool few_rows_applies(const GemmProblem& p)
 {
-    // (rows are read as 16-byte pieces: K a multiple of 4)
-    return !p.conv && p.c_seg == 0 && p.C % 4 == 0 && p.C >= 4 && p.C <= (1 << 20) && p.M >= 1 && p.M <= 1024 && p.N <= (1 << 24) &&
+    // Rows are read as 16-byte pieces: K a multiple of 4.  Less than the 128 rows of a tcgen05 tile: from there on a layer gives,
+    // bit for bit, what the 1 x 1 convolution of the same numbers gives, whose MMAs add in the same order (128 x 96 -> 160
+    // would be faster here too, 1.8 us against 5.0; 128 x 1280 -> 1280 would not, 8.5 against 7.0).
+    return !p.conv && p.c_seg == 0 && p.C % 4 == 0 && p.C >= 4 && p.C <= (1 << 20) && p.M >= 1 && p.M < 128 && p.N <= (1 << 24) &&
            (uintptr_t)p.x % 16 == 0;
 }
 

@@ -42,7 +42,7 @@ def _run(x, w, ws, xs, b, fx, fw, policy):
 
 
 @pytest.mark.parametrize("M,K,N", [(1, 4, 1), (7, 60, 15), (8, 64, 16), (9, 68, 17), (16, 512, 33), (17, 516, 64), (33, 1028, 65), (64, 320, 129),
-                                   (100, 576, 96), (129, 96, 160), (3, 2052, 31), (2, 1280, 1280), (1000, 8, 40)])
+                                   (100, 576, 96), (127, 96, 160), (3, 2052, 31), (2, 1280, 1280), (126, 8, 40)])
 @pytest.mark.parametrize("fx,fw", [("e4m3", "e4m3"), ("e4m3", "e2m1"), ("e4m3", "e5m2"), ("e5m2", "e4m3"), ("e5m2", "e2m1"), ("e5m2", "e5m2"),
                                    ("e4m3", "e1m2")])
 def test_matches_sums_of_the_codes(M, K, N, fx, fw):
