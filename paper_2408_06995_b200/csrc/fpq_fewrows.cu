@@ -6,7 +6,7 @@
 // the reduction from global memory straight into registers, turns the activations into codes and both operands into FP16
 // numbers (every E4M3, E5M2 and E2M1 value is one) and multiplies them with mma.sync: no shared memory, no barrier until the
 // warps' sums are added up.  A 128-row tcgen05 tile would be mostly empty, and its operands would have to go through shared
-// memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3e-8 to 8e-8, theirs 3e-8 to 9e-8).
+// memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3e-8 to 7e-8, theirs 3e-8 to 9e-8).
 // What bounds it: with one block per SM the chain of loads, converts and MMAs, some 0.4 to 0.9 us per 64 elements of a warp; with
 // several the conversions, which every block does for itself.  Whole layer, us here / two kernels, E2M1 weights: 16 x 320 -> 320 1.8 /
 // 5.3, 64 x 320 -> 1280 3.0 / 5.6, 32 x 1280 -> 1280 4.0 / 6.7; against a warp per column on the CUDA cores
@@ -176,13 +176,20 @@ __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const
         }
         if (k0 + WARPS * KG < g.K)
             load(k0 + WARPS * KG);
+        // (the MMA cuts off what it adds to an accumulator, so a sum of 64 products starts from zero and is added by an FP32 addition)
+        float part[NT][4] = {};
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             const uint32_t av[4] = {a[0][s][0], R == 1 ? 0u : a[R - 1][s][0], a[0][s][1], R == 1 ? 0u : a[R - 1][s][1]};
 #pragma unroll
             for (int j = 0; j < NT; ++j)
-                mma_f16(acc[j], av, b[j][s][0], b[j][s][1]);
+                mma_f16(part[j], av, b[j][s][0], b[j][s][1]);
         }
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                acc[j][h] += part[j][h];
     }
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
