@@ -129,21 +129,6 @@ fpq_status launch_sgemm_nt(const float* P, int64_t ldp, const float* Q, int64_t 
                            int64_t J, int64_t R, cudaStream_t st);
 fpq_status launch_round_harden(const float* alpha, int64_t N, int64_t K, uint8_t* bits, cudaStream_t st);
 
-// The same step from A^T A on the INT8 tensor cores (fpq_gram.cu): what it keeps in the workspace, and its estimated time.
-constexpr int SLICED_MAX_K = 8192;
-struct SlicedPlan {
-    bool applies;
-    int64_t K16, Mp;           // rows of the planes of E and S, of A^T
-    int BN, tiles, slices, rows;   // A^T A: column tile, tiles, slices of `rows` rows
-    int grad_BN;
-    double us;
-    size_t off_E, off_DQ, off_RG, off_lam, off_PE, off_PA, off_PG, off_SP, off_S, off_PM, off_eE, off_eA, off_eG, off_ticket, bytes;
-};
-SlicedPlan sliced_plan(int64_t M, int64_t N, int64_t K);
-fpq_status launch_sliced_step(const SlicedPlan& p, const float* w, const float* scale, const QFormat& f, float* alpha, const float* a,
-                              int64_t M, int64_t N, int64_t K, float reg, float lr, float* grad, double* loss, void* workspace,
-                              cudaStream_t st);
-
 // C = P Q^T in FP32 on the tensor cores (three TF32 products per term): P [I][ldp], Q [J][ldq], reduction of
 // length R contiguous in both, cut into slices of kb_per_split 32-wide blocks.  epi 0: slice z is written to
 // C + z * split_stride, row-major [I][ldc]; epi 1 (one slice): C[j][i] (leading dimension ldc) and *sq_sum += the sum of the

@@ -3,7 +3,7 @@
 // and of its gradient with respect to alpha, for a bias-free linear layer with FP32 calibration
 // activations A [M][K].  The paper runs this step in FP32, and the contractions keep at least that: the
 // direct form as three TF32 tensor-core products per FP32 product (fpq_tf32.cu), or FP32 multiply-adds on the CUDA cores
-// where rows are no multiple of 4 floats; the form with A^T A in exact sums of digits.
+// where rows are no multiple of 4 floats; the form with A^T A in double.
 //
 //   prepare_kernel          E = Wq(alpha) - W and dWq/dalpha per weight; A^T for the TF32 contractions
 // direct form
@@ -11,7 +11,9 @@
 //   sgemm128<true>          reduction is cut into slices that reduce_d_kernel adds
 //   the same, <false>       partial sums of D^T A over slices of the M rows
 //   grad_finalize_kernel    slices added in a fixed order, chain rule, sum of lambda, optional descent update
-// or, where that is less work (make_plan), from A^T A: fpq_gram.cu
+// with many calibration rows (make_plan), where D^T A = E (A^T A) and sum D^2 = <E (A^T A), E> are less work
+//   gram_kernel             A^T A in double, slices of rows; gram_reduce_kernel adds them
+//   gram_grad_kernel        E (A^T A) in double, both losses, chain rule, optional descent update
 //
 //   harden_kernel           the inference rule: decision bit = (sigma(alpha) >= 0.5)
 //   unfold_kernel           a convolution's input rows, so that the same step serves convolution weights
@@ -20,7 +22,6 @@
 #include <mutex>
 
 #include "fpq_kernels.h"
-#include "fpq_softround.cuh"
 
 namespace fpq {
 
@@ -29,6 +30,23 @@ namespace {
 constexpr int TILE = 128;      // output tile edge
 constexpr int BK = 16;         // reduction elements per shared-memory stage
 constexpr int LDS = TILE + 4;  // padded row length of a stage (floats)
+
+// sigma(alpha), sigma (1 - sigma) and u = 2 |sigma - 0.5| = tanh(|alpha| / 2), each from expressions without
+// cancellation (1 - sigma and sigma - 0.5 formed by subtraction lose most of their bits once sigma saturates,
+// and the regulariser raises u to the 19th power).
+struct SoftTerms {
+    float sig, sp, u;
+};
+__device__ __forceinline__ SoftTerms soft_terms(float al)
+{
+    float t = expf(-fabsf(al));
+    float inv = 1.0f / (1.0f + t);
+    SoftTerms o;
+    o.sig = al >= 0.f ? inv : t * inv;
+    o.sp = t * inv * inv;
+    o.u = tanhf(0.5f * fabsf(al));
+    return o;
+}
 
 // Two FP32 values in one 64-bit register, and the packed multiply-add on such pairs (each half an IEEE fused
 // multiply-add, round to nearest): half the issue slots of two scalar instructions.
@@ -47,6 +65,55 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Adds one value per thread over the block and then into *dst (one atomic per block).
+__device__ __forceinline__ void block_atomic_add(double v, double* dst)
+{
+    __shared__ double warp_part[32];
+    v = warp_sum(v);
+    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0)
+        warp_part[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        int nw = (blockDim.x + 31) >> 5;
+        double s = lane < nw ? warp_part[lane] : 0.0;
+        s = warp_sum(s);
+        if (lane == 0)
+            atomicAdd(dst, s);
+    }
+}
+
+// Learned-rounding equation of Sec. V-B with the sigmoid kept soft, for one weight.
+struct SoftWeight {
+    float e, dq;               // Wq(alpha) - w, dWq/dalpha
+};
+__device__ __forceinline__ SoftWeight soft_weight(float wv, float al, float g, float r, float c, const QFormat& f, bool& nan)
+{
+    const float t = __fmul_rn(wv, r);
+    if (t != t) {
+        nan = true;
+        return {0.f, 0.f};
+    }
+    const SoftTerms st = soft_terms(al);
+    const float a = fminf(fmaxf(t, -c), c);
+    const int Eb = (int)((__float_as_uint(a) >> 23) & 0xffu);
+    const int e_eff = max(Eb - 127, 1 - f.B);                                 // binade whose step applies
+    const float s = __uint_as_float((uint32_t)(e_eff - f.m + 127) << 23);     // step, a power of two
+    const float s_inv = __uint_as_float((uint32_t)(f.m - e_eff + 127) << 23);
+    const float fl = floorf(a * s_inv);                                       // exact: power-of-two scaling
+    const float pre = s * (fl + st.sig);
+    const float q = fminf(fmaxf(pre, -c), c);
+    return {fmaf(g, q, -wv), (pre >= -c && pre <= c) ? g * s * st.sp : 0.f};
+}
+
 // The first blocks: E and dWq/dalpha, four weights per thread (VEC, rows of a multiple of four) or one; block 0 empties
 // the losses.  The others, where A is transposed: one 32 x 32 tile of A^T each.  One launch: both are short.
 template <bool VEC>
@@ -54,7 +121,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ 
                                                       const float* __restrict__ alpha, float* __restrict__ E,
                                                       float* __restrict__ DQ, double* __restrict__ loss, int64_t N, int64_t K,
                                                       int weight_blocks, const float* __restrict__ A, int64_t M,
-                                                      float* __restrict__ AT, int64_t Mp,
+                                                      float* __restrict__ AT, int64_t Mp, unsigned* __restrict__ ticket,
                                                       int* __restrict__ status)
 {
     __shared__ float tile[32][33];
@@ -75,6 +142,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ 
     }
     if (blockIdx.x == 0 && threadIdx.x < 2)
         loss[threadIdx.x] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 2)
+        *ticket = 0;
     constexpr int V = VEC ? 4 : 1;
     const float c = __uint_as_float(f.cmax_bits);
     const int64_t per_row = K / V, total = N * per_row;
@@ -260,6 +329,18 @@ __global__ void __launch_bounds__(256, 2) sgemm128(const float* __restrict__ P, 
         block_atomic_add((double)sq, sq_sum);
 }
 
+// gradient of one weight's alpha: g * dWq/dalpha + reg * dlambda/dalpha; lam += lambda(alpha)
+__device__ __forceinline__ float weight_gradient(float g, float dq, float al, float reg, float& lam)
+{
+    const SoftTerms st = soft_terms(al);
+    const float u = st.u;
+    const float u2 = u * u, u4 = u2 * u2, u8 = u4 * u4, u16 = u8 * u8;
+    lam += 1.0f - u16 * u4;
+    const float u19 = u16 * u2 * u;
+    const float dlam = -40.0f * u19 * (al > 0.f ? 1.f : (al < 0.f ? -1.f : 0.f)) * st.sp;
+    return fmaf(g, dq, reg * dlam);
+}
+
 // grad = (2 / (M N)) (sum of the slices of D^T A) * dWq/dalpha + reg * dlambda/dalpha; alpha -= lr * grad when
 // lr != 0; sum of lambda.  Thread 0 of block 0 turns the sum of squares into the mean.
 // VEC: four weights per thread.  Few blocks, each ending in two atomics: those of a thousand blocks took longer than the
@@ -311,6 +392,271 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(const float* __restr
             store(alpha + i, al);
     }
     block_atomic_add((double)lam, loss + 1);
+}
+
+// ---- the gradient from S = A^T A, in double ----------------------------------------------------------------------
+// sum D^2 = <E S, E> squares what cancels in D = A E^T, and descent makes E small along the rows' leading directions, where
+// all of it cancels.  With S and E S in FP32 the loss of 4096 rows of rank 32 was up to 93 % off and negative at times; in
+// double (products of FP32 numbers are exact) it is closer than the FP32 sum of squares.  The FP64 matrix instructions give
+// 37 TFLOP/s and bound both kernels (70 % busy in gram_kernel, 42 % in gram_grad_kernel, whose blocks are short): 4096 x 320
+// rows and 960 x 320 weights 43.8 us for the whole step; with S in TF32 products 29.5, the direct form 59.6.
+
+// d += a b: 8 x 8 += (8 x 4) (4 x 8); lane l holds a[l / 4][l % 4], b[l % 4][l / 4], d[l / 4][2 (l % 4) + 0, 1]
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b)
+{
+    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+// 16 bytes to shared memory, zeros where there is nothing
+__device__ __forceinline__ void copy16(uint32_t to, const void* from, bool there)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
+}
+
+// S: 64 x 64 tiles on and above the diagonal, each over slices of the rows (blockIdx.y); slice z of tile t goes to SP + (z *
+// tiles + t) * 4096.  Stages of 32 rows; four warps have 32 x 32 outputs each, twice, for half of a stage's rows.
+// Rows of shared memory are 72 floats: the 4 x 8 elements of a fragment lie in 32 banks.
+constexpr int ST = 64, S_ROWS = 32, S_STAGES = 4, S_LD = ST + 8, S_STAGE = 2 * S_ROWS * S_LD;
+constexpr int S_SMEM = S_STAGES * S_STAGE * 4;
+static_assert(S_SMEM >= ST * ST * 8, "the second half's sums");
+__global__ void __launch_bounds__(256, 2) gram_kernel(const float* __restrict__ A, int64_t M, int64_t K, int tiles, int64_t per,
+                                                      double* __restrict__ SP)
+{
+    extern __shared__ __align__(16) float gsm[];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, half = warp >> 2;
+    int ti = 0, left = (int)blockIdx.x;
+    for (; left >= tiles - ti; ++ti)
+        left -= tiles - ti;
+    const int64_t i0 = (int64_t)ti * ST, j0 = (int64_t)(ti + left) * ST;
+    const int64_t m_lo = (int64_t)blockIdx.y * per, m_hi = min(m_lo + per, M);
+    const int wi = (warp & 1) * 32, wj = (warp >> 1 & 1) * 32;
+    auto fetch = [&](int stage, int64_t m) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(gsm + stage * S_STAGE);
+        const int row = t / 16, c = t % 16 * 4;
+#pragma unroll
+        for (int q = 0; q < S_ROWS; q += 16) {
+            const int64_t at = m + row + q;
+            const uint32_t to = dst + ((row + q) * S_LD + c) * 4;
+            const bool in_i = at < m_hi && i0 + c < K, in_j = at < m_hi && j0 + c < K;
+            copy16(to, in_i ? A + at * K + i0 + c : A, in_i);
+            copy16(to + S_ROWS * S_LD * 4, in_j ? A + at * K + j0 + c : A, in_j);
+        }
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int stages = (int)((m_hi - m_lo + S_ROWS - 1) / S_ROWS);
+#pragma unroll
+    for (int s = 0; s < S_STAGES - 1; ++s) {
+        if (s < stages)
+            fetch(s, m_lo + s * S_ROWS);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    double acc[4][4][2] = {};
+    for (int s = 0; s < stages; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(S_STAGES - 2) : "memory");
+        __syncthreads();                               // (and everybody is done with the stage that is filled next)
+        if (s + S_STAGES - 1 < stages)
+            fetch((s + S_STAGES - 1) % S_STAGES, m_lo + (int64_t)(s + S_STAGES - 1) * S_ROWS);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* p = gsm + s % S_STAGES * S_STAGE + (half * (S_ROWS / 2) + (lane & 3)) * S_LD + (lane >> 2);
+#pragma unroll
+        for (int k = 0; k < S_ROWS / 2; k += 4) {
+            double a[4], b[4];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                a[f] = (double)p[k * S_LD + wi + 8 * f];
+                b[f] = (double)p[(S_ROWS + k) * S_LD + wj + 8 * f];
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    mma_f64(acc[x][y], a[x], b[y]);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    double* other = reinterpret_cast<double*>(gsm);
+    double* out = SP + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (ST * ST);
+    const int at = (wi + (lane >> 2)) * ST + wj + 2 * (lane & 3);
+    if (half) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                *reinterpret_cast<double2*>(other + at + 8 * x * ST + 8 * y) = make_double2(acc[x][y][0], acc[x][y][1]);
+    }
+    __syncthreads();
+    if (!half) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const double2 o = *reinterpret_cast<const double2*>(other + at + 8 * x * ST + 8 * y);
+                *reinterpret_cast<double2*>(out + at + 8 * x * ST + 8 * y) = make_double2(acc[x][y][0] + o.x, acc[x][y][1] + o.y);
+            }
+    }
+}
+
+// S [K][K] = the slices added in their order, both triangles.  A block has 8 rows of a tile (blockIdx.y), a thread two columns.
+__global__ void __launch_bounds__(256) gram_reduce_kernel(const double* __restrict__ SP, int slices, int tiles, double* __restrict__ S,
+                                                          int64_t K)
+{
+    __shared__ double turn[8][ST + 1];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int ti = 0, left = (int)blockIdx.x;
+    for (; left >= tiles - ti; ++ti)
+        left -= tiles - ti;
+    const int64_t i0 = (int64_t)ti * ST + blockIdx.y * 8, j0 = (int64_t)(ti + left) * ST;
+    const int row = threadIdx.x / 32, c = threadIdx.x % 32 * 2;
+    const double* p = SP + (int64_t)blockIdx.x * (ST * ST) + (blockIdx.y * 8 + row) * ST + c;
+    double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int z = 0; z < slices; ++z) {
+        const double2 v = *reinterpret_cast<const double2*>(p + (int64_t)z * gridDim.x * (ST * ST));
+        sum.x += v.x, sum.y += v.y;
+    }
+    if (i0 + row < K && j0 + c < K)                    // (K is even)
+        *reinterpret_cast<double2*>(S + (i0 + row) * K + j0 + c) = sum;
+    turn[row][c] = sum.x, turn[row][c + 1] = sum.y;
+    __syncthreads();
+    const int col = threadIdx.x / 4, r = threadIdx.x % 4 * 2;
+    if (left && j0 + col < K && i0 + r < K)
+        *reinterpret_cast<double2*>(S + (j0 + col) * K + i0 + r) = make_double2(turn[r][col], turn[r + 1][col]);
+}
+
+// The rest of the step from S in one kernel: a ROWS x 64 tile of E S per block, reduced over all of K, then what
+// grad_finalize_kernel does.  S is symmetric, so both operands are read as they lie.  64 reduction elements per stage, three
+// stages of asynchronous copies; each of the eight warps has half of the columns and a quarter of a stage's elements, and
+// the quarters' sums are added through shared memory.  Rows are padded so that a fragment's elements lie in different banks.
+constexpr int GK = 64, GR = 64, G_STAGES = 3;
+constexpr int GE_LD = GR + 4, GS_LD = GK + 4, GO_LD = GK + 2;      // floats of E, doubles of S, doubles of a sum
+__host__ __device__ constexpr int gram_stage(int rows) { return rows * GE_LD * 4 + GR * GS_LD * 8; }      // bytes
+constexpr int gram_smem(int rows)
+{
+    return G_STAGES * gram_stage(rows) > 4 * rows * GO_LD * 8 ? G_STAGES * gram_stage(rows) : 4 * rows * GO_LD * 8;
+}
+template <int ROWS>
+__global__ void __launch_bounds__(256, 1) gram_grad_kernel(const float* __restrict__ E, const double* __restrict__ S,
+                                                           const float* __restrict__ DQ, float* __restrict__ alpha,
+                                                           float* __restrict__ grad, double* __restrict__ loss,
+                                                           unsigned* __restrict__ ticket, int64_t N, int64_t K, double coef,
+                                                           double inv_mn, float reg, float lr, int vec)
+{
+    constexpr int F = ROWS / 8;
+    extern __shared__ __align__(16) uint8_t gsm8[];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, col0 = (warp & 1) * 32, part = warp >> 1;
+    const int64_t n0 = (int64_t)blockIdx.x * ROWS, k0 = (int64_t)blockIdx.y * GK;
+    auto fetch = [&](int stage, int64_t r0) {
+        const uint32_t e = (uint32_t)__cvta_generic_to_shared(gsm8 + stage * gram_stage(ROWS)), s = e + ROWS * GE_LD * 4;
+#pragma unroll
+        for (int id = t; id < ROWS * (GR / 4); id += 256) {
+            const int row = id / (GR / 4), c = id % (GR / 4) * 4;
+            const bool there = n0 + row < N && r0 + c < K;
+            copy16(e + (row * GE_LD + c) * 4, there ? E + (n0 + row) * K + r0 + c : E, there);
+        }
+#pragma unroll
+        for (int id = t; id < GR * (GK / 2); id += 256) {
+            const int row = id / (GK / 2), c = id % (GK / 2) * 2;
+            const bool there = r0 + row < K && k0 + c < K;
+            copy16(s + (row * GS_LD + c) * 8, there ? S + (r0 + row) * K + k0 + c : S, there);
+        }
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int stages = (int)((K + GR - 1) / GR);
+#pragma unroll
+    for (int i = 0; i < G_STAGES - 1; ++i) {
+        if (i < stages)
+            fetch(i, (int64_t)i * GR);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    double acc[F][4][2] = {};
+    for (int i = 0; i < stages; ++i) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(G_STAGES - 2) : "memory");
+        __syncthreads();                               // (and everybody is done with the stage that is filled next)
+        if (i + G_STAGES - 1 < stages)
+            fetch((i + G_STAGES - 1) % G_STAGES, (int64_t)(i + G_STAGES - 1) * GR);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const uint8_t* stage = gsm8 + i % G_STAGES * gram_stage(ROWS);
+        const float* es = reinterpret_cast<const float*>(stage) + (lane >> 2) * GE_LD + part * (GR / 4) + (lane & 3);
+        const double* ss = reinterpret_cast<const double*>(stage + ROWS * GE_LD * 4) + (part * (GR / 4) + (lane & 3)) * GS_LD +
+                           col0 + (lane >> 2);
+#pragma unroll
+        for (int r = 0; r < GR / 4; r += 4) {
+            double b[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                b[y] = ss[r * GS_LD + 8 * y];
+#pragma unroll
+            for (int x = 0; x < F; ++x) {
+                const double a = (double)es[8 * x * GE_LD + r];
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    mma_f64(acc[x][y], a, b[y]);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    double* sums = reinterpret_cast<double*>(gsm8);
+#pragma unroll
+    for (int x = 0; x < F; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+            *reinterpret_cast<double2*>(sums + (part * ROWS + 8 * x + (lane >> 2)) * GO_LD + col0 + 8 * y + 2 * (lane & 3)) =
+                make_double2(acc[x][y][0], acc[x][y][1]);
+    __syncthreads();
+    float lam = 0.f;
+    double sq = 0.0;
+    for (int id = t; id < ROWS * GK / 4; id += 256) {
+        const int row = id / (GK / 4), c = id % (GK / 4) * 4;
+        if (n0 + row >= N || k0 + c >= K)
+            continue;
+        const int64_t at = (n0 + row) * K + k0 + c;
+        const float4 dq = *reinterpret_cast<const float4*>(DQ + at), e = *reinterpret_cast<const float4*>(E + at);
+        float al[4], gr[4];
+        if (vec) {
+            const float4 v = *reinterpret_cast<const float4*>(alpha + at);
+            al[0] = v.x, al[1] = v.y, al[2] = v.z, al[3] = v.w;
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                al[v] = alpha[at + v];
+        }
+        const float d[4] = {dq.x, dq.y, dq.z, dq.w}, ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            double g = 0.0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                g += sums[(q * ROWS + row) * GO_LD + c + v];
+            sq = fma(g, (double)ev[v], sq);
+            gr[v] = weight_gradient((float)(coef * g), d[v], al[v], reg, lam);
+            al[v] = al[v] - lr * gr[v];
+        }
+        if (vec) {
+            *reinterpret_cast<float4*>(grad + at) = make_float4(gr[0], gr[1], gr[2], gr[3]);
+            if (lr != 0.f)
+                *reinterpret_cast<float4*>(alpha + at) = make_float4(al[0], al[1], al[2], al[3]);
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                grad[at + v] = gr[v];
+                if (lr != 0.f)
+                    alpha[at + v] = al[v];
+            }
+        }
+    }
+    block_atomic_add((double)lam, loss + 1);
+    __syncthreads();                                   // (the helper's shared memory is used again)
+    block_atomic_add(sq * inv_mn, loss);
+    // a sum of squares: rounding must not leave it below zero (the block that comes last looks)
+    if (t == 0) {
+        __threadfence();
+        if (atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1) {
+            __threadfence();
+            if (__ldcg(loss) < 0.0)
+                *loss = 0.0;
+        }
+    }
 }
 
 // D = sum over the reduction slices of the first contraction (fixed order), and the sum of its squares.
@@ -388,9 +734,20 @@ struct Plan {
     int kb_per_split_tc, splits_tc;
     int kb_per_split1_tc, splits1_tc;       // first contraction: sliced too when it has few output tiles
     size_t off_AT, off_DT;
-    SlicedPlan sliced;
-    bool use_sliced;
+    // with A^T A: 64-wide tiles per side, slices of M
+    int gram, tiles_s, slices_s;
+    int64_t rows_s;
+    size_t off_SP, off_S, off_ticket;
 };
+
+// Rows of gram_grad_kernel's tiles: the fewest whose blocks all run at once, one per SM; with several rounds of them, 64.
+int gram_tile_rows(int64_t N, int64_t K)
+{
+    for (int rows : {32, 40, 48})
+        if ((N + rows - 1) / rows * ((K + 63) / 64) <= 148)
+            return rows;
+    return 64;
+}
 
 // As many slices of a reduction of length R as still fit into one wave of two resident blocks per SM (one more
 // would add a second, nearly empty wave), each at least 128 long.
@@ -457,37 +814,67 @@ Plan make_plan(int64_t M, int64_t N, int64_t K)
     o += (size_t)round_up(K * p.Mp * 4, 256);
     p.off_DT = o;
     o += (size_t)round_up(N * p.Mp * 4, 256);
-    // The sums of digits (fpq_gram.cu), where they are faster than the direct form, whose estimate is fitted to 20 shapes within 16 %
-    // (us, digits / direct, M x N x K: 8192 x 2560 x 320 47 / 195, 8192 x 1000 x 1000 123 / 223, 4096 x 960 x 320 30 / 60, 2048 x 640 x 640
-    // 43 / 52, 8192 x 320 x 320 40 / 45, 150 x 500 x 900 38 / 40; 2048 x 640 x 1280 87 / 74, 94 x 200 x 1164 42 / 35, 64 x 2560 x 2560 248 / 99).
-    // Rows that are no multiple of 4 floats: 777 x 1000 x 333 28 / 69.
-    p.sliced = sliced_plan(M, N, K);
-    const double mnk = (double)M * (double)N * (double)K;
-    const double direct = K % 4 == 0 ? 29.6 + 13.9 * mnk / 1e9 + (3.55 * (double)M + 10.5 * (double)N) * (double)K / 1e6 : 30.0 + mnk / 9e6;
-    p.use_sliced = p.sliced.applies && p.sliced.us < direct;
-    // A shape asks for what it always did, so that a workspace that a program holds still fits: the direct form's buffers,
-    // and where calibration rows abound room for A^T A in double, in 64 x 64 tiles of up to 64 slices, beside them.
     {
-        const int64_t side = (K + 63) / 64, tiles = side * (side + 1) / 2, stages = (M + 31) / 32;
-        int64_t best = 0, slices = 1;
+        // E (A^T A) in place of (A E^T)^T A: half of M K^2 and N K^2 products in double instead of 2 M N K on the TF32 tensor
+        // cores.  The slices of M with the shortest rounds of blocks (a stage of 32 rows 1.25 us, the sums' way out two of
+        // them), the rounds of gram_grad_kernel's blocks over K (42 ns per row of a tile and 64 of K), against the direct
+        // form's products (us so / direct, M x N x K: 4096 x 960 x 320 43.8 / 59.6, 8192 x 2560 x 320 88.4 / 195.5, 1024 x 512 x 256 22.9 /
+        // 38.0, 139 x 1394 x 192 19.2 / 32.4, 2048 x 320 x 320 30.9 / 33.0, 8192 x 320 x 320 59.5 / 43.8, 2048 x 640 x 640 68.5 / 50.8,
+        // 1024 x 2560 x 640 132 / 72.8, 94 x 19 x 1164, whose 19 blocks reduce 19 times 64 elements each, 50.3 / 35.0).
+        p.tiles_s = (int)((K + ST - 1) / ST);
+        const int64_t tiles = (int64_t)p.tiles_s * (p.tiles_s + 1) / 2, stages = (M + S_ROWS - 1) / S_ROWS;
+        int64_t best = 0;
         for (int64_t want = 1; want <= 64 && want <= stages; ++want) {
-            const int64_t each = (stages + want - 1) / want, n = (stages + each - 1) / each;
-            const int64_t cost = (tiles * n + 147) / 148 * (each + 2);
-            if (best == 0 || cost < best)
-                best = cost, slices = n;
+            const int64_t each = (stages + want - 1) / want, slices = (stages + each - 1) / each;
+            const int64_t cost = (tiles * slices + 147) / 148 * (each + 2);
+            if (best == 0 || cost < best) {
+                best = cost;
+                p.slices_s = (int)slices;
+                p.rows_s = each * S_ROWS;
+            }
         }
-        int64_t rows = 64;
-        for (int64_t r : {48, 40, 32})
-            if ((N + r - 1) / r * side <= 148)
-                rows = r;
-        const int64_t rounds = ((N + rows - 1) / rows * side + 147) / 148;
-        const double with = 8.0 + 1.25 * (double)best + (double)rounds * (6.0 + 0.042 * (double)(rows * side));
-        if (K % 4 == 0 && with <= 28.0 + 2.0 * mnk / 83e6)
-            o += (size_t)round_up(slices * tiles * 4096 * 8, 256) + (size_t)round_up(K * K * 8, 256);
+        const int rows = gram_tile_rows(N, K);
+        const int64_t rounds = ((N + rows - 1) / rows * p.tiles_s + 147) / 148;
+        const double gram = 8.0 + 1.25 * (double)best + (double)rounds * (6.0 + 0.042 * rows * p.tiles_s);
+        p.gram = K % 4 == 0 && gram <= 28.0 + 2.0 * (double)M * (double)N * (double)K / 83e6;
     }
+    if (p.gram) {
+        const int64_t tiles = (int64_t)p.tiles_s * (p.tiles_s + 1) / 2;
+        p.off_SP = o;
+        o += (size_t)round_up((int64_t)p.slices_s * tiles * ST * ST * 8, 256);
+        p.off_S = o;
+        o += (size_t)round_up(K * K * 8, 256);
+    }
+    p.off_ticket = o;
     o += 256;
-    p.bytes = p.use_sliced && p.sliced.bytes > o ? p.sliced.bytes : o;
+    p.bytes = o;
     return p;
+}
+
+// most dynamic shared memory of a kernel, set once per device
+template <typename Kernel>
+bool allow_smem(Kernel kernel, int bytes, bool (&set)[64])
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+        return false;
+    if (!set[dev])
+        set[dev] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    return set[dev];
+}
+
+template <int ROWS>
+cudaError_t launch_gram_grad(const float* E, const double* S, const float* DQ, float* alpha, float* grad, double* loss, unsigned* ticket,
+                             int64_t N, int64_t K, double coef, double inv_mn, float reg, float lr, cudaStream_t st)
+{
+    static bool set[64] = {};
+    if (!allow_smem(gram_grad_kernel<ROWS>, gram_smem(ROWS), set))
+        return cudaErrorUnknown;
+    const int vec = (uintptr_t)alpha % 16 == 0 && (uintptr_t)grad % 16 == 0;
+    return launch_overlapped(gram_grad_kernel<ROWS>, dim3((unsigned)((N + ROWS - 1) / ROWS), (unsigned)((K + GK - 1) / GK)), 256,
+                             gram_smem(ROWS), st, E, S, DQ, alpha, grad, loss, ticket, N, K, coef, inv_mn, reg, lr, vec);
 }
 
 }  // namespace
@@ -499,8 +886,6 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
                               void* workspace, cudaStream_t st)
 {
     Plan p = make_plan(M, N, K);
-    if (p.use_sliced)
-        return launch_sliced_step(p.sliced, w, scale, f, alpha, a, M, N, K, reg, lr, grad, loss, workspace, st);
     char* ws = (char*)workspace;
     float* E = (float*)(ws + p.off_E);
     float* DQ = (float*)(ws + p.off_DQ);
@@ -514,14 +899,15 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
     const float coef = (float)(2.0 * inv_mn);
     const bool tc = tf32x3_applies(a, K, E, K, M, N, K) && M <= (1 << 21) && N <= (1 << 21) && K <= (1 << 21);
     float* AT = (float*)(ws + p.off_AT);
+    unsigned* ticket = (unsigned*)(ws + p.off_ticket);
     {
         const bool vec = K % 4 == 0 && (uintptr_t)w % 16 == 0 && (uintptr_t)alpha % 16 == 0;
         const int weight_blocks = grid_for(vec ? N * K / 4 : N * K);
-        const int64_t blocks = weight_blocks + (tc ? ((M + 31) / 32) * ((K + 31) / 32) : 0);
+        const int64_t blocks = weight_blocks + (tc && !p.gram ? ((M + 31) / 32) * ((K + 31) / 32) : 0);
         if (blocks > 0x7fffffff)
             return FPQ_ERR_SHAPE;
         if (launch_overlapped(vec ? prepare_kernel<true> : prepare_kernel<false>, dim3((unsigned)blocks), 256, 0, st, w, scale, f,
-                              alpha, E, DQ, loss, N, K, weight_blocks, a, M, AT, p.Mp, status) != cudaSuccess)
+                              alpha, E, DQ, loss, N, K, weight_blocks, a, M, AT, p.Mp, ticket, status) != cudaSuccess)
             return FPQ_ERR_CUDA;
     }
     auto finalize = [&](int splits) {
@@ -533,6 +919,22 @@ fpq_status launch_round_learn(const float* w, const float* scale, const QFormat&
                    ? FPQ_OK
                    : FPQ_ERR_CUDA;
     };
+    if (tc && p.gram) {
+        double* SP = (double*)(ws + p.off_SP);
+        double* S = (double*)(ws + p.off_S);
+        const unsigned tiles = (unsigned)(p.tiles_s * (p.tiles_s + 1) / 2);
+        static bool set[64] = {};
+        if (!allow_smem(gram_kernel, S_SMEM, set) ||
+            launch_overlapped(gram_kernel, dim3(tiles, (unsigned)p.slices_s), 256, S_SMEM, st, a, M, K, p.tiles_s, p.rows_s, SP) !=
+                cudaSuccess ||
+            launch_overlapped(gram_reduce_kernel, dim3(tiles, ST / 8), 256, 0, st, SP, p.slices_s, p.tiles_s, S, K) != cudaSuccess)
+            return FPQ_ERR_CUDA;
+        const int rows = gram_tile_rows(N, K);
+        const auto launch = rows == 32 ? launch_gram_grad<32> : rows == 40 ? launch_gram_grad<40>
+                            : rows == 48 ? launch_gram_grad<48> : launch_gram_grad<64>;
+        return launch(E, S, DQ, alpha, grad, loss, ticket, N, K, 2.0 * inv_mn, inv_mn, reg, lr, st) == cudaSuccess ? FPQ_OK
+                                                                                                                  : FPQ_ERR_CUDA;
+    }
     if (tc) {
         // Both contractions on the tensor cores (three TF32 products per FP32 product): D^T = (A E^T)^T is written
         // transposed by the first one's epilogue, so that the second one, D^T A, again reduces over the contiguous

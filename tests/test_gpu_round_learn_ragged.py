@@ -1,5 +1,4 @@
-"""The rounding-learning step from A^T A on the INT8 tensor cores: ragged tiles and slices, columns of very different size, and
-operands that are not finite."""
+"""The rounding-learning step at ragged sizes, with columns of very different size, and with operands that are not finite."""
 import numpy as np
 import pytest
 import torch
@@ -29,8 +28,7 @@ def _reference(w, scale, alpha, a):
     return (d * d).mean(), c * (d.T @ ad), c.abs() * (noise @ (ad.abs().T @ ad.abs()))
 
 
-# a row and column; less and more than a tile of either product; slices of less than 256 rows, of several times 256, a last one of
-# few rows; rows of no multiple of 4 and of 16
+# a row and column; less and more than a tile of either product; few and many rows; rows of no multiple of 4 and of 16
 @pytest.mark.parametrize("M,N,K", [(1, 1, 1), (31, 129, 47), (257, 127, 33), (600, 130, 129), (5000, 64, 95), (300, 513, 260),
                                    (8192, 130, 200), (9000, 257, 321), (2049, 300, 640), (40, 2000, 17)])
 def test_sizes(M, N, K):
@@ -50,7 +48,6 @@ def test_columns_of_very_different_size():
     a[:, 8] = 1e-42
     grad, _ = fpq.fpq_round_learn_step(w, scale, fpq.E2M1, alpha, a, 0.0)
     _, want, noise = _reference(w, scale, alpha, a)
-    # (a whole number of 32 bits per entry of A: 2^-32 of its column's largest magnitude, some 2^-24 of the sums of magnitudes)
     assert bool(((grad.double() - want).abs() <= 2 * noise + 2.0 ** -19 * want.abs() + 1e-38).all())
 
 
