@@ -175,6 +175,8 @@ fpq_status fpq_prepare_weight(const uint8_t* codes, fpq_format fmt, const fpq_la
  * FPQ_ERR_UNSUPPORTED otherwise.
  * workspace: fpq_linear_workspace_size bytes, 128-byte aligned; contents are
  * scratch.
+ * y may be x or overlap it: the layer then runs as two kernels under every route policy, and x is read whole before
+ * y is written.  Nothing else may overlap y or the workspace (in the host-buffer forms neither may x and y).
  */
 size_t fpq_linear_workspace_size(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format fw);
 fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_scale, float x_scale,
@@ -185,7 +187,8 @@ fpq_status fpq_linear(const float* x, const void* w_prepared, const float* w_sca
  * Quantized 2-D convolution (cross-correlation, zero padding, square stride):
  * x FP32 NCHW [B][C][H][W], y FP32 NCHW [B][C_out][H_out][W_out],
  * H_out = (H + 2 pad - R) / stride + 1.  Same arithmetic as fpq_linear with
- * k running over (c, r, s); padding contributes code 0.
+ * k running over (c, r, s); padding contributes code 0.  y must not overlap x (a layer that runs as one kernel stores
+ * while it still reads).
  */
 size_t fpq_conv2d_workspace_size(int B, int C, int H, int W, int C_out, int R, int S, int pad,
                                  int stride, fpq_format fx, fpq_format fw);

@@ -687,7 +687,9 @@ static fpq_status linear_impl(const float* x, const void* w_prepared, const floa
     if (!aligned(x, 16) || !aligned(y, 16) || !aligned(w_prepared, 128) || !aligned(w_scale, 4) ||
         (bias && !aligned(bias, 4)))
         return FPQ_ERR_ALIGN;
-    if (g_path_policy == FPQ_PATH_FUSED || g_path_policy == FPQ_PATH_AUTO) {
+    // y on top of x: only the two kernels have read all of x before the first store
+    const bool apart = (uintptr_t)x + (uintptr_t)(M * K) * 4 <= (uintptr_t)y || (uintptr_t)y + (uintptr_t)(M * N) * 4 <= (uintptr_t)x;
+    if (apart && (g_path_policy == FPQ_PATH_FUSED || g_path_policy == FPQ_PATH_AUTO)) {
         // few rows: one kernel, the codes stay in registers
         GemmProblem p = linear_problem(M, N, K, fx, fw);
         p.x = x, p.w_prepared = w_prepared, p.w_scale = w_scale, p.x_scale = x_scale, p.bias = bias, p.y = y;
@@ -702,7 +704,7 @@ static fpq_status linear_impl(const float* x, const void* w_prepared, const floa
     }
     // a handful of rows (time-embedding projections): one pass over the weights on the CUDA cores,
     // whatever the route policy says; the workspace is not touched
-    if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(whole, K, N, is_e2m1(fw) ? 1 : 0)) {
+    if (apart && !is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(whole, K, N, is_e2m1(fw) ? 1 : 0)) {
         if (!status_word())
             return FPQ_ERR_CUDA;
         return launch_small_m_linear(x, (int)M, (int)K, w_prepared, is_e2m1(fw) ? 1 : 0, (int)N, w_scale, x_scale, bias, y,
@@ -710,7 +712,7 @@ static fpq_status linear_impl(const float* x, const void* w_prepared, const floa
     }
     // one kernel: the activations are quantized inside the contraction's operand staging
     // (AUTO takes the two-kernel route: measured faster on B200 so far)
-    if (g_path_policy == FPQ_PATH_FUSED && is_e4m3_native(fx)) {
+    if (apart && g_path_policy == FPQ_PATH_FUSED && is_e4m3_native(fx)) {
         s = linear_contract_impl(workspace, ws_bytes, w_prepared, w_scale, x_scale, fx, fw, bias, y, M, N, K, stream, 0,
                                  x);
         if (s != FPQ_ERR_UNSUPPORTED)
