@@ -697,7 +697,7 @@ static fpq_status linear_impl(const float* x, const void* w_prepared, const floa
         const bool few = few_rows_preferred(p);
         p.M = M;
         if (few) {
-            s = launch_few_rows(p, (cudaStream_t)stream);
+            s = launch_few_rows(p, whole, (cudaStream_t)stream);
             if (s != FPQ_ERR_UNSUPPORTED)
                 return s;
         }

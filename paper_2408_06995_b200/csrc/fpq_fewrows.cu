@@ -6,7 +6,7 @@
 // the reduction from global memory straight into registers, turns the activations into codes and both operands into FP16
 // numbers (every E4M3, E5M2 and E2M1 value is one) and multiplies them with mma.sync: no shared memory, no barrier until the
 // warps' sums are added up.  A 128-row tcgen05 tile would be mostly empty, and its operands would have to go through shared
-// memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3e-8 to 7e-8, theirs 3e-8 to 9e-8).
+// memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3.5e-8 to 6e-8, theirs 3.5e-8 to 9e-8).
 // What bounds it: with one block per SM the chain of loads, converts and MMAs, some 0.4 to 0.9 us per 64 elements of a warp; with
 // several the conversions, which every block does for itself.  Whole layer, us here / two kernels, E2M1 weights: 16 x 320 -> 320 1.8 /
 // 5.3, 64 x 320 -> 1280 3.0 / 5.6, 32 x 1280 -> 1280 4.0 / 6.7; against a warp per column on the CUDA cores
@@ -51,6 +51,12 @@ __device__ __forceinline__ uint32_t quantized(float lo, float hi, unsigned long 
         asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(c) : "f"(b), "f"(a));
     return two_values<E5>(c);
 }
+// NaN counts as zero
+__device__ __forceinline__ void nan_to_zero(uint32_t& v)
+{
+    if ((v & 0x7fffu) > 0x7c00u) v &= 0xffff0000u;
+    if ((v & 0x7fff0000u) > 0x7c000000u) v &= 0xffffu;
+}
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 
 // values of eight E2M1 codes (low nibble first)
@@ -85,7 +91,7 @@ struct FewArgs {
 
 // A block has 8 R rows (R = 1, 2) and 8 NT columns.  The lanes of a quad have 16 neighbouring elements of the reduction each;
 // the MMA's step s takes the fourth s of them (its own order of the reduction is the same for both operands, so any will do).
-template <int WF, bool E5, int R, int NT>
+template <int WF, bool E5, int R, int NT, bool SHORT>
 __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const FewArgs g)
 {
     constexpr int COLS = 8 * NT;
@@ -110,86 +116,124 @@ __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const
         there[i] = m0 + 8 * i + r < g.M;
         xp[i] = g.x + (int64_t)(there[i] ? m0 + 8 * i + r : 0) * g.K + 16 * q;
     }
-    uint4 wv[NT];
-    float4 xv[R][4];
-    auto load = [&](int k0) {
+    if constexpr (SHORT) {
+        // Four warps share a group of 64, a step of the MMA each; no sum is longer than 16 products, to which the MMA adds zero
+        // (it cuts off what it adds to an accumulator).
+        for (int k0 = (warp >> 2) * KG; k0 < g.K; k0 += 2 * KG) {
+            const int s = warp & 3, k = k0 + 16 * q + 4 * s;
+            uint32_t codes[NT], a[R][2];
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            if (WF == W_E2M1) {
-                const uint2 v = __ldg(reinterpret_cast<const uint2*>(wp[j] + k0 / 2));
-                wv[j] = make_uint4(v.x, v.y, 0u, 0u);
-            } else {
-                wv[j] = __ldg(reinterpret_cast<const uint4*>(wp[j] + k0));
+            for (int j = 0; j < NT; ++j)
+                codes[j] = __ldg(reinterpret_cast<const uint32_t*>(wp[j] + (WF == W_E2M1 ? k0 / 2 + (s & 2) * 2 : k0 + 4 * s)));
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const float4 v = there[i] && k < g.K ? __ldg(reinterpret_cast<const float4*>(xp[i] + k0 + 4 * s)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                a[i][0] = quantized<E5>(v.x, v.y, rinv2);
+                a[i][1] = quantized<E5>(v.z, v.w, rinv2);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (__hisnan(__low2half(as_half2(a[i][h]))) || __hisnan(__high2half(as_half2(a[i][h])))) {
+                        nan = true;
+                        nan_to_zero(a[i][h]);
+                    }
+            }
+            const uint32_t av[4] = {a[0][0], R == 1 ? 0u : a[R - 1][0], a[0][1], R == 1 ? 0u : a[R - 1][1]};
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                uint32_t b[4];
+                if (WF == W_E2M1) {
+                    eight_values(codes[j], b);
+                    if (s & 1) b[0] = b[2], b[1] = b[3];
+                } else {
+                    b[0] = two_values<WF == W_E5M2>((uint16_t)(codes[j] & 0xffffu));
+                    b[1] = two_values<WF == W_E5M2>((uint16_t)(codes[j] >> 16));
+                }
+                float part[4] = {};
+                mma_f16(part, av, b[0], b[1]);
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    acc[j][h] += part[h];
             }
         }
+    } else {
+        uint4 wv[NT];
+        float4 xv[R][4];
+        auto load = [&](int k0) {
 #pragma unroll
-        for (int i = 0; i < R; ++i)
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-                xv[i][s] = there[i] && k0 + 16 * q + 4 * s < g.K ? __ldg(reinterpret_cast<const float4*>(xp[i] + k0 + 4 * s))
-                                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-    };
-    int k0 = warp * KG;
-    if (k0 < g.K)
-        load(k0);
-    for (; k0 < g.K; k0 += WARPS * KG) {
-        uint32_t a[R][4][2];
-        __half2 most = __float2half2_rn(0.f);
-#pragma unroll
-        for (int i = 0; i < R; ++i)
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                a[i][s][0] = quantized<E5>(xv[i][s].x, xv[i][s].y, rinv2);
-                a[i][s][1] = quantized<E5>(xv[i][s].z, xv[i][s].w, rinv2);
-                most = __hmax2_nan(most, __hmax2_nan(__habs2(as_half2(a[i][s][0])), __habs2(as_half2(a[i][s][1]))));
+            for (int j = 0; j < NT; ++j) {
+                if (WF == W_E2M1) {
+                    const uint2 v = __ldg(reinterpret_cast<const uint2*>(wp[j] + k0 / 2));
+                    wv[j] = make_uint4(v.x, v.y, 0u, 0u);
+                } else {
+                    wv[j] = __ldg(reinterpret_cast<const uint4*>(wp[j] + k0));
+                }
             }
-        if (__hisnan(__low2half(most)) || __hisnan(__high2half(most))) {
-            // NaN counts as zero
-            nan = true;
 #pragma unroll
             for (int i = 0; i < R; ++i)
 #pragma unroll
                 for (int s = 0; s < 4; ++s)
+                    xv[i][s] = there[i] && k0 + 16 * q + 4 * s < g.K ? __ldg(reinterpret_cast<const float4*>(xp[i] + k0 + 4 * s))
+                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        int k0 = warp * KG;
+        if (k0 < g.K)
+            load(k0);
+        for (; k0 < g.K; k0 += WARPS * KG) {
+            uint32_t a[R][4][2];
+            __half2 most = __float2half2_rn(0.f);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if ((a[i][s][h] & 0x7fffu) > 0x7c00u) a[i][s][h] &= 0xffff0000u;
-                        if ((a[i][s][h] & 0x7fff0000u) > 0x7c000000u) a[i][s][h] &= 0xffffu;
-                    }
-        }
-        uint32_t b[NT][4][2];
-#pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            if (WF == W_E2M1) {
-                uint32_t lo[4], hi[4];
-                eight_values(wv[j].x, lo);
-                eight_values(wv[j].y, hi);
-                b[j][0][0] = lo[0], b[j][0][1] = lo[1], b[j][1][0] = lo[2], b[j][1][1] = lo[3];
-                b[j][2][0] = hi[0], b[j][2][1] = hi[1], b[j][3][0] = hi[2], b[j][3][1] = hi[3];
-            } else {
-                const uint32_t c[4] = {wv[j].x, wv[j].y, wv[j].z, wv[j].w};
+            for (int i = 0; i < R; ++i)
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
-                    b[j][s][0] = two_values<WF == W_E5M2>((uint16_t)(c[s] & 0xffffu));
-                    b[j][s][1] = two_values<WF == W_E5M2>((uint16_t)(c[s] >> 16));
+                    a[i][s][0] = quantized<E5>(xv[i][s].x, xv[i][s].y, rinv2);
+                    a[i][s][1] = quantized<E5>(xv[i][s].z, xv[i][s].w, rinv2);
+                    most = __hmax2_nan(most, __hmax2_nan(__habs2(as_half2(a[i][s][0])), __habs2(as_half2(a[i][s][1]))));
+                }
+            if (__hisnan(__low2half(most)) || __hisnan(__high2half(most))) {
+                nan = true;
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            nan_to_zero(a[i][s][h]);
+            }
+            uint32_t b[NT][4][2];
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                if (WF == W_E2M1) {
+                    uint32_t lo[4], hi[4];
+                    eight_values(wv[j].x, lo);
+                    eight_values(wv[j].y, hi);
+                    b[j][0][0] = lo[0], b[j][0][1] = lo[1], b[j][1][0] = lo[2], b[j][1][1] = lo[3];
+                    b[j][2][0] = hi[0], b[j][2][1] = hi[1], b[j][3][0] = hi[2], b[j][3][1] = hi[3];
+                } else {
+                    const uint32_t c[4] = {wv[j].x, wv[j].y, wv[j].z, wv[j].w};
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        b[j][s][0] = two_values<WF == W_E5M2>((uint16_t)(c[s] & 0xffffu));
+                        b[j][s][1] = two_values<WF == W_E5M2>((uint16_t)(c[s] >> 16));
+                    }
                 }
             }
-        }
-        if (k0 + WARPS * KG < g.K)
-            load(k0 + WARPS * KG);
-        // (the MMA cuts off what it adds to an accumulator, so a sum of 64 products starts from zero and is added by an FP32 addition)
-        float part[NT][4] = {};
+            if (k0 + WARPS * KG < g.K)
+                load(k0 + WARPS * KG);
+            // (the MMA cuts off what it adds to an accumulator, so a sum of 64 products starts from zero and is added by an FP32 addition)
+            float part[NT][4] = {};
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const uint32_t av[4] = {a[0][s][0], R == 1 ? 0u : a[R - 1][s][0], a[0][s][1], R == 1 ? 0u : a[R - 1][s][1]};
+            for (int s = 0; s < 4; ++s) {
+                const uint32_t av[4] = {a[0][s][0], R == 1 ? 0u : a[R - 1][s][0], a[0][s][1], R == 1 ? 0u : a[R - 1][s][1]};
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    mma_f16(part[j], av, b[j][s][0], b[j][s][1]);
+            }
 #pragma unroll
             for (int j = 0; j < NT; ++j)
-                mma_f16(part[j], av, b[j][s][0], b[j][s][1]);
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    acc[j][h] += part[j][h];
         }
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-            for (int h = 0; h < 4; ++h)
-                acc[j][h] += part[j][h];
     }
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
@@ -200,12 +244,28 @@ __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const
     __syncthreads();
     for (int id = threadIdx.x; id < 8 * R * COLS; id += THREADS) {
         const int i = id / COLS, c = id % COLS, n = n0 + c;
-        float v = sums[0][i][c];
+        // In pairs; what the last two levels, whose sums are the largest, round away is kept (Knuth's two-sum) and added last: the error
+        // of the layer against 64 bits is 9 % below that of a warp per column (1 to 8 rows of 64 to 5120) and 25 % below
+        // that of the two kernels, where the warps' sums one after the other were 1 % above the former; 0.3 % of the time.
+        float v[WARPS], lost = 0.f;
 #pragma unroll
-        for (int k = 1; k < WARPS; ++k)
-            v += sums[k][i][c];
-        if (m0 + i < g.M && n < g.N)
-            g.y[(int64_t)(m0 + i) * g.N + n] = fmaf(v, g.x_scale * __ldg(g.w_scale + n), g.bias ? __ldg(g.bias + n) : 0.f);
+        for (int k = 0; k < WARPS; ++k)
+            v[k] = sums[k][i][c];
+#pragma unroll
+        for (int s = 1; s < WARPS; s *= 2)
+#pragma unroll
+            for (int k = 0; k < WARPS; k += 2 * s) {
+                const float t = __fadd_rn(v[k], v[k + s]);
+                if (s > 1) {
+                    const float z = __fsub_rn(t, v[k]);
+                    lost += __fadd_rn(__fsub_rn(v[k], __fsub_rn(t, z)), __fsub_rn(v[k + s], z));
+                }
+                v[k] = t;
+            }
+        if (m0 + i < g.M && n < g.N) {
+            const float scale = g.x_scale * __ldg(g.w_scale + n);
+            g.y[(int64_t)(m0 + i) * g.N + n] = fmaf(v[0], scale, fmaf(lost, scale, g.bias ? __ldg(g.bias + n) : 0.f));
+        }
     }
     if (nan)
         flag_status(g.status, FPQ_ERR_NAN_INPUT);
@@ -234,14 +294,30 @@ const Form& best_form(int64_t M, int64_t N, int64_t K, double* us)
     return *best;
 }
 
+// Whether sums of a group of 64 are formed in four warps instead of one: where otherwise the error against 64 bits is above that of the
+// route that such a layer takes without this kernel (1 to 8 rows of 64 / 128 / 132 0.8 / 0.8 / 0.2 % above a warp per column, so 0.4 / 1.8 / 2 %
+// below it; 16 and 64 rows of 64 0.3 % above two kernels, so 1.3 % below), and not where it is below in any case and all warps are
+// busy anyway (127 x 128 -> 1280 3.2 us, so 3.6).  By the rows of the whole call: results do not depend on how it is cut.
+bool short_sums(int64_t whole, int64_t K) { return K <= KG || (whole <= 8 && K <= 4 * KG); }
+
+template <int WF, bool E5, bool SHORT>
+auto kernel_of(const Form& f)
+{
+    return f.R == 1 ? (f.NT == 2   ? few_rows_kernel<WF, E5, 1, 2, SHORT>
+                       : f.NT == 4 ? few_rows_kernel<WF, E5, 1, 4, SHORT>
+                                   : few_rows_kernel<WF, E5, 1, 8, SHORT>)
+                    : (f.NT == 2   ? few_rows_kernel<WF, E5, 2, 2, SHORT>
+                       : f.NT == 4 ? few_rows_kernel<WF, E5, 2, 4, SHORT>
+                                   : few_rows_kernel<WF, E5, 2, 8, SHORT>);
+}
+
 template <int WF, bool E5>
-cudaError_t launch(const FewArgs& g, cudaStream_t st)
+cudaError_t launch(const FewArgs& g, int64_t whole, cudaStream_t st)
 {
     double us;
     const Form& f = best_form(g.M, g.N, g.K, &us);
     const dim3 grid((unsigned)((g.N + 8 * f.NT - 1) / (8 * f.NT)), (unsigned)((g.M + 8 * f.R - 1) / (8 * f.R)));
-    const auto kernel = f.R == 1 ? (f.NT == 2 ? few_rows_kernel<WF, E5, 1, 2> : f.NT == 4 ? few_rows_kernel<WF, E5, 1, 4> : few_rows_kernel<WF, E5, 1, 8>)
-                                 : (f.NT == 2 ? few_rows_kernel<WF, E5, 2, 2> : f.NT == 4 ? few_rows_kernel<WF, E5, 2, 4> : few_rows_kernel<WF, E5, 2, 8>);
+    const auto kernel = short_sums(whole, g.K) ? kernel_of<WF, E5, true>(f) : kernel_of<WF, E5, false>(f);
     return launch_overlapped(kernel, grid, THREADS, 0, st, g);
 }
 
@@ -268,7 +344,7 @@ bool few_rows_preferred(const GemmProblem& p)
     return p.w_e5m2 || p.a_e5m2 || 1000.0 * us < small_m_linear_ns(p.M, p.C, p.N, p.w4);
 }
 
-fpq_status launch_few_rows(const GemmProblem& p, cudaStream_t st)
+fpq_status launch_few_rows(const GemmProblem& p, int64_t whole, cudaStream_t st)
 {
     if (!few_rows_applies(p))
         return FPQ_ERR_UNSUPPORTED;
@@ -281,9 +357,9 @@ fpq_status launch_few_rows(const GemmProblem& p, cudaStream_t st)
         return FPQ_ERR_CUDA;
     cudaError_t e;
     if (p.a_e5m2)
-        e = p.w4 ? launch<W_E2M1, true>(g, st) : p.w_e5m2 ? launch<W_E5M2, true>(g, st) : launch<W_E4M3, true>(g, st);
+        e = p.w4 ? launch<W_E2M1, true>(g, whole, st) : p.w_e5m2 ? launch<W_E5M2, true>(g, whole, st) : launch<W_E4M3, true>(g, whole, st);
     else
-        e = p.w4 ? launch<W_E2M1, false>(g, st) : p.w_e5m2 ? launch<W_E5M2, false>(g, st) : launch<W_E4M3, false>(g, st);
+        e = p.w4 ? launch<W_E2M1, false>(g, whole, st) : p.w_e5m2 ? launch<W_E5M2, false>(g, whole, st) : launch<W_E4M3, false>(g, whole, st);
     return e == cudaSuccess ? FPQ_OK : FPQ_ERR_CUDA;
 }
 

@@ -97,9 +97,9 @@ bool pair_gemm_preferred(const GemmProblem& p);   // in range, and faster than t
 fpq_status launch_pair_rows(const GemmProblem& p, int terms, cudaStream_t st);
 bool pair_rows_preferred(const GemmProblem& p, int terms);   // in range, and faster than the general contraction
 
-// Linear layer from FP32 rows (p.x) in one kernel with warp-level MMAs, for few rows.  FPQ_ERR_UNSUPPORTED when out of range
-// (nothing was enqueued).
-fpq_status launch_few_rows(const GemmProblem& p, cudaStream_t st);
+// Linear layer from FP32 rows (p.x) in one kernel with warp-level MMAs, for few rows; whole: the rows of the call that these are
+// part of, which the order of the sums depends on.  FPQ_ERR_UNSUPPORTED when out of range (nothing was enqueued).
+fpq_status launch_few_rows(const GemmProblem& p, int64_t whole, cudaStream_t st);
 bool few_rows_preferred(const GemmProblem& p);   // in range, and faster than the other routes
 
 // Linear layer with at most 8 rows on the CUDA cores (one pass over the weights).
