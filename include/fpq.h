@@ -152,9 +152,9 @@ fpq_status fpq_prepare_weight(const uint8_t* codes, fpq_format fmt, const fpq_la
  * x FP32 [M][K] row-major, y FP32 [M][N] row-major, both 16-byte aligned; bias
  * [N] or NULL.  The activations are quantized with (fx, x_scale) exactly as
  * fpq_quantize_act does; products are exact and accumulated in FP32 on the
- * tensor cores (layers of at most 8 rows with K a multiple of 4 run on the CUDA
- * cores instead: the same exact products, another order of the FP32 additions;
- * the workspace is then left untouched).  Supported operand pairs: fx = E4M3 bias 7 FPQ_SAT_NATIVE or
+ * tensor cores (layers of fewer than 128 rows with K a multiple of 4 may run as one
+ * kernel, and those of at most 8 rows on the CUDA cores, see fpq_linear_contraction: the
+ * same exact products, another order of the FP32 additions; the workspace is then left untouched).  Supported operand pairs: fx = E4M3 bias 7 FPQ_SAT_NATIVE or
  * fx = E5M2 bias 15 FPQ_SAT_NATIVE (the two 8-bit types the tensor cores read; Sec. V-A searches the
  * activation encodings too) with
  * fw = E4M3 bias 7 FPQ_SAT_NATIVE, fw = E5M2 bias 15 FPQ_SAT_NATIVE, fw = E2M1 bias 1, or any fw that fpq_prepare_weight
@@ -433,7 +433,8 @@ fpq_status fpq_round_learn_harden(const float* alpha, int64_t N, int64_t K, uint
  *                         linear layers of few rows keep the codes in registers, other linear layers
  *                         and stride-1 convolutions use the general fused form; other geometries fall
  *                         back to two kernels.
- *   FPQ_PATH_TWO_KERNELS  always *_quantize_input followed by *_contract.
+ *   FPQ_PATH_TWO_KERNELS  always *_quantize_input followed by *_contract (but for linear layers of up to 8 rows that
+ *                         are FPQ_CONTRACTION_CUDA_CORES, see below).
  *   FPQ_PATH_TWO_KERNELS_NARROW  the same, and the contraction never takes its CTA-pair form (M = 256
  *                         MMAs for long reductions with many tiles): for measurements and tests.
  *   FPQ_PATH_AUTO         the library's choice per shape (default): the CTA-pair kernel, or that of
@@ -458,12 +459,14 @@ int32_t fpq_conv2d_route(int B, int C, int H, int W, int C_out, int R, int S, in
                          fpq_format fx, fpq_format fw);
 
 /*
- * Which contraction kernel runs behind the activation-quantize kernel for this shape under the current policy (for
- * logs, benchmarks and tests; nothing is launched):
+ * Which contraction kernel runs behind the activation-quantize kernel, or in its place, for this shape under the current
+ * policy (for logs, benchmarks and tests; pointer alignment is assumed to be as documented and x and y to lie apart;
+ * nothing is launched):
  *   FPQ_CONTRACTION_GENERAL     128-row tiles, the reduction shared by a cluster where that pays;
  *   FPQ_CONTRACTION_PAIRS       256-row tiles on CTA pairs;
- *   FPQ_CONTRACTION_CUDA_CORES  a linear layer of a few rows as one kernel on the CUDA cores, no quantize kernel;
+ *   FPQ_CONTRACTION_CUDA_CORES  a linear layer of up to 8 rows as one kernel on the CUDA cores, no quantize kernel;
  *   FPQ_CONTRACTION_OTHER       the FP32 grid-value route;
+ *   FPQ_CONTRACTION_FEW_ROWS    a linear layer of fewer than 128 rows as one kernel with warp-level MMAs, no quantize kernel;
  *   negative                    FPQ_ERR_FORMAT or FPQ_ERR_SHAPE.
  * A convolution that takes FPQ_ROUTE_PAIR_FUSED or FPQ_ROUTE_FUSED runs neither kernel.
  */
@@ -471,7 +474,8 @@ enum {
     FPQ_CONTRACTION_GENERAL = 0,
     FPQ_CONTRACTION_PAIRS = 1,
     FPQ_CONTRACTION_CUDA_CORES = 2,
-    FPQ_CONTRACTION_OTHER = 3
+    FPQ_CONTRACTION_OTHER = 3,
+    FPQ_CONTRACTION_FEW_ROWS = 4
 };
 int32_t fpq_linear_contraction(int64_t M, int64_t N, int64_t K, fpq_format fx, fpq_format fw);
 int32_t fpq_conv2d_contraction(int B, int C, int H, int W, int C_out, int R, int S, int pad, int stride,

@@ -25,7 +25,7 @@ OK = 0
 ERR_NULL, ERR_FORMAT, ERR_SHAPE, ERR_ALIGN, ERR_UNSUPPORTED = -1, -2, -3, -4, -5
 ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_NAN_INPUT, ERR_TOO_LARGE, ERR_SCALE = -6, -7, -8, -9, -10, -11
 ROUTE_TWO_KERNELS, ROUTE_FUSED, ROUTE_PAIR_FUSED, ROUTE_OTHER = 0, 1, 2, 3
-CONTRACTION_GENERAL, CONTRACTION_PAIRS, CONTRACTION_CUDA_CORES, CONTRACTION_OTHER = 0, 1, 2, 3
+CONTRACTION_GENERAL, CONTRACTION_PAIRS, CONTRACTION_CUDA_CORES, CONTRACTION_OTHER, CONTRACTION_FEW_ROWS = 0, 1, 2, 3, 4
 STATIC_SCRATCH_BYTES = 8 << 20
 SAT_PAPER, SAT_NATIVE = 0, 1
 LINEAR, CONV2D = 0, 1

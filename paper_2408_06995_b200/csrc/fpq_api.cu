@@ -1468,8 +1468,11 @@ int32_t fpq_linear_contraction(int64_t M, int64_t N, int64_t K, fpq_format fx, f
         K = 2 * padded_c(K), fw = term;
     } else if (act_terms_pair(fx, fw, &terms)) {
         K = terms * padded_c(K), fx = classify_weight(fx).e5m2 ? kE5M2Native : kE4M3Native;
-    } else if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(M, K, N, is_e2m1(fw) ? 1 : 0)) {
-        return FPQ_CONTRACTION_CUDA_CORES;
+    } else {
+        if ((g_path_policy == FPQ_PATH_FUSED || g_path_policy == FPQ_PATH_AUTO) && few_rows_preferred(linear_problem(M, N, K, fx, fw)))
+            return FPQ_CONTRACTION_FEW_ROWS;
+        if (!is_e5m2_native(fw) && is_e4m3_native(fx) && small_m_linear_preferred(M, K, N, is_e2m1(fw) ? 1 : 0))
+            return FPQ_CONTRACTION_CUDA_CORES;
     }
     return pairs && pair_rows_preferred(linear_problem(M, N, K, fx, fw), 1) ? FPQ_CONTRACTION_PAIRS : FPQ_CONTRACTION_GENERAL;
 }

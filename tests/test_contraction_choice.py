@@ -5,8 +5,8 @@ import pytest
 import paper_2408_06995_b200 as fpq
 
 E4M3, E5M2, E2M1, E3M4, E2M5, E1M2 = fpq.E4M3, fpq.E5M2, fpq.E2M1, fpq.E3M4, fpq.E2M5, fpq.E1M2
-GENERAL, PAIRS, FEW_ROWS, OTHER = (fpq.CONTRACTION_GENERAL, fpq.CONTRACTION_PAIRS, fpq.CONTRACTION_CUDA_CORES,
-                                   fpq.CONTRACTION_OTHER)
+GENERAL, PAIRS, CUDA_CORES, OTHER, FEW_ROWS = (fpq.CONTRACTION_GENERAL, fpq.CONTRACTION_PAIRS, fpq.CONTRACTION_CUDA_CORES,
+                                               fpq.CONTRACTION_OTHER, fpq.CONTRACTION_FEW_ROWS)
 
 
 # test_gpu_pair_rows.py and test_gpu_ragged_columns.py
@@ -20,8 +20,11 @@ def test_linear_layers_on_pairs(fx, fw, M, K, N):
 
 
 @pytest.mark.parametrize("fx,fw,M,K,N,form", [
-    (E4M3, E2M1, 8192, 320, 960, GENERAL), (E4M3, E2M1, 64, 5120, 320, GENERAL), (E4M3, E3M4, 300, 640, 65, GENERAL),
-    (E4M3, E2M1, 2, 1280, 1280, FEW_ROWS), (E4M3, E2M1, 8, 5120, 10240, GENERAL), (E4M3, fpq.Format(6, 1, 31), 64, 64, 64, OTHER)])
+    (E4M3, E2M1, 8192, 320, 960, GENERAL), (E4M3, E2M1, 64, 5120, 320, FEW_ROWS), (E4M3, E3M4, 300, 640, 65, GENERAL),
+    (E4M3, E2M1, 2, 1280, 1280, FEW_ROWS), (E4M3, E2M1, 8, 5120, 10240, FEW_ROWS), (E4M3, fpq.Format(6, 1, 31), 64, 64, 64, OTHER),
+    (E5M2, E4M3, 64, 320, 320, FEW_ROWS), (E4M3, E1M2, 100, 640, 320, FEW_ROWS), (E4M3, E2M1, 127, 5120, 10240, GENERAL),
+    (E4M3, E4M3, 127, 320, 320, FEW_ROWS), (E4M3, E4M3, 128, 320, 320, GENERAL), (E4M3, E4M3, 64, 322, 320, GENERAL),
+    (E4M3, E4M3, 1, 96, 160, CUDA_CORES), (E4M3, E3M4, 8, 320, 320, GENERAL)])
 def test_other_linear_layers(fx, fw, M, K, N, form):
     assert fpq.fpq_linear_contraction(M, N, K, fx, fw) == form
 
@@ -36,6 +39,19 @@ def test_other_linear_layers(fx, fw, M, K, N, form):
 def test_convolutions_on_pairs(B, C, H, W, Co, stride):
     for fw in (E4M3, E2M1):
         assert fpq.fpq_conv2d_contraction(B, C, H, W, Co, 3, 3, 1, stride, E4M3, fw) == PAIRS
+
+
+# the kernels for few rows under each policy: one with warp-level MMAs where the route may be one kernel, the one on the CUDA cores always
+@pytest.mark.parametrize("M,K,N,alone,never", [(2, 1280, 1280, FEW_ROWS, CUDA_CORES), (64, 5120, 320, FEW_ROWS, GENERAL),
+                                               (8, 5120, 10240, FEW_ROWS, GENERAL), (1, 4, 1, CUDA_CORES, CUDA_CORES)])
+def test_few_rows_by_policy(M, K, N, alone, never):
+    try:
+        for policy, form in ((fpq.PATH_AUTO, alone), (fpq.PATH_FUSED, alone), (fpq.PATH_TWO_KERNELS, never),
+                             (fpq.PATH_TWO_KERNELS_NARROW, never)):
+            fpq.fpq_set_path_policy(policy)
+            assert fpq.fpq_linear_contraction(M, N, K, E4M3, E2M1) == form
+    finally:
+        fpq.fpq_set_path_policy(fpq.PATH_AUTO)
 
 
 def test_policies_and_errors():
