@@ -271,20 +271,32 @@ __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const
         flag_status(g.status, FPQ_ERR_NAN_INPUT);
 }
 
-// Rows and columns of a block.  us: a launch with its first round trip and one block per SM; more per 64 elements of a warp's
-// chain; and what every further block of an SM adds, and adds per 64 elements (measured; sums over 8 warps, so K / 512 steps).
+// Whether sums of a group of 64 are formed in four warps instead of one: where otherwise the error against 64 bits is above that of the
+// route that such a layer takes without this kernel (8 rows of 64 / 128 / 136 0.8 / 1.4 / 0.3 % above a warp per column, so 0.4 / 1.8 / 2 %
+// below it, and below it in any case from 144 on; 16 and 64 rows of 64 0.3 % above two kernels, so 1.3 % below), and nowhere else: where all
+// warps are busy anyway it takes longer (127 x 128 -> 1280 3.2 us, so 3.6; 8 x 256 -> 7680 2.1 and 2.8).  By the rows of the whole call:
+// results do not depend on how it is cut.
+bool short_sums(int64_t whole, int64_t K) { return K <= KG || (whole <= 8 && K < 2 * KG + 16); }
+
+// Rows and columns of a block.  us: a launch with its first round trip and one block per SM; more per 512 elements of the reduction;
+// and what every further block of an SM adds, and adds per 512 elements.  Fitted to the choices at 1896 shapes of 1 to 127 rows, 64 to
+// 5120 elements and 64 to 10240 columns with either size of weights: what is chosen takes 0.5 % more than the fastest of the forms and the two
+// kernels.  (Of 4700 others 8 take more than 1.1 times as long as without this kernel, at most 1.19; with whole steps of 512 and a
+// time of the two kernels that did not know the rows 48, at most 1.47: 24 x 1024 -> 10240 11.2 us, two kernels 7.9.)
 struct Form {
     int R, NT;
     double first, first_step, more, more_step;
 };
-constexpr Form FORMS[] = {{1, 2, 1.40, 0.41, 0.25, 0.38}, {1, 4, 1.55, 0.45, 0.20, 0.45}, {1, 8, 1.87, 0.58, 1.30, 0.58},
-                          {2, 2, 1.35, 0.72, 0.10, 0.64}, {2, 4, 1.50, 0.77, 0.30, 0.73}, {2, 8, 2.05, 0.90, 1.05, 0.90}};
-const Form& best_form(int64_t M, int64_t N, int64_t K, double* us)
+constexpr Form FORMS[] = {{1, 2, 1.39, 0.29, 0.29, 0.33}, {1, 4, 1.45, 0.34, 0.44, 0.54}, {1, 8, 1.82, 0.71, 1.28, 0.75},
+                          {2, 4, 1.77, 0.76, 0.47, 0.78}, {2, 8, 2.57, 0.87, 1.58, 1.03}};
+const Form& best_form(int64_t M, int64_t N, int64_t K, int64_t whole, double* us)
 {
     const Form* best = nullptr;
     for (const Form& f : FORMS) {
+        if (f.R == 2 && f.NT == 8 && short_sums(whole, K))
+            continue;                                  // (never the fastest; not built)
         const int64_t blocks = (N + 8 * f.NT - 1) / (8 * f.NT) * ((M + 8 * f.R - 1) / (8 * f.R));
-        const double steps = (double)((K + WARPS * KG - 1) / (WARPS * KG)), per_sm = (double)((blocks + 147) / 148);
+        const double steps = (double)K / (WARPS * KG), per_sm = (double)((blocks + 147) / 148);
         const double t = f.first + steps * f.first_step + (per_sm - 1.0) * (f.more + steps * f.more_step);
         if (!best || t < *us) {
             best = &f;
@@ -294,28 +306,21 @@ const Form& best_form(int64_t M, int64_t N, int64_t K, double* us)
     return *best;
 }
 
-// Whether sums of a group of 64 are formed in four warps instead of one: where otherwise the error against 64 bits is above that of the
-// route that such a layer takes without this kernel (1 to 8 rows of 64 / 128 / 132 0.8 / 0.8 / 0.2 % above a warp per column, so 0.4 / 1.8 / 2 %
-// below it; 16 and 64 rows of 64 0.3 % above two kernels, so 1.3 % below), and not where it is below in any case and all warps are
-// busy anyway (127 x 128 -> 1280 3.2 us, so 3.6).  By the rows of the whole call: results do not depend on how it is cut.
-bool short_sums(int64_t whole, int64_t K) { return K <= KG || (whole <= 8 && K <= 4 * KG); }
-
 template <int WF, bool E5, bool SHORT>
 auto kernel_of(const Form& f)
 {
     return f.R == 1 ? (f.NT == 2   ? few_rows_kernel<WF, E5, 1, 2, SHORT>
                        : f.NT == 4 ? few_rows_kernel<WF, E5, 1, 4, SHORT>
                                    : few_rows_kernel<WF, E5, 1, 8, SHORT>)
-                    : (f.NT == 2   ? few_rows_kernel<WF, E5, 2, 2, SHORT>
-                       : f.NT == 4 ? few_rows_kernel<WF, E5, 2, 4, SHORT>
-                                   : few_rows_kernel<WF, E5, 2, 8, SHORT>);
+           : SHORT || f.NT == 4 ? few_rows_kernel<WF, E5, 2, 4, SHORT>
+                                : few_rows_kernel<WF, E5, 2, 8, false>;
 }
 
 template <int WF, bool E5>
 cudaError_t launch(const FewArgs& g, int64_t whole, cudaStream_t st)
 {
     double us;
-    const Form& f = best_form(g.M, g.N, g.K, &us);
+    const Form& f = best_form(g.M, g.N, g.K, whole, &us);
     const dim3 grid((unsigned)((g.N + 8 * f.NT - 1) / (8 * f.NT)), (unsigned)((g.M + 8 * f.R - 1) / (8 * f.R)));
     const auto kernel = short_sums(whole, g.K) ? kernel_of<WF, E5, true>(f) : kernel_of<WF, E5, false>(f);
     return launch_overlapped(kernel, grid, THREADS, 0, st, g);
@@ -337,11 +342,11 @@ bool few_rows_preferred(const GemmProblem& p)
     if (!few_rows_applies(p))
         return false;
     double us;
-    best_form(p.M, p.N, p.C, &us);
-    if (1000.0 * us > two_kernels_ns(p.C, p.N))
+    best_form(p.M, p.N, p.C, p.M, &us);
+    if (1000.0 * us > two_kernels_ns(p.M, p.C, p.N))
         return false;
-    // (a single row of a short reduction: 96 -> 160 1.4 us there, 1.6 here)
-    return p.w_e5m2 || p.a_e5m2 || 1000.0 * us < small_m_linear_ns(p.M, p.C, p.N, p.w4);
+    // (0.88: the form on the CUDA cores is up to 15 % below its estimate at the smallest sizes; 1 x 64 -> 320 1.33 us there, 1.53 here)
+    return p.w_e5m2 || p.a_e5m2 || 1000.0 * us < 0.88 * small_m_linear_ns(p.M, p.C, p.N, p.w4);
 }
 
 fpq_status launch_few_rows(const GemmProblem& p, int64_t whole, cudaStream_t st)

@@ -105,7 +105,7 @@ bool few_rows_preferred(const GemmProblem& p);   // in range, and faster than th
 // Linear layer with at most 8 rows on the CUDA cores (one pass over the weights).
 bool small_m_linear_preferred(int64_t M, int64_t K, int64_t N, int w4);
 double small_m_linear_ns(int64_t M, int64_t K, int64_t N, int w4);   // its estimated time (1e30: out of range) ...
-double two_kernels_ns(int64_t K, int64_t N);                          // ... and that of a quantize kernel and a contraction of few rows
+double two_kernels_ns(int64_t M, int64_t K, int64_t N);               // ... and that of a quantize kernel and a contraction of few rows
 fpq_status launch_small_m_linear(const float* x, int M, int K, const void* w_prepared, int w4, int N, const float* w_scale,
                                  float x_scale, const float* bias, float* y, cudaStream_t st);
 

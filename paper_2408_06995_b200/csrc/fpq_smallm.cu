@@ -176,9 +176,16 @@ static bool in_range(int64_t M, int64_t K, int64_t N)
 
 double small_m_linear_ns(int64_t M, int64_t K, int64_t N, int w4) { return in_range(M, K, N) ? plan_small(M, K, N, w4).ns : 1e30; }
 
-double two_kernels_ns(int64_t K, int64_t N)
+double two_kernels_ns(int64_t M, int64_t K, int64_t N)
 {
-    return 4200.0 + 2.8 * (double)(K < 320 ? K : 320) + 0.3 * (double)(K > 320 ? K - 320 : 0) + 3.3e-4 * (double)N * (double)K + 0.05 * (double)N;
+    const double head = (double)(K < 320 ? K : 320), tail = (double)(K > 320 ? K - 320 : 0), weights = (double)N * (double)K;
+    const double few = 4200.0 + 2.8 * head + 0.3 * tail + 3.3e-4 * weights + 0.05 * (double)N;
+    if (M <= SMALLM_MAX_ROWS)
+        return few;
+    // (fitted to 9894 shapes of 9 to 127 rows and up to 13 us, 7 % rms; up to 24 rows large weights take longer: 9 x 5120 -> 10240 23.7 us,
+    // 32 x 5120 -> 10240 15.5; 24 x 1920 -> 5120 9.9, 32 x 1920 -> 5120 7.4)
+    const double more = 4350.0 + 2.44 * head + 0.385 * tail + 2.2e-4 * weights + 0.018 * (double)N + 3.6 * (double)M;
+    return M <= 24 && few > more ? few : more;
 }
 
 // Whether one pass on the CUDA cores is expected to be faster than the quantize kernel and the contraction, whose
@@ -187,7 +194,7 @@ double two_kernels_ns(int64_t K, int64_t N)
 // 8.2 / 9.8, 8 rows 37 / 9.8; 5120 -> 320, 4 rows 5.2 / 7.2, 8 rows 8.5 / 7.3).
 bool small_m_linear_preferred(int64_t M, int64_t K, int64_t N, int w4)
 {
-    return in_range(M, K, N) && plan_small(M, K, N, w4).ns <= two_kernels_ns(K, N);
+    return in_range(M, K, N) && plan_small(M, K, N, w4).ns <= two_kernels_ns(M, K, N);
 }
 
 template <bool W4, int MR, int KS>

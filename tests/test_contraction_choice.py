@@ -54,6 +54,15 @@ def test_few_rows_by_policy(M, K, N, alone, never):
         fpq.fpq_set_path_policy(fpq.PATH_AUTO)
 
 
+# what measured faster (us, one kernel / two: 11.2 / 7.9, 8.0 / 6.2, 10.0 / 7.9, 7.4 / 6.2; 2.9 / 5.0, 3.7 / 5.2, 16 / 23, 8.1 / 9.9, 3.6 / 6.6, 6.8 / 8.2)
+@pytest.mark.parametrize("M,K,N,form", [
+    (24, 1024, 10240, GENERAL), (48, 512, 7680, GENERAL), (20, 1024, 10240, GENERAL), (48, 1024, 3840, GENERAL), (48, 64, 5120, FEW_ROWS),
+    (120, 100, 1920, FEW_ROWS), (9, 5120, 10240, FEW_ROWS), (24, 1920, 5120, FEW_ROWS), (64, 1280, 640, FEW_ROWS), (112, 2560, 1280, FEW_ROWS)])
+def test_few_rows_or_two_kernels(M, K, N, form):
+    for fw in (E4M3, E2M1):
+        assert fpq.fpq_linear_contraction(M, N, K, E4M3, fw) == form
+
+
 def test_policies_and_errors():
     L = fpq.lib()
     try:
