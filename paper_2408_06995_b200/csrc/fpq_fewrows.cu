@@ -8,9 +8,9 @@
 // warps' sums are added up.  A 128-row tcgen05 tile would be mostly empty, and its operands would have to go through shared
 // memory first.  Products are exact and sums FP32, as on the other routes (error against 64 bits 3.5e-8 to 6e-8, theirs 3.5e-8 to 9e-8).
 // What bounds it: with one block per SM the chain of loads, converts and MMAs, some 0.4 to 0.9 us per 64 elements of a warp; with
-// several the conversions, which every block does for itself.  Whole layer, us here / two kernels, E2M1 weights: 16 x 320 -> 320 1.8 /
-// 5.3, 64 x 320 -> 1280 3.0 / 5.6, 32 x 1280 -> 1280 4.0 / 6.7; against a warp per column on the CUDA cores
-// (fpq_smallm.cu): 2 x 1280 -> 1280 2.4 / 3.8, 8 x 320 -> 1280 1.8 / 4.8, 8 x 1280 -> 1280 2.8 / 6.2.
+// several the conversions, which every block does for itself.  Whole layer, us here / two kernels, E2M1 weights: 16 x 320 -> 320 1.7 /
+// 5.3, 64 x 320 -> 1280 3.2 / 5.4, 8 x 1280 -> 1280 2.8 / 6.3, 32 x 1280 -> 1280 3.6 / 6.6; against a warp per column on the CUDA cores
+// (fpq_smallm.cu): 2 x 1280 -> 1280 2.4 / 3.8, 8 x 320 -> 1280 1.8 / 4.7.
 #include <cuda_fp16.h>
 
 #include "fpq_common.cuh"
@@ -263,8 +263,9 @@ __global__ void __launch_bounds__(THREADS, NT < 8 ? 2 : 1) few_rows_kernel(const
                 v[k] = t;
             }
         if (m0 + i < g.M && n < g.N) {
-            const float scale = g.x_scale * __ldg(g.w_scale + n);
-            g.y[(int64_t)(m0 + i) * g.N + n] = fmaf(v[0], scale, fmaf(lost, scale, g.bias ? __ldg(g.bias + n) : 0.f));
+            const float scale = g.x_scale * __ldg(g.w_scale + n), low = lost * scale;
+            // (nothing where that is not finite: with an infinite scale the result is infinite, not 0 * infinity)
+            g.y[(int64_t)(m0 + i) * g.N + n] = fmaf(v[0], scale, (g.bias ? __ldg(g.bias + n) : 0.f) + (fabsf(low) < INFINITY ? low : 0.f));
         }
     }
     if (nan)

@@ -188,7 +188,8 @@ double two_kernels_ns(int64_t M, int64_t K, int64_t N)
     return M <= 24 && few > more ? few : more;
 }
 
-// Whether one pass on the CUDA cores is expected to be faster than the quantize kernel and the contraction, whose
+// Whether one pass on the CUDA cores is expected to be faster than the quantize kernel and the contraction (where the route may be one
+// kernel, few_rows_preferred is asked first and leaves this one layers of few columns and single rows of short reductions), whose
 // time in chains of its kind is fitted by two_kernels_ns (us, here / there: 1280 -> 1280, 4-bit weights, 2 rows 3.9 / 6.3,
 // 8 rows 9.4 / 6.5; 1280 -> 10240, one row 11.7 / 8.9; 5120 -> 10240, 8 rows 156 / 23; 8-bit weights: 1280 -> 10240, one row
 // 8.2 / 9.8, 8 rows 37 / 9.8; 5120 -> 320, 4 rows 5.2 / 7.2, 8 rows 8.5 / 7.3).

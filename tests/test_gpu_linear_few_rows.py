@@ -25,12 +25,14 @@ def _layer(M, K, N, fw, seed, fx="e4m3", bias=True):
     return x, w, ws, xs, b
 
 
-def _run(x, w, ws, xs, b, fx, fw, policy=fpq.PATH_AUTO):
+def _run(x, w, ws, xs, b, fx, fw, policy=fpq.PATH_AUTO, out_scale=None):
     M, K = x.shape
     N = w.shape[0]
     gfx, gfw = FORMATS[fx][0], FORMATS[fw][0]
     sc = torch.from_numpy(ws).cuda()
     prep = fpq.fpq_prepare_weight(fpq.fpq_quantize_weight(torch.from_numpy(w).cuda(), sc, gfw), gfw, fpq.LINEAR, N, K)
+    if out_scale is not None:
+        sc = torch.from_numpy(out_scale).cuda()
     y = torch.full((M + 2, N), float("nan"), device="cuda")
     ws_ = torch.empty(max(256, fpq.fpq_linear_workspace_size(M, N, K, gfx, gfw)), dtype=torch.uint8, device="cuda")
     try:
@@ -99,6 +101,21 @@ def test_smallest_and_plain_sizes(M, K, N, fx, fw):
     # (either of the kernels for few rows: at most K / 32 + 5 FP32 roundings on the CUDA cores, see above for the other)
     n = max(4 + (K / 512 + 4) / 2, (K / 32 + 5) / 2)
     assert np.all(np.abs(y - want) <= n * 2.0 ** -23 * terms + 2 * np.spacing(np.abs(want).astype(np.float32)) + 2.0 ** -23 * np.abs(want))
+
+
+@pytest.mark.parametrize("M,K,N", [(9, 1280, 40), (20, 1900, 351), (33, 60, 1432), (33, 1392, 2946)])
+@pytest.mark.parametrize("fx,fw", [("e4m3", "e4m3"), ("e5m2", "e5m2")])
+def test_scales_that_overflow(M, K, N, fx, fw):
+    x, w, ws, xs, b = _layer(M, K, N, fw, 6, fx)
+    out = ws.copy()
+    out[[0, 7, 11, 14, N - 1]] = [np.inf, 3e38, -np.inf, 3e38 / 64, np.nan]
+    x, xs = x * np.float32(1024), xs * 1024              # (the product of the scales overflows, or the result does)
+    assert fpq.fpq_linear_contraction(M, N, K, FORMATS[fx][0], FORMATS[fw][0]) == fpq.CONTRACTION_FEW_ROWS
+    y, two = (_run(x, w, ws, xs, b, fx, fw, policy, out) for policy in (fpq.PATH_AUTO, fpq.PATH_TWO_KERNELS))
+    assert np.isinf(y).any()
+    for n in (0, 7, 11, 14, N - 1):
+        assert np.array_equal(np.where(np.isfinite(y[:, n]), 0.0, y[:, n]), np.where(np.isfinite(two[:, n]), 0.0, two[:, n]), equal_nan=True)
+    fpq.fpq_read_status()
 
 
 # a NaN in either group of eight rows of a block, in the last row and the last column, in sums of one warp and of four
