@@ -121,6 +121,11 @@ def gpu_layer(L, ws, xs, use_bias=True, route="auto"):
     return {"auto": y0, "fused": y1, "two": y2}[route]
 
 
+def routes(L):
+    """The routes whose results have to be held to the oracle: where few rows may take a kernel of their own, the two kernels too."""
+    return ("auto", "two") if L.kind == "linear" and L.M < 128 else ("auto",)
+
+
 def oracle_layer(L, ws, xs, idx=None, use_bias=True):
     _, ofw = FMT[L.wfmt]
     rb = O.pack_bits(L.bits) if L.bits is not None else None

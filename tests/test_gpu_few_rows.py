@@ -1,12 +1,13 @@
-"""Linear layers of a few rows: one pass over the weights with a column per warp or shared by two or four, ragged numbers of
-columns and of reduction steps, and the sizes beside the line where the tensor cores take over; against the CPU oracle."""
+"""Linear layers of a few rows, by default and on the routes without the kernel that takes most of them: one pass over the weights with
+a column per warp or shared by two or four, ragged numbers of columns and of reduction steps, and the sizes beside the line
+where the tensor cores take over; against the CPU oracle."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2408_06995_b200 as fpq
 from paper_2408_06995_b200 import inputs as I
-from _helpers import assert_close, gpu_layer, layer_scales, oracle_layer
+from _helpers import assert_close, gpu_layer, layer_scales, oracle_layer, routes
 
 pytestmark = pytest.mark.gpu
 
@@ -18,9 +19,9 @@ pytestmark = pytest.mark.gpu
 def test_few_rows(M, K, N, wfmt):
     L = I.draw(I.linear_layer("few", M, K, N, wfmt), 31, M, "silu", 0.02, True)
     ws, xs = layer_scales(L)
-    y = gpu_layer(L, ws, xs)
     yo, ab = oracle_layer(L, ws, xs)
-    assert_close(y, yo, ab)
+    for route in routes(L):
+        assert_close(gpu_layer(L, ws, xs, route=route), yo, ab)
 
 
 def test_nan_in_a_row_is_reported():
@@ -42,6 +43,6 @@ def test_nan_in_a_row_is_reported():
 def test_shared_tiles(M, K, N, wfmt):
     L = I.draw(I.linear_layer("shared", M, K, N, wfmt), 32, M, "silu", 0.02, True)
     ws, xs = layer_scales(L)
-    y = gpu_layer(L, ws, xs)
     yo, ab = oracle_layer(L, ws, xs)
-    assert_close(y, yo, ab)
+    for route in routes(L):
+        assert_close(gpu_layer(L, ws, xs, route=route), yo, ab)

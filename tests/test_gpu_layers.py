@@ -10,17 +10,19 @@ import torch
 import oracle as O
 import paper_2408_06995_b200 as fpq
 from paper_2408_06995_b200 import inputs as I
-from _helpers import FMT, Guarded, assert_close, gpu_layer, gpu_prepare, layer_scales, oracle_layer, sample_indices
+from _helpers import FMT, Guarded, assert_close, gpu_layer, gpu_prepare, layer_scales, oracle_layer, routes, sample_indices
 
 pytestmark = pytest.mark.gpu
 
 
 def _check_full(L, use_bias=True):
     ws, xs = layer_scales(L)
-    y = gpu_layer(L, ws, xs, use_bias)
     yr, ab = oracle_layer(L, ws, xs, None, use_bias)
-    assert y.shape == yr.shape
-    return assert_close(y, yr, ab)
+    for route in routes(L):
+        y = gpu_layer(L, ws, xs, use_bias, route)
+        assert y.shape == yr.shape
+        worst = assert_close(y, yr, ab)
+    return worst
 
 
 def _tile_edges(L):

@@ -5,7 +5,7 @@ import torch
 
 import paper_2408_06995_b200 as fpq
 from paper_2408_06995_b200 import inputs as I
-from _helpers import assert_close, gpu_layer, layer_scales, oracle_layer, sample_indices
+from _helpers import assert_close, gpu_layer, layer_scales, oracle_layer, routes, sample_indices
 
 pytestmark = pytest.mark.gpu
 
@@ -17,10 +17,10 @@ pytestmark = pytest.mark.gpu
 def test_ragged_columns(M, K, N, wfmt):
     L = I.draw(I.linear_layer("ragged", M, K, N, wfmt), 33, M, "silu", 0.02, True)
     ws, xs = layer_scales(L)
-    y = gpu_layer(L, ws, xs).reshape(-1)
-    idx = sample_indices(y.size, min(y.size, 200000), 7)
+    idx = sample_indices(M * N, min(M * N, 200000), 7)
     yo, ab = oracle_layer(L, ws, xs, idx)
-    assert_close(y[idx], yo, ab)
+    for route in routes(L):
+        assert_close(gpu_layer(L, ws, xs, route=route).reshape(-1)[idx], yo, ab)
 
 
 @pytest.mark.parametrize("M,K,N", [(2048, 2560, 638), (300, 640, 65), (1111, 1300, 1283), (700, 640, 65)])

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2408_06995_b200 import inputs as I
-from _helpers import layer_scales, gpu_layer, oracle_layer, assert_close, sample_indices
+from _helpers import layer_scales, gpu_layer, oracle_layer, assert_close, routes, sample_indices
 
 pytestmark = pytest.mark.gpu
 
@@ -40,8 +40,9 @@ def test_random_layers_match_the_oracle(seed):
         L = _random_layer(rng, j)
         I.draw(L, 80 + seed, 10 * j, ["normal", "silu", "t4"][j % 3], 0.03, True)
         ws, xs = layer_scales(L)
-        y = gpu_layer(L, ws, xs)                        # both routes, asserted equal
-        idx = sample_indices(y.size, min(y.size, 400), j, [0, y.size - 1])
-        yr, ab = oracle_layer(L, ws, xs, idx)
-        assert np.all(np.isfinite(y)), (seed, j, L.name)
-        assert_close(y.reshape(-1)[idx], yr, ab)
+        for route in routes(L):
+            y = gpu_layer(L, ws, xs, route=route)           # both routes, asserted equal
+            idx = sample_indices(y.size, min(y.size, 400), j, [0, y.size - 1])
+            yr, ab = oracle_layer(L, ws, xs, idx)
+            assert np.all(np.isfinite(y)), (seed, j, L.name)
+            assert_close(y.reshape(-1)[idx], yr, ab)
