@@ -198,8 +198,8 @@ fpq_status fpq_conv2d(const float* x, const void* w_prepared, const float* w_sca
                       size_t ws_bytes, void* stream);
 
 /*
- * The two stages of fpq_linear / fpq_conv2d as separate calls (the layer call
- * is exactly stage 1 followed by stage 2 on the same stream):
+ * The two stages of fpq_linear / fpq_conv2d as separate calls (a layer call that runs
+ * as two kernels is exactly stage 1 followed by stage 2 on the same stream):
  *   stage 1, *_quantize_input: activation quantize (Sec. IV-B rounding equation,
  *            static per-tensor scale) written to `workspace` in the operand
  *            layout of the contraction (linear: [M][K rounded up to 16] codes;
