@@ -338,6 +338,7 @@ def test_two_kernel_route_matches_the_oracle_and_the_fused_call(wfmt):
     ("conv", (5, 130, 32, 32, 140, 1)),       # 5 images in 5 slices
     ("linear", (4096, 320, 320)),             # sliced by rows
     ("linear", (3000, 640, 200)),             # 3000 rows in 8 unequal slices
+    ("linear", (900, 320, 2048)),             # slices of fewer rows than the kernel for few rows takes
     ("linear", (4096, 130, 322)),             # rows are not 16-byte multiples: one slice
 ])
 def test_host_forms_equal_the_device_forms(kind, shape):
